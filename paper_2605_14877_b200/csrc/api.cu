@@ -22,9 +22,8 @@ struct TcState;
 int tc_create(const heatkv_config& cfg, void* k_pool, void* v_pool, uint64_t pool_rows, TcState** out);
 void tc_destroy(TcState* st);
 bool tc_ready(const TcState* st);
-bool tc_supported(const TcState* st, const AttnParams& p, int d, int n_seq, bool calib);
-cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int d, int n_seq, bool calib, cudaStream_t stream,
-                           int* launches);
+bool tc_supported(const TcState* st, const AttnParams& p, int d, int n_seq);
+cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int n_seq, cudaStream_t stream);
 int tc_split_slot_floats(int d);
 cudaError_t launch_wait_expiry(uint32_t* status, uint32_t* result, cudaStream_t stream);
 struct CalibTcState;
@@ -33,6 +32,7 @@ int calib_tc_create(const heatkv_config& cfg, void* dev_table, cudaStream_t stre
 void calib_tc_destroy(CalibTcState* st);
 bool calib_tc_ready(const CalibTcState* st);
 bool calib_tc_supported(const CalibTcState* st, const AttnParams& p, int d, int n_seq);
+void calib_tc_step_descs(const CalibTcState* st, int step, const int2** descs, int* n_slots);
 cudaError_t launch_calib_tc(CalibTcState* st, const AttnParams& p, int n_seq, cudaStream_t stream);
 cudaError_t launch_calib_tc_steps(CalibTcState* st, const AttnParams& p, int n_seq, const int* steps, const int* t_q,
                                   const int* q_tok0, int n_steps, int q_tokens, int k_tokens, int64_t bias_step_stride,
@@ -659,7 +659,7 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
   p.layer = layer;
   const bool stores = step + 1 < ctx->cfg.K;                  // the last scale is never cached
   const int choice = ctx->cfg.kernel;
-  bool use_tc = choice != HEATKV_KERNEL_GENERIC && tc_supported(ctx->tc, p, ctx->cfg.d, n_seq, false);
+  bool use_tc = choice != HEATKV_KERNEL_GENERIC && tc_supported(ctx->tc, p, ctx->cfg.d, n_seq);
   // AUTO: steps of 256 queries and more, and steps of 128 and more once the call holds 64 (sequence, head) units:
   // from there on the warp-level kernel is bound by its mma.sync rate (144 queries, 128 units: 52 us against 23 us)
   if (choice == HEATKV_KERNEL_AUTO && !(p.t_q >= 256 || (p.t_q >= 128 && (int64_t)n_seq * ctx->cfg.H >= 64))) use_tc = false;
@@ -719,15 +719,14 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
   if (fuse) p.append_tiles = (ctx->cfg.t[step] + HEATKV_PAGE_TOKENS - 1) / HEATKV_PAGE_TOKENS + 1;
   cudaError_t e;
   if (use_tc) {
-    int n = 0;
     try {
       choose_split(ctx, seq_ids, n_seq, step, layer, &p);
     } catch (const std::bad_alloc&) {
       return HEATKV_ERR_HOST_MEMORY;
     }
-    e = launch_attn_tc(ctx->tc, p, ctx->cfg.d, n_seq, false, stream, &n);
-    ctx->launches += n;
-    ctx->kstats.attention_tcgen05 += n;
+    e = launch_attn_tc(ctx->tc, p, n_seq, stream);
+    ctx->launches += 1;
+    ctx->kstats.attention_tcgen05 += 1;
   } else {
     fill_head_table(ctx, seq_ids, n_seq, step, layer, &p);
     e = launch_attn_generic(p, ctx->cfg.d, n_seq, false, stream);
@@ -806,12 +805,23 @@ int heatkv_calibrate_scores(heatkv_ctx* ctx, int layer, int step, int n_seq, con
   p.step = step;
   p.layer = layer;
   p.beta_row = beta_accum + (((int64_t)layer * ctx->cfg.H) * ctx->cfg.K + step) * ctx->cfg.K;
-  // without an attention output the pass is S = Q K^T plus bookkeeping: the tensor-memory kernel takes it
+  // Steps of 256 queries and more run on tensor memory: without an output the pass is S = Q K^T plus bookkeeping (the
+  // calibration kernel), with one it is the attention kernel with that bookkeeping beside its softmax (13 scales, 16 heads,
+  // 2 sequences: 1.24 ms a pass against 6.05 ms on the warp-level kernel).
   const int choice = ctx->cfg.kernel;
-  bool use_tc = !out && choice != HEATKV_KERNEL_GENERIC && calib_tc_supported(ctx->calib_tc, p, ctx->cfg.d, n_seq);
+  const int64_t items = (int64_t)ctx->cfg.H * ((p.t_q + 255) / 256);
+  bool use_tc = choice != HEATKV_KERNEL_GENERIC && calib_tc_supported(ctx->calib_tc, p, ctx->cfg.d, n_seq) &&
+                (!out || (tc_supported(ctx->tc, p, ctx->cfg.d, n_seq) && items * n_seq <= INT32_MAX));
   if (choice == HEATKV_KERNEL_AUTO && p.t_q < 256) use_tc = false;
-  cudaError_t e = use_tc ? launch_calib_tc(ctx->calib_tc, p, n_seq, stream)
-                         : launch_attn_generic(p, ctx->cfg.d, n_seq, true, stream);
+  cudaError_t e;
+  if (use_tc && out) {
+    calib_tc_step_descs(ctx->calib_tc, step, &p.full_descs, &p.full_slots);
+    p.n_seq = n_seq;
+    p.items_per_seq = (int)items;
+    e = launch_attn_tc(ctx->tc, p, n_seq, stream);
+  } else {
+    e = use_tc ? launch_calib_tc(ctx->calib_tc, p, n_seq, stream) : launch_attn_generic(p, ctx->cfg.d, n_seq, true, stream);
+  }
   ctx->launches += 1;
   (use_tc ? ctx->kstats.calibration_tcgen05 : ctx->kstats.calibration_generic) += 1;
   return e == cudaSuccess ? HEATKV_OK : HEATKV_ERR_CUDA;

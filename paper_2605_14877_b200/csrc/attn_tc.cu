@@ -101,6 +101,9 @@ struct Slot {
   int seg;
 };
 
+// FULL (calibration with an attention output): every key comes from the caller's tensor, and the descriptors, cut at
+// source-scale borders, number its rows.
+template <bool FULL>
 __device__ __forceinline__ Slot get_slot(int i, const int2* descs, int n_desc, int n_slots, int64_t base_row,
                                          int t_own, int step) {
   Slot s;
@@ -108,7 +111,7 @@ __device__ __forceinline__ Slot get_slot(int i, const int2* descs, int n_desc, i
   if (!valid) i = n_slots - 1;                      // padding half-tile: re-read finite data, mask everything
   if (i < n_desc) {
     int2 d = descs[i];
-    s.pool_row = (int)(base_row + d.x);
+    s.pool_row = FULL ? -(d.x + 1) : (int)(base_row + d.x);
     s.n_valid = d.y & 0xff;
     s.seg = (d.y >> 8) & 0xff;
   } else {
@@ -125,6 +128,7 @@ __device__ __forceinline__ Slot get_slot(int i, const int2* descs, int n_desc, i
 struct Item {
   int head, seq, n_split, sub, piece, qp, q0, nq, j0, n_tiles, slot_base, ctr_base, n_desc, n_slots, desc_begin;
 };
+template <bool FULL>
 __device__ __forceinline__ Item read_item(const volatile int32_t* ring, const AttnParams& p, int n_qp) {
   Item it;
   it.head = ring[W_HEAD];
@@ -140,7 +144,7 @@ __device__ __forceinline__ Item read_item(const volatile int32_t* ring, const At
   it.qp = it.sub % n_qp;
   it.q0 = it.qp * (2 * BM);
   it.nq = (it.q0 + BM < p.t_q) ? 2 : 1;             // does tile B hold any query?
-  it.n_slots = it.n_desc + (p.n_own + HALF - 1) / HALF;
+  it.n_slots = FULL ? it.n_desc : it.n_desc + (p.n_own + HALF - 1) / HALF;
   // this item's run of key tiles: [j0, j0 + n_tiles) of the head's ceil(n_slots / 2)
   const int piece_tiles = (tiles + it.n_split - 1) / it.n_split;
   it.j0 = it.piece * piece_tiles;
@@ -148,7 +152,10 @@ __device__ __forceinline__ Item read_item(const volatile int32_t* ring, const At
   return it;
 }
 
-template <int D>
+// FULL: heatkv_calibrate_scores with an attention output.  The softmax warps also keep, for every query row, the
+// probability mass of each source scale (a half-tile lies inside one scale; finished scales are parked in the warp's
+// output staging buffer) and add the step's row of beta (Eq. 2) at the end of the item.
+template <int D, bool FULL>
 __global__ void __launch_bounds__(THREADS, 1)
 attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Maps maps) {
   using L = Layout<D>;
@@ -245,68 +252,81 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
       // heads finds the item.
       const int seq = idx % p.n_seq;
       const int item = idx / p.n_seq;
-      PlanView pv(p.seqs[seq].plan);
-      if (lane == 0) ring[W_KIND] = NOTHING;            // sequences of a call may differ in item count
-      __syncwarp();
-      int before = 0, slots_before = 0, ctrs_before = 0;
-      for (int base = 0; base < p.H; base += 32) {
-        const int i = base + lane;
-        int h = 0, tiles = 0, ns = 0, cnt = 0;
-        if (i < p.H) {
-          if (p.table_heads > 0) {                            // the host put the per-head table into the launch parameters
-            h = p.table_head[i];
-            tiles = p.table_tiles[i];
-            ns = p.table_split[i];
-          } else {
-            h = pv.order()[u + i];
-            tiles = (pv.attn_cnt()[u + h] + own_slots + 1) >> 1;
-            ns = p.split_tiles > 0 ? (tiles + p.split_tiles - 1) / p.split_tiles : 1;
-          }
-          cnt = n_qp * ns;
-        }
-        const int scnt = ns > 1 ? cnt : 0, ccnt = ns > 1 ? n_qp : 0;
-        int inc = cnt, sinc = scnt, cinc = ccnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int v0 = __shfl_up_sync(0xffffffffu, inc, o), v1 = __shfl_up_sync(0xffffffffu, sinc, o),
-                    v2 = __shfl_up_sync(0xffffffffu, cinc, o);
-          if (lane >= o) { inc += v0; sinc += v1; cinc += v2; }
-        }
-        const int excl = before + inc - cnt;
-        const bool mine = cnt > 0 && item >= excl && item < excl + cnt;
-        if (mine) {
-          ring[W_HEAD] = h;
+      if (lane == 0) {
+        ring[W_KIND] = FULL ? ATTENTION : NOTHING;      // sequences of a call may differ in item count
+        if (FULL) {                                     // all heads alike: query tile pair fastest
+          ring[W_HEAD] = item / n_qp;
           ring[W_SEQ] = seq;
-          ring[W_TILES] = tiles;
-          ring[W_NSPLIT] = ns;
-          ring[W_SUB] = item - excl;                        // piece * n_qp + query tile pair
-          ring[W_SLOT] = slots_before + sinc - scnt;        // first partial slot of this head
-          ring[W_CTR] = ctrs_before + cinc - ccnt;          // first arrival counter group of this head
-          ring[W_DESC] = pv.attn_begin()[u + h];
-          ring[W_NDESC] = pv.attn_cnt()[u + h];
-          ring[W_KIND] = ATTENTION;
+          ring[W_TILES] = (p.full_slots + 1) >> 1;
+          ring[W_NSPLIT] = 1;
+          ring[W_SUB] = item % n_qp;
+          ring[W_SLOT] = ring[W_CTR] = ring[W_DESC] = 0;
+          ring[W_NDESC] = p.full_slots;
         }
-        const bool any = __any_sync(0xffffffffu, mine);
-        before += __shfl_sync(0xffffffffu, inc, 31);
-        slots_before += __shfl_sync(0xffffffffu, sinc, 31);
-        ctrs_before += __shfl_sync(0xffffffffu, cinc, 31);
-        if (any) break;
       }
       __syncwarp();
+      if (!FULL) {
+        PlanView pv(p.seqs[seq].plan);
+        int before = 0, slots_before = 0, ctrs_before = 0;
+        for (int base = 0; base < p.H; base += 32) {
+          const int i = base + lane;
+          int h = 0, tiles = 0, ns = 0, cnt = 0;
+          if (i < p.H) {
+            if (p.table_heads > 0) {                            // the host put the per-head table into the launch parameters
+              h = p.table_head[i];
+              tiles = p.table_tiles[i];
+              ns = p.table_split[i];
+            } else {
+              h = pv.order()[u + i];
+              tiles = (pv.attn_cnt()[u + h] + own_slots + 1) >> 1;
+              ns = p.split_tiles > 0 ? (tiles + p.split_tiles - 1) / p.split_tiles : 1;
+            }
+            cnt = n_qp * ns;
+          }
+          const int scnt = ns > 1 ? cnt : 0, ccnt = ns > 1 ? n_qp : 0;
+          int inc = cnt, sinc = scnt, cinc = ccnt;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const int v0 = __shfl_up_sync(0xffffffffu, inc, o), v1 = __shfl_up_sync(0xffffffffu, sinc, o),
+                      v2 = __shfl_up_sync(0xffffffffu, cinc, o);
+            if (lane >= o) { inc += v0; sinc += v1; cinc += v2; }
+          }
+          const int excl = before + inc - cnt;
+          const bool mine = cnt > 0 && item >= excl && item < excl + cnt;
+          if (mine) {
+            ring[W_HEAD] = h;
+            ring[W_SEQ] = seq;
+            ring[W_TILES] = tiles;
+            ring[W_NSPLIT] = ns;
+            ring[W_SUB] = item - excl;                        // piece * n_qp + query tile pair
+            ring[W_SLOT] = slots_before + sinc - scnt;        // first partial slot of this head
+            ring[W_CTR] = ctrs_before + cinc - ccnt;          // first arrival counter group of this head
+            ring[W_DESC] = pv.attn_begin()[u + h];
+            ring[W_NDESC] = pv.attn_cnt()[u + h];
+            ring[W_KIND] = ATTENTION;
+          }
+          const bool any = __any_sync(0xffffffffu, mine);
+          before += __shfl_sync(0xffffffffu, inc, 31);
+          slots_before += __shfl_sync(0xffffffffu, sinc, 31);
+          ctrs_before += __shfl_sync(0xffffffffu, cinc, 31);
+          if (any) break;
+        }
+        __syncwarp();
+      }
       const bool is_attn = ring[W_KIND] == ATTENTION;
       Item im;
-      if (is_attn) im = read_item(ring, p, n_qp);
+      if (is_attn) im = read_item<FULL>(ring, p, n_qp);
       __syncwarp();
       if (leader) mbar_arrive(bar(ITEM_FULL + slot));
       if (!is_attn) continue;
-      const int2* descs = pv.descs() + im.desc_begin;
-      const int64_t base_row = p.seqs[seq].base_row;
+      const int2* descs = FULL ? p.full_descs : PlanView(p.seqs[seq].plan).descs() + im.desc_begin;
+      const int64_t base_row = FULL ? 0 : p.seqs[seq].base_row;
       for (int j = 0; j < im.n_tiles && ok; ++j, ++g) {
         const uint32_t st = g % KV_STAGES;
         const uint32_t use = g / KV_STAGES;
         Slot sl[2];
         for (int hf = 0; hf < 2; ++hf)
-          sl[hf] = get_slot(2 * (im.j0 + j) + hf, descs, im.n_desc, im.n_slots, base_row, p.n_own, p.step);
+          sl[hf] = get_slot<FULL>(2 * (im.j0 + j) + hf, descs, im.n_desc, im.n_slots, base_row, p.n_own, p.step);
         // K first: the S product of the next tile needs it earliest
         if (use > 0) ok = warp_wait(bar(K_EMPTY + st), (use - 1) & 1, abort_flag, p.status);
         if (!ok) break;
@@ -402,7 +422,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
       const int kind = ring[W_KIND];
       if (kind == STOP) break;
       if (kind == ATTENTION) {
-        const Item im = read_item(ring, p, n_qp);
+        const Item im = read_item<FULL>(ring, p, n_qp);
         const int nq = im.nq, n_tiles = im.n_tiles;
         const uint32_t st0 = g % KV_STAGES, par0 = (g / KV_STAGES) & 1;
 #pragma unroll
@@ -521,7 +541,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
         // Only what the tile loop needs stays in registers; the epilogue reads the ring entry again.
         int n_tiles, nq;
         {
-          const Item im = read_item(ring, p, n_qp);
+          const Item im = read_item<FULL>(ring, p, n_qp);
           n_tiles = im.n_tiles;
           nq = im.nq;
         }
@@ -530,16 +550,21 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
           const int2* descs;
           const float* bias_h;
           {
-            const Item im = read_item(ring, p, n_qp);
+            const Item im = read_item<FULL>(ring, p, n_qp);
             j0 = im.j0; n_desc = im.n_desc; n_slots = im.n_slots;
-            descs = PlanView(p.seqs[im.seq].plan).descs() + im.desc_begin;
+            descs = FULL ? p.full_descs : PlanView(p.seqs[im.seq].plan).descs() + im.desc_begin;
             bias_h = p.seg_bias ? p.seg_bias + im.head * p.K : nullptr;
           }
           float m_ref = -INFINITY, l_sum = 0.f;
+          // FULL: the scale whose mass is being collected (warp-uniform; scales arrive in ascending order, each as one
+          // run of half-tiles, and every scale up to the step has some) and the masses of the finished ones
+          int cur_seg = 0;
+          float cur_mass = 0.f;
+          float* masses = reinterpret_cast<float*>(stage) + lane;      // [scale][32 rows]
           for (int j = 0; j < n_tiles && ok; ++j) {
             const uint32_t ph = (cx + j) & 1;
-            Slot s0 = get_slot(2 * (j0 + j), descs, n_desc, n_slots, 0, p.n_own, p.step);       // row numbers unused here
-            Slot s1 = get_slot(2 * (j0 + j) + 1, descs, n_desc, n_slots, 0, p.n_own, p.step);
+            Slot s0 = get_slot<FULL>(2 * (j0 + j), descs, n_desc, n_slots, 0, p.n_own, p.step);       // row numbers unused here
+            Slot s1 = get_slot<FULL>(2 * (j0 + j) + 1, descs, n_desc, n_slots, 0, p.n_own, p.step);
             const float b0 = bias_h ? bias_h[s0.seg] * LOG2E : 0.f;
             const float b1 = bias_h ? bias_h[s1.seg] * LOG2E : 0.f;
             ok = __all_sync(0xffffffffu, mbar_wait(bar(S_FULL + x), ph, abort_flag, p.status));
@@ -598,6 +623,10 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
               }
               tmem_wait_st();
               l_sum *= f;
+              if (FULL) {
+                cur_mass *= f;
+                for (int s = 0; s < cur_seg; ++s) masses[s * 32] *= f;
+              }
             }
             if (grow) m_ref = m_new;
             // p = exp2(logit - m_ref); row sum in fp32; P as bf16 pairs into the columns S occupied
@@ -632,6 +661,19 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             tmem_wait_st();
             tc_fence_before();
             mbar_arrive(bar(P_FULL + 2 * x));                      // the PV product of keys 0..63 may start
+            if (FULL) {
+              float sa, sb;
+              unpack2(sum2, sa, sb);
+              const float half = sa + sb;
+              l_sum += half;
+              sum2 = pack2(0.f, 0.f);
+              if (s0.seg != cur_seg) {
+                masses[cur_seg * 32] = cur_mass;
+                cur_seg = s0.seg;
+                cur_mass = 0.f;
+              }
+              cur_mass += half;
+            }
             exp_chunk(r2, bb1, 2);
             exp_chunk(r3, bb1, 3);
             float sa, sb;
@@ -640,13 +682,34 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             tmem_wait_st();
             tc_fence_before();
             mbar_arrive(bar(P_FULL + 2 * x + 1));
+            if (FULL && s1.n_valid > 0) {
+              if (s1.seg != cur_seg) {
+                masses[cur_seg * 32] = cur_mass;
+                cur_seg = s1.seg;
+                cur_mass = 0.f;
+              }
+              cur_mass += sa + sb;
+            }
           }
           if (ok) ok = __all_sync(0xffffffffu, mbar_wait(bar(PV_DONE + x), items_x & 1, abort_flag, p.status));
           ++items_x;
           cx += n_tiles;
-          const Item im = read_item(ring, p, n_qp);
+          const Item im = read_item<FULL>(ring, p, n_qp);
           const int seq = im.seq;
           const int q_row0 = im.q0 + x * BM;
+          if (FULL && ok) {
+            // Eq. 2: mean over the step's rows of mass(row, scale) / rowsum(row); rows past t_q are padding
+            const float inv_t = 1.f / (float)p.t_q;
+            const float w = q_row0 + row < p.t_q ? inv_t / l_sum : 0.f;
+            float* beta = p.beta_row + (int64_t)im.head * p.K * p.K;
+            for (int s = 0; s <= p.step; ++s) {
+              float v = (s == cur_seg ? cur_mass : masses[s * 32]) * w;
+#pragma unroll
+              for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+              if (lane == 0) atomicAdd(beta + s, v);
+            }
+            __syncwarp();                                   // the buffer now takes output rows
+          }
           __nv_bfloat16* dst = p.out + seq * p.o_seq + im.head * p.o_head + (int64_t)q_row0 * p.o_tok;
           // Normalised rows leave through this warp's staging buffer: per group of 32 columns every thread
           // parks its 64 bytes (16-byte chunks, chunk ^ (row / 2 mod 4) against bank conflicts), then four
@@ -893,19 +956,22 @@ int tc_create(const heatkv_config& cfg, void* k_pool, void* v_pool, uint64_t poo
   st->encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   if (!encode_2d(st, &st->k_pool, k_pool, pool_rows) || !encode_2d(st, &st->v_pool, v_pool, pool_rows))
     return HEATKV_OK;
-  const void* kern = cfg.d == 128 ? (const void*)tc::attn_tc_kernel<128> : (const void*)tc::attn_tc_kernel<64>;
   const int smem = cfg.d == 128 ? (int)tc::Layout<128>::SM_ALLOC : (int)tc::Layout<64>::SM_ALLOC;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
-    cudaGetLastError();
-    return HEATKV_OK;
+  const void* kernels[2] = {cfg.d == 128 ? (const void*)tc::attn_tc_kernel<128, false> : (const void*)tc::attn_tc_kernel<64, false>,
+                            cfg.d == 128 ? (const void*)tc::attn_tc_kernel<128, true> : (const void*)tc::attn_tc_kernel<64, true>};
+  for (const void* kern : kernels) {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+      cudaGetLastError();
+      return HEATKV_OK;
+    }
+    // the register hand-over inside the kernel must fit in what the launch really allocates
+    cudaFuncAttributes attr;
+    if (cudaFuncGetAttributes(&attr, kern) != cudaSuccess) {
+      cudaGetLastError();
+      return HEATKV_OK;
+    }
+    if (attr.numRegs * tc::THREADS < 128 * tc::REGS_SMALL + 256 * tc::REGS_SOFTMAX) return HEATKV_ERR_CUDA;
   }
-  // the register hand-over inside the kernel must fit in what the launch really allocates
-  cudaFuncAttributes attr;
-  if (cudaFuncGetAttributes(&attr, kern) != cudaSuccess) {
-    cudaGetLastError();
-    return HEATKV_OK;
-  }
-  if (attr.numRegs * tc::THREADS < 128 * tc::REGS_SMALL + 256 * tc::REGS_SOFTMAX) return HEATKV_ERR_CUDA;
   int dev = 0, n_sm = 0;
   if (cudaGetDevice(&dev) == cudaSuccess &&
       cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n_sm > 0)
@@ -920,8 +986,8 @@ bool tc_ready(const TcState* st) { return st && st->ready; }
 
 int tc_split_slot_floats(int d) { return d == 64 ? tc::Layout<64>::SPLIT_SLOT_FLOATS : tc::Layout<128>::SPLIT_SLOT_FLOATS; }
 
-bool tc_supported(const TcState* st, const AttnParams& p, int d, int n_seq, bool calib) {
-  if (!st || !st->ready || calib || d != st->d || n_seq > 65535) return false;
+bool tc_supported(const TcState* st, const AttnParams& p, int d, int n_seq) {
+  if (!st || !st->ready || d != st->d || n_seq > 65535) return false;
   // TMA needs 16-byte aligned bases (checked by the caller) and strides that are multiples of 16 bytes
   const int64_t s[6] = {p.q_seq, p.q_head, p.q_tok, p.kv_seq, p.kv_head, p.kv_tok};
   for (int64_t v : s)
@@ -929,9 +995,9 @@ bool tc_supported(const TcState* st, const AttnParams& p, int d, int n_seq, bool
   return true;
 }
 
-cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int d, int n_seq, bool calib, cudaStream_t stream,
-                           int* launches) {
-  (void)d; (void)calib;
+// Attention of a scale step (p.items_per_seq work items per sequence) or, with p.full_slots > 0, calibration with an
+// attention output over all p.n_own keys of p.k_new / p.v_new.
+cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int n_seq, cudaStream_t stream) {
   tc::Maps maps;
   maps.k_pool = st->k_pool;
   maps.v_pool = st->v_pool;
@@ -945,9 +1011,14 @@ cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int d, int n_seq, b
   q.attn_items = p.items_per_seq * n_seq;
   q.store_items = p.append_tiles * p.H * n_seq;
   dim3 grid((unsigned)std::min(q.attn_items, st->n_sm));
-  if (st->d == 128) tc::attn_tc_kernel<128><<<grid, tc::THREADS, tc::Layout<128>::SM_ALLOC, stream>>>(q, maps);
-  else tc::attn_tc_kernel<64><<<grid, tc::THREADS, tc::Layout<64>::SM_ALLOC, stream>>>(q, maps);
-  *launches = 1;
+  const bool full = p.full_slots > 0;
+  if (st->d == 128) {
+    if (full) tc::attn_tc_kernel<128, true><<<grid, tc::THREADS, tc::Layout<128>::SM_ALLOC, stream>>>(q, maps);
+    else tc::attn_tc_kernel<128, false><<<grid, tc::THREADS, tc::Layout<128>::SM_ALLOC, stream>>>(q, maps);
+  } else {
+    if (full) tc::attn_tc_kernel<64, true><<<grid, tc::THREADS, tc::Layout<64>::SM_ALLOC, stream>>>(q, maps);
+    else tc::attn_tc_kernel<64, false><<<grid, tc::THREADS, tc::Layout<64>::SM_ALLOC, stream>>>(q, maps);
+  }
   return cudaGetLastError();
 }
 

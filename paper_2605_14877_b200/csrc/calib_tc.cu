@@ -446,6 +446,12 @@ void calib_tc_destroy(CalibTcState* st) { delete st; }
 
 bool calib_tc_ready(const CalibTcState* st) { return st && st->ready; }
 
+// The step's key half-tiles on the device.
+void calib_tc_step_descs(const CalibTcState* st, int step, const int2** descs, int* n_slots) {
+  *descs = st->dev_descs + st->first[step];
+  *n_slots = st->count[step];
+}
+
 bool calib_tc_supported(const CalibTcState* st, const AttnParams& p, int d, int n_seq) {
   if (!st || !st->ready || d != st->d || n_seq > 65535 || p.H > 65535) return false;
   const int64_t s[6] = {p.q_seq, p.q_head, p.q_tok, p.kv_seq, p.kv_head, p.kv_tok};

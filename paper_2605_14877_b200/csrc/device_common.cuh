@@ -49,6 +49,10 @@ struct AttnParams {
   int32_t longest_piece;          // host report: longest piece among the heads that are cut (0: none is)
   int32_t append_tiles;           // > 0: the launch also stores the step's K/V (paged layout): that many destination
                                   // half-tile slots per (sequence, head) follow the attention work
+  // tensor-memory kernel, calibration with an attention output (full_slots > 0): the step's key half-tiles, cut at
+  // source-scale borders ({first key row, rows | scale << 8})
+  const int2* full_descs;
+  int32_t full_slots;
   int32_t attn_items, store_items;  // tensor-memory kernel: attention work items; cache-update items (destination half-tiles)
   float* split_partials;          // [n_seq * slots_per_seq][SPLIT_SLOT_FLOATS]
   uint32_t* split_counters;       // [n_seq * ctrs_per_seq], zero between launches

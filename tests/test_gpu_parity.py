@@ -431,6 +431,31 @@ def test_calibration_tensor_memory_kernel_outlier_keys(hk):
     assert np.allclose(beta.sum(axis=-1), 1.0, atol=2e-4)
 
 
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+@pytest.mark.parametrize("outliers", [False, True], ids=["plain_bias", "outlier_keys"])
+def test_calibration_with_output_tensor_memory_kernel(hk, d, outliers):
+    """Attention output and scale masses from one tcgen05 launch per step, every step forced through it: one-row tiles,
+    odd half-tile counts, several items per head; with outlier keys the running reference (and with it the masses of
+    the scales already finished) moves in the middle of a row."""
+    sh = W.Shape("mid", L=1, H=3, d=d, sides=W.SIDES_13[:10], n_seq=2, s=3)
+    bias = None if outliers else W.seg_bias_prior_lognormal(sh, 8)
+
+    def mutate(q, k, v):
+        k = k.clone()
+        k[:, :, 200:203] *= 8.0
+        k[:, :, 700] *= 12.0
+        # One key may carry a whole row, so |O| reaches max|V| = 4.2 and the two bf16 roundings (P and O, 2^-9 relative
+        # each) allow 4.2 * 2^-8 = 0.0165; V scaled by 1/4 (exact) brings that bound to 0.0041, inside the 1e-2 bar.
+        return q, k, v * 0.25
+
+    beta, scas, cas, ref = _calibrate(hk, sh, seeds=[5], bias=bias, with_out=True, kernel=hk.KERNEL_TCGEN05,
+                                      mutate=mutate if outliers else None)
+    mask = ref > 1e-5
+    assert np.all(np.abs(beta - ref)[mask] <= RTOL_BETA * ref[mask])
+    assert np.allclose(beta.sum(axis=-1), 1.0, atol=2e-4)
+    assert np.all(np.triu(beta, 1) == 0)
+
+
 def test_config2_calibration_full_size(hk):
     """Sec. 3.1, Eq. 2 and Eq. 4 at the size the bench calibrates at: 13 scales, 2 sequences x 16 heads, bias on
     the current scale, automatic kernel choice (tensor-memory kernel for the seven steps of 256 tokens and more:
