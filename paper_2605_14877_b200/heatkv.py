@@ -72,11 +72,14 @@ class Strides(C.Structure):
     @classmethod
     def of(cls, q: torch.Tensor, kv: torch.Tensor, o: Optional[torch.Tensor] = None) -> "Strides":
         """Strides of [n_seq, H, t, d] views (d contiguous)."""
-        o = q if o is None else o
-        for x in (q, kv, o):
-            assert x.dim() == 4 and x.stride(3) == 1
-        return cls(q.stride(0), q.stride(1), q.stride(2), kv.stride(0), kv.stride(1), kv.stride(2),
-                   o.stride(0), o.stride(1), o.stride(2))
+        sq, skv = q.stride(), kv.stride()
+        return cls._of(sq, skv, sq if o is None else o.stride())
+
+    @classmethod
+    def _of(cls, sq, skv, so) -> "Strides":
+        for s in (sq, skv, so):
+            assert len(s) == 4 and s[3] == 1
+        return cls(*sq[:3], *skv[:3], *so[:3])
 
 
 class AllocStats(C.Structure):
@@ -162,7 +165,8 @@ for _n in exported_symbols():
 
 def _stream(stream) -> int:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        # the handle itself: building the Stream object around it (torch.cuda.current_stream) costs 3 us a call
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -182,6 +186,8 @@ def _check(rc: int, where: str) -> None:
 
 
 def _ids(seq_ids: Sequence[int]):
+    if isinstance(seq_ids, C.Array):                   # converted before (Session.generate)
+        return seq_ids, len(seq_ids)
     return (C.c_int * len(seq_ids))(*[int(i) for i in seq_ids]), len(seq_ids)
 
 

@@ -53,14 +53,17 @@ class Session:
     def run_layer_step(self, seq_ids, layer: int, step: int, q, k, v, out, seg_bias=None, fused: bool = False) -> None:
         """q, k, v, out: [n_seq, H, n_tokens, d] tensors holding all scales; uses the slice of `step`.
         `fused`: one heatkv_attention_append call instead of attention followed by the cache update."""
-        lo, hi = self.step_slices(step)
-        qs, ks, vs, os_ = q[:, :, lo:hi], k[:, :, lo:hi], v[:, :, lo:hi], out[:, :, lo:hi]
-        st = hk.Strides.of(qs, ks, os_)
+        # The step's slice as base pointers: building the four views x[:, :, lo:hi] costs 8 us, as much as the launch.
+        lo = self.c[step] - self.t[step]
+        sq, sk, so = q.stride(), k.stride(), out.stride()
+        qp, op = q.data_ptr() + 2 * lo * sq[2], out.data_ptr() + 2 * lo * so[2]
+        kp, vp = k.data_ptr() + 2 * lo * sk[2], v.data_ptr() + 2 * lo * sk[2]
+        st = hk.Strides._of(sq, sk, so)
         if fused:
-            hk.heatkv_attention_append(self.ctx, seq_ids, layer, step, qs, ks, vs, st, seg_bias, os_)
+            hk.heatkv_attention_append(self.ctx, seq_ids, layer, step, qp, kp, vp, st, seg_bias, op)
             return
-        hk.heatkv_scale_attention(self.ctx, seq_ids, layer, step, qs, ks, vs, st, seg_bias, os_)
-        hk.heatkv_append_compact(self.ctx, seq_ids, layer, step, ks, vs, st)
+        hk.heatkv_scale_attention(self.ctx, seq_ids, layer, step, qp, kp, vp, st, seg_bias, op)
+        hk.heatkv_append_compact(self.ctx, seq_ids, layer, step, kp, vp, st)
 
     def pre_step(self, seq_ids, step: int) -> None:
         hk.heatkv_append_compact(self.ctx, seq_ids, -1, step, None, None, None)
@@ -69,6 +72,7 @@ class Session:
                  bias_of: Optional[Callable[[int, int], Optional[torch.Tensor]]] = None,
                  after: Optional[Callable[[int, int], None]] = None, fused: bool = False) -> None:
         """Whole sweep: steps outer, layers inner.  `after(step, layer)` runs after each layer."""
+        seq_ids = hk._ids(seq_ids)[0]
         for step in range(self.K):
             self.pre_step(seq_ids, step)
             for layer in range(self.L):
