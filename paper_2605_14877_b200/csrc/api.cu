@@ -12,7 +12,7 @@
 #include "internal.h"
 
 namespace heatkv {
-cudaError_t launch_attn_generic(const AttnParams& p, int d, int n_seq, bool calib, cudaStream_t stream);
+cudaError_t launch_attn_generic(const AttnParams& p, int d, int n_seq, bool calib, int n_sm, cudaStream_t stream);
 cudaError_t launch_calibrate_static(const AttnParams& p, int d, int n_seq, cudaStream_t stream, bool* too_large);
 cudaError_t launch_append(const CopyParams& p, int n_seq, cudaStream_t stream);
 cudaError_t launch_compact(const CopyParams& p, int n_seq, cudaStream_t stream);
@@ -729,7 +729,7 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
     ctx->kstats.attention_tcgen05 += 1;
   } else {
     fill_head_table(ctx, seq_ids, n_seq, step, layer, &p);
-    e = launch_attn_generic(p, ctx->cfg.d, n_seq, false, stream);
+    e = launch_attn_generic(p, ctx->cfg.d, n_seq, false, ctx->n_sm, stream);
     ctx->launches += 1;
     ctx->kstats.attention_generic += 1;
   }
@@ -820,7 +820,7 @@ int heatkv_calibrate_scores(heatkv_ctx* ctx, int layer, int step, int n_seq, con
     p.items_per_seq = (int)items;
     e = launch_attn_tc(ctx->tc, p, n_seq, stream);
   } else {
-    e = use_tc ? launch_calib_tc(ctx->calib_tc, p, n_seq, stream) : launch_attn_generic(p, ctx->cfg.d, n_seq, true, stream);
+    e = use_tc ? launch_calib_tc(ctx->calib_tc, p, n_seq, stream) : launch_attn_generic(p, ctx->cfg.d, n_seq, true, ctx->n_sm, stream);
   }
   ctx->launches += 1;
   (use_tc ? ctx->kstats.calibration_tcgen05 : ctx->kstats.calibration_generic) += 1;
@@ -875,7 +875,7 @@ int heatkv_calibrate_scores_steps(heatkv_ctx* ctx, int layer, int step_begin, in
     g.seg_bias = seg_bias;
     g.cal_bias_stride = H * K;
     g.beta_row = beta_layer;
-    if (launch_attn_generic(g, ctx->cfg.d, n_seq, true, stream) != cudaSuccess) return HEATKV_ERR_CUDA;
+    if (launch_attn_generic(g, ctx->cfg.d, n_seq, true, ctx->n_sm, stream) != cudaSuccess) return HEATKV_ERR_CUDA;
     ctx->launches += 1;
     ctx->kstats.calibration_generic += 1;
   }

@@ -1,7 +1,8 @@
 // Generic ragged attention kernel (warp-level MMA, online softmax), used for the small,
 // bandwidth / latency bound scale steps and for calibration.
 //
-// One CTA = 64 queries of one (sequence, head); 4 warps x 16 query rows.  Keys arrive as a
+// One CTA = 64 queries of one (sequence, head); 4 warps x 16 query rows, or two such groups of warps that take the key
+// half-tiles in turn and meet at the end.  Keys arrive as a
 // sequence of half-tiles of up to 64 rows: first the head's retained prior keys, listed by
 // the plan's page table (Sec. 3.3: the head-scales not in A_k), then the step's own keys
 // from k_new.  In calibration mode (Eq. 2) every key comes from k_full and the per-row
@@ -14,17 +15,18 @@ namespace heatkv {
 
 constexpr int GM = 64;    // queries per CTA
 constexpr int GN = 64;    // keys per half-tile
-constexpr int GTHREADS = 128;
+constexpr int GTHREADS = 128; // threads of one group
 constexpr int GSTAGES = 2;   // key/value half-tiles in flight or in use per CTA (3 measured no faster: the small steps are bound by the warp-level MMA rate)
 
-template <int D>
+template <int D, int GROUPS = 1>
 struct GenericSmem {
   static constexpr int TILE_BYTES = GN * D * 2;
-  // q | k[GSTAGES] | v[GSTAGES] | seg_sum[GM][16] | seg_ref[GM][16]
+  // q | per group: k[GSTAGES] | v[GSTAGES] | then seg_sum[GM][16] | seg_ref[GM][16]
   static constexpr int Q_OFF = 0;
   static constexpr int K_OFF = GM * D * 2;
   static constexpr int V_OFF = K_OFF + GSTAGES * TILE_BYTES;
-  static constexpr int SEG_OFF = V_OFF + GSTAGES * TILE_BYTES;
+  static constexpr int GROUP_BYTES = 2 * GSTAGES * TILE_BYTES;
+  static constexpr int SEG_OFF = K_OFF + GROUPS * GROUP_BYTES;
   static constexpr int BYTES = SEG_OFF + 2 * GM * HEATKV_MAX_K * 4;
   static constexpr int ATTN_BYTES = SEG_OFF;             // without the calibration sums: two CTAs of head_dim 128 fit an SM
 };
@@ -35,17 +37,19 @@ __device__ __forceinline__ uint32_t tile_off(int r, int ch) {
   return (uint32_t)((r * (D / 8) + (ch ^ (r & 7))) * 16);
 }
 
-// copies `rows` rows (row-major, D bf16 each, `stride` elements apart) into a swizzled tile;
-// rows >= n_valid are zero-filled.
-template <int D>
+// copies n_valid rows (row-major, D bf16 each, `stride` elements apart) into a swizzled tile; rows from there to the
+// next multiple of 16 (what the products read) are zero-filled.
+template <int D, int THREADS = GTHREADS>
 __device__ __forceinline__ void load_tile(uint32_t smem_base, const __nv_bfloat16* src, int64_t stride,
                                           int n_valid, int tid) {
   constexpr int CH = D / 8;
-  constexpr int ROWS_PER_PASS = GTHREADS / CH;
+  constexpr int ROWS_PER_PASS = THREADS / CH;
   const int ch = tid % CH;
   const int r0 = tid / CH;
+  const int rows = (n_valid + 15) & ~15;
 #pragma unroll
   for (int r = r0; r < GN; r += ROWS_PER_PASS) {
+    if (r >= rows) break;
     const bool ok = r < n_valid;
     const __nv_bfloat16* p = ok ? src + (int64_t)r * stride + ch * 8 : src;
     cp_async16(smem_base + tile_off<D>(r, ch), p, ok ? 16 : 0);
@@ -58,11 +62,19 @@ __device__ __forceinline__ void load_tile(uint32_t smem_base, const __nv_bfloat1
 constexpr int STATIC_PARTIAL_FLOATS = 1 << 20;
 static __device__ __align__(256) float g_static_partials[STATIC_PARTIAL_FLOATS];
 
-template <int D, bool CALIB, bool PARTIALS = false>
-__global__ void __launch_bounds__(GTHREADS, 2) attn_generic_kernel(const __grid_constant__ AttnParams p) {
+__device__ __forceinline__ void group_sync(int grp) {
+  asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "n"(GTHREADS) : "memory");
+}
+
+// GROUPS = 2: a launch that leaves SMs idle is a chain of key half-tiles (1.4 to 2 us each: copies, products at the
+// warp-level rate, softmax) per CTA; two groups of warps halve it.  GROUPS_MEASURED
+template <int D, bool CALIB, bool PARTIALS = false, int GROUPS = 1>
+__global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_kernel(const __grid_constant__ AttnParams p) {
   extern __shared__ __align__(128) unsigned char smem[];
-  using SM = GenericSmem<D>;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  using SM = GenericSmem<D, GROUPS>;
+  static_assert(GROUPS == 1 || !CALIB, "the scale masses are kept by one group");
+  const int grp = GROUPS == 1 ? 0 : __shfl_sync(0xffffffffu, (int)threadIdx.x / GTHREADS, 0);
+  const int tid = threadIdx.x - grp * GTHREADS, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, qd = lane & 3;
   // attention: grid = (query tiles, sequences, heads by descending key count), so the heaviest heads of
   // every sequence are dispatched first; calibration: grid = (query tiles, heads, sequences)
@@ -72,11 +84,11 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_generic_kernel(const __grid_
     const int64_t src = sq * p.kv_seq + hd * p.kv_head;
     if (p.k8_pool)
       append_half_tile_fp8(p.seqs[sq].plan, p.pool_base[sq], (p.step * p.L + p.layer) * p.H + hd, j, p.k_new + src,
-                           p.v_new + src, p.kv_tok, p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, D, threadIdx.x, GTHREADS);
+                           p.v_new + src, p.kv_tok, p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, D, threadIdx.x, GTHREADS * GROUPS);
     else
       append_half_tile(p.seqs[sq].plan, p.seqs[sq].base_row, (p.step * p.L + p.layer) * p.H + hd, j, p.k_new + src,
                        p.v_new + src, p.kv_tok, const_cast<__nv_bfloat16*>(p.k_pool), const_cast<__nv_bfloat16*>(p.v_pool),
-                       D, threadIdx.x, GTHREADS);
+                       D, threadIdx.x, GTHREADS * GROUPS);
     return;
   }
   const int seq = CALIB ? blockIdx.z : blockIdx.y;
@@ -122,14 +134,16 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_generic_kernel(const __grid_
   const int n_tiles = n_desc + n_own_tiles;
 
   const uint32_t sbase = smem_u32(smem);
+  const uint32_t gbase = sbase + grp * SM::GROUP_BYTES;    // K_OFF / V_OFF of this group's stages count from here
   float* seg_sum = reinterpret_cast<float*>(smem + SM::SEG_OFF);
   float* seg_ref = seg_sum + GM * HEATKV_MAX_K;
 
   const __nv_bfloat16* kown = p.k_new + seq * p.kv_seq + head * p.kv_head;
   const __nv_bfloat16* vown = p.v_new ? p.v_new + seq * p.kv_seq + head * p.kv_head : nullptr;
 
-  // descriptors are fetched one tile ahead of the copy they steer: `dsc_next` belongs to the tile issued next
-  int2 dsc_next = n_desc > 0 ? descs[0] : make_int2(0, 0);
+  // descriptors are fetched one tile ahead of the copy they steer: `dsc_next` belongs to the tile issued next.
+  // The group's i-th tile is tile grp + i * GROUPS of the CTA.
+  int2 dsc_next = n_desc > grp ? descs[grp] : make_int2(0, 0);
   auto issue_tile = [&](int j, int stage) {
     const __nv_bfloat16 *ks, *vs;
     int64_t stride;
@@ -148,18 +162,18 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_generic_kernel(const __grid_
       stride = p.kv_tok;
       nv = min(GN, n_own - jj * GN);
     }
-    load_tile<D>(sbase + SM::K_OFF + stage * SM::TILE_BYTES, ks, stride, nv, tid);
-    if (vs) load_tile<D>(sbase + SM::V_OFF + stage * SM::TILE_BYTES, vs, stride, nv, tid);
-    if (j + 1 < n_desc) dsc_next = descs[j + 1];
+    load_tile<D>(gbase + SM::K_OFF + stage * SM::TILE_BYTES, ks, stride, nv, tid);
+    if (vs) load_tile<D>(gbase + SM::V_OFF + stage * SM::TILE_BYTES, vs, stride, nv, tid);
+    if (j + GROUPS < n_desc) dsc_next = descs[j + GROUPS];
   };
 
   // ---- prologue: Q tile and the first GSTAGES - 1 key tiles, one copy group each (empty groups keep the count)
   {
     const __nv_bfloat16* qsrc = q_base + seq * p.q_seq + head * p.q_head + (int64_t)q0 * p.q_tok;
-    load_tile<D>(sbase + SM::Q_OFF, qsrc, p.q_tok, min(GM, t_q - q0), tid);
+    load_tile<D, GTHREADS * GROUPS>(sbase + SM::Q_OFF, qsrc, p.q_tok, min(GM, t_q - q0), threadIdx.x);
     cp_async_commit();
-    for (int j = 0; j < GSTAGES - 1; ++j) {
-      if (j < n_tiles) issue_tile(j, j);
+    for (int i = 0; i < GSTAGES - 1; ++i) {
+      if (grp + i * GROUPS < n_tiles) issue_tile(grp + i * GROUPS, i);
       cp_async_commit();
     }
   }
@@ -186,12 +200,16 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_generic_kernel(const __grid_
   float m_run[2] = {-INFINITY, -INFINITY};
   float l_run[2] = {0.f, 0.f};
 
-  for (int j = 0; j < n_tiles; ++j) {
-    const int stage = j % GSTAGES;
+  const bool has_rows = q0 + warp * 16 < t_q;          // a warp without query rows only helps with the copies
+  for (int i = 0, j = grp; j < n_tiles; ++i, j += GROUPS) {
+    const int stage = i % GSTAGES;
     cp_async_wait<GSTAGES - 2>();                      // all groups but the newest GSTAGES - 2: tile j is among them
-    __syncthreads();                                   // tile j landed for everyone; everyone left tile j-1
-    if (j + GSTAGES - 1 < n_tiles) issue_tile(j + GSTAGES - 1, (j + GSTAGES - 1) % GSTAGES);   // into tile j-1's stage
+    if (GROUPS == 1) __syncthreads();                  // tile j landed for everyone; everyone left the tile before
+    else group_sync(grp);
+    if (j + (GSTAGES - 1) * GROUPS < n_tiles)          // into the stage of the tile before
+      issue_tile(j + (GSTAGES - 1) * GROUPS, (i + GSTAGES - 1) % GSTAGES);
     cp_async_commit();
+    if (!has_rows) continue;
 
     // tile attributes (warp-uniform)
     int nv, seg_lo, seg_hi, col0 = 0;
@@ -212,15 +230,16 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_generic_kernel(const __grid_
       }
     }
 
-    // ---- S = Q K^T
+    // ---- S = Q K^T (a tile of a small scale has few keys: its empty groups of 16 are skipped throughout)
     float s[GN / 8][4];
 #pragma unroll
     for (int i = 0; i < GN / 8; ++i) s[i][0] = s[i][1] = s[i][2] = s[i][3] = 0.f;
-    const uint32_t kbase = sbase + SM::K_OFF + stage * SM::TILE_BYTES;
+    const uint32_t kbase = gbase + SM::K_OFF + stage * SM::TILE_BYTES;
 #pragma unroll
     for (int ks = 0; ks < D / 16; ++ks) {
 #pragma unroll
       for (int np = 0; np < GN / 16; ++np) {
+        if (np * 16 >= nv) break;
         uint32_t b[4];
         int r = np * 16 + (lane & 7) + (lane >> 4) * 8;
         int ch = ks * 2 + ((lane >> 3) & 1);
@@ -237,6 +256,7 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_generic_kernel(const __grid_
     float mx[2] = {-INFINITY, -INFINITY};
 #pragma unroll
     for (int n = 0; n < GN / 8; ++n) {
+      if ((n & ~1) * 8 >= nv) break;
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         int col = n * 8 + qd * 2 + (e & 1);
@@ -264,6 +284,7 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_generic_kernel(const __grid_
     float psum[2] = {0.f, 0.f};
 #pragma unroll
     for (int n = 0; n < GN / 8; ++n) {
+      if ((n & ~1) * 8 >= nv) break;
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         float pv = exp2f(s[n][e] - m_run[e >> 1]);
@@ -311,9 +332,10 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_generic_kernel(const __grid_
         o[i][2] *= corr[1];
         o[i][3] *= corr[1];
       }
-      const uint32_t vbase = sbase + SM::V_OFF + stage * SM::TILE_BYTES;
+      const uint32_t vbase = gbase + SM::V_OFF + stage * SM::TILE_BYTES;
 #pragma unroll
       for (int kk = 0; kk < GN / 16; ++kk) {
+        if (kk * 16 >= nv) break;
         uint32_t pa[4];
         pa[0] = pack_bf16(s[2 * kk][0], s[2 * kk][1]);
         pa[1] = pack_bf16(s[2 * kk][2], s[2 * kk][3]);
@@ -332,6 +354,43 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_generic_kernel(const __grid_
     }
   }
   cp_async_wait<0>();
+
+  if (GROUPS == 2) {
+    // ---- the second group's partial result joins the first's (through the copy stages, which nobody reads any more)
+    __syncthreads();
+    float* part = reinterpret_cast<float*>(smem + SM::K_OFF) + tid;
+    constexpr int STAT = D / 8 * 4 * GTHREADS;
+    if (grp == 1) {
+      if (has_rows) {
+#pragma unroll
+        for (int i = 0; i < D / 8; ++i)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) part[(i * 4 + e) * GTHREADS] = o[i][e];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          part[STAT + r * GTHREADS] = m_run[r];
+          part[STAT + (2 + r) * GTHREADS] = l_run[r];
+        }
+      }
+    }
+    __syncthreads();
+    if (grp == 0 && has_rows) {
+      float w0[2], w1[2];
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const float m1 = part[STAT + r * GTHREADS];     // -inf when the second group had no tile; ours is finite
+        const float m = fmaxf(m_run[r], m1);
+        w0[r] = exp2f(m_run[r] - m);
+        w1[r] = exp2f(m1 - m);
+        l_run[r] = l_run[r] * w0[r] + part[STAT + (2 + r) * GTHREADS] * w1[r];
+      }
+#pragma unroll
+      for (int i = 0; i < D / 8; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          o[i][e] = o[i][e] * w0[e >> 1] + part[(i * 4 + e) * GTHREADS] * w1[e >> 1];
+    }
+  }
 
   // ---- epilogue
   float inv_l[2];
@@ -372,6 +431,7 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_generic_kernel(const __grid_
   if (p.out) {
     __syncthreads();                                   // all warps are done with the K/V stages
     // stage the bf16 tile in shared memory (reusing the Q region), then 16-byte row stores
+    if (grp == 0 && has_rows) {
 #pragma unroll
     for (int n = 0; n < D / 8; ++n) {
       int r0 = warp * 16 + g;
@@ -380,10 +440,11 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_generic_kernel(const __grid_
       *reinterpret_cast<uint32_t*>(smem + SM::Q_OFF + tile_off<D>(r0, n) + qd * 4) = lo;
       *reinterpret_cast<uint32_t*>(smem + SM::Q_OFF + tile_off<D>(r0 + 8, n) + qd * 4) = hi;
     }
+    }
     __syncthreads();
     constexpr int CH = D / 8;
     __nv_bfloat16* dst = p.out + seq * p.o_seq + head * p.o_head + (int64_t)q0 * p.o_tok;
-    for (int i = tid; i < GM * CH; i += GTHREADS) {
+    for (int i = threadIdx.x; i < GM * CH; i += GTHREADS * GROUPS) {
       int r = i / CH, ch = i % CH;
       if (q0 + r < t_q) {
         int4 v = *reinterpret_cast<const int4*>(smem + SM::Q_OFF + tile_off<D>(r, ch));
@@ -410,10 +471,10 @@ __global__ void reduce_partials_kernel(const float* partials, float* beta_row, i
 
 constexpr int MAX_DEVICES = 64;
 
-template <int D, bool CALIB>
+template <int D, bool CALIB, int GROUPS = 1>
 static cudaError_t launch_one(const AttnParams& p, int n_seq, cudaStream_t stream) {
-  auto kern = attn_generic_kernel<D, CALIB>;
-  constexpr int bytes = CALIB ? GenericSmem<D>::BYTES : GenericSmem<D>::ATTN_BYTES;
+  auto kern = attn_generic_kernel<D, CALIB, false, GROUPS>;
+  constexpr int bytes = CALIB ? GenericSmem<D>::BYTES : GenericSmem<D, GROUPS>::ATTN_BYTES;
   // the attribute belongs to the (function, device) pair: set it once on every device that launches
   static std::atomic<bool> configured[MAX_DEVICES];
   int dev = -1;
@@ -427,7 +488,7 @@ static cudaError_t launch_one(const AttnParams& p, int n_seq, cudaStream_t strea
   }
   const int q_tiles = CALIB && p.cal_n > 0 ? p.cal_tile_begin[p.cal_n] : (p.t_q + GM - 1) / GM;
   dim3 grid(q_tiles + (CALIB ? 0 : p.append_tiles), CALIB ? p.H : n_seq, CALIB ? n_seq : p.H);
-  kern<<<grid, GTHREADS, bytes, stream>>>(p);
+  kern<<<grid, GTHREADS * GROUPS, bytes, stream>>>(p);
   return cudaGetLastError();
 }
 
@@ -485,10 +546,15 @@ cudaError_t launch_calibrate_static(const AttnParams& p_in, int d, int n_seq, cu
   return cudaGetLastError();
 }
 
-cudaError_t launch_attn_generic(const AttnParams& p, int d, int n_seq, bool calib, cudaStream_t stream) {
-  if (d == 128) return calib ? launch_one<128, true>(p, n_seq, stream) : launch_one<128, false>(p, n_seq, stream);
-  if (d == 64) return calib ? launch_one<64, true>(p, n_seq, stream) : launch_one<64, false>(p, n_seq, stream);
-  return cudaErrorInvalidValue;
+// `n_sm`: SMs of the device.  Two groups of warps per CTA while every CTA has an SM to itself and heads see more than one
+// key half-tile; a fuller launch keeps two single-group CTAs per SM (the same warps per SM, and nothing to merge).
+cudaError_t launch_attn_generic(const AttnParams& p, int d, int n_seq, bool calib, int n_sm, cudaStream_t stream) {
+  if (d != 64 && d != 128) return cudaErrorInvalidValue;
+  if (calib) return d == 128 ? launch_one<128, true>(p, n_seq, stream) : launch_one<64, true>(p, n_seq, stream);
+  const int64_t ctas = (int64_t)((p.t_q + GM - 1) / GM) * n_seq * p.H;
+  if (p.step > 0 && ctas <= n_sm)
+    return d == 128 ? launch_one<128, false, 2>(p, n_seq, stream) : launch_one<64, false, 2>(p, n_seq, stream);
+  return d == 128 ? launch_one<128, false>(p, n_seq, stream) : launch_one<64, false>(p, n_seq, stream);
 }
 
 }  // namespace heatkv
