@@ -75,6 +75,7 @@ __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_ke
   static_assert(GROUPS == 1 || !CALIB, "the scale masses are kept by one group");
   const int grp = GROUPS == 1 ? 0 : __shfl_sync(0xffffffffu, (int)threadIdx.x / GTHREADS, 0);
   const int tid = threadIdx.x - grp * GTHREADS, warp = tid >> 5, lane = tid & 31;
+  pdl_trigger();
   const int g = lane >> 2, qd = lane & 3;
   // attention: grid = (query tiles, sequences, heads by descending key count), so the heaviest heads of
   // every sequence are dispatched first; calibration: grid = (query tiles, heads, sequences)
@@ -82,6 +83,7 @@ __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_ke
     // cache update riding on this launch: one CTA per (destination half-tile, sequence, head)
     const int sq = blockIdx.y, hd = blockIdx.z, j = blockIdx.x - (p.t_q + GM - 1) / GM;
     const int64_t src = sq * p.kv_seq + hd * p.kv_head;
+    pdl_wait();
     if (p.k8_pool)
       append_half_tile_fp8(p.seqs[sq].plan, p.pool_base[sq], (p.step * p.L + p.layer) * p.H + hd, j, p.k_new + src,
                            p.v_new + src, p.kv_tok, p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, D, threadIdx.x, GTHREADS * GROUPS);
@@ -167,6 +169,7 @@ __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_ke
     if (j + GROUPS < n_desc) dsc_next = descs[j + GROUPS];
   };
 
+  pdl_wait();
   // ---- prologue: Q tile and the first GSTAGES - 1 key tiles, one copy group each (empty groups keep the count)
   {
     const __nv_bfloat16* qsrc = q_base + seq * p.q_seq + head * p.q_head + (int64_t)q0 * p.q_tok;
@@ -459,6 +462,8 @@ __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_ke
 __global__ void reduce_partials_kernel(const float* partials, float* beta_row, int n_qtiles, int H, int n_seq, int K,
                                        int step) {
   const int head = blockIdx.x, sg = threadIdx.x;
+  pdl_trigger();
+  pdl_wait();
   if (sg > step) return;
   float acc = 0.f;
   for (int seq = 0; seq < n_seq; ++seq)
@@ -488,8 +493,7 @@ static cudaError_t launch_one(const AttnParams& p, int n_seq, cudaStream_t strea
   }
   const int q_tiles = CALIB && p.cal_n > 0 ? p.cal_tile_begin[p.cal_n] : (p.t_q + GM - 1) / GM;
   dim3 grid(q_tiles + (CALIB ? 0 : p.append_tiles), CALIB ? p.H : n_seq, CALIB ? n_seq : p.H);
-  kern<<<grid, GTHREADS * GROUPS, bytes, stream>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(kern, grid, GTHREADS * GROUPS, bytes, stream, p);
 }
 
 // Calibration pass whose scratch is the static array above.  Returns cudaErrorInvalidValue when the
@@ -528,7 +532,7 @@ cudaError_t launch_calibrate_static(const AttnParams& p_in, int d, int n_seq, cu
       if (e != cudaSuccess) return e;
       configured[dev][which].store(true, std::memory_order_release);
     }
-    kern<<<grid, GTHREADS, GenericSmem<128>::BYTES, stream>>>(p);
+    e = launch_pdl(kern, grid, GTHREADS, GenericSmem<128>::BYTES, stream, p);
   } else if (d == 64) {
     auto kern = attn_generic_kernel<64, true, true>;
     if (!configured[dev][which].load(std::memory_order_acquire)) {
@@ -536,14 +540,13 @@ cudaError_t launch_calibrate_static(const AttnParams& p_in, int d, int n_seq, cu
       if (e != cudaSuccess) return e;
       configured[dev][which].store(true, std::memory_order_release);
     }
-    kern<<<grid, GTHREADS, GenericSmem<64>::BYTES, stream>>>(p);
+    e = launch_pdl(kern, grid, GTHREADS, GenericSmem<64>::BYTES, stream, p);
   } else {
     return cudaErrorInvalidValue;
   }
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  reduce_partials_kernel<<<p.H, HEATKV_MAX_K, 0, stream>>>(p.partials, p.beta_row, n_qtiles, p.H, n_seq, p.K, p.step);
-  return cudaGetLastError();
+  return launch_pdl(reduce_partials_kernel, p.H, HEATKV_MAX_K, 0, stream, (const float*)p.partials, p.beta_row, n_qtiles, p.H,
+                    n_seq, p.K, p.step);
 }
 
 // `n_sm`: SMs of the device.  Two groups of warps per CTA while every CTA has an SM to itself and heads see more than one

@@ -178,6 +178,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
   const int u = (p.step * p.L + p.layer) * p.H;
   const int n_qp = (p.t_q + 2 * BM - 1) / (2 * BM);
 
+  pdl_trigger();
   if (threadIdx.x == 0) {
     *abort_flag = *reinterpret_cast<volatile uint32_t*>(p.status) != 0;   // an earlier CTA gave up: do not wait again
     for (int x = 0; x < 2; ++x) {
@@ -209,6 +210,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_ptr_smem;
+  pdl_wait();
 
   // register budget per warpgroup: 128*72 + 256*216 <= 64K
   if (warp < 4) {
@@ -1012,14 +1014,11 @@ cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int n_seq, cudaStre
   q.store_items = p.append_tiles * p.H * n_seq;
   dim3 grid((unsigned)std::min(q.attn_items, st->n_sm));
   const bool full = p.full_slots > 0;
-  if (st->d == 128) {
-    if (full) tc::attn_tc_kernel<128, true><<<grid, tc::THREADS, tc::Layout<128>::SM_ALLOC, stream>>>(q, maps);
-    else tc::attn_tc_kernel<128, false><<<grid, tc::THREADS, tc::Layout<128>::SM_ALLOC, stream>>>(q, maps);
-  } else {
-    if (full) tc::attn_tc_kernel<64, true><<<grid, tc::THREADS, tc::Layout<64>::SM_ALLOC, stream>>>(q, maps);
-    else tc::attn_tc_kernel<64, false><<<grid, tc::THREADS, tc::Layout<64>::SM_ALLOC, stream>>>(q, maps);
-  }
-  return cudaGetLastError();
+  if (st->d == 128)
+    return launch_pdl(full ? tc::attn_tc_kernel<128, true> : tc::attn_tc_kernel<128, false>, grid, tc::THREADS,
+                      tc::Layout<128>::SM_ALLOC, stream, q, maps);
+  return launch_pdl(full ? tc::attn_tc_kernel<64, true> : tc::attn_tc_kernel<64, false>, grid, tc::THREADS,
+                    tc::Layout<64>::SM_ALLOC, stream, q, maps);
 }
 
 }  // namespace heatkv

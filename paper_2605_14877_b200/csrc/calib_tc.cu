@@ -129,6 +129,7 @@ calib_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Ma
   const int nq = (q0 + BM < t_q) ? 2 : 1;               // does tile B hold any query?
   const int n_tiles = (n_slots + 1) / 2;
 
+  pdl_trigger();
   if (threadIdx.x == 0) {
     *abort_flag = *reinterpret_cast<volatile uint32_t*>(p.status) != 0;   // an earlier CTA gave up: do not wait again
     for (int i = 0; i < HEATKV_MAX_K; ++i) acc_smem[i] = 0.f;
@@ -154,6 +155,7 @@ calib_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Ma
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_ptr_smem;
+  pdl_wait();
 
   // register budget per warpgroup: 128*40 + 512*104 <= 640*96
   if (warp < 4) {
@@ -507,10 +509,10 @@ cudaError_t launch_calib_tc_steps(CalibTcState* st, const AttnParams& p, int n_s
   tab.cta_begin[n_steps] = ctas;
   dim3 grid((unsigned)ctas);
   if (st->d == 128)
-    calib::calib_tc_kernel<128><<<grid, calib::THREADS, calib::SM_ALLOC, stream>>>(p, maps, st->dev_descs, tab, n_seq, bias_step_stride);
-  else
-    calib::calib_tc_kernel<64><<<grid, calib::THREADS, calib::SM_ALLOC, stream>>>(p, maps, st->dev_descs, tab, n_seq, bias_step_stride);
-  return cudaGetLastError();
+    return launch_pdl(calib::calib_tc_kernel<128>, grid, calib::THREADS, calib::SM_ALLOC, stream, p, maps, st->dev_descs, tab,
+                      n_seq, bias_step_stride);
+  return launch_pdl(calib::calib_tc_kernel<64>, grid, calib::THREADS, calib::SM_ALLOC, stream, p, maps, st->dev_descs, tab, n_seq,
+                    bias_step_stride);
 }
 
 // One step: p.q = the step's queries, p.t_q of them; p.k_new = all p.n_own keys; p.beta_row = beta_accum[layer][0][step]

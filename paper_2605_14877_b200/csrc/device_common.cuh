@@ -116,6 +116,29 @@ struct PlanView {
   __device__ __forceinline__ const int32_t* src_rows() const { return w + w[17]; }   // fp8 cache only
 };
 
+// Programmatic dependent launch: every kernel lets the next one of the stream be set up while it runs (pdl_trigger, first
+// thing).  A kernel started with launch_pdl touches nothing that an earlier kernel may still write, nor anything an earlier
+// kernel may still read, before all of them are complete (pdl_wait, in every CTA, so that waiting for one kernel waits for
+// all before it).  Launch parameters and plan blobs (uploaded before any launch that names them) may be read before
+// that.  Back to back, the launches of a 256 x 256 preview (28 of them) take 235 us instead of 290, those of a tiny image
+// (4) 18 instead of 24.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
