@@ -457,6 +457,262 @@ __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_ke
   }
 }
 
+// ---------------------------------------------------------------------------------- attention of the small steps
+// What bounds a small scale step is the chain of one CTA: descriptors, the first copies, then per key half-tile the
+// products at the warp-level rate (a 16 x 16 x 128 chunk, S and PV, takes a warp about 0.5 us) and the softmax.  So a CTA
+// is 16 queries and four warps, one per SM sub-partition, that take 16 keys of every half-tile each and meet once at the
+// end in shared memory, where all threads normalise and write.  The step's own keys, whose place needs no descriptor,
+// come first.  2 sequences x 16 heads, back to back, against 64 queries per CTA with two groups of four warps:
+// 4 queries 3.3 against 4.0 us, 36: 6.4 against 6.8, 64: 7.9 against 8.8, 144: 11.7 against 12.4.  K and V are read once per
+// 16 queries, so a launch that fills the SMs is better off with the 64-query CTAs (8 sequences, 64 queries: 12.4 against
+// 9.1 us).
+constexpr int SKEYS = 16;      // keys of a half-tile one warp takes
+constexpr int SGROUPS = GN / SKEYS;
+constexpr int SSTAGES = 3;
+
+template <int D>
+struct SmallSmem {
+  static constexpr int ROWS = 16;
+  static constexpr int CHUNK_BYTES = SKEYS * D * 2;                 // K or V of one warp and stage
+  static constexpr int Q_OFF = 0;
+  static constexpr int KV_OFF = ROWS * D * 2;                       // [warp][stage][K | V]
+  static constexpr int KV_BYTES = SGROUPS * SSTAGES * 2 * CHUNK_BYTES;
+  static constexpr int PART_STRIDE = D + 8;                         // floats per row of a partial O (8: no bank conflicts)
+  static constexpr int PART_BYTES = SGROUPS * ROWS * PART_STRIDE * 4;      // takes the place of the copy stages
+  static constexpr int STAT_OFF = KV_OFF + (KV_BYTES > PART_BYTES ? KV_BYTES : PART_BYTES);   // [reference | sum][warp][row]
+  static constexpr int BYTES = STAT_OFF + 2 * SGROUPS * ROWS * 4;
+};
+
+template <int D>
+__global__ void __launch_bounds__(GTHREADS, 2) attn_small_kernel(const __grid_constant__ AttnParams p) {
+  using SM = SmallSmem<D>;
+  extern __shared__ __align__(128) unsigned char smem[];
+  pdl_trigger();
+  const int q_tiles = (p.t_q + SM::ROWS - 1) / SM::ROWS;
+  if ((int)blockIdx.x >= q_tiles) {
+    // cache update riding on this launch: one CTA per (destination half-tile, sequence, head)
+    const int sq = blockIdx.y, hd = blockIdx.z, j = blockIdx.x - q_tiles;
+    const int64_t src = sq * p.kv_seq + hd * p.kv_head;
+    pdl_wait();
+    if (p.k8_pool)
+      append_half_tile_fp8(p.seqs[sq].plan, p.pool_base[sq], (p.step * p.L + p.layer) * p.H + hd, j, p.k_new + src,
+                           p.v_new + src, p.kv_tok, p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, D, threadIdx.x, GTHREADS);
+    else
+      append_half_tile(p.seqs[sq].plan, p.seqs[sq].base_row, (p.step * p.L + p.layer) * p.H + hd, j, p.k_new + src,
+                       p.v_new + src, p.kv_tok, const_cast<__nv_bfloat16*>(p.k_pool), const_cast<__nv_bfloat16*>(p.v_pool),
+                       D, threadIdx.x, GTHREADS);
+    return;
+  }
+  const int grp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const int g = lane >> 2, qd = lane & 3;
+  const int seq = blockIdx.y, q0 = blockIdx.x * SM::ROWS;
+  int head, n_desc;
+  const int2* descs;
+  if (p.table_heads > 0) {
+    head = p.table_head[blockIdx.z];
+    descs = reinterpret_cast<const int2*>(p.seqs[seq].plan + p.table_desc_begin[blockIdx.z]);
+    n_desc = p.table_ndesc[blockIdx.z];
+  } else {
+    PlanView pv(p.seqs[seq].plan);
+    const int u = (p.step * p.L + p.layer) * p.H;
+    head = pv.order()[u + blockIdx.z];                   // heavy heads first
+    descs = pv.descs() + pv.attn_begin()[u + head];
+    n_desc = pv.attn_cnt()[u + head];
+  }
+  const int64_t base_row = p.seqs[seq].base_row;
+  const int n_own_tiles = (p.n_own + GN - 1) / GN, n_tiles = n_own_tiles + n_desc;
+  const uint32_t sbase = smem_u32(smem);
+  const uint32_t kvbase = sbase + SM::KV_OFF + grp * (SSTAGES * 2 * SM::CHUNK_BYTES);
+  const __nv_bfloat16* kown = p.k_new + seq * p.kv_seq + head * p.kv_head;
+  const __nv_bfloat16* vown = p.v_new + seq * p.kv_seq + head * p.kv_head;
+
+  // This warp's keys of tile j: rows [16 sub, 16 sub + n) of it.  The assignment turns with the tile, so that short tiles
+  // do not all fall to the same warps.  `dsc` is the tile's descriptor (used past the own tiles).
+  auto part_of = [&](int j, int2 dsc, int& sub) {
+    sub = (grp + 2 * j) & (SGROUPS - 1);
+    const int nv = j < n_own_tiles ? p.n_own - j * GN : dsc.y & 0xff;
+    return min(SKEYS, max(0, nv - sub * SKEYS));
+  };
+  auto load_chunk = [&](uint32_t dst, const __nv_bfloat16* src, int64_t stride, int n) {
+    constexpr int CH = D / 8;
+#pragma unroll
+    for (int i = lane; i < SKEYS * CH; i += 32) {
+      const int r = i / CH, ch = i % CH;
+      const bool ok = r < n;
+      cp_async16(dst + tile_off<D>(r, ch), ok ? src + (int64_t)r * stride + ch * 8 : src, ok ? 16 : 0);
+    }
+  };
+  auto issue = [&](int j, int2 dsc, int stage) {
+    int sub;
+    const int n = part_of(j, dsc, sub);
+    if (n <= 0) return;
+    const uint32_t dst = kvbase + stage * 2 * SM::CHUNK_BYTES;
+    if (j < n_own_tiles) {
+      const int64_t off = (int64_t)(j * GN + sub * SKEYS) * p.kv_tok;
+      load_chunk(dst, kown + off, p.kv_tok, n);
+      load_chunk(dst + SM::CHUNK_BYTES, vown + off, p.kv_tok, n);
+    } else {
+      const int64_t off = (base_row + dsc.x + sub * SKEYS) * D;
+      load_chunk(dst, p.k_pool + off, D, n);
+      load_chunk(dst + SM::CHUNK_BYTES, p.v_pool + off, D, n);
+    }
+  };
+  auto desc_of = [&](int j) { return j >= n_own_tiles && j < n_tiles ? descs[j - n_own_tiles] : make_int2(0, 0); };
+
+  // descriptors run SSTAGES tiles ahead of the products: ahead[i] belongs to the i-th tile from the current one
+  int2 ahead[SSTAGES];
+#pragma unroll
+  for (int i = 0; i < SSTAGES; ++i) ahead[i] = desc_of(i);
+  pdl_wait();
+  {
+    constexpr int CH = D / 8;
+    const __nv_bfloat16* qsrc = p.q + seq * p.q_seq + head * p.q_head + (int64_t)q0 * p.q_tok;
+#pragma unroll
+    for (int i = threadIdx.x; i < SM::ROWS * CH; i += GTHREADS) {
+      const int r = i / CH, ch = i % CH;
+      const bool ok = q0 + r < p.t_q;
+      cp_async16(sbase + SM::Q_OFF + tile_off<D>(r, ch), ok ? qsrc + (int64_t)r * p.q_tok + ch * 8 : qsrc, ok ? 16 : 0);
+    }
+  }
+  cp_async_commit();
+#pragma unroll
+  for (int i = 0; i < SSTAGES - 1; ++i) {
+    if (i < n_tiles) issue(i, ahead[i], i);
+    cp_async_commit();
+  }
+  cp_async_wait<SSTAGES - 1>();                          // Q has landed
+  __syncthreads();
+  uint32_t qf[D / 16][4];
+#pragma unroll
+  for (int ks = 0; ks < D / 16; ++ks)
+    ldmatrix_x4(qf[ks], sbase + SM::Q_OFF + tile_off<D>((lane & 7) + ((lane >> 3) & 1) * 8, ks * 2 + (lane >> 4)));
+
+  float o[D / 8][4];
+#pragma unroll
+  for (int i = 0; i < D / 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
+  float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
+  const float LOG2E = 1.4426950408889634f;
+  const float* bias_h = p.seg_bias ? p.seg_bias + head * p.K : nullptr;
+
+  for (int j = 0; j < n_tiles; ++j) {
+    const int stage = j % SSTAGES;
+    const int2 dsc = ahead[0];
+#pragma unroll
+    for (int i = 0; i + 1 < SSTAGES; ++i) ahead[i] = ahead[i + 1];
+    ahead[SSTAGES - 1] = desc_of(j + SSTAGES);
+    cp_async_wait<SSTAGES - 2>();
+    __syncwarp();                                        // the warp's chunk landed; every lane left the one before
+    if (j + SSTAGES - 1 < n_tiles) issue(j + SSTAGES - 1, ahead[SSTAGES - 2], (j + SSTAGES - 1) % SSTAGES);
+    cp_async_commit();
+    int sub;
+    const int n = part_of(j, dsc, sub);
+    if (n <= 0) continue;
+
+    const uint32_t kb = kvbase + stage * 2 * SM::CHUNK_BYTES, vb = kb + SM::CHUNK_BYTES;
+    float s[2][4] = {};
+#pragma unroll
+    for (int ks = 0; ks < D / 16; ++ks) {
+      uint32_t b[4];
+      ldmatrix_x4(b, kb + tile_off<D>((lane & 7) + (lane >> 4) * 8, ks * 2 + ((lane >> 3) & 1)));
+      mma_bf16(s[0], qf[ks], b[0], b[1]);
+      mma_bf16(s[1], qf[ks], b[2], b[3]);
+    }
+    const float bias = bias_h ? bias_h[j < n_own_tiles ? p.step : (dsc.y >> 8) & 0xff] * LOG2E : 0.f;
+    float mx[2] = {-INFINITY, -INFINITY}, psum[2] = {0.f, 0.f}, corr[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float v = i * 8 + qd * 2 + (e & 1) < n ? fmaf(s[i][e], p.scale_log2, bias) : -INFINITY;
+        s[i][e] = v;
+        mx[e >> 1] = fmaxf(mx[e >> 1], v);
+      }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 1));
+      mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 2));
+      const float m_new = fmaxf(m_run[r], mx[r]);
+      corr[r] = exp2f(m_run[r] - m_new);
+      m_run[r] = m_new;
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        s[i][e] = exp2f(s[i][e] - m_run[e >> 1]);
+        psum[e >> 1] += s[i][e];
+      }
+    l_run[0] = l_run[0] * corr[0] + psum[0];
+    l_run[1] = l_run[1] * corr[1] + psum[1];
+    if (__any_sync(0xffffffffu, corr[0] != 1.f || corr[1] != 1.f)) {
+#pragma unroll
+      for (int i = 0; i < D / 8; ++i) {
+        o[i][0] *= corr[0];
+        o[i][1] *= corr[0];
+        o[i][2] *= corr[1];
+        o[i][3] *= corr[1];
+      }
+    }
+    uint32_t pa[4] = {pack_bf16(s[0][0], s[0][1]), pack_bf16(s[0][2], s[0][3]), pack_bf16(s[1][0], s[1][1]),
+                      pack_bf16(s[1][2], s[1][3])};
+#pragma unroll
+    for (int dp = 0; dp < D / 16; ++dp) {
+      uint32_t b[4];
+      ldmatrix_x4_trans(b, vb + tile_off<D>((lane & 7) + ((lane >> 3) & 1) * 8, dp * 2 + (lane >> 4)));
+      mma_bf16(o[2 * dp], pa, b[0], b[1]);
+      mma_bf16(o[2 * dp + 1], pa, b[2], b[3]);
+    }
+  }
+  cp_async_wait<0>();
+  __syncthreads();                                       // the copy stages are free: the partial results take their place
+
+  float* part = reinterpret_cast<float*>(smem + SM::KV_OFF);
+  float* stat = reinterpret_cast<float*>(smem + SM::STAT_OFF);
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int row = g + r * 8;
+    float l = l_run[r];
+    l += __shfl_xor_sync(0xffffffffu, l, 1);
+    l += __shfl_xor_sync(0xffffffffu, l, 2);
+    if (qd == 0) {
+      stat[grp * SM::ROWS + row] = m_run[r];
+      stat[(SGROUPS + grp) * SM::ROWS + row] = l;
+    }
+    float* dst = part + (grp * SM::ROWS + row) * SM::PART_STRIDE + qd * 2;
+#pragma unroll
+    for (int i = 0; i < D / 8; ++i) *reinterpret_cast<float2*>(dst + i * 8) = make_float2(o[i][2 * r], o[i][2 * r + 1]);
+  }
+  __syncthreads();
+  constexpr int CH = D / 8;
+  __nv_bfloat16* out = p.out + seq * p.o_seq + head * p.o_head + (int64_t)q0 * p.o_tok;
+#pragma unroll
+  for (int i = threadIdx.x; i < SM::ROWS * CH; i += GTHREADS) {
+    const int row = i / CH, ch = i % CH;
+    if (q0 + row >= p.t_q) continue;
+    // every row sees at least one key, so the largest reference is finite; a warp without keys weighs nothing
+    float w[SGROUPS], m = -INFINITY, l = 0.f, acc[8] = {};
+#pragma unroll
+    for (int k = 0; k < SGROUPS; ++k) m = fmaxf(m, stat[k * SM::ROWS + row]);
+#pragma unroll
+    for (int k = 0; k < SGROUPS; ++k) {
+      w[k] = exp2f(stat[k * SM::ROWS + row] - m);
+      l = fmaf(stat[(SGROUPS + k) * SM::ROWS + row], w[k], l);
+    }
+    const float inv = 1.f / l;
+#pragma unroll
+    for (int k = 0; k < SGROUPS; ++k) {
+      const float4* src = reinterpret_cast<const float4*>(part + (k * SM::ROWS + row) * SM::PART_STRIDE + ch * 8);
+      const float4 a = src[0], b = src[1];
+      const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+      for (int e = 0; e < 8; ++e) acc[e] = fmaf(v[e], w[k], acc[e]);
+    }
+    *reinterpret_cast<int4*>(out + (int64_t)row * p.o_tok + ch * 8) =
+        make_int4((int)pack_bf16(acc[0] * inv, acc[1] * inv), (int)pack_bf16(acc[2] * inv, acc[3] * inv),
+                  (int)pack_bf16(acc[4] * inv, acc[5] * inv), (int)pack_bf16(acc[6] * inv, acc[7] * inv));
+  }
+}
+
 // beta[head][step][sg] += sum of the partials of that head in the order (sequence, query tile, warp):
 // one thread per (head, source scale), so the result does not depend on scheduling.
 __global__ void reduce_partials_kernel(const float* partials, float* beta_row, int n_qtiles, int H, int n_seq, int K,
@@ -476,24 +732,41 @@ __global__ void reduce_partials_kernel(const float* partials, float* beta_row, i
 
 constexpr int MAX_DEVICES = 64;
 
-template <int D, bool CALIB, int GROUPS = 1>
-static cudaError_t launch_one(const AttnParams& p, int n_seq, cudaStream_t stream) {
-  auto kern = attn_generic_kernel<D, CALIB, false, GROUPS>;
-  constexpr int bytes = CALIB ? GenericSmem<D>::BYTES : GenericSmem<D, GROUPS>::ATTN_BYTES;
-  // the attribute belongs to the (function, device) pair: set it once on every device that launches
+// the attribute belongs to the (function, device) pair: set it once on every device that launches
+template <auto KERN>
+static cudaError_t allow_smem(int bytes) {
   static std::atomic<bool> configured[MAX_DEVICES];
   int dev = -1;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= MAX_DEVICES) return cudaErrorInvalidDevice;
   if (!configured[dev].load(std::memory_order_acquire)) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    e = cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e != cudaSuccess) return e;
     configured[dev].store(true, std::memory_order_release);
   }
+  return cudaSuccess;
+}
+
+template <int D, bool CALIB, int GROUPS = 1>
+static cudaError_t launch_one(const AttnParams& p, int n_seq, cudaStream_t stream) {
+  constexpr auto kern = attn_generic_kernel<D, CALIB, false, GROUPS>;
+  constexpr int bytes = CALIB ? GenericSmem<D>::BYTES : GenericSmem<D, GROUPS>::ATTN_BYTES;
+  cudaError_t e = allow_smem<kern>(bytes);
+  if (e != cudaSuccess) return e;
   const int q_tiles = CALIB && p.cal_n > 0 ? p.cal_tile_begin[p.cal_n] : (p.t_q + GM - 1) / GM;
   dim3 grid(q_tiles + (CALIB ? 0 : p.append_tiles), CALIB ? p.H : n_seq, CALIB ? n_seq : p.H);
   return launch_pdl(kern, grid, GTHREADS * GROUPS, bytes, stream, p);
+}
+
+template <int D>
+static cudaError_t launch_small(const AttnParams& p, int n_seq, cudaStream_t stream) {
+  constexpr auto kern = attn_small_kernel<D>;
+  constexpr int bytes = SmallSmem<D>::BYTES;
+  cudaError_t e = allow_smem<kern>(bytes);
+  if (e != cudaSuccess) return e;
+  dim3 grid((p.t_q + SmallSmem<D>::ROWS - 1) / SmallSmem<D>::ROWS + p.append_tiles, n_seq, p.H);
+  return launch_pdl(kern, grid, GTHREADS, bytes, stream, p);
 }
 
 // Calibration pass whose scratch is the static array above.  Returns cudaErrorInvalidValue when the
@@ -549,13 +822,17 @@ cudaError_t launch_calibrate_static(const AttnParams& p_in, int d, int n_seq, cu
                     n_seq, p.K, p.step);
 }
 
-// `n_sm`: SMs of the device.  Two groups of warps per CTA while every CTA has an SM to itself and heads see more than one
-// key half-tile; a fuller launch keeps two single-group CTAs per SM (the same warps per SM, and nothing to merge).
+// `n_sm`: SMs of the device.  16-query CTAs while two of them per SM hold the launch (or the step has no more queries than
+// that: then nothing is read twice); else two groups of warps per 64-query CTA while every CTA has an SM to itself and heads
+// see more than one key half-tile; a fuller launch keeps two single-group CTAs per SM (the same warps per SM, and nothing
+// to merge).
 cudaError_t launch_attn_generic(const AttnParams& p, int d, int n_seq, bool calib, int n_sm, cudaStream_t stream) {
   if (d != 64 && d != 128) return cudaErrorInvalidValue;
   if (calib) return d == 128 ? launch_one<128, true>(p, n_seq, stream) : launch_one<64, true>(p, n_seq, stream);
-  const int64_t ctas = (int64_t)((p.t_q + GM - 1) / GM) * n_seq * p.H;
-  if (p.step > 0 && ctas <= n_sm)
+  const int64_t units = (int64_t)n_seq * p.H;
+  if (p.t_q <= 16 || (p.t_q + 15) / 16 * units <= 2 * n_sm)
+    return d == 128 ? launch_small<128>(p, n_seq, stream) : launch_small<64>(p, n_seq, stream);
+  if (p.step > 0 && (p.t_q + GM - 1) / GM * units <= n_sm)
     return d == 128 ? launch_one<128, false, 2>(p, n_seq, stream) : launch_one<64, false, 2>(p, n_seq, stream);
   return d == 128 ? launch_one<128, false>(p, n_seq, stream) : launch_one<64, false>(p, n_seq, stream);
 }

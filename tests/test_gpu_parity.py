@@ -235,6 +235,21 @@ def test_attention_with_cache_update_in_one_call(hk, layout, kernel):
         assert n == sh.K * sh.L                      # one launch per (step, layer): every update here is small
 
 
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+@pytest.mark.parametrize("H,n_seq", [(3, 2), (24, 4)], ids=["few_units", "many_units"])
+def test_small_steps_ragged_sizes(hk, d, H, n_seq):
+    """Query and key counts around the edges of the warp-level kernels' tiles (16 queries, 16 keys of a 64-key half-tile:
+    9, 16, 25, 49, 81, 121), with few units (16-query CTAs throughout) and with many (both 64-query forms); the cache
+    update rides along."""
+    sh = W.Shape("ragged_small", L=1, H=H, d=d, sides=(1, 3, 4, 5, 7, 9, 11), n_seq=n_seq, s=2)
+    scores = W.synthetic_scas(sh, 11)
+    ref = O.heatkv_schedule(scores, 0.5, sh.s, sh.sides)
+    bias = W.seg_bias_prior_lognormal(sh, 11)
+    heads = None if H < 8 else [(0, 0, 0), (3, 0, H - 1), (1, 0, 7), (2, 0, 16)]
+    _run_full_parity(hk, sh, ref, lambda ses: ses.schedule(scas=scores, b=0.5), hk.LAYOUT_PAGED, bias=bias,
+                     kernel=hk.KERNEL_GENERIC, check_heads=heads, fused=True)
+
+
 def test_config2_one_call_per_step_all_units(hk):
     sh = W.CFG2
     scores = W.synthetic_scas(sh, 0)
