@@ -1,21 +1,23 @@
-"""Builds libheatkv.so (CUDA kernels + C ABI) in-tree for sm_100a with nvcc."""
+"""Builds libheatkv.so (CUDA kernels + C ABI) in-tree for sm_100a with nvcc, and the call sequencer _native beside it."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libheatkv.so")
+NATIVE = os.path.join(HERE, "_native" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 SOURCES = ["schedule.cpp", "plan.cpp", "split.cpp", "api.cu", "attn_generic.cu", "attn_tc.cu", "calib_tc.cu", "cache_kernels.cu"]
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(NATIVE):
         return True
-    lib_t = os.path.getmtime(LIB)
+    lib_t = min(os.path.getmtime(LIB), os.path.getmtime(NATIVE))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "heatkv.h")]
     return any(os.path.getmtime(p) > lib_t for p in deps)
 
@@ -48,6 +50,9 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
         raise RuntimeError("nvcc failed")
     link = [nvcc, "-shared", "-o", LIB] + objs + ["-gencode", "arch=compute_100a,code=sm_100a", "-lcudart"]
     subprocess.run(link, check=True)
+    subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                    "-I", os.path.join(ROOT, "include"), os.path.join(CSRC, "native_module.c"), "-o", NATIVE, "-L", HERE,
+                    "-l:libheatkv.so", "-Wl,-rpath,$ORIGIN"], check=True)
     return LIB
 
 

@@ -73,10 +73,7 @@ class Strides(C.Structure):
     def of(cls, q: torch.Tensor, kv: torch.Tensor, o: Optional[torch.Tensor] = None) -> "Strides":
         """Strides of [n_seq, H, t, d] views (d contiguous)."""
         sq, skv = q.stride(), kv.stride()
-        return cls._of(sq, skv, sq if o is None else o.stride())
-
-    @classmethod
-    def _of(cls, sq, skv, so) -> "Strides":
+        so = sq if o is None else o.stride()
         for s in (sq, skv, so):
             assert len(s) == 4 and s[3] == 1
         return cls(*sq[:3], *skv[:3], *so[:3])
@@ -186,8 +183,6 @@ def _check(rc: int, where: str) -> None:
 
 
 def _ids(seq_ids: Sequence[int]):
-    if isinstance(seq_ids, C.Array):                   # converted before (Session.generate)
-        return seq_ids, len(seq_ids)
     return (C.c_int * len(seq_ids))(*[int(i) for i in seq_ids]), len(seq_ids)
 
 

@@ -7,7 +7,10 @@ from typing import Callable, Optional, Sequence
 
 import torch
 
+from . import _native
 from . import heatkv as hk
+
+_native.set_hooks(hk._check, torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
 
 
 class Session:
@@ -53,17 +56,7 @@ class Session:
     def run_layer_step(self, seq_ids, layer: int, step: int, q, k, v, out, seg_bias=None, fused: bool = False) -> None:
         """q, k, v, out: [n_seq, H, n_tokens, d] tensors holding all scales; uses the slice of `step`.
         `fused`: one heatkv_attention_append call instead of attention followed by the cache update."""
-        # The step's slice as base pointers: building the four views x[:, :, lo:hi] costs 8 us, as much as the launch.
-        lo = self.c[step] - self.t[step]
-        sq, sk, so = q.stride(), k.stride(), out.stride()
-        qp, op = q.data_ptr() + 2 * lo * sq[2], out.data_ptr() + 2 * lo * so[2]
-        kp, vp = k.data_ptr() + 2 * lo * sk[2], v.data_ptr() + 2 * lo * sk[2]
-        st = hk.Strides._of(sq, sk, so)
-        if fused:
-            hk.heatkv_attention_append(self.ctx, seq_ids, layer, step, qp, kp, vp, st, seg_bias, op)
-            return
-        hk.heatkv_scale_attention(self.ctx, seq_ids, layer, step, qp, kp, vp, st, seg_bias, op)
-        hk.heatkv_append_compact(self.ctx, seq_ids, layer, step, kp, vp, st)
+        _native.run_layer_step(self.ctx, seq_ids, layer, step, self.c[step] - self.t[step], q, k, v, out, seg_bias, fused)
 
     def pre_step(self, seq_ids, step: int) -> None:
         hk.heatkv_append_compact(self.ctx, seq_ids, -1, step, None, None, None)
@@ -72,12 +65,5 @@ class Session:
                  bias_of: Optional[Callable[[int, int], Optional[torch.Tensor]]] = None,
                  after: Optional[Callable[[int, int], None]] = None, fused: bool = False) -> None:
         """Whole sweep: steps outer, layers inner.  `after(step, layer)` runs after each layer."""
-        seq_ids = hk._ids(seq_ids)[0]
-        for step in range(self.K):
-            self.pre_step(seq_ids, step)
-            for layer in range(self.L):
-                q, k, v = qkv_of_layer(layer)
-                bias = bias_of(layer, step) if bias_of else None
-                self.run_layer_step(seq_ids, layer, step, q, k, v, out_of_layer(layer), bias, fused)
-                if after:
-                    after(step, layer)
+        _native.generate(self.ctx, seq_ids, tuple(c - t for c, t in zip(self.c, self.t)), self.L, qkv_of_layer, out_of_layer,
+                         bias_of, after, fused)
