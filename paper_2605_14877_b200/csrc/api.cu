@@ -303,7 +303,7 @@ void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int 
   for (int i = 1; i < n_seq && one_plan; ++i) one_plan = ctx->seqs[seq_ids[i]].plan == ctx->seqs[seq_ids[0]].plan;
   const std::vector<int> tiles = ordered_tiles(pe0, step, layer, own_slots);
   const int H = (int)tiles.size();
-  for (int t : tiles) one_plan = one_plan && t <= 32767;
+  for (int t : tiles) one_plan = one_plan && t <= 16383;          // half-tile counts travel as 16 bits
   const uint64_t key = (pe0.uid << 24) ^ ((uint64_t)step << 20) ^ ((uint64_t)layer << 8) ^ (uint64_t)n_seq ^
                        (one_plan ? 0ull : 1ull << 63);
   auto fits = [&](const SplitShape& sh) {
@@ -344,8 +344,13 @@ void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int 
   p->table_heads = 0;
   p->longest_piece = 0;
   if (one_plan) {
-    const int32_t* order = pe0.plan.blob.data() + pe0.plan.header().off_order + pe0.sched.at(step, layer, 0);
+    const PlanHeader& hdr = pe0.plan.header();
+    const int32_t* blob = pe0.plan.blob.data();
+    const size_t at = pe0.sched.at(step, layer, 0);
+    const int32_t *order = blob + hdr.off_order + at, *cnt = blob + hdr.off_attn_cnt + at, *begin = blob + hdr.off_attn_begin + at;
     for (int i = 0; i < H; ++i) {
+      p->table_ndesc[i] = (int16_t)cnt[order[i]];
+      p->table_desc_begin[i] = hdr.off_desc + 2 * begin[order[i]];
       p->table_head[i] = (int16_t)order[i];
       p->table_tiles[i] = (int16_t)tiles[i];
       p->table_split[i] = (int16_t)ch.ns[i];

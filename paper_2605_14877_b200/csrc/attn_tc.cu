@@ -210,7 +210,8 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_ptr_smem;
-  pdl_wait();
+  // (every role waits for the launches before this one where it first touches what they may still use; the MMA warp only
+  // follows the others' barriers)
 
   // register budget per warpgroup: 128*72 + 256*216 <= 64K
   if (warp < 4) {
@@ -230,6 +231,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
       // one fetch past the end, so the launch makes exactly attn_items fetches and the last resets the counter.
       int idx = blockIdx.x;
       if (it > 0) {
+        if (it == 1) pdl_wait();
         uint32_t old = 0;
         if (lane == 0) {
           old = atomicAdd(work_counter, 1u);
@@ -303,8 +305,8 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             ring[W_SUB] = item - excl;                        // piece * n_qp + query tile pair
             ring[W_SLOT] = slots_before + sinc - scnt;        // first partial slot of this head
             ring[W_CTR] = ctrs_before + cinc - ccnt;          // first arrival counter group of this head
-            ring[W_DESC] = pv.attn_begin()[u + h];
-            ring[W_NDESC] = pv.attn_cnt()[u + h];
+            ring[W_DESC] = p.table_heads > 0 ? p.table_desc_begin[i] : pv.w[4] + 2 * pv.attn_begin()[u + h];
+            ring[W_NDESC] = p.table_heads > 0 ? (int)p.table_ndesc[i] : pv.attn_cnt()[u + h];
             ring[W_KIND] = ATTENTION;
           }
           const bool any = __any_sync(0xffffffffu, mine);
@@ -321,7 +323,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
       __syncwarp();
       if (leader) mbar_arrive(bar(ITEM_FULL + slot));
       if (!is_attn) continue;
-      const int2* descs = FULL ? p.full_descs : PlanView(p.seqs[seq].plan).descs() + im.desc_begin;
+      const int2* descs = FULL ? p.full_descs : reinterpret_cast<const int2*>(p.seqs[seq].plan + im.desc_begin);
       const int64_t base_row = FULL ? 0 : p.seqs[seq].base_row;
       for (int j = 0; j < im.n_tiles && ok; ++j, ++g) {
         const uint32_t st = g % KV_STAGES;
@@ -329,6 +331,8 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
         Slot sl[2];
         for (int hf = 0; hf < 2; ++hf)
           sl[hf] = get_slot<FULL>(2 * (im.j0 + j) + hf, descs, im.n_desc, im.n_slots, base_row, p.n_own, p.step);
+        // the first item is decoded and its descriptors are read while the launch before may still run
+        if (g == 0) pdl_wait();
         // K first: the S product of the next tile needs it earliest
         if (use > 0) ok = warp_wait(bar(K_EMPTY + st), (use - 1) & 1, abort_flag, p.status);
         if (!ok) break;
@@ -503,6 +507,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
     // Each warp takes destination half-tiles of (sequence, head) units from a counter of its own and copies
     // their rows while the other warps work on attention items.  Every store warp of the launch ends with one
     // fetch past the end; the last of those store_items + 2 * CTAs fetches resets the counter.
+    pdl_wait();
     uint32_t* store_counter = p.status + STORE_COUNTER_WORD;
     const uint32_t fetches = (uint32_t)p.store_items + 2u * gridDim.x;
     for (;;) {
@@ -531,6 +536,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
     const float LOG2E = 1.4426950408889634f;
     uint32_t cx = 0;                                    // key tiles of this query tile so far (all items)
     uint32_t items_x = 0;                               // items in which this query tile held rows so far
+    pdl_wait();
     bool ok = true;
     for (uint32_t it = 0; ok; ++it) {
       const uint32_t slot = it & 1;
@@ -554,7 +560,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
           {
             const Item im = read_item<FULL>(ring, p, n_qp);
             j0 = im.j0; n_desc = im.n_desc; n_slots = im.n_slots;
-            descs = FULL ? p.full_descs : PlanView(p.seqs[im.seq].plan).descs() + im.desc_begin;
+            descs = FULL ? p.full_descs : reinterpret_cast<const int2*>(p.seqs[im.seq].plan + im.desc_begin);
             bias_h = p.seg_bias ? p.seg_bias + im.head * p.K : nullptr;
           }
           float m_ref = -INFINITY, l_sum = 0.f;
