@@ -141,9 +141,10 @@ typedef struct {
  * exactly.  Attention in such a context is attention over x^ for the cached scales (the step's own K/V come
  * from k_new / v_new unquantised, as always): before the attention kernel runs, the call expands the visible
  * head-scales of its (layer, step) into bf16 staging rows inside the arena (stage_bytes), and the attention
- * kernels read those; the update after the layer quantises the new rows on their way into the pool.  Inputs
- * must be finite.  Only the paged layout is supported; heatkv_attention_append runs the expansion as a kernel of its
- * own, and the update inside the attention launch only on the generic kernel (small steps).  A call whose sequences need more staging rows than stage_bytes holds returns
+ * kernels read those (the warp-level kernel of the smallest steps reads the codes themselves); the update after the layer
+ * quantises the new rows on their way into the pool.  Inputs must be finite.  Only the paged layout is supported; in
+ * heatkv_attention_append the update rides on the attention launch of the warp-level kernel (small steps) and on the
+ * expansion before the tensor-memory kernel.  A call whose sequences need more staging rows than stage_bytes holds returns
  * HEATKV_ERR_OUT_OF_PAGES (rows needed per sequence: the largest number of visible 64-row half-tiles of any
  * (layer, step) of its schedule, times 64).
  *

@@ -17,7 +17,8 @@ cudaError_t launch_calibrate_static(const AttnParams& p, int d, int n_seq, cudaS
 cudaError_t launch_append(const CopyParams& p, int n_seq, cudaStream_t stream);
 cudaError_t launch_compact(const CopyParams& p, int n_seq, cudaStream_t stream);
 cudaError_t launch_append_fp8(const CopyParams& p, int n_seq, cudaStream_t stream);
-cudaError_t launch_dequant_fp8(const CopyParams& p, int n_seq, int slots, cudaStream_t stream);
+cudaError_t launch_stage_fp8(const CopyParams& p, int n_seq, int slots, bool update, cudaStream_t stream);
+bool attn_is_small(int t_q, int64_t units, int n_sm);
 struct TcState;
 int tc_create(const heatkv_config& cfg, void* k_pool, void* v_pool, uint64_t pool_rows, TcState** out);
 void tc_destroy(TcState* st);
@@ -289,6 +290,8 @@ void fill_head_table(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, i
     p->table_ndesc[i] = (int16_t)cnt[order[i]];
     p->table_desc_begin[i] = hdr.off_desc + 2 * begin[order[i]];
   }
+  p->off_desc = hdr.off_desc;
+  p->off_src = hdr.off_src;
   p->table_heads = pe0.sched.H;
 }
 
@@ -669,10 +672,13 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
   // from there on the warp-level kernel is bound by its mma.sync rate (144 queries, 128 units: 52 us against 23 us)
   if (choice == HEATKV_KERNEL_AUTO && !(p.t_q >= 256 || (p.t_q >= 128 && (int64_t)n_seq * ctx->cfg.H >= 64))) use_tc = false;
   if (choice == HEATKV_KERNEL_TCGEN05 && !use_tc) return HEATKV_ERR_INVALID_ARG;   // never a silent substitute
+  bool updated = false;                                       // the cache update already went along
   if (ctx->fp8) {
-    // The attention kernels read bf16 rows: expand the visible head-scales of this (layer, step) from the code
-    // pools into the staging rows first (every sequence gets the rows its plan needs, one after the other),
-    // then point the kernels' row numbering at them.
+    // The attention kernels read bf16 rows (all but the small-step kernel): expand the visible head-scales of this (layer,
+    // step) from the code pools into the staging rows first (every sequence gets the rows its plan needs, one after the
+    // other), then point the kernels' row numbering at them.  The tensor-memory kernel does not carry the quantising
+    // update (the same branch in its spare warps measured 1.5 % on the bf16 path's largest launch and 8 % on its
+    // smallest); there it goes with the expansion.
     CopyParams cp;
     std::memset(&cp, 0, sizeof(cp));
     cp.k_pool = ctx->k_pool; cp.v_pool = ctx->v_pool;
@@ -692,8 +698,15 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
       next += (uint64_t)count * HEATKV_PAGE_TOKENS;
     }
     if (next > ctx->stage_rows) return HEATKV_ERR_OUT_OF_PAGES;
-    if (launch_dequant_fp8(cp, n_seq, slots, stream) != cudaSuccess) return HEATKV_ERR_CUDA;
-    if (slots > 0) {
+    p.direct8 = !use_tc && attn_is_small(p.t_q, (int64_t)n_seq * ctx->cfg.H, ctx->n_sm);
+    updated = with_update && stores && use_tc;
+    if (updated) {
+      cp.k_new = p.k_new; cp.v_new = p.v_new;
+      cp.kv_seq = s.kv_seq; cp.kv_head = s.kv_head; cp.kv_tok = s.kv_tok;
+      cp.t_k = ctx->cfg.t[step];
+    }
+    if (!p.direct8 && (slots > 0 || updated)) {
+      if (launch_stage_fp8(cp, n_seq, slots, updated, stream) != cudaSuccess) return HEATKV_ERR_CUDA;
       ctx->launches += 1;
       ctx->kstats.other += 1;
     }
@@ -703,9 +716,7 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
     }
     p.k8_pool = ctx->k8_pool; p.v8_pool = ctx->v8_pool; p.k_exp = ctx->k_exp; p.v_exp = ctx->v_exp;
   }
-  // fp8 cache: only the generic kernel carries the quantising update (the same branch in the tensor-memory kernel's
-  // spare warps measured 1.5 % on the bf16 path's largest launch and 8 % on its smallest)
-  bool fuse = with_update && stores && ctx->cfg.layout == HEATKV_LAYOUT_PAGED && !(ctx->fp8 && use_tc);
+  bool fuse = with_update && stores && ctx->cfg.layout == HEATKV_LAYOUT_PAGED && !updated;
   if (fuse) {
     // The tensor-memory kernel copies the new rows with two spare warps per SM beside the attention work, so
     // the update rides along whatever its size.  The generic kernel carries it as extra CTAs of its own
@@ -740,7 +751,7 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
   }
   if (e != cudaSuccess) return HEATKV_ERR_CUDA;
   if (!with_update) return HEATKV_OK;
-  if (fuse || !stores) {
+  if (fuse || updated || !stores) {
     for (int i = 0; i < n_seq; ++i) ctx->seqs[seq_ids[i]].done_step[layer] = (int16_t)step;
     return HEATKV_OK;
   }

@@ -479,11 +479,15 @@ struct SmallSmem {
   static constexpr int KV_BYTES = SGROUPS * SSTAGES * 2 * CHUNK_BYTES;
   static constexpr int PART_STRIDE = D + 8;                         // floats per row of a partial O (8: no bank conflicts)
   static constexpr int PART_BYTES = SGROUPS * ROWS * PART_STRIDE * 4;      // takes the place of the copy stages
-  static constexpr int STAT_OFF = KV_OFF + (KV_BYTES > PART_BYTES ? KV_BYTES : PART_BYTES);   // [reference | sum][warp][row]
+  static_assert(PART_BYTES <= KV_BYTES, "partial results");
+  static constexpr int STAT_OFF = KV_OFF + KV_BYTES;   // [reference | sum][warp][row]
   static constexpr int BYTES = STAT_OFF + 2 * SGROUPS * ROWS * 4;
 };
 
-template <int D>
+// FP8: the cached keys are read from the code pools themselves (a chunk's codes land in its place in shared memory and are
+// widened there), so a small step of such a context needs no expansion launch before it (4 x 16 units, 4 queries: 6.4 -> 3.5 us,
+// 64 queries: 12.3 -> 8.1).
+template <int D, bool FP8>
 __global__ void __launch_bounds__(GTHREADS, 2) attn_small_kernel(const __grid_constant__ AttnParams p) {
   using SM = SmallSmem<D>;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -519,12 +523,19 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_small_kernel(const __grid_co
     descs = pv.descs() + pv.attn_begin()[u + head];
     n_desc = pv.attn_cnt()[u + head];
   }
-  const int64_t base_row = p.seqs[seq].base_row;
+  const int64_t base_row = FP8 ? p.pool_base[seq] : p.seqs[seq].base_row;
   const int n_own_tiles = (p.n_own + GN - 1) / GN, n_tiles = n_own_tiles + n_desc;
   const uint32_t sbase = smem_u32(smem);
   const uint32_t kvbase = sbase + SM::KV_OFF + grp * (SSTAGES * 2 * SM::CHUNK_BYTES);
   const __nv_bfloat16* kown = p.k_new + seq * p.kv_seq + head * p.kv_head;
   const __nv_bfloat16* vown = p.v_new + seq * p.kv_seq + head * p.kv_head;
+
+  const int32_t* src_rows = nullptr;                     // FP8: the pool rows behind the head's descriptors
+  if (FP8) {
+    const int32_t* plan = p.seqs[seq].plan;
+    const int off_desc = p.table_heads > 0 ? p.off_desc : plan[4], off_src = p.table_heads > 0 ? p.off_src : plan[17];
+    src_rows = plan + off_src + (reinterpret_cast<const int32_t*>(descs) - (plan + off_desc)) / 2;
+  }
 
   // This warp's keys of tile j: rows [16 sub, 16 sub + n) of it.  The assignment turns with the tile, so that short tiles
   // do not all fall to the same warps.  `dsc` is the tile's descriptor (used past the own tiles).
@@ -542,7 +553,16 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_small_kernel(const __grid_co
       cp_async16(dst + tile_off<D>(r, ch), ok ? src + (int64_t)r * stride + ch * 8 : src, ok ? 16 : 0);
     }
   };
-  auto issue = [&](int j, int2 dsc, int stage) {
+  auto load_codes = [&](uint32_t dst, const uint8_t* src, int n) {          // rows of D codes, one after the other
+    constexpr int CH = D / 16;
+#pragma unroll
+    for (int i = lane; i < SKEYS * CH; i += 32) {
+      const bool ok = i / CH < n;
+      cp_async16(dst + i * 16, ok ? src + i * 16 : src, ok ? 16 : 0);
+    }
+  };
+  // FP8: exponent byte of K row `lane` (lanes 0..15) or V row `lane - 16` of the chunk
+  auto issue = [&](int j, int2 dsc, int stage, int& exponent) {
     int sub;
     const int n = part_of(j, dsc, sub);
     if (n <= 0) return;
@@ -551,16 +571,50 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_small_kernel(const __grid_co
       const int64_t off = (int64_t)(j * GN + sub * SKEYS) * p.kv_tok;
       load_chunk(dst, kown + off, p.kv_tok, n);
       load_chunk(dst + SM::CHUNK_BYTES, vown + off, p.kv_tok, n);
+    } else if (FP8) {
+      const int64_t r0 = base_row + dsc.x + sub * SKEYS;
+      load_codes(dst, p.k8_pool + r0 * D, n);
+      load_codes(dst + SM::CHUNK_BYTES, p.v8_pool + r0 * D, n);
+      const int r = lane & 15;
+      exponent = r < n ? (lane < 16 ? p.k_exp : p.v_exp)[r0 + r] : 0;
     } else {
       const int64_t off = (base_row + dsc.x + sub * SKEYS) * D;
       load_chunk(dst, p.k_pool + off, D, n);
       load_chunk(dst + SM::CHUNK_BYTES, p.v_pool + off, D, n);
     }
   };
-  auto desc_of = [&](int j) { return j >= n_own_tiles && j < n_tiles ? descs[j - n_own_tiles] : make_int2(0, 0); };
+  // codes of a chunk -> bf16 rows in the swizzled layout, in place
+  auto widen = [&](unsigned char* chunk, int exponent, int first_lane) {
+    constexpr int CH = D / 8, PER_LANE = SKEYS * CH / 32;
+    uint2 c[PER_LANE];
+#pragma unroll
+    for (int i = 0; i < PER_LANE; ++i) c[i] = *reinterpret_cast<const uint2*>(chunk + (lane + 32 * i) * 8);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < PER_LANE; ++i) {
+      const int r = (lane + 32 * i) / CH, ch = (lane + 32 * i) % CH;
+      const float scale = pow2f(__shfl_sync(0xffffffffu, exponent, first_lane + r));
+      const uint32_t w[4] = {c[i].x & 0xffffu, c[i].x >> 16, c[i].y & 0xffffu, c[i].y >> 16};
+      uint32_t o[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float lo, hi;
+        from_e4m3x2(w[q], lo, hi);
+        o[q] = pack_bf16(lo * scale, hi * scale);          // exact, as in the expansion kernel
+      }
+      *reinterpret_cast<int4*>(chunk + tile_off<D>(r, ch)) = make_int4((int)o[0], (int)o[1], (int)o[2], (int)o[3]);
+    }
+  };
+  auto desc_of = [&](int j) {
+    if (j < n_own_tiles || j >= n_tiles) return make_int2(0, 0);
+    int2 d = descs[j - n_own_tiles];
+    if (FP8) d.x = src_rows[j - n_own_tiles];
+    return d;
+  };
 
   // descriptors run SSTAGES tiles ahead of the products: ahead[i] belongs to the i-th tile from the current one
   int2 ahead[SSTAGES];
+  int exps[SSTAGES] = {};
 #pragma unroll
   for (int i = 0; i < SSTAGES; ++i) ahead[i] = desc_of(i);
   pdl_wait();
@@ -577,7 +631,7 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_small_kernel(const __grid_co
   cp_async_commit();
 #pragma unroll
   for (int i = 0; i < SSTAGES - 1; ++i) {
-    if (i < n_tiles) issue(i, ahead[i], i);
+    if (i < n_tiles) issue(i, ahead[i], i, exps[i]);
     cp_async_commit();
   }
   cp_async_wait<SSTAGES - 1>();                          // Q has landed
@@ -600,15 +654,23 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_small_kernel(const __grid_co
 #pragma unroll
     for (int i = 0; i + 1 < SSTAGES; ++i) ahead[i] = ahead[i + 1];
     ahead[SSTAGES - 1] = desc_of(j + SSTAGES);
+    const int exponent = exps[0];
+#pragma unroll
+    for (int i = 0; i + 1 < SSTAGES; ++i) exps[i] = exps[i + 1];
     cp_async_wait<SSTAGES - 2>();
     __syncwarp();                                        // the warp's chunk landed; every lane left the one before
-    if (j + SSTAGES - 1 < n_tiles) issue(j + SSTAGES - 1, ahead[SSTAGES - 2], (j + SSTAGES - 1) % SSTAGES);
+    if (j + SSTAGES - 1 < n_tiles) issue(j + SSTAGES - 1, ahead[SSTAGES - 2], (j + SSTAGES - 1) % SSTAGES, exps[SSTAGES - 2]);
     cp_async_commit();
     int sub;
     const int n = part_of(j, dsc, sub);
     if (n <= 0) continue;
 
     const uint32_t kb = kvbase + stage * 2 * SM::CHUNK_BYTES, vb = kb + SM::CHUNK_BYTES;
+    if (FP8 && j >= n_own_tiles) {
+      widen(smem + (kb - sbase), exponent, 0);
+      widen(smem + (vb - sbase), exponent, 16);
+      __syncwarp();
+    }
     float s[2][4] = {};
 #pragma unroll
     for (int ks = 0; ks < D / 16; ++ks) {
@@ -759,9 +821,9 @@ static cudaError_t launch_one(const AttnParams& p, int n_seq, cudaStream_t strea
   return launch_pdl(kern, grid, GTHREADS * GROUPS, bytes, stream, p);
 }
 
-template <int D>
+template <int D, bool FP8>
 static cudaError_t launch_small(const AttnParams& p, int n_seq, cudaStream_t stream) {
-  constexpr auto kern = attn_small_kernel<D>;
+  constexpr auto kern = attn_small_kernel<D, FP8>;
   constexpr int bytes = SmallSmem<D>::BYTES;
   cudaError_t e = allow_smem<kern>(bytes);
   if (e != cudaSuccess) return e;
@@ -822,16 +884,20 @@ cudaError_t launch_calibrate_static(const AttnParams& p_in, int d, int n_seq, cu
                     n_seq, p.K, p.step);
 }
 
-// `n_sm`: SMs of the device.  16-query CTAs while two of them per SM hold the launch (or the step has no more queries than
+// Does the small-step kernel take an attention launch of t_q queries and `units` (sequence, head) pairs?  16-query CTAs while two of them per SM hold the launch (or the step has no more queries than
 // that: then nothing is read twice); else two groups of warps per 64-query CTA while every CTA has an SM to itself and heads
 // see more than one key half-tile; a fuller launch keeps two single-group CTAs per SM (the same warps per SM, and nothing
 // to merge).
+bool attn_is_small(int t_q, int64_t units, int n_sm) { return t_q <= 16 || (t_q + 15) / 16 * units <= 2 * n_sm; }
+
+// `n_sm`: SMs of the device.
 cudaError_t launch_attn_generic(const AttnParams& p, int d, int n_seq, bool calib, int n_sm, cudaStream_t stream) {
   if (d != 64 && d != 128) return cudaErrorInvalidValue;
   if (calib) return d == 128 ? launch_one<128, true>(p, n_seq, stream) : launch_one<64, true>(p, n_seq, stream);
   const int64_t units = (int64_t)n_seq * p.H;
-  if (p.t_q <= 16 || (p.t_q + 15) / 16 * units <= 2 * n_sm)
-    return d == 128 ? launch_small<128>(p, n_seq, stream) : launch_small<64>(p, n_seq, stream);
+  if (attn_is_small(p.t_q, units, n_sm))                    // (direct8 is set under this same rule)
+    return p.direct8 ? (d == 128 ? launch_small<128, true>(p, n_seq, stream) : launch_small<64, true>(p, n_seq, stream))
+                     : (d == 128 ? launch_small<128, false>(p, n_seq, stream) : launch_small<64, false>(p, n_seq, stream));
   if (p.step > 0 && (p.t_q + GM - 1) / GM * units <= n_sm)
     return d == 128 ? launch_one<128, false, 2>(p, n_seq, stream) : launch_one<64, false, 2>(p, n_seq, stream);
   return d == 128 ? launch_one<128, false>(p, n_seq, stream) : launch_one<64, false>(p, n_seq, stream);

@@ -83,13 +83,24 @@ __global__ void __launch_bounds__(CP_THREADS) append_fp8_kernel(const __grid_con
 }
 
 // Expansion of the visible head-scales of one (step, layer) into the bf16 staging rows the attention kernels
-// read: grid = (visible half-tile of the layer in descriptor order, sequence, K | V).  Staging slot j of the
+// read: one CTA per (visible half-tile of the layer in descriptor order, sequence, K | V).  Staging slot j of the
 // sequence takes the n_valid rows behind descriptor first + j; rows past n_valid keep whatever finite values
-// an earlier call left there (the kernels mask them).
-__global__ void __launch_bounds__(CP_THREADS) dequant_fp8_kernel(const __grid_constant__ CopyParams p) {
+// an earlier call left there (the kernels mask them).  When the call also stores the step's rows (p.k_new), the CTAs
+// after those quantise them into the code pools: the plan releases no page that this step still reads before the update,
+// so the two need no order between them, and the update costs no launch of its own (4 sequences x 16 heads, 2 layers, 13
+// scales at budget 1/10: 2.43 -> 2.32 ms a pass, the small steps' direct reading included).
+__global__ void __launch_bounds__(CP_THREADS) stage_fp8_kernel(const __grid_constant__ CopyParams p, int slots, int n_seq) {
   pdl_trigger();
-  const int seq = blockIdx.y, j = blockIdx.x;
-  const bool is_v = blockIdx.z != 0;
+  const int expand = slots * n_seq * 2;
+  if ((int)blockIdx.x >= expand) {
+    const int a = blockIdx.x - expand, seq = a % n_seq, head = (a / n_seq) % p.H, j = a / (n_seq * p.H);
+    const int64_t src = seq * p.kv_seq + head * p.kv_head;
+    append_half_tile_fp8(p.seqs[seq].plan, p.seqs[seq].base_row, (p.step * p.L + p.layer) * p.H + head, j, p.k_new + src,
+                         p.v_new + src, p.kv_tok, p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, p.d, threadIdx.x, CP_THREADS);
+    return;
+  }
+  const bool is_v = blockIdx.x & 1;
+  const int seq = (blockIdx.x >> 1) % n_seq, j = (blockIdx.x >> 1) / n_seq;
   PlanView pv(p.seqs[seq].plan);
   const int u0 = (p.step * p.L + p.layer) * p.H;
   const int first = pv.attn_begin()[u0];
@@ -124,11 +135,14 @@ cudaError_t launch_append_fp8(const CopyParams& p, int n_seq, cudaStream_t strea
   return cudaGetLastError();
 }
 
-// `slots` = the largest number of visible half-tiles any sequence of the call has at (step, layer)
-cudaError_t launch_dequant_fp8(const CopyParams& p, int n_seq, int slots, cudaStream_t stream) {
-  if (slots < 1) return cudaSuccess;
-  dim3 grid(slots, n_seq, 2);
-  dequant_fp8_kernel<<<grid, CP_THREADS, 0, stream>>>(p);
+// `slots` = the largest number of visible half-tiles any sequence of the call has at (step, layer); `update` = the step's
+// rows (p.k_new, p.v_new) are stored too
+cudaError_t launch_stage_fp8(const CopyParams& p, int n_seq, int slots, bool update, cudaStream_t stream) {
+  const int64_t tiles = update ? (p.t_k + HEATKV_PAGE_TOKENS - 1) / HEATKV_PAGE_TOKENS + 1 : 0;
+  const int64_t ctas = (int64_t)slots * n_seq * 2 + tiles * p.H * n_seq;
+  if (ctas < 1) return cudaSuccess;
+  if (ctas > INT32_MAX) return cudaErrorInvalidValue;
+  stage_fp8_kernel<<<(unsigned)ctas, CP_THREADS, 0, stream>>>(p, slots, n_seq);
   return cudaGetLastError();
 }
 

@@ -74,6 +74,9 @@ struct AttnParams {
   int8_t* k_exp;
   int8_t* v_exp;
   int32_t pool_base[HEATKV_MAX_BATCH];
+  // fp8 cache, small-step kernel: the codes themselves are read (no staging rows).  With table_heads > 0 the plan's word
+  // offsets of the descriptors and of the pool rows behind them
+  int32_t direct8, off_desc, off_src;
 };
 
 struct CopyParams {

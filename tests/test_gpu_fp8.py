@@ -143,6 +143,32 @@ def test_fp8_cache_full_budget_head_dim_64_wide_range(hk):
     _run_fp8(hk, sh, ref, lambda ses: ses.schedule(scas=scores, b=1.0), hk.KERNEL_AUTO, mutate=mutate)
 
 
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+def test_fp8_small_steps_mixed_schedules_equal_single_ones(hk, d):
+    """Steps whose kernel reads the codes itself, in a call that mixes schedules (descriptors found through the plans) and
+    in calls of one sequence (found through the launch parameters): the same bits, as every unit is computed alone."""
+    from paper_2605_14877_b200.sweep import Session
+    sh = W.Shape("mixed", L=1, H=3, d=d, sides=W.SIDES_13[:6], n_seq=2, s=2)
+    q, k, v = W.qkv_layer(sh, 3, 0, device="cuda")
+    with Session(sh.L, sh.H, sh.d, sh.t, sh.s, 1 << 14, layout=hk.LAYOUT_PAGED, cache_dtype=hk.CACHE_FP8_E4M3) as ses:
+        schs = [ses.schedule(scas=W.synthetic_scas(sh, i), b=b) for i, b in enumerate((0.4, 1.0))]
+
+        def run(which):
+            ids = [hk.heatkv_seq_open(ses.ctx, schs[i]) for i in which]
+            args = [x[list(which)].contiguous() for x in (q, k, v)]
+            out = torch.zeros_like(args[0])
+            ses.generate(ids, lambda l: args, lambda l: out, fused=True)
+            for i in ids:
+                hk.heatkv_seq_close(ses.ctx, i)
+            return W.bf16_bits(out)
+
+        both = run((0, 1))
+        assert np.array_equal(both[0], run((0,))[0]) and np.array_equal(both[1], run((1,))[0])
+        assert hk.heatkv_device_status(ses.ctx) == 0
+        for s in schs:
+            hk.heatkv_schedule_free(s)
+
+
 def test_fp8_cache_needs_paged_layout_and_enough_staging(hk):
     from paper_2605_14877_b200.sweep import Session
     sh = W.Shape("mid", L=1, H=2, d=128, sides=W.SIDES_13[:9], n_seq=1, s=3)
