@@ -14,7 +14,7 @@
 //   warps 4-7   softmax of tile A, warps 8-11 softmax of tile B: one thread per query row
 //               reads its row of S from TMEM, keeps the running max / sum, writes P (bf16)
 //               back into the columns S occupied, and rescales O only when the row max grew
-//               by more than 2^8 since the last reference (the sum keeps the same reference,
+//               by more than 2^32 since the last reference (the sum keeps the same reference,
 //               so the result is exact).  The same warps write the item's result.
 // TMEM columns: S_A/P_A 0..127, S_B/P_B 128..255, O_A 256..383, O_B 384..511.
 // The MMA order S_A S_B (PV_A S_A' PV_B S_B')* lets the softmax of one tile overlap the
