@@ -83,6 +83,7 @@ enum Bar : uint32_t {
 constexpr uint32_t BAR_TMEM_PTR = N_BARS * 8;                  // offsets inside the barrier region
 constexpr uint32_t BAR_ABORT = BAR_TMEM_PTR + 4;
 constexpr uint32_t BAR_RING = 256;                             // 2 entries x int32[16]
+constexpr float SUM_LIMIT = 4294967296.f;                      // 2^RESCALE_THRESHOLD: no term of a sum below it is above it
 enum ItemKind : int { ATTENTION = 0, STOP = 2, NOTHING = 3 };
 // ring entry words
 enum ItemWord : int { W_KIND = 0, W_HEAD, W_SEQ, W_TILES, W_NSPLIT, W_SUB, W_SLOT, W_CTR, W_DESC, W_NDESC };
@@ -164,6 +165,10 @@ __global__ void __launch_bounds__(THREADS, 1)
 attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Maps maps) {
   using L = Layout<D>;
   constexpr int NCH = L::NCH;
+  // Where the softmax itself weighs most: half the tensor work per exponential (64-wide heads), or masses to keep besides
+  // (FULL).  Measured: generation with 64-wide heads 1.673 -> 1.629 ms, calibration with output (128-wide) 1.186 -> 1.142;
+  // 128-wide generation, where a product's latency is the larger part of the chain, was 0.3 to 0.8 % slower with it.
+  constexpr bool SPECULATE = FULL || D == 64;
   constexpr uint32_t TILE_BYTES = L::TILE_BYTES, SM_Q = L::SM_Q, SM_K = L::SM_K, SM_V = L::SM_V, SM_OUT = L::SM_OUT,
                      SM_BAR = L::SM_BAR, SM_TMEM_PTR = L::SM_BAR + BAR_TMEM_PTR, SM_ABORT = L::SM_BAR + BAR_ABORT,
                      SM_RING = L::SM_BAR + BAR_RING;
@@ -592,49 +597,6 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
                 if (i + 32 >= s1.n_valid) r3[i] = 0xff800000u;
               }
             }
-            // row maximum: the logit is raw * scale + bias(half) with scale > 0, so take the raw maxima
-            // (eight independent chains keep the dependent depth short)
-            float mq[8];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              mq[c] = fmaxf(__uint_as_float(r0[c]), __uint_as_float(r1[c]));
-              mq[4 + c] = fmaxf(__uint_as_float(r2[c]), __uint_as_float(r3[c]));
-            }
-#pragma unroll
-            for (int i = 4; i < 32; i += 4) {
-#pragma unroll
-              for (int c = 0; c < 4; ++c) {
-                mq[c] = fmax3(mq[c], __uint_as_float(r0[i + c]), __uint_as_float(r1[i + c]));
-                mq[4 + c] = fmax3(mq[4 + c], __uint_as_float(r2[i + c]), __uint_as_float(r3[i + c]));
-              }
-            }
-            const float mx0 = fmaxf(fmaxf(mq[0], mq[1]), fmaxf(mq[2], mq[3]));
-            const float mx1 = fmaxf(fmaxf(mq[4], mq[5]), fmaxf(mq[6], mq[7]));
-            const float mx = fmaxf(fmaf(mx0, p.scale_log2, b0), fmaf(mx1, p.scale_log2, b1));
-            const float m_new = fmaxf(m_ref, mx);
-            const bool grow = m_new > m_ref + RESCALE_THRESHOLD;   // also true on the first tile (m_ref = -inf)
-            if (j > 0 && __any_sync(0xffffffffu, grow)) {
-              // O_x holds tiles < j relative to m_ref: rescale the rows whose reference moves.  O_x is complete:
-              // S_x of this tile was issued after the PV products of tile j - 1 by the same thread, and the
-              // commit behind S_FULL covers every product issued before it.
-              const float f = grow ? exp2f(m_ref - m_new) : 1.f;
-#pragma unroll
-              for (int c = 0; c < D / 32; ++c) {
-                uint32_t r[32];
-                tmem_ld32(t_o + c * 32, r);
-                tmem_wait_ld();
-#pragma unroll
-                for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * f);
-                tmem_st32(t_o + c * 32, r);
-              }
-              tmem_wait_st();
-              l_sum *= f;
-              if (FULL) {
-                cur_mass *= f;
-                for (int s = 0; s < cur_seg; ++s) masses[s * 32] *= f;
-              }
-            }
-            if (grow) m_ref = m_new;
             // p = exp2(logit - m_ref); row sum in fp32; P as bf16 pairs into the columns S occupied
             // (keys 32c..32c+31 -> P columns 16c..16c+15; the whole row of S is already in registers).
             // One pair in four takes the polynomial on the FMA pipe, the rest the MUFU unit: the tile's
@@ -642,28 +604,110 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             // the tile's two products.
             const uint64_t scale2 = pack2(p.scale_log2, p.scale_log2);
             uint64_t sum2 = pack2(0.f, 0.f);
-            auto exp_chunk = [&](const uint32_t (&rc)[32], uint64_t bb2, int c) {
-              uint32_t pk[16];
+            float top = 0.f;                                         // the largest argument that went to the polynomial
+            auto exps = [&](const uint32_t (&rc)[32], uint64_t bb2, uint32_t (&pk)[16]) {
 #pragma unroll
               for (int i = 0; i < 32; i += 2) {
                 const uint64_t xx = fma2(pack2(__uint_as_float(rc[i]), __uint_as_float(rc[i + 1])), scale2, bb2);
-                float e0, e1;
+                float e0, e1, x0, x1;
+                unpack2(xx, x0, x1);
                 if (((i >> 1) & POLY_MASK) == POLY_MASK) {
                   exp2_poly2(xx, e0, e1);
+                  if (SPECULATE) top = fmax3(top, x0, x1);
                 } else {
-                  float x0, x1;
-                  unpack2(xx, x0, x1);
                   e0 = ex2_approx(x0);
                   e1 = ex2_approx(x1);
                 }
                 sum2 = add2(sum2, pack2(e0, e1));
                 pk[i >> 1] = pack_bf16(e0, e1);
               }
+            };
+            auto exp_chunk = [&](const uint32_t (&rc)[32], uint64_t bb2, int c) {
+              uint32_t pk[16];
+              exps(rc, bb2, pk);
               tmem_st16(t_s + c * 16, pk);
             };
-            const uint64_t bb0 = pack2(b0 - m_ref, b0 - m_ref), bb1 = pack2(b1 - m_ref, b1 - m_ref);
-            exp_chunk(r0, bb0, 0);
-            exp_chunk(r1, bb0, 1);
+            // The reference moves seldom.  SPECULATE: from the second tile on, the first half's exponentials are taken against the
+            // present one, and their sum tells whether it still serves (the polynomial's arguments are looked at too: it is
+            // meaningless above 2^127); only the second half's maximum is computed, beside them.
+            bool take_max = true;
+            uint32_t pk0[16], pk1[16];
+            if (SPECULATE && j > 0) {
+              const uint64_t bb0 = pack2(b0 - m_ref, b0 - m_ref);
+              exps(r0, bb0, pk0);
+              exps(r1, bb0, pk1);
+              float ma[4];
+#pragma unroll
+              for (int c = 0; c < 4; ++c) ma[c] = fmaxf(__uint_as_float(r2[c]), __uint_as_float(r3[c]));
+#pragma unroll
+              for (int i = 4; i < 32; ++i) ma[i & 3] = fmax3(ma[i & 3], __uint_as_float(r2[i]), __uint_as_float(r3[i]));
+              const float m1 = fmaf(fmaxf(fmaxf(ma[0], ma[1]), fmaxf(ma[2], ma[3])), p.scale_log2, b1);
+              float sa, sb;
+              unpack2(sum2, sa, sb);
+              take_max = __any_sync(0xffffffffu, !(sa + sb <= SUM_LIMIT && fmaxf(top, m1 - m_ref) <= RESCALE_THRESHOLD));
+              if (take_max) {                                        // S is still there: load the half again
+                sum2 = pack2(0.f, 0.f);
+                tmem_ld32(t_s, r0);
+                tmem_ld32(t_s + 32, r1);
+                tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                  if (i >= s0.n_valid) r0[i] = 0xff800000u;
+                  if (i + 32 >= s0.n_valid) r1[i] = 0xff800000u;
+                }
+              }
+            }
+            if (take_max) {
+              // row maximum: the logit is raw * scale + bias(half) with scale > 0, so take the raw maxima
+              // (eight independent chains keep the dependent depth short)
+              float mq[8];
+#pragma unroll
+              for (int c = 0; c < 4; ++c) {
+                mq[c] = fmaxf(__uint_as_float(r0[c]), __uint_as_float(r1[c]));
+                mq[4 + c] = fmaxf(__uint_as_float(r2[c]), __uint_as_float(r3[c]));
+              }
+#pragma unroll
+              for (int i = 4; i < 32; i += 4) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                  mq[c] = fmax3(mq[c], __uint_as_float(r0[i + c]), __uint_as_float(r1[i + c]));
+                  mq[4 + c] = fmax3(mq[4 + c], __uint_as_float(r2[i + c]), __uint_as_float(r3[i + c]));
+                }
+              }
+              const float mx0 = fmaxf(fmaxf(mq[0], mq[1]), fmaxf(mq[2], mq[3]));
+              const float mx1 = fmaxf(fmaxf(mq[4], mq[5]), fmaxf(mq[6], mq[7]));
+              const float mx = fmaxf(fmaf(mx0, p.scale_log2, b0), fmaf(mx1, p.scale_log2, b1));
+              const float m_new = fmaxf(m_ref, mx);
+              const bool grow = m_new > m_ref + RESCALE_THRESHOLD;   // also true on the first tile (m_ref = -inf)
+              if (j > 0 && __any_sync(0xffffffffu, grow)) {
+                // O_x holds tiles < j relative to m_ref: rescale the rows whose reference moves.  O_x is complete:
+                // S_x of this tile was issued after the PV products of tile j - 1 by the same thread, and the
+                // commit behind S_FULL covers every product issued before it.
+                const float f = grow ? exp2f(m_ref - m_new) : 1.f;
+#pragma unroll
+                for (int c = 0; c < D / 32; ++c) {
+                  uint32_t r[32];
+                  tmem_ld32(t_o + c * 32, r);
+                  tmem_wait_ld();
+#pragma unroll
+                  for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * f);
+                  tmem_st32(t_o + c * 32, r);
+                }
+                tmem_wait_st();
+                l_sum *= f;
+                if (FULL) {
+                  cur_mass *= f;
+                  for (int s = 0; s < cur_seg; ++s) masses[s * 32] *= f;
+                }
+              }
+              if (grow) m_ref = m_new;
+              const uint64_t bb0 = pack2(b0 - m_ref, b0 - m_ref);
+              exp_chunk(r0, bb0, 0);
+              exp_chunk(r1, bb0, 1);
+            } else {
+              tmem_st16(t_s, pk0);
+              tmem_st16(t_s + 16, pk1);
+            }
             tmem_wait_st();
             tc_fence_before();
             mbar_arrive(bar(P_FULL + 2 * x));                      // the PV product of keys 0..63 may start
@@ -680,6 +724,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
               }
               cur_mass += half;
             }
+            const uint64_t bb1 = pack2(b1 - m_ref, b1 - m_ref);
             exp_chunk(r2, bb1, 2);
             exp_chunk(r3, bb1, 3);
             float sa, sb;

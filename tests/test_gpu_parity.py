@@ -231,6 +231,25 @@ def test_tensor_memory_kernel_lagging_reference(hk, d):
                      kernel=hk.KERNEL_TCGEN05, check_cache=False, fused=True, mutate=mutate)
 
 
+@pytest.mark.parametrize("where", ["first_half", "second_half"])
+def test_tensor_memory_kernel_outlier_keys_head_dim_64(hk, where):
+    """64-wide heads take a tile's exponentials before its maximum is known: keys scaled by 40 (logits of +-100 and more, past the
+    polynomial's range) in either half of later tiles, at positions of both exponential forms, must still move the reference."""
+    sh = W.Shape("outlier64", L=1, H=2, d=64, sides=W.SIDES_13[:11], n_seq=2, s=3)
+    scores = W.synthetic_scas(sh, 2)
+    ref = O.heatkv_schedule(scores, 0.5, sh.s, sh.sides)
+
+    def mutate(l, q, k, v):
+        k = k.clone()
+        tok = torch.arange(k.shape[2], device=k.device)
+        pick = (tok >= 300) & (tok % 41 == 0) & ((tok % 128 < 64) == (where == "first_half"))
+        k[:, :, pick] *= 40
+        return q, k, v * 0.25                      # |O| below 1.1, so the two bf16 roundings stay within 0.0041 (bar 1e-2)
+
+    _run_full_parity(hk, sh, ref, lambda ses: ses.schedule(scas=scores, b=0.5), hk.LAYOUT_PAGED,
+                     kernel=hk.KERNEL_TCGEN05, check_cache=False, fused=True, mutate=mutate)
+
+
 def test_tensor_memory_kernel_full_cache(hk):
     """b = 1: long page tables (up to 4121 prior keys), tcgen05 kernel, no bias."""
     sh = W.Shape("full128", L=1, H=2, d=128, sides=W.SIDES_13[:12], n_seq=1, s=3)
