@@ -215,6 +215,16 @@ __device__ __forceinline__ bool elect_one() {
   asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(pred));
   return pred != 0;
 }
+// The same for a converged warp with the vote inside the loop: one vote per try, and a provably uniform result.
+__device__ __forceinline__ bool warp_wait_vote(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t* status) {
+  for (uint32_t it = 0; it < WAIT_LIMIT; ++it) {
+    if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+    if ((it & 31u) == 31u && __any_sync(0xffffffffu, *abort_flag)) return false;
+  }
+  *abort_flag = 1;
+  atomicOr(status, 1u);
+  return false;
+}
 __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t* status) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status));
 }
