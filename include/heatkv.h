@@ -95,8 +95,9 @@ typedef struct {
   uint64_t arena_bytes;          /* metadata region + scratch region + K pool + V pool     */
   uint64_t meta_bytes;           /* bytes of the arena set aside for plans; 0 = default    */
   uint64_t scratch_bytes;        /* bytes of the arena for partial results of heads whose key range is
-                                    split over several CTAs; 0 = default (1/8 of the arena, at most
-                                    128 MiB); too little only disables splitting                    */
+                                    split over several CTAs, an eighth of it (at most 32 MiB) for the
+                                    plans' merged tables; 0 = default (1/8 of the arena, at most
+                                    128 MiB); too little only disables both                         */
   int32_t cache_dtype;           /* heatkv_cache_dtype; FP8_E4M3 needs the paged layout                    */
   int32_t reserved0;
   uint64_t stage_bytes;          /* FP8_E4M3 only: bytes of the arena for the bf16 staging rows one attention
@@ -245,17 +246,19 @@ int heatkv_schedule_footprint(const heatkv_schedule* sch, int layout, int64_t* p
                               int64_t* reserved_rows);
 
 /* The plan a sequence of this schedule runs under `layout`, as the flat int32 table the
- * kernels read (HOST copy, for inspection and tests): a 20-word header {L, H, K, n_desc,
+ * kernels read (HOST copy, for inspection and tests): a 24-word header {L, H, K, n_desc,
  * word offsets of: desc, attn_begin, attn_cnt, app_begin, app_cnt, order, move, pre_begin,
- * pre_cnt, post_begin, post_cnt, then n_move, total_words, 3 spare} followed by the tables.
+ * pre_cnt, post_begin, post_cnt, then n_move, total_words, 1 spare, word offsets of run_desc,
+ * run_begin, run_cnt, 3 spare} followed by the tables.
  * desc = {row relative to the reservation, n_valid | source_scale << 8}; move = {src, dst, n, 0};
- * the per-(step, layer, head) tables are indexed (step*L + layer)*H + head.
+ * the per-(step, layer, head) tables are indexed (step*L + layer)*H + head.  run_* = attn_* for
+ * calls without seg_bias: rows that follow one another share half-tiles across source scales.
  * Call with words == NULL to get *n_words, then with a buffer of that many int32.        */
 int heatkv_schedule_plan(const heatkv_schedule* sch, int layout, int32_t* words, int64_t* n_words);
 /* The same for a context with the fp8 cache (paged layout): the attention descriptors of every (step, layer) carry
  * staging rows -- consecutive 64-row slots in descriptor order across the layer's heads -- and header word 17 is the
  * word offset of an extra table int32[n_desc] with the pool row behind every descriptor (append descriptors keep
- * pool rows).  *stage_rows (optional) = staging rows one sequence needs in an attention call: 64 per visible
+ * pool rows); word 21 is the same for run_desc.  *stage_rows (optional) = staging rows one sequence needs in an attention call: 64 per visible
  * half-tile of its busiest (step, layer).  Pure host code. */
 int heatkv_schedule_plan_fp8(const heatkv_schedule* sch, int32_t* words, int64_t* n_words, int64_t* stage_rows);
 

@@ -94,6 +94,8 @@ struct PlanEntry {
   Schedule sched;
   Plan plan;
   uint64_t meta_off = 0, meta_len = 0;
+  uint64_t run_off = 0, run_len = 0;    // merged attention tables on the device (run_len 0: none), both from the arena's start
+  int32_t run_shift = 0;                // what takes a word offset inside them from the host's blob to the device
   int refs = 0;
 };
 
@@ -126,7 +128,7 @@ struct heatkv_ctx {
   int8_t* v_exp = nullptr;
   uint64_t stage_rows = 0;
   uint32_t* status = nullptr;
-  RangeAlloc rows, metas;
+  RangeAlloc rows, metas, run_tables;
   std::vector<std::unique_ptr<PlanEntry>> plans;
   std::vector<Seq> seqs;
   uint64_t reserved_rows = 0, peak_reserved = 0, meta_used = 0;
@@ -157,13 +159,15 @@ int find_or_load_plan(heatkv_ctx* ctx, const Schedule& s, cudaStream_t stream, i
   e->sched = s;
   int rc = build_plan(s, ctx->cfg.layout, &e->plan, ctx->fp8);
   if (rc != HEATKV_OK) return rc;
-  uint64_t bytes = ((uint64_t)e->plan.blob.size() * 4 + META_ALIGN - 1) / META_ALIGN * META_ALIGN;
+  const uint64_t plain_words = (uint64_t)e->plan.header().off_run_desc;
+  uint64_t bytes = (plain_words * 4 + META_ALIGN - 1) / META_ALIGN * META_ALIGN;
   uint64_t off = 0;
   bool ok = ctx->metas.alloc(bytes, &off);
   if (!ok) {                                    // drop resident plans nobody uses and retry
     for (auto& pe : ctx->plans)
       if (pe && pe->refs == 0) {
         ctx->metas.release(pe->meta_off, pe->meta_len);
+        if (pe->run_len) ctx->run_tables.release(pe->run_off, pe->run_len);
         ctx->meta_used -= pe->meta_len;
         pe.reset();
       }
@@ -172,13 +176,27 @@ int find_or_load_plan(heatkv_ctx* ctx, const Schedule& s, cudaStream_t stream, i
   if (!ok) return HEATKV_ERR_OUT_OF_PAGES;
   e->meta_off = off;
   e->meta_len = bytes;
-  if (cudaMemcpyAsync(ctx->meta + off, e->plan.blob.data(), e->plan.blob.size() * 4, cudaMemcpyHostToDevice,
-                      stream) != cudaSuccess) {
+  // The merged tables go to a region of their own: a plan that finds no room there does without them.
+  PlanHeader& h = *reinterpret_cast<PlanHeader*>(e->plan.blob.data());
+  const uint64_t run_words = e->plan.blob.size() - plain_words;
+  uint64_t run_len = (run_words * 4 + META_ALIGN - 1) / META_ALIGN * META_ALIGN;
+  if (ctx->run_tables.alloc(run_len, &e->run_off)) {
+    e->run_len = run_len;
+    e->run_shift = (int32_t)((int64_t)(e->run_off - off) / 4 - (int64_t)plain_words);
+  }
+  auto shift_runs = [&](int32_t by) { h.off_run_desc += by; h.off_run_begin += by; h.off_run_cnt += by; h.off_run_src += by; };
+  shift_runs(e->run_shift);
+  cudaError_t up = cudaMemcpyAsync(ctx->meta + off, e->plan.blob.data(), plain_words * 4, cudaMemcpyHostToDevice, stream);
+  if (up == cudaSuccess && e->run_len)
+    up = cudaMemcpyAsync(ctx->meta + e->run_off, e->plan.blob.data() + plain_words, run_words * 4, cudaMemcpyHostToDevice, stream);
+  // the blob is pageable host memory: wait so the vector may be touched again safely
+  if (up == cudaSuccess) up = cudaStreamSynchronize(stream);
+  shift_runs(-e->run_shift);
+  if (up != cudaSuccess) {
     ctx->metas.release(off, bytes);
+    if (e->run_len) ctx->run_tables.release(e->run_off, e->run_len);
     return HEATKV_ERR_CUDA;
   }
-  // the blob is pageable host memory: wait so the vector may be touched again safely
-  if (cudaStreamSynchronize(stream) != cudaSuccess) return HEATKV_ERR_CUDA;
   ctx->meta_used += bytes;
   size_t slot = ctx->plans.size();
   for (size_t i = 0; i < ctx->plans.size(); ++i)
@@ -259,13 +277,20 @@ int gather_seqs(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int layer, int s
   return HEATKV_OK;
 }
 
+// A call reads the merged attention tables when no bias per scale is given and every sequence's plan has them.
+bool all_have_runs(const heatkv_ctx* ctx, const int* seq_ids, int n_seq) {
+  for (int i = 0; i < n_seq; ++i)
+    if (!ctx->plans[ctx->seqs[seq_ids[i]].plan]->run_len) return false;
+  return true;
+}
+
 // ---- key-range splitting of the tensor-memory attention kernel -----------------------------------------
 // Key tiles of the heads of (step, layer), in the plan's dispatch order (descending key count).
-std::vector<int> ordered_tiles(const PlanEntry& pe, int step, int layer, int own_slots) {
+std::vector<int> ordered_tiles(const PlanEntry& pe, int step, int layer, int own_slots, bool runs) {
   const Schedule& s = pe.sched;
   const PlanHeader& h = pe.plan.header();
   const int32_t* blob = pe.plan.blob.data();
-  const int32_t* cnt = blob + h.off_attn_cnt + s.at(step, layer, 0);
+  const int32_t* cnt = blob + attn_tables(h, runs).cnt + s.at(step, layer, 0);
   const int32_t* order = blob + h.off_order + s.at(step, layer, 0);
   std::vector<int> t(s.H);
   for (int i = 0; i < s.H; ++i) t[i] = (cnt[order[i]] + own_slots + 1) / 2;
@@ -283,15 +308,17 @@ void fill_head_table(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, i
   const PlanHeader& hdr = pe0.plan.header();
   const int32_t* blob = pe0.plan.blob.data();
   const int at = pe0.sched.at(step, layer, 0);
-  const int32_t *order = blob + hdr.off_order + at, *cnt = blob + hdr.off_attn_cnt + at, *begin = blob + hdr.off_attn_begin + at;
+  const AttnTables tab = attn_tables(hdr, p->runs);
+  const int32_t shift = p->runs ? pe0.run_shift : 0;
+  const int32_t *order = blob + hdr.off_order + at, *cnt = blob + tab.cnt + at, *begin = blob + tab.begin + at;
   for (int i = 0; i < pe0.sched.H; ++i) {
     if (cnt[order[i]] > 32767) return;
     p->table_head[i] = (int16_t)order[i];
     p->table_ndesc[i] = (int16_t)cnt[order[i]];
-    p->table_desc_begin[i] = hdr.off_desc + 2 * begin[order[i]];
+    p->table_desc_begin[i] = tab.desc + shift + 2 * begin[order[i]];
   }
-  p->off_desc = hdr.off_desc;
-  p->off_src = hdr.off_src;
+  p->off_desc = tab.desc + shift;
+  p->off_src = tab.src + shift;
   p->table_heads = pe0.sched.H;
 }
 
@@ -304,11 +331,11 @@ void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int 
   const PlanEntry& pe0 = *ctx->plans[ctx->seqs[seq_ids[0]].plan];
   bool one_plan = pe0.sched.H <= 64;
   for (int i = 1; i < n_seq && one_plan; ++i) one_plan = ctx->seqs[seq_ids[i]].plan == ctx->seqs[seq_ids[0]].plan;
-  const std::vector<int> tiles = ordered_tiles(pe0, step, layer, own_slots);
+  const std::vector<int> tiles = ordered_tiles(pe0, step, layer, own_slots, p->runs);
   const int H = (int)tiles.size();
   for (int t : tiles) one_plan = one_plan && t <= 16383;          // half-tile counts travel as 16 bits
   const uint64_t key = (pe0.uid << 24) ^ ((uint64_t)step << 20) ^ ((uint64_t)layer << 8) ^ (uint64_t)n_seq ^
-                       (one_plan ? 0ull : 1ull << 63);
+                       (one_plan ? 0ull : 1ull << 63) ^ (p->runs ? 1ull << 62 : 0ull);
   auto fits = [&](const SplitShape& sh) {
     return (uint64_t)sh.slots * n_seq <= ctx->split_slots &&
            (uint64_t)sh.ctrs * n_seq * SPLIT_CTRS_PER_GROUP <= ctx->split_ctrs;
@@ -329,7 +356,7 @@ void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int 
         const int pi = ctx->seqs[seq_ids[i]].plan;
         if (pi == last_plan) continue;
         last_plan = pi;
-        const std::vector<int> t = ordered_tiles(*ctx->plans[pi], step, layer, own_slots);
+        const std::vector<int> t = ordered_tiles(*ctx->plans[pi], step, layer, own_slots, p->runs);
         std::vector<int> ns(t.size());
         for (size_t k = 0; k < t.size(); ++k) ns[k] = split_pieces_for(t[k], lm);
         const SplitShape sh = split_shape(t, ns, n_qp);
@@ -350,10 +377,11 @@ void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int 
     const PlanHeader& hdr = pe0.plan.header();
     const int32_t* blob = pe0.plan.blob.data();
     const size_t at = pe0.sched.at(step, layer, 0);
-    const int32_t *order = blob + hdr.off_order + at, *cnt = blob + hdr.off_attn_cnt + at, *begin = blob + hdr.off_attn_begin + at;
+    const AttnTables tab = attn_tables(hdr, p->runs);
+    const int32_t *order = blob + hdr.off_order + at, *cnt = blob + tab.cnt + at, *begin = blob + tab.begin + at;
     for (int i = 0; i < H; ++i) {
       p->table_ndesc[i] = (int16_t)cnt[order[i]];
-      p->table_desc_begin[i] = hdr.off_desc + 2 * begin[order[i]];
+      p->table_desc_begin[i] = tab.desc + (p->runs ? pe0.run_shift : 0) + 2 * begin[order[i]];
       p->table_head[i] = (int16_t)order[i];
       p->table_tiles[i] = (int16_t)tiles[i];
       p->table_split[i] = (int16_t)ch.ns[i];
@@ -445,10 +473,13 @@ int heatkv_create(const heatkv_config* cfg, void* stream_, heatkv_ctx** out) {
   {   // scratch region: arrival counters first (kept zero between launches), then the partial-result slots
     const uint64_t ctr_bytes = std::min<uint64_t>(scratch / 4, 256u << 10) / 1024 * 1024;
     const uint64_t slot_bytes = (uint64_t)tc_split_slot_floats(cfg->d) * 4;
+    // ... and at its end the plans' merged attention tables (half a megabyte for 13 scales of 4 layers x 30 heads)
+    const uint64_t run_bytes = std::min<uint64_t>(scratch / 8, 32u << 20) / 1024 * 1024;
+    ctx->run_tables.reset(meta + scratch - run_bytes, run_bytes);
     ctx->split_counters = reinterpret_cast<uint32_t*>(ctx->meta + meta);
     ctx->split_ctrs = ctr_bytes / 4;
     ctx->split_partials = reinterpret_cast<float*>(ctx->meta + meta + ctr_bytes);
-    ctx->split_slots = (scratch - ctr_bytes) / slot_bytes;
+    ctx->split_slots = (scratch - ctr_bytes - run_bytes) / slot_bytes;
     if (ctr_bytes && cudaMemsetAsync(ctx->split_counters, 0, ctr_bytes, stream) != cudaSuccess) return HEATKV_ERR_CUDA;
     int dev = 0, n_sm = 0;
     if (cudaGetDevice(&dev) == cudaSuccess &&
@@ -662,6 +693,7 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
   p.v_new = static_cast<const __nv_bfloat16*>(v_new);
   p.out = static_cast<__nv_bfloat16*>(out);
   p.seg_bias = seg_bias;
+  p.runs = !seg_bias && all_have_runs(ctx, seq_ids, n_seq);
   p.t_q = p.n_own = ctx->cfg.t[step];
   p.step = step;
   p.layer = layer;
@@ -683,6 +715,7 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
     std::memset(&cp, 0, sizeof(cp));
     cp.k_pool = ctx->k_pool; cp.v_pool = ctx->v_pool;
     cp.k8_pool = ctx->k8_pool; cp.v8_pool = ctx->v8_pool; cp.k_exp = ctx->k_exp; cp.v_exp = ctx->v_exp;
+    cp.runs = p.runs;
     cp.step = step; cp.layer = layer; cp.H = ctx->cfg.H; cp.K = ctx->cfg.K; cp.L = ctx->cfg.L; cp.d = ctx->cfg.d;
     uint64_t next = 0;
     int slots = 0;
@@ -691,8 +724,9 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
       const PlanHeader& hd = pe.plan.header();
       const int32_t* blob = pe.plan.blob.data();
       const size_t u0 = pe.sched.at(step, layer, 0), u1 = pe.sched.at(step, layer, pe.sched.H - 1);
-      const int count = blob[hd.off_attn_begin + u1] + blob[hd.off_attn_cnt + u1] - blob[hd.off_attn_begin + u0];
-      slots = std::max(slots, count);
+      auto half_tiles = [&](const AttnTables& t) { return blob[t.begin + u1] + blob[t.cnt + u1] - blob[t.begin + u0]; };
+      const int count = half_tiles(attn_tables(hd, false));   // rows are set aside for either form of the tables
+      slots = std::max(slots, half_tiles(attn_tables(hd, p.runs)));
       cp.seqs[i] = p.seqs[i];
       cp.stage_base[i] = (int32_t)next;
       next += (uint64_t)count * HEATKV_PAGE_TOKENS;
@@ -779,6 +813,7 @@ int heatkv_attention_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int l
   AttnParams p;
   std::memset(&p, 0, sizeof(p));
   p.t_q = p.n_own = ctx->cfg.t[step];
+  p.runs = all_have_runs(ctx, seq_ids, n_seq);                  // (a call without a per-scale bias)
   try {
     choose_split(ctx, seq_ids, n_seq, step, layer, &p);
   } catch (const std::bad_alloc&) {

@@ -127,8 +127,8 @@ __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_ke
       PlanView pv(p.seqs[seq].plan);
       const int u = (p.step * p.L + p.layer) * p.H;
       head = pv.order()[u + blockIdx.z];                   // heavy heads first
-      descs = pv.descs() + pv.attn_begin()[u + head];
-      n_desc = pv.attn_cnt()[u + head];
+      descs = pv.attn_descs(p.runs) + pv.attn_begin(p.runs)[u + head];
+      n_desc = pv.attn_cnt(p.runs)[u + head];
     }
     base_row = p.seqs[seq].base_row;
   }
@@ -520,8 +520,8 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_small_kernel(const __grid_co
     PlanView pv(p.seqs[seq].plan);
     const int u = (p.step * p.L + p.layer) * p.H;
     head = pv.order()[u + blockIdx.z];                   // heavy heads first
-    descs = pv.descs() + pv.attn_begin()[u + head];
-    n_desc = pv.attn_cnt()[u + head];
+    descs = pv.attn_descs(p.runs) + pv.attn_begin(p.runs)[u + head];
+    n_desc = pv.attn_cnt(p.runs)[u + head];
   }
   const int64_t base_row = FP8 ? p.pool_base[seq] : p.seqs[seq].base_row;
   const int n_own_tiles = (p.n_own + GN - 1) / GN, n_tiles = n_own_tiles + n_desc;
@@ -533,7 +533,8 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_small_kernel(const __grid_co
   const int32_t* src_rows = nullptr;                     // FP8: the pool rows behind the head's descriptors
   if (FP8) {
     const int32_t* plan = p.seqs[seq].plan;
-    const int off_desc = p.table_heads > 0 ? p.off_desc : plan[4], off_src = p.table_heads > 0 ? p.off_src : plan[17];
+    const int off_desc = p.table_heads > 0 ? p.off_desc : plan[p.runs ? 18 : 4];
+    const int off_src = p.table_heads > 0 ? p.off_src : plan[p.runs ? 21 : 17];
     src_rows = plan + off_src + (reinterpret_cast<const int32_t*>(descs) - (plan + off_desc)) / 2;
   }
 

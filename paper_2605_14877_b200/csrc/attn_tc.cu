@@ -291,7 +291,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
               ns = p.table_split[i];
             } else {
               h = pv.order()[u + i];
-              tiles = (pv.attn_cnt()[u + h] + own_slots + 1) >> 1;
+              tiles = (pv.attn_cnt(p.runs)[u + h] + own_slots + 1) >> 1;
               ns = p.split_tiles > 0 ? (tiles + p.split_tiles - 1) / p.split_tiles : 1;
             }
             cnt = n_qp * ns;
@@ -314,8 +314,8 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             ring[W_SUB] = item - excl;                        // piece * n_qp + query tile pair
             ring[W_SLOT] = slots_before + sinc - scnt;        // first partial slot of this head
             ring[W_CTR] = ctrs_before + cinc - ccnt;          // first arrival counter group of this head
-            ring[W_DESC] = p.table_heads > 0 ? p.table_desc_begin[i] : pv.w[4] + 2 * pv.attn_begin()[u + h];
-            ring[W_NDESC] = p.table_heads > 0 ? (int)p.table_ndesc[i] : pv.attn_cnt()[u + h];
+            ring[W_DESC] = p.table_heads > 0 ? p.table_desc_begin[i] : pv.w[p.runs ? 18 : 4] + 2 * pv.attn_begin(p.runs)[u + h];
+            ring[W_NDESC] = p.table_heads > 0 ? (int)p.table_ndesc[i] : pv.attn_cnt(p.runs)[u + h];
             ring[W_KIND] = ATTENTION;
           }
           const bool any = __any_sync(0xffffffffu, mine);

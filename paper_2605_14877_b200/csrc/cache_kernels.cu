@@ -103,11 +103,11 @@ __global__ void __launch_bounds__(CP_THREADS) stage_fp8_kernel(const __grid_cons
   const int seq = (blockIdx.x >> 1) % n_seq, j = (blockIdx.x >> 1) / n_seq;
   PlanView pv(p.seqs[seq].plan);
   const int u0 = (p.step * p.L + p.layer) * p.H;
-  const int first = pv.attn_begin()[u0];
-  const int count = pv.attn_begin()[u0 + p.H - 1] + pv.attn_cnt()[u0 + p.H - 1] - first;
+  const int first = pv.attn_begin(p.runs)[u0];
+  const int count = pv.attn_begin(p.runs)[u0 + p.H - 1] + pv.attn_cnt(p.runs)[u0 + p.H - 1] - first;
   if (j >= count) return;
-  const int n = pv.descs()[first + j].y & 0xff;
-  const int64_t src_row = p.seqs[seq].base_row + pv.src_rows()[first + j];
+  const int n = pv.attn_descs(p.runs)[first + j].y & 0xff;
+  const int64_t src_row = p.seqs[seq].base_row + pv.src_rows(p.runs)[first + j];
   const int64_t dst_row = (int64_t)p.stage_base[seq] + (int64_t)j * HEATKV_PAGE_TOKENS;
   const uint8_t* codes = (is_v ? p.v8_pool : p.k8_pool) + src_row * p.d;
   const int8_t* exps = (is_v ? p.v_exp : p.k_exp) + src_row;

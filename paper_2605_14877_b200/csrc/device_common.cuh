@@ -77,6 +77,7 @@ struct AttnParams {
   // fp8 cache, small-step kernel: the codes themselves are read (no staging rows).  With table_heads > 0 the plan's word
   // offsets of the descriptors and of the pool rows behind them
   int32_t direct8, off_desc, off_src;
+  int32_t runs;                   // no per-scale bias: the plan's merged attention tables (PlanView)
 };
 
 struct CopyParams {
@@ -96,6 +97,7 @@ struct CopyParams {
   int8_t* k_exp;
   int8_t* v_exp;
   int32_t stage_base[HEATKV_MAX_BATCH];
+  int32_t runs;                   // as in AttnParams
 };
 
 // ---- plan blob accessors (see PlanHeader in internal.h: word offsets from the blob start)
@@ -106,8 +108,11 @@ struct PlanView {
   __device__ __forceinline__ int H() const { return w[1]; }
   __device__ __forceinline__ int K() const { return w[2]; }
   __device__ __forceinline__ const int2* descs() const { return reinterpret_cast<const int2*>(w + w[4]); }
-  __device__ __forceinline__ const int32_t* attn_begin() const { return w + w[5]; }
-  __device__ __forceinline__ const int32_t* attn_cnt() const { return w + w[6]; }
+  // tables of the attention; `runs`: those of calls without a per-scale bias, whose half-tiles may cross scales
+  __device__ __forceinline__ const int2* attn_descs(bool runs) const { return reinterpret_cast<const int2*>(w + w[runs ? 18 : 4]); }
+  __device__ __forceinline__ const int32_t* attn_begin(bool runs) const { return w + w[runs ? 19 : 5]; }
+  __device__ __forceinline__ const int32_t* attn_cnt(bool runs) const { return w + w[runs ? 20 : 6]; }
+  __device__ __forceinline__ const int32_t* src_rows(bool runs) const { return w + w[runs ? 21 : 17]; }   // fp8 cache only
   __device__ __forceinline__ const int32_t* app_begin() const { return w + w[7]; }
   __device__ __forceinline__ const int32_t* app_cnt() const { return w + w[8]; }
   __device__ __forceinline__ const int32_t* order() const { return w + w[9]; }
@@ -116,7 +121,6 @@ struct PlanView {
   __device__ __forceinline__ const int32_t* pre_cnt() const { return w + w[12]; }
   __device__ __forceinline__ const int32_t* post_begin() const { return w + w[13]; }
   __device__ __forceinline__ const int32_t* post_cnt() const { return w + w[14]; }
-  __device__ __forceinline__ const int32_t* src_rows() const { return w + w[17]; }   // fp8 cache only
 };
 
 // Programmatic dependent launch: every kernel lets the next one of the stream be set up while it runs (pdl_trigger, first

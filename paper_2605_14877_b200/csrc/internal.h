@@ -51,8 +51,20 @@ struct PlanHeader {
   int32_t total_words;
   int32_t off_src;         // fp8 cache only, else 0: int32[n_desc] pool row (relative to the reservation) behind
                            // every descriptor; the attention descriptors then carry staging rows instead
+  // The same attention tables once more for calls without a per-scale bias, where a half-tile need not stay inside one scale:
+  // neighbouring rows of one head make one run, cut every 64 rows.  They are the end of the blob; on the device they lie in a
+  // region of their own (or, when that is full, not at all), and these offsets, still from the blob's start, lead there
+  int32_t off_run_desc, off_run_begin, off_run_cnt, off_run_src;
   int32_t pad[2];
 };
+// What a call's attention reads: word offsets of the descriptors, of each head's first and count, and (fp8) of the pool rows.
+struct AttnTables {
+  int32_t desc, begin, cnt, src;
+};
+inline AttnTables attn_tables(const PlanHeader& h, bool runs) {
+  if (runs) return {h.off_run_desc, h.off_run_begin, h.off_run_cnt, h.off_run_src};
+  return {h.off_desc, h.off_attn_begin, h.off_attn_cnt, h.off_src};
+}
 static_assert(sizeof(PlanHeader) % 16 == 0, "header must keep 16-byte alignment");
 
 struct Plan {

@@ -39,6 +39,7 @@ class Session:
             torch.cuda.synchronize(self.device)
             hk.heatkv_destroy(self.ctx)
             self.ctx = None
+            self.arena = self._arena_view = None       # the device memory goes with the context, not with the last reference
 
     def __enter__(self):
         return self

@@ -351,6 +351,41 @@ def test_key_range_splitting_is_used_and_exact(hk):
                      kernel=hk.KERNEL_AUTO)
 
 
+@pytest.mark.parametrize("layout", [0, 1], ids=["ragged", "paged"])
+def test_merged_tables_are_optional(hk, layout):
+    """A plan whose merged attention tables find no room on the device (none here: 1 KB of scratch) runs on its per-scale ones,
+    also in a call together with a plan that has them (room for one plan's).  The same generation each way: both outputs are
+    within 1e-2 of the oracle elsewhere in this file, so they lie within 2e-2 of one another."""
+    from paper_2605_14877_b200.sweep import Session
+    sh = W.Shape("mid", L=1, H=6, d=128, sides=W.SIDES_13[:10], n_seq=2, s=3)
+    q, k, v = W.qkv_layer(sh, 0, 0, device="cuda")
+    outs = []
+    for scratch in (1 << 26, 1024, None):
+        if scratch is None:                       # an eighth of the scratch holds the tables of one plan, not of two
+            cfg = hk.Config.make(sh.L, sh.H, sh.d, sh.t, sh.s)
+            sch = hk.heatkv_build_schedule(cfg, scas=W.synthetic_scas(sh, 3), b=0.6)
+            words = hk.heatkv_schedule_plan(sch, layout)
+            hk.heatkv_schedule_free(sch)
+            one = (len(words) - int(words[18])) * 4
+            assert one > 1280                     # so that what is left of the last KB holds no second one
+            scratch = 8 * ((one + 255) // 256 * 256 + 1023 & ~1023)
+        with Session(sh.L, sh.H, sh.d, sh.t, sh.s, pool_rows=2 * sh.H * (sh.c[-2] + 64 * sh.K), layout=layout,
+                     scratch_bytes=scratch) as ses:
+            schs = [ses.schedule(scas=W.synthetic_scas(sh, seed), b=0.6) for seed in (3, 4)]
+            ids = [hk.heatkv_seq_open(ses.ctx, s) for s in schs]
+            out = torch.zeros_like(q)
+            ses.generate(ids, lambda l: (q, k, v), lambda l: out)
+            torch.cuda.synchronize()
+            assert hk.heatkv_device_status(ses.ctx) == 0
+            outs.append(out.float())
+            for i in ids:
+                hk.heatkv_seq_close(ses.ctx, i)
+            for s in schs:
+                hk.heatkv_schedule_free(s)
+    assert (outs[1] - outs[0]).abs().max().item() <= 2e-2
+    assert torch.equal(outs[1], outs[2])          # one plan without them: the whole call goes without
+
+
 def test_split_heads_are_reproducible_bit_for_bit(hk):
     """Pieces of a cut head are merged in piece order whichever arrives last: the same generation run four
     times gives identical output bits (steps of this workload are cut, see the test above)."""

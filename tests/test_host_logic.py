@@ -381,6 +381,53 @@ def test_split_plan_rejects_bad_input():
         hk.heatkv_split_plan([4, 0], n_qp=1, n_seq=1)
 
 
+@pytest.mark.parametrize("layout", [0, 1], ids=["ragged", "paged"])
+def test_plan_merged_tables_list_the_same_rows(hk, layout):
+    """The attention tables of calls without a bias: the same rows in the same order as the per-scale ones, in half-tiles
+    of at most 64 that only end where the rows stop being neighbours; with the fp8 cache the same through its row table."""
+    sh = W.Shape("mid", L=3, H=4, d=128, sides=W.SIDES_13[:11], n_seq=1, s=3)
+    cfg = hk.Config.make(sh.L, sh.H, sh.d, sh.t, sh.s)
+    sch = hk.heatkv_build_schedule(cfg, scas=W.synthetic_scas(sh, 4), b=0.3)
+    words = hk.heatkv_schedule_plan(sch, layout)
+    fp8 = hk.heatkv_schedule_plan_fp8(sch)[0] if layout == 1 else None
+    hk.heatkv_schedule_free(sch)
+    P = _Plan(words)
+    n = P.K * P.L * P.H
+
+    def tables(w):
+        off_desc, off_begin, off_cnt = (int(x) for x in w[18:21])
+        return (w[off_desc:], w[off_begin: off_begin + n].reshape(P.K, P.L, P.H), w[off_cnt: off_cnt + n].reshape(P.K, P.L, P.H))
+
+    desc, begin, cnt = tables(words)
+    fewer = 0
+    for k in range(P.K):
+        for l in range(P.L):
+            for h in range(P.H):
+                want, _ = P.rows(P.attn_begin[k, l, h], P.attn_cnt[k, l, h])
+                mine = desc[2 * begin[k, l, h]: 2 * (begin[k, l, h] + cnt[k, l, h])].reshape(-1, 2)
+                got = []
+                for i, (row, meta) in enumerate(mine):
+                    nv = int(meta) & 0xff
+                    assert 1 <= nv <= 64
+                    if got and got[-1] + 1 == row:                     # cut only because the half-tile before is full
+                        assert int(mine[i - 1, 1]) & 0xff == 64
+                    got += list(range(int(row), int(row) + nv))
+                assert got == want
+                assert cnt[k, l, h] <= P.attn_cnt[k, l, h]
+                fewer += int(P.attn_cnt[k, l, h] - cnt[k, l, h])
+    assert fewer > 0
+    if fp8 is not None:
+        fdesc, fbegin, fcnt = tables(fp8)
+        total = int(fcnt.sum())
+        src = fp8[int(fp8[21]): int(fp8[21]) + total]
+        assert np.array_equal(fbegin, begin) and np.array_equal(fcnt, cnt)
+        assert np.array_equal(src, desc[: 2 * total: 2]) and np.array_equal(fdesc[1: 2 * total: 2], desc[1: 2 * total: 2])
+        for k in range(P.K):
+            for l in range(P.L):
+                first, end = int(begin[k, l, 0]), int(begin[k, l, -1] + cnt[k, l, -1])
+                assert np.array_equal(fdesc[2 * first: 2 * end: 2], 64 * np.arange(end - first))
+
+
 def test_fp8_plan_renumbers_attention_rows_into_staging_slots(hk):
     """Plan of a context with the fp8 cache against the plain paged plan of the same schedule: same tables, the
     attention descriptors of every (step, layer) sit in consecutive 64-row staging slots in descriptor order, the
