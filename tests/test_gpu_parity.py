@@ -250,6 +250,32 @@ def test_tensor_memory_kernel_outlier_keys_head_dim_64(hk, where):
                      kernel=hk.KERNEL_TCGEN05, check_cache=False, fused=True, mutate=mutate)
 
 
+@pytest.mark.parametrize("token_major", [False, True], ids=["head_major", "token_major"])
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+def test_tensor_memory_kernel_writes_its_own_rows_only(hk, d, token_major):
+    """The output leaves in boxes of 32 rows: at token counts around multiples of 32 and 128 a step fills its rows of every head
+    and sequence and leaves the rows behind them alone."""
+    from paper_2605_14877_b200.sweep import Session
+    sh = W.Shape("guard", L=1, H=3, d=d, sides=(1, 5, 6, 8, 11, 12, 16, 17), n_seq=2, s=1)
+    q, k, v = W.qkv_layer(sh, 0, 0, device="cuda")
+    shape = (sh.n_seq, sh.c[-1] + 64, sh.H, d) if token_major else (sh.n_seq, sh.H, sh.c[-1] + 64, d)
+    buf = torch.full(shape, 7.0, dtype=torch.bfloat16, device="cuda")
+    out = buf.transpose(1, 2) if token_major else buf
+    with Session(sh.L, sh.H, sh.d, sh.t, sh.s, pool_rows=2 * sh.H * (sh.c[-2] + 64 * sh.K), kernel=hk.KERNEL_TCGEN05) as ses:
+        sch = ses.schedule(scas=W.synthetic_scas(sh, 3), b=1.0)
+        ids = [hk.heatkv_seq_open(ses.ctx, sch) for _ in range(sh.n_seq)]
+
+        def after(step, layer):
+            torch.cuda.synchronize()
+            lo, hi = ses.step_slices(step)
+            assert (out[:, :, hi:] == 7.0).all(), step
+            assert not (out[:, :, lo:hi] == 7.0).all(dim=-1).any(), step
+
+        ses.generate(ids, lambda l: (q, k, v), lambda l: out, None, after)
+        assert hk.heatkv_device_status(ses.ctx) == 0
+        hk.heatkv_schedule_free(sch)
+
+
 def test_tensor_memory_kernel_full_cache(hk):
     """b = 1: long page tables (up to 4121 prior keys), tcgen05 kernel, no bias."""
     sh = W.Shape("full128", L=1, H=2, d=128, sides=W.SIDES_13[:12], n_seq=1, s=3)
