@@ -571,6 +571,25 @@ def test_calibration_with_output_tensor_memory_kernel(hk, d, outliers):
     assert np.all(np.triu(beta, 1) == 0)
 
 
+@pytest.mark.parametrize("side", [6, 7], ids=["t36", "t49"])
+def test_calibration_with_output_kernel_choice(hk, side):
+    """Automatic choice with an output: 36 queries on the warp-level kernel, 49 on tensor memory; either matches the oracle."""
+    from paper_2605_14877_b200.sweep import Session
+    sh = W.Shape("choice", L=1, H=3, d=128, sides=(1, 3, side), n_seq=2, s=1)
+    beta, scas, cas, ref = _calibrate(hk, sh, seeds=[5], bias=W.seg_bias_prior_lognormal(sh, 8), with_out=True)
+    mask = ref > 1e-5
+    assert np.all(np.abs(beta - ref)[mask] <= RTOL_BETA * ref[mask])
+    with Session(sh.L, sh.H, sh.d, sh.t, sh.s, pool_rows=64) as ses:
+        q, k, v = W.qkv_layer(sh, 0, 0, device="cuda")
+        lo, hi = ses.step_slices(2)
+        qs, out = q[:, :, lo:hi], torch.zeros_like(q[:, :, lo:hi])
+        acc = torch.zeros(sh.L, sh.H, sh.K, sh.K, dtype=torch.float32, device="cuda")
+        hk.heatkv_calibrate_scores(ses.ctx, 0, 2, sh.n_seq, qs, k, v, hk.Strides.of(qs, k, out), None, acc, out)
+        torch.cuda.synchronize()
+        st = hk.heatkv_kernel_launches(ses.ctx)
+        assert (st.calibration_tcgen05, st.calibration_generic) == ((0, 1) if side == 6 else (1, 0))
+
+
 def test_config2_calibration_full_size(hk):
     """Sec. 3.1, Eq. 2 and Eq. 4 at the size the bench calibrates at: 13 scales, 2 sequences x 16 heads, bias on
     the current scale, automatic kernel choice (tensor-memory kernel for the seven steps of 256 tokens and more:
