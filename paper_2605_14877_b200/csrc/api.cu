@@ -582,7 +582,7 @@ int heatkv_schedule_footprint(const heatkv_schedule* sch, int layout, int64_t* p
   Plan plan;
   int rc;
   try {
-    rc = build_plan(sch->s, layout, &plan);
+    rc = build_plan(sch->s, layout, &plan, false, false);
   } catch (const std::bad_alloc&) {
     return HEATKV_ERR_HOST_MEMORY;
   }

@@ -67,7 +67,8 @@ __device__ __forceinline__ void group_sync(int grp) {
 }
 
 // GROUPS = 2: a launch that leaves SMs idle is a chain of key half-tiles (1.4 to 2 us each: copies, products at the
-// warp-level rate, softmax) per CTA; two groups of warps halve it.  GROUPS_MEASURED
+// warp-level rate, softmax) per CTA; two groups of warps halve it.  Back to back, 2 sequences x 16 heads:
+// 144 queries 19.8 us with one group and 12.4 with two, 64: 11.6 and 8.8, 36: 8.7 and 6.8.
 template <int D, bool CALIB, bool PARTIALS = false, int GROUPS = 1>
 __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_kernel(const __grid_constant__ AttnParams p) {
   extern __shared__ __align__(128) unsigned char smem[];

@@ -112,6 +112,7 @@ int build_schedule(const heatkv_config& cfg, const double* scas, const double* c
 // `fp8`: plan for a context with the fp8 cache (paged layout only): the attention descriptors of every
 // (step, layer) are renumbered to consecutive 64-row staging slots, in descriptor order across the layer's heads,
 // and a table of the pool rows behind them is added.
-int build_plan(const Schedule& sch, int layout, Plan* out, bool fp8 = false);
+// `tables` false: only the footprint (peak, reserved rows), not the blob
+int build_plan(const Schedule& sch, int layout, Plan* out, bool fp8 = false, bool tables = true);
 
 }  // namespace heatkv

@@ -44,16 +44,19 @@ struct Builder {
   void merge_runs() {
     run_begin.assign(attn_begin.size(), 0);
     run_cnt.assign(attn_begin.size(), 0);
+    run_descs.resize(descs.size());
+    Desc* out = run_descs.data();
     for (size_t u = 0; u < attn_begin.size(); ++u) {
-      run_begin[u] = (int32_t)run_descs.size();
+      run_begin[u] = (int32_t)(out - run_descs.data());
       for (int i = attn_begin[u], end = i + attn_cnt[u]; i < end;) {
         const int row = descs[i].row, scale = descs[i].meta >> 8;
         int n = 0;
         for (; i < end && descs[i].row == row + n; ++i) n += descs[i].meta & 0xff;
-        for (int off = 0; off < n; off += P) run_descs.push_back({row + off, pack_meta(std::min(P, n - off), scale)});
+        for (int off = 0; off < n; off += P) *out++ = {row + off, pack_meta(std::min(P, n - off), scale)};
       }
-      run_cnt[u] = (int32_t)run_descs.size() - run_begin[u];
+      run_cnt[u] = (int32_t)(out - run_descs.data()) - run_begin[u];
     }
+    run_descs.resize(out - run_descs.data());
   }
   void finish(Plan* out) {
     PlanHeader h{};
@@ -61,6 +64,9 @@ struct Builder {
     h.n_desc = (int32_t)descs.size();
     h.n_move = (int32_t)moves.size();
     std::vector<int32_t>& b = out->blob;
+    b.clear();
+    b.reserve(sizeof(PlanHeader) / 4 + 2 * (descs.size() + run_descs.size()) + 4 * moves.size() + 12 * attn_begin.size() +
+              src.size() + run_src.size() + 64);
     b.assign(sizeof(PlanHeader) / 4, 0);
     auto put = [&](const void* p, size_t bytes) {
       while (b.size() % 4) b.push_back(0);               // 16-byte alignment of every table
@@ -114,7 +120,7 @@ void fill_order(const Schedule& S, Builder& B) {
 
 }  // namespace
 
-int build_plan(const Schedule& S, int layout, Plan* out, bool fp8) {
+int build_plan(const Schedule& S, int layout, Plan* out, bool fp8, bool tables) {
   if (layout != HEATKV_LAYOUT_PAGED && layout != HEATKV_LAYOUT_RAGGED) return HEATKV_ERR_INVALID_ARG;
   if (fp8 && layout != HEATKV_LAYOUT_PAGED) return HEATKV_ERR_INVALID_ARG;
   const int L = S.L, H = S.H, K = S.K, s = S.s, T = L * H;
@@ -314,6 +320,7 @@ int build_plan(const Schedule& S, int layout, Plan* out, bool fp8) {
   }
   out->peak_tokens = peak_tokens;
   out->stage_rows = 0;
+  if (!tables) return HEATKV_OK;
   B.merge_runs();
   if (fp8) {
     // The attention kernels read bf16 staging rows that the call fills from the fp8 pool just before: the
