@@ -149,6 +149,11 @@ __device__ __forceinline__ Item read_item(const volatile int32_t* ring, const At
   it.qp = it.sub % n_qp;
   it.q0 = it.qp * (2 * BM);
   it.nq = (it.q0 + BM < p.t_q) ? 2 : 1;             // does tile B hold any query?
+  if (FULL) {                                       // one query tile of the pair (W_SLOT: 0 both, 1 the first, 2 the second)
+    const int single = ring_word(ring, W_SLOT);
+    if (single > 0) it.nq = 1;
+    if (single == 2) it.q0 += BM;
+  }
   it.n_slots = FULL ? it.n_desc : it.n_desc + (p.n_own + HALF - 1) / HALF;
   // this item's run of key tiles: [j0, j0 + n_tiles) of the head's ceil(n_slots / 2)
   const int piece_tiles = (tiles + it.n_split - 1) / it.n_split;
@@ -263,8 +268,10 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
       // from the host's table, else from the launch's longest run), and every (piece, query tile pair) is
       // one item, pieces outermost.  A prefix sum over the
       // heads finds the item.
-      const int seq = idx % p.n_seq;
-      const int item = idx / p.n_seq;
+      // (FULL: past full_whole the items are single query tiles, so that the last round of CTAs is not half empty)
+      const int pair = FULL && idx > p.full_whole ? p.full_whole + (idx - p.full_whole) / 2 : idx;
+      const int seq = pair % p.n_seq;
+      const int item = pair / p.n_seq;
       if (lane == 0) {
         ring[W_KIND] = FULL ? ATTENTION : NOTHING;      // sequences of a call may differ in item count
         if (FULL) {                                     // all heads alike: query tile pair fastest
@@ -273,7 +280,9 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
           ring[W_TILES] = (p.full_slots + 1) >> 1;
           ring[W_NSPLIT] = 1;
           ring[W_SUB] = item % n_qp;
-          ring[W_SLOT] = ring[W_CTR] = ring[W_DESC] = 0;
+          ring[W_CTR] = ring[W_DESC] = 0;
+          ring[W_SLOT] = idx < p.full_whole ? 0 : 1 + ((idx - p.full_whole) & 1);
+          if (ring[W_SLOT] == 2 && item % n_qp * (2 * BM) + BM >= p.t_q) ring[W_KIND] = NOTHING;
           ring[W_NDESC] = p.full_slots;
         }
       }
@@ -561,12 +570,12 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
           nq = im.nq;
         }
         if (x < nq) {
-          int j0, n_desc, n_slots;
+          int j0, n_desc, n_slots, q0;
           const int2* descs;
           const float* bias_h;
           {
             const Item im = read_item<FULL>(ring, p, n_qp);
-            j0 = im.j0; n_desc = im.n_desc; n_slots = im.n_slots;
+            j0 = im.j0; n_desc = im.n_desc; n_slots = im.n_slots; q0 = im.q0;
             descs = FULL ? p.full_descs : reinterpret_cast<const int2*>(p.seqs[im.seq].plan + im.desc_begin);
             bias_h = p.seg_bias ? p.seg_bias + im.head * p.K : nullptr;
           }
@@ -579,7 +588,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
           int j = 0;
           // FULL: a warp whose 32 rows all lie past the last query hands on whatever is there (its rows of O and its masses go
           // nowhere): a calibration pass 1.130 -> 1.115 ms.  Generation measured 0.3 to 0.8 % slower with the branch.
-          const bool no_rows = FULL && ring_word(ring, W_SUB) % n_qp * (2 * BM) + x * BM + (warp & 3) * 32 >= p.t_q;
+          const bool no_rows = FULL && q0 + x * BM + (warp & 3) * 32 >= p.t_q;
           for (; no_rows && j < n_tiles && ok; ++j) {
             ok = __all_sync(0xffffffffu, mbar_wait(bar(S_FULL + x), (cx + j) & 1, abort_flag, p.status));
             mbar_arrive(bar(P_FULL + 2 * x));
@@ -1084,6 +1093,19 @@ cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int n_seq, cudaStre
   q.store_items = p.append_tiles * p.H * n_seq;
   dim3 grid((unsigned)std::min(q.attn_items, st->n_sm));
   const bool full = p.full_slots > 0;
+  if (full) {
+    // Items of calibration are all of one length, so a partly filled last round costs as much as a full one.  Where its single
+    // query tiles would still all run at once it is issued as those (a tile alone is quicker per key tile than one of a
+    // pair): 2 sequences x 16 heads, 256 queries 16.7 -> 14.7 us, 400: 24.0 -> 21.7, 1600: 123.2 -> 117.6; a pass 1.105 -> 1.073 ms.
+    const int total = q.attn_items, n_qp = (p.t_q + 2 * tc::BM - 1) / (2 * tc::BM), whole = total / st->n_sm * st->n_sm;
+    const bool tail_single = p.t_q - (n_qp - 1) * 2 * tc::BM <= tc::BM;
+    int singles = 0;
+    for (int i = whole; i < total; ++i) singles += (tail_single && i / n_seq % n_qp == n_qp - 1) ? 1 : 2;
+    const bool cut = singles <= st->n_sm && total < INT32_MAX - 2 * st->n_sm;
+    q.full_whole = cut ? whole : total;
+    if (cut) q.attn_items = whole + 2 * (total - whole);
+    grid = dim3((unsigned)std::min(q.attn_items, st->n_sm));
+  }
   if (st->d == 128)
     return launch_pdl(full ? tc::attn_tc_kernel<128, true> : tc::attn_tc_kernel<128, false>, grid, tc::THREADS,
                       tc::Layout<128>::SM_ALLOC, stream, q, maps);

@@ -78,6 +78,7 @@ struct AttnParams {
   // offsets of the descriptors and of the pool rows behind them
   int32_t direct8, off_desc, off_src;
   int32_t runs;                   // no per-scale bias: the plan's merged attention tables (PlanView)
+  int32_t full_whole;             // calibration with output: work items before this one hold a pair of query tiles, later ones one
 };
 
 struct CopyParams {
