@@ -37,9 +37,9 @@ __device__ __forceinline__ uint32_t tile_off(int r, int ch) {
   return (uint32_t)((r * (D / 8) + (ch ^ (r & 7))) * 16);
 }
 
-// copies n_valid rows (row-major, D bf16 each, `stride` elements apart) into a swizzled tile; rows from there to the
-// next multiple of 16 (what the products read) are zero-filled.
-template <int D, int THREADS = GTHREADS>
+// copies n_valid rows (row-major, D bf16 each, `stride` elements apart) into a swizzled tile; the rows behind them that the
+// products read are zero-filled: all of the tile's (WHOLE), or those up to the next multiple of 16.
+template <int D, bool WHOLE, int THREADS = GTHREADS>
 __device__ __forceinline__ void load_tile(uint32_t smem_base, const __nv_bfloat16* src, int64_t stride,
                                           int n_valid, int tid) {
   constexpr int CH = D / 8;
@@ -49,7 +49,7 @@ __device__ __forceinline__ void load_tile(uint32_t smem_base, const __nv_bfloat1
   const int rows = (n_valid + 15) & ~15;
 #pragma unroll
   for (int r = r0; r < GN; r += ROWS_PER_PASS) {
-    if (r >= rows) break;
+    if (!WHOLE && r >= rows) break;
     const bool ok = r < n_valid;
     const __nv_bfloat16* p = ok ? src + (int64_t)r * stride + ch * 8 : src;
     cp_async16(smem_base + tile_off<D>(r, ch), p, ok ? 16 : 0);
@@ -73,10 +73,15 @@ template <int D, bool CALIB, bool PARTIALS = false, int GROUPS = 1>
 __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_kernel(const __grid_constant__ AttnParams p) {
   extern __shared__ __align__(128) unsigned char smem[];
   using SM = GenericSmem<D, GROUPS>;
+  // Two groups run a launch that is bound by latency: there the empty 16-key groups of a short tile, and warps without query
+  // rows, are skipped.  With one group the launch fills the GPU, and the branches cost more than they save: 1024 queries
+  // x 512 units 1951 -> 1287 us without them, allocation-free calibration over 13 scales 6.73 -> 4.70 ms, 64 queries
+  // x 512 units 22.1 -> 17.8 us.
+  constexpr bool SKIP = GROUPS == 2;
   static_assert(GROUPS == 1 || !CALIB, "the scale masses are kept by one group");
   const int grp = GROUPS == 1 ? 0 : __shfl_sync(0xffffffffu, (int)threadIdx.x / GTHREADS, 0);
   const int tid = threadIdx.x - grp * GTHREADS, warp = tid >> 5, lane = tid & 31;
-  pdl_trigger();
+  if (!PARTIALS) pdl_trigger();                        // (its follower, one small reduction, took SM slots from the tail: 64-wide heads 3 %)
   const int g = lane >> 2, qd = lane & 3;
   // attention: grid = (query tiles, sequences, heads by descending key count), so the heaviest heads of
   // every sequence are dispatched first; calibration: grid = (query tiles, heads, sequences)
@@ -165,8 +170,8 @@ __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_ke
       stride = p.kv_tok;
       nv = min(GN, n_own - jj * GN);
     }
-    load_tile<D>(gbase + SM::K_OFF + stage * SM::TILE_BYTES, ks, stride, nv, tid);
-    if (vs) load_tile<D>(gbase + SM::V_OFF + stage * SM::TILE_BYTES, vs, stride, nv, tid);
+    load_tile<D, !SKIP>(gbase + SM::K_OFF + stage * SM::TILE_BYTES, ks, stride, nv, tid);
+    if (vs) load_tile<D, !SKIP>(gbase + SM::V_OFF + stage * SM::TILE_BYTES, vs, stride, nv, tid);
     if (j + GROUPS < n_desc) dsc_next = descs[j + GROUPS];
   };
 
@@ -174,7 +179,7 @@ __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_ke
   // ---- prologue: Q tile and the first GSTAGES - 1 key tiles, one copy group each (empty groups keep the count)
   {
     const __nv_bfloat16* qsrc = q_base + seq * p.q_seq + head * p.q_head + (int64_t)q0 * p.q_tok;
-    load_tile<D, GTHREADS * GROUPS>(sbase + SM::Q_OFF, qsrc, p.q_tok, min(GM, t_q - q0), threadIdx.x);
+    load_tile<D, !SKIP, GTHREADS * GROUPS>(sbase + SM::Q_OFF, qsrc, p.q_tok, min(GM, t_q - q0), threadIdx.x);
     cp_async_commit();
     for (int i = 0; i < GSTAGES - 1; ++i) {
       if (grp + i * GROUPS < n_tiles) issue_tile(grp + i * GROUPS, i);
@@ -204,7 +209,7 @@ __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_ke
   float m_run[2] = {-INFINITY, -INFINITY};
   float l_run[2] = {0.f, 0.f};
 
-  const bool has_rows = q0 + warp * 16 < t_q;          // a warp without query rows only helps with the copies
+  const bool has_rows = !SKIP || q0 + warp * 16 < t_q;  // SKIP: a warp without query rows only helps with the copies
   for (int i = 0, j = grp; j < n_tiles; ++i, j += GROUPS) {
     const int stage = i % GSTAGES;
     cp_async_wait<GSTAGES - 2>();                      // all groups but the newest GSTAGES - 2: tile j is among them
@@ -234,7 +239,7 @@ __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_ke
       }
     }
 
-    // ---- S = Q K^T (a tile of a small scale has few keys: its empty groups of 16 are skipped throughout)
+    // ---- S = Q K^T
     float s[GN / 8][4];
 #pragma unroll
     for (int i = 0; i < GN / 8; ++i) s[i][0] = s[i][1] = s[i][2] = s[i][3] = 0.f;
@@ -243,7 +248,7 @@ __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_ke
     for (int ks = 0; ks < D / 16; ++ks) {
 #pragma unroll
       for (int np = 0; np < GN / 16; ++np) {
-        if (np * 16 >= nv) break;
+        if (SKIP && np * 16 >= nv) break;
         uint32_t b[4];
         int r = np * 16 + (lane & 7) + (lane >> 4) * 8;
         int ch = ks * 2 + ((lane >> 3) & 1);
@@ -260,7 +265,7 @@ __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_ke
     float mx[2] = {-INFINITY, -INFINITY};
 #pragma unroll
     for (int n = 0; n < GN / 8; ++n) {
-      if ((n & ~1) * 8 >= nv) break;
+      if (SKIP && (n & ~1) * 8 >= nv) break;
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         int col = n * 8 + qd * 2 + (e & 1);
@@ -288,7 +293,7 @@ __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_ke
     float psum[2] = {0.f, 0.f};
 #pragma unroll
     for (int n = 0; n < GN / 8; ++n) {
-      if ((n & ~1) * 8 >= nv) break;
+      if (SKIP && (n & ~1) * 8 >= nv) break;
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         float pv = exp2f(s[n][e] - m_run[e >> 1]);
@@ -339,7 +344,7 @@ __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_ke
       const uint32_t vbase = gbase + SM::V_OFF + stage * SM::TILE_BYTES;
 #pragma unroll
       for (int kk = 0; kk < GN / 16; ++kk) {
-        if (kk * 16 >= nv) break;
+        if (SKIP && kk * 16 >= nv) break;
         uint32_t pa[4];
         pa[0] = pack_bf16(s[2 * kk][0], s[2 * kk][1]);
         pa[1] = pack_bf16(s[2 * kk][2], s[2 * kk][3]);
