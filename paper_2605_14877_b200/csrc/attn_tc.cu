@@ -343,6 +343,8 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
       if (!is_attn) continue;
       const int2* descs = FULL ? p.full_descs : reinterpret_cast<const int2*>(p.seqs[seq].plan + im.desc_begin);
       const int64_t base_row = FULL ? 0 : p.seqs[seq].base_row;
+      const int q_head = map_index(im.head, p.q_head), q_seq = map_index(seq, p.q_seq);
+      const int kv_head = map_index(im.head, p.kv_head), kv_seq = map_index(seq, p.kv_seq);
       for (int j = 0; j < im.n_tiles && ok; ++j, ++g) {
         const uint32_t st = g % KV_STAGES;
         const uint32_t use = g / KV_STAGES;
@@ -362,7 +364,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             for (int ch = 0; ch < NCH; ++ch) {
               uint32_t dst = sbase + SM_K + st * TILE_BYTES + ch * HALF_COLS_BYTES + hf * SLOT_BYTES;
               if (sl[hf].pool_row >= 0) tma_load_2d(dst, &maps.k_pool, ch * 64, sl[hf].pool_row, bar(K_FULL + st));
-              else tma_load_4d(dst, &maps.k_own, ch * 64, -sl[hf].pool_row - 1, im.head, seq, bar(K_FULL + st));
+              else tma_load_4d(dst, &maps.k_own, ch * 64, -sl[hf].pool_row - 1, kv_head, kv_seq, bar(K_FULL + st));
             }
         }
         if (j == 0) {
@@ -380,7 +382,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
               for (int ch = 0; ch < NCH; ++ch)
                 for (int hf = 0; hf < 2; ++hf)
                   tma_load_4d(sbase + SM_Q + x * TILE_BYTES + ch * HALF_COLS_BYTES + hf * SLOT_BYTES, &maps.q, ch * 64,
-                              im.q0 + x * BM + hf * HALF, im.head, seq, bar(Q_FULL + x));
+                              im.q0 + x * BM + hf * HALF, q_head, q_seq, bar(Q_FULL + x));
             }
           }
           if (!ok) break;
@@ -395,7 +397,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             for (int ch = 0; ch < NCH; ++ch) {
               uint32_t dst = sbase + SM_V + st * TILE_BYTES + ch * HALF_COLS_BYTES + hf * SLOT_BYTES;
               if (sl[hf].pool_row >= 0) tma_load_2d(dst, &maps.v_pool, ch * 64, sl[hf].pool_row, bar(V_FULL + st));
-              else tma_load_4d(dst, &maps.v_own, ch * 64, -sl[hf].pool_row - 1, im.head, seq, bar(V_FULL + st));
+              else tma_load_4d(dst, &maps.v_own, ch * 64, -sl[hf].pool_row - 1, kv_head, kv_seq, bar(V_FULL + st));
             }
         }
         __syncwarp();
@@ -806,8 +808,8 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0 && any_row) {
-              tma_store_4d(&maps.out, smem_u32(buf), c * 32, q_row0 + (warp & 3) * 32, p.o_head > 0 ? im.head : 0,
-                           p.o_seq > 0 ? seq : 0);
+              tma_store_4d(&maps.out, smem_u32(buf), c * 32, q_row0 + (warp & 3) * 32, map_index(im.head, p.o_head),
+                           map_index(seq, p.o_seq));
               bulk_commit();
             }
           };
@@ -1005,14 +1007,11 @@ bool encode_2d(TcState* st, CUtensorMap* m, void* base, uint64_t rows) {
 // [n_seq, H, t, d] view with element strides -> 4-D map (d, token, head, sequence)
 bool encode_4d(TcState* st, CUtensorMap* m, const void* base, int t, int H, int n_seq, int64_t s_tok, int64_t s_head,
                int64_t s_seq, bool output = false) {
-  cuuint64_t dims[4] = {(cuuint64_t)st->d, (cuuint64_t)t, (cuuint64_t)H, (cuuint64_t)n_seq};
-  // a stride of 0 is not encodable; a dimension of extent 1 may carry any positive stride
-  auto fix = [](int64_t s) { return (cuuint64_t)((s > 0 ? s : 8) * 2); };
-  cuuint64_t strides[3] = {fix(s_tok), fix(s_head), fix(s_seq)};
+  const tc::MapShape g = tc::map_shape(st->d, t, H, n_seq, s_tok, s_head, s_seq);
   // inputs: 64 x 64 boxes; the output leaves in a warp's 32 rows x 32 columns
   cuuint32_t box[4] = {output ? 32u : 64u, output ? 32u : (cuuint32_t)tc::HALF, 1, 1};
   cuuint32_t estr[4] = {1, 1, 1, 1};
-  return st->encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
+  return st->encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), g.dims, g.strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, output ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }

@@ -100,7 +100,9 @@ __device__ __forceinline__ HalfTile get_half(int i, const int2* descs, int n_slo
   return h;
 }
 
-template <int D>
+// SHARED: a head or sequence stride is 0.  An instantiation of its own because the two index choices of the producer cost
+// the other one its registers (112 bytes of spill loads, one calibration batch of recorded steps 0.726 -> 0.755 ms).
+template <int D, bool SHARED>
 __global__ void __launch_bounds__(THREADS, 1)
 calib_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Maps maps, const int2* __restrict__ all_descs,
                 const __grid_constant__ StepTable tab, int n_seq, int64_t bias_step_stride) {
@@ -171,10 +173,12 @@ calib_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Ma
           for (int ch = 0; ch < NCH; ++ch)
             for (int hf = 0; hf < 2; ++hf)
               tma_load_4d(sbase + SM_Q + x * TILE_BYTES + ch * HALF_COLS_BYTES + hf * SLOT_BYTES, &maps.q, ch * 64,
-                          q_tok + x * BM + hf * HALF, head, seq, bar(Q_FULL + x));
+                          q_tok + x * BM + hf * HALF, SHARED ? map_index(head, p.q_head) : head,
+                          SHARED ? map_index(seq, p.q_seq) : seq, bar(Q_FULL + x));
         }
       }
       bool ok = true;
+      const int kv_head = SHARED ? map_index(head, p.kv_head) : head, kv_seq = SHARED ? map_index(seq, p.kv_seq) : seq;
       for (int j = 0; j < n_tiles && ok; ++j) {
         const int st = j % K_STAGES;
         const uint32_t use = (uint32_t)(j / K_STAGES);
@@ -188,7 +192,7 @@ calib_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Ma
           for (int hf = 0; hf < 2; ++hf)
             for (int ch = 0; ch < NCH; ++ch)
               tma_load_4d(sbase + SM_K + st * TILE_BYTES + ch * HALF_COLS_BYTES + hf * SLOT_BYTES, &maps.k, ch * 64,
-                          hf == 0 ? h0.row : h1.row, head, seq, bar(K_FULL + st));
+                          hf == 0 ? h0.row : h1.row, kv_head, kv_seq, bar(K_FULL + st));
         }
         __syncwarp();
       }
@@ -383,6 +387,11 @@ struct CalibTcState {
   bool ready = false;
 };
 
+static auto calib_kernel(int d, bool shared) {
+  if (shared) return d == 128 ? calib::calib_tc_kernel<128, true> : calib::calib_tc_kernel<64, true>;
+  return d == 128 ? calib::calib_tc_kernel<128, false> : calib::calib_tc_kernel<64, false>;
+}
+
 uint64_t calib_tc_desc_bytes(const heatkv_config& cfg) {
   uint64_t n = 0;
   for (int step = 0; step < cfg.K; ++step)
@@ -428,18 +437,20 @@ int calib_tc_create(const heatkv_config& cfg, void* dev_table, cudaStream_t stre
   // later calls may come on other streams: the table must be in place before create returns
   if (cudaStreamSynchronize(stream) != cudaSuccess) return HEATKV_ERR_CUDA;
   st->dev_descs = static_cast<const int2*>(dev_table);
-  const void* kern = cfg.d == 128 ? (const void*)calib::calib_tc_kernel<128> : (const void*)calib::calib_tc_kernel<64>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)calib::SM_ALLOC) != cudaSuccess) {
-    cudaGetLastError();
-    return HEATKV_OK;
+  for (const bool shared : {false, true}) {
+    const auto kern = calib_kernel(cfg.d, shared);
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)calib::SM_ALLOC) != cudaSuccess) {
+      cudaGetLastError();
+      return HEATKV_OK;
+    }
+    cudaFuncAttributes attr;
+    if (cudaFuncGetAttributes(&attr, kern) != cudaSuccess) {
+      cudaGetLastError();
+      return HEATKV_OK;
+    }
+    // the register hand-over inside the kernel must fit in what the launch really allocates
+    if (attr.numRegs * calib::THREADS < 128 * calib::REGS_UTIL + 512 * calib::REGS_SOFTMAX) return HEATKV_ERR_CUDA;
   }
-  cudaFuncAttributes attr;
-  if (cudaFuncGetAttributes(&attr, kern) != cudaSuccess) {
-    cudaGetLastError();
-    return HEATKV_OK;
-  }
-  // the register hand-over inside the kernel must fit in what the launch really allocates
-  if (attr.numRegs * calib::THREADS < 128 * calib::REGS_UTIL + 512 * calib::REGS_SOFTMAX) return HEATKV_ERR_CUDA;
   st->ready = true;
   return HEATKV_OK;
 }
@@ -465,12 +476,10 @@ bool calib_tc_supported(const CalibTcState* st, const AttnParams& p, int d, int 
 namespace {
 bool encode_4d(CalibTcState* st, CUtensorMap* m, const void* base, int t, int H, int n_seq, int64_t s_tok, int64_t s_head,
                int64_t s_seq) {
-  cuuint64_t dims[4] = {(cuuint64_t)st->d, (cuuint64_t)t, (cuuint64_t)H, (cuuint64_t)n_seq};
-  auto fix = [](int64_t s) { return (cuuint64_t)((s > 0 ? s : 8) * 2); };
-  cuuint64_t strides[3] = {fix(s_tok), fix(s_head), fix(s_seq)};
+  const tc::MapShape g = tc::map_shape(st->d, t, H, n_seq, s_tok, s_head, s_seq);
   cuuint32_t box[4] = {64, (cuuint32_t)calib::HALF, 1, 1};
   cuuint32_t estr[4] = {1, 1, 1, 1};
-  return st->encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
+  return st->encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), g.dims, g.strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -508,10 +517,8 @@ cudaError_t launch_calib_tc_steps(CalibTcState* st, const AttnParams& p, int n_s
   }
   tab.cta_begin[n_steps] = ctas;
   dim3 grid((unsigned)ctas);
-  if (st->d == 128)
-    return launch_pdl(calib::calib_tc_kernel<128>, grid, calib::THREADS, calib::SM_ALLOC, stream, p, maps, st->dev_descs, tab,
-                      n_seq, bias_step_stride);
-  return launch_pdl(calib::calib_tc_kernel<64>, grid, calib::THREADS, calib::SM_ALLOC, stream, p, maps, st->dev_descs, tab, n_seq,
+  const bool shared = (p.H > 1 && (p.q_head == 0 || p.kv_head == 0)) || (n_seq > 1 && (p.q_seq == 0 || p.kv_seq == 0));
+  return launch_pdl(calib_kernel(st->d, shared), grid, calib::THREADS, calib::SM_ALLOC, stream, p, maps, st->dev_descs, tab, n_seq,
                     bias_step_stride);
 }
 

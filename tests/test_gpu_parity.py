@@ -484,6 +484,41 @@ def _calibrate(hk, sh, seeds, bias=None, with_out=False, kernel=None, mutate=Non
     return beta, scas, cas, ref
 
 
+def _shared(x, over):
+    """The first sequence's (dim 0) or head's (dim 1) part of x for all of them: a view of stride 0."""
+    for dim in over:
+        x = x.narrow(dim, 0, 1).expand(*[x.shape[i] if i == dim else -1 for i in range(4)])
+    return x
+
+
+@pytest.mark.parametrize("q_over,kv_over", [((), (1,)), ((0,), (0, 1)), ((0, 1), (0,))], ids=["kv_heads", "all_seqs", "q_both"])
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+def test_activations_shared_by_heads_or_sequences(hk, d, q_over, kv_over):
+    """Strides of 0 along heads or sequences: generation on both kernels (steps of 1 to 400 queries), calibration step by step
+    with and without an output, and all steps in one call."""
+    from paper_2605_14877_b200.sweep import Session
+    sh = W.Shape("shared", L=1, H=3, d=d, sides=(1, 2, 4, 7, 12, 16, 20), n_seq=2, s=2)
+    scores = W.synthetic_scas(sh, 6)
+    ref = O.heatkv_schedule(scores, 0.6, sh.s, sh.sides)
+    bias = W.seg_bias_prior_lognormal(sh, 6)
+    for kernel in (hk.KERNEL_AUTO, hk.KERNEL_TCGEN05):
+        _run_full_parity(hk, sh, ref, lambda ses: ses.schedule(scas=scores, b=0.6), hk.LAYOUT_PAGED, bias=bias, kernel=kernel,
+                         fused=True, mutate=lambda l, q, k, v: (_shared(q, q_over), _shared(k, kv_over), _shared(v, kv_over)))
+        for with_out in (False, True):
+            beta, _, _, want = _calibrate(hk, sh, seeds=[5], bias=bias, with_out=with_out, kernel=kernel,
+                                          mutate=lambda q, k, v: (_shared(q, q_over), _shared(k, kv_over), _shared(v, kv_over)))
+            mask = want > 1e-5
+            assert np.all(np.abs(beta - want)[mask] <= RTOL_BETA * want[mask])
+        with Session(sh.L, sh.H, sh.d, sh.t, sh.s, pool_rows=64, kernel=kernel) as ses:
+            q, k, _ = W.qkv_layer(sh, 5, 0, device="cuda")
+            q, k = _shared(q, q_over), _shared(k, kv_over)
+            acc = torch.zeros(sh.L, sh.H, sh.K, sh.K, dtype=torch.float32, device="cuda")
+            hk.heatkv_calibrate_scores_steps(ses.ctx, 0, 0, sh.K, sh.n_seq, q, k, hk.Strides.of(q, k),
+                                             torch.from_numpy(bias).cuda()[0].contiguous(), acc)
+            beta = hk.heatkv_finalize_scores(ses.ctx, acc, sh.n_seq, sh.L, sh.H, sh.K)[0]
+            assert np.all(np.abs(beta - want)[mask] <= RTOL_BETA * want[mask])
+
+
 def test_calibration_tiny_four_samples(hk):
     sh = W.TINY
     beta, scas, cas, ref = _calibrate(hk, sh, seeds=range(4))
