@@ -224,8 +224,9 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_ptr_smem, 0);
-  // (every role waits for the launches before this one where it first touches what they may still use; the MMA warp only
-  // follows the others' barriers)
+  // (every role waits for the launches before this one where it first touches what they may still use, and before its first
+  // wait for another role: the tries of a bounded wait are for this CTA's own copies and products, not for a launch that is
+  // still running)
 
   // register budget per warpgroup: 128*72 + 256*216 <= 64K
   if (warp < 4) {
@@ -424,6 +425,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
     const uint32_t lead = elect_one();
     constexpr uint32_t IDESC_S = instr_desc(BM, BN, 0, 0);     // Q, K both K-major
     constexpr uint32_t IDESC_PV = instr_desc(BM, D, 0, 1);     // P from TMEM, V MN-major
+    pdl_wait();
     bool ok = true;
     // 64-wide heads wait with the vote in the loop (1.621 -> 1.588 ms); for 128-wide ones it measured 1 to 2 % slower
     auto mma_wait = [&](uint32_t b, uint32_t parity) {

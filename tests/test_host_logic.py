@@ -466,3 +466,21 @@ def test_fp8_plan_renumbers_attention_rows_into_staging_slots(hk):
         b0, n = int(pb[u]), int(pc[u])
         assert not is_attn[b0: b0 + n].any() and np.array_equal(fd[b0: b0 + n, 0], pd[b0: b0 + n, 0])
     assert stage_rows == 64 * busiest and busiest > 0
+
+
+def test_bounded_waits_start_after_the_launch_before():
+    """Kernels that may start while the launch before them runs: no role of a CTA begins a bounded wait (it gives up after a
+    number of tries) before it has waited for that launch, whose run time is not the CTA's."""
+    bounded = re.compile(r"\b(?:warp_wait|warp_wait_vote|mbar_wait|mbar_wait_hint|mma_wait)\(bar\(")
+    roles = 0
+    for name in ("attn_tc.cu", "calib_tc.cu"):
+        with open(os.path.join(ROOT, "paper_2605_14877_b200", "csrc", name)) as f:
+            body = f.read()
+        body = body[body.index(name.replace(".cu", "_kernel(")):]
+        common, *parts = re.split(r"// -{40,} ", body)
+        for part in parts:
+            first = bounded.search(part)
+            if first:
+                assert "pdl_wait();" in common + part[: first.start()], (name, part.splitlines()[0])
+                roles += 1
+    assert roles == 6                                       # copies, products, softmax of either kernel
