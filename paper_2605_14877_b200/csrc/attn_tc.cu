@@ -792,8 +792,11 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
           // store writes the 32 rows, clipping those past the last query.  The halves of the buffer alternate.  Loads from the
           // buffer and 16-byte stores by all lanes took 3000 to 3700 cycles of every item; image pair at 20x 2.219 -> 2.183 ms, eight
           // images at 10x 3.659 -> 3.623, ragged 2.492 -> 2.458, preview 162.8 -> 158.7 us, 64-wide heads as before.
+          // A warp without a row below the last query writes nothing, the buffer included: its last store may still be reading one
+          // half, and only a store of its own for every group would make the wait for all but the newest one cover that half.
           const bool any_row = q_row0 + (warp & 3) * 32 < p.t_q;
           auto store_rows = [&](const float (&acc)[32], float inv, int c) {
+            if (!any_row) return;
             unsigned char* buf = stage + (c & 1) * 2048;
             if (lane == 0) bulk_wait_read<1>();                 // the store before the last has read this half
             __syncwarp();
@@ -809,7 +812,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
-            if (lane == 0 && any_row) {
+            if (lane == 0) {
               tma_store_4d(&maps.out, smem_u32(buf), c * 32, q_row0 + (warp & 3) * 32, map_index(im.head, p.o_head),
                            map_index(seq, p.o_seq));
               bulk_commit();

@@ -276,6 +276,31 @@ def test_tensor_memory_kernel_writes_its_own_rows_only(hk, d, token_major):
         hk.heatkv_schedule_free(sch)
 
 
+@pytest.mark.parametrize("calibrate", [False, True], ids=["generation", "calibration"])
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+def test_tensor_memory_kernel_rows_survive_an_item_without_rows(hk, d, calibrate):
+    """400 queries x 320 (sequence, head) units: more items than SMs, and in every second one three warps hold no query, right
+    after an item whose rows may still be leaving their staging buffers.  All rows against attention in 64 bits."""
+    from paper_2605_14877_b200.sweep import Session
+    sh = W.Shape("norows", L=1, H=16, d=d, sides=(1, 20), n_seq=20, s=1)
+    q, k, v = W.qkv_layer(sh, 0, 0, device="cuda")
+    out = torch.zeros_like(q)
+    with Session(sh.L, sh.H, sh.d, sh.t, sh.s, pool_rows=sh.n_seq * sh.H * 128, kernel=hk.KERNEL_TCGEN05) as ses:
+        if calibrate:
+            acc = torch.zeros(sh.L, sh.H, sh.K, sh.K, dtype=torch.float32, device="cuda")
+            qs, os_ = q[:, :, 1:], out[:, :, 1:]
+            hk.heatkv_calibrate_scores(ses.ctx, 0, 1, sh.n_seq, qs, k, v, hk.Strides.of(qs, k, os_), None, acc, os_)
+        else:
+            sch = ses.schedule(scas=W.synthetic_scas(sh, 3), b=1.0)
+            ids = [hk.heatkv_seq_open(ses.ctx, sch) for _ in range(sh.n_seq)]
+            ses.generate(ids, lambda l: (q, k, v), lambda l: out)
+            hk.heatkv_schedule_free(sch)
+        torch.cuda.synchronize()
+        assert hk.heatkv_device_status(ses.ctx) == 0
+    p = torch.softmax(q[:, :, 1:].double() @ k.double().transpose(2, 3) / math.sqrt(d), dim=-1)
+    assert (out[:, :, 1:].double() - p @ v.double()).abs().max().item() <= ATOL_MAX
+
+
 def test_tensor_memory_kernel_full_cache(hk):
     """b = 1: long page tables (up to 4121 prior keys), tcgen05 kernel, no bias."""
     sh = W.Shape("full128", L=1, H=2, d=128, sides=W.SIDES_13[:12], n_seq=1, s=3)
