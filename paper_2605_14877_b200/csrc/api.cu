@@ -252,6 +252,9 @@ void fill_common(const heatkv_ctx* ctx, AttnParams* p, const heatkv_strides& s) 
   p->q_seq = s.q_seq; p->q_head = s.q_head; p->q_tok = s.q_tok;
   p->kv_seq = s.kv_seq; p->kv_head = s.kv_head; p->kv_tok = s.kv_tok;
   p->o_seq = s.o_seq; p->o_head = s.o_head; p->o_tok = s.o_tok;
+  auto mask = [](int64_t stride) { return stride > 0 ? ~0 : 0; };
+  p->q_head_mask = mask(s.q_head); p->q_seq_mask = mask(s.q_seq);
+  p->kv_head_mask = mask(s.kv_head); p->kv_seq_mask = mask(s.kv_seq);
   p->H = ctx->cfg.H; p->K = ctx->cfg.K; p->L = ctx->cfg.L;
   p->scale_log2 = ctx->sm_scale * 1.4426950408889634f;
   for (int i = 0; i < HEATKV_MAX_K; ++i) p->c[i] = i < ctx->cfg.K ? ctx->c[i] : 0x7fffffff;

@@ -344,8 +344,8 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
       if (!is_attn) continue;
       const int2* descs = FULL ? p.full_descs : reinterpret_cast<const int2*>(p.seqs[seq].plan + im.desc_begin);
       const int64_t base_row = FULL ? 0 : p.seqs[seq].base_row;
-      const int q_head = map_index(im.head, p.q_head), q_seq = map_index(seq, p.q_seq);
-      const int kv_head = map_index(im.head, p.kv_head), kv_seq = map_index(seq, p.kv_seq);
+      const int q_head = im.head & p.q_head_mask, q_seq = seq & p.q_seq_mask;
+      const int kv_head = im.head & p.kv_head_mask, kv_seq = seq & p.kv_seq_mask;
       for (int j = 0; j < im.n_tiles && ok; ++j, ++g) {
         const uint32_t st = g % KV_STAGES;
         const uint32_t use = g / KV_STAGES;
@@ -813,8 +813,8 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) {
-              tma_store_4d(&maps.out, smem_u32(buf), c * 32, q_row0 + (warp & 3) * 32, map_index(im.head, p.o_head),
-                           map_index(seq, p.o_seq));
+              tma_store_4d(&maps.out, smem_u32(buf), c * 32, q_row0 + (warp & 3) * 32, p.o_head > 0 ? im.head : 0,
+                           p.o_seq > 0 ? seq : 0);
               bulk_commit();
             }
           };

@@ -173,12 +173,12 @@ calib_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Ma
           for (int ch = 0; ch < NCH; ++ch)
             for (int hf = 0; hf < 2; ++hf)
               tma_load_4d(sbase + SM_Q + x * TILE_BYTES + ch * HALF_COLS_BYTES + hf * SLOT_BYTES, &maps.q, ch * 64,
-                          q_tok + x * BM + hf * HALF, SHARED ? map_index(head, p.q_head) : head,
-                          SHARED ? map_index(seq, p.q_seq) : seq, bar(Q_FULL + x));
+                          q_tok + x * BM + hf * HALF, SHARED ? head & p.q_head_mask : head,
+                          SHARED ? seq & p.q_seq_mask : seq, bar(Q_FULL + x));
         }
       }
       bool ok = true;
-      const int kv_head = SHARED ? map_index(head, p.kv_head) : head, kv_seq = SHARED ? map_index(seq, p.kv_seq) : seq;
+      const int kv_head = SHARED ? head & p.kv_head_mask : head, kv_seq = SHARED ? seq & p.kv_seq_mask : seq;
       for (int j = 0; j < n_tiles && ok; ++j) {
         const int st = j % K_STAGES;
         const uint32_t use = (uint32_t)(j / K_STAGES);

@@ -54,6 +54,9 @@ struct AttnParams {
   const int2* full_descs;
   int32_t full_slots;
   int32_t attn_items, store_items;  // tensor-memory kernel: attention work items; cache-update items (destination half-tiles)
+  // tensor-memory kernels: 0 for a head or sequence stride of 0, else all ones; an index along such a dimension goes through
+  // it.  (Beside the item count because a CTA's first copies wait for it.)
+  int32_t q_head_mask, q_seq_mask, kv_head_mask, kv_seq_mask;
   float* split_partials;          // [n_seq * slots_per_seq][SPLIT_SLOT_FLOATS]
   uint32_t* split_counters;       // [n_seq * ctrs_per_seq], zero between launches
   // with table_heads > 0: per head in dispatch order, the half-tile descriptors of its visible

@@ -79,7 +79,7 @@ __device__ __forceinline__ bool mbar_wait_hint(uint32_t bar, uint32_t parity, vo
 
 // Tensor maps of [n_seq, H, t, d] views.  A head or sequence stride of 0 (one tensor shared by all heads or sequences) has no
 // place in a map: such a dimension gets extent 1 (its stride is then not used; any legal one will do), and whoever addresses
-// the map takes index 0 along it.
+// the map takes index 0 along it (AttnParams::q_head_mask and the three beside it).
 struct MapShape {
   cuuint64_t dims[4], strides[3];
 };
@@ -88,7 +88,6 @@ inline MapShape map_shape(int d, int t, int H, int n_seq, int64_t s_tok, int64_t
   return {{(cuuint64_t)d, (cuuint64_t)t, (cuuint64_t)(s_head > 0 ? H : 1), (cuuint64_t)(s_seq > 0 ? n_seq : 1)},
           {bytes(s_tok), bytes(s_head), bytes(s_seq)}};
 }
-__device__ __forceinline__ int map_index(int i, int64_t stride) { return stride > 0 ? i : 0; }
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
   asm volatile(
