@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_ke
   float o[D / 8][4];
 #pragma unroll
   for (int i = 0; i < D / 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
-  float m_run[2] = {-INFINITY, -INFINITY};
+  float m_run[2] = {NO_MAX, NO_MAX};
   float l_run[2] = {0.f, 0.f};
 
   const bool has_rows = !SKIP || q0 + warp * 16 < t_q;  // SKIP: a warp without query rows only helps with the copies
@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_ke
       float w0[2], w1[2];
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
-        const float m1 = part[STAT + r * GTHREADS];     // -inf when the second group had no tile; ours is finite
+        const float m1 = part[STAT + r * GTHREADS];     // NO_MAX when the second group had no tile
         const float m = fmaxf(m_run[r], m1);
         w0[r] = exp2f(m_run[r] - m);
         w1[r] = exp2f(m1 - m);
@@ -651,7 +651,7 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_small_kernel(const __grid_co
   float o[D / 8][4];
 #pragma unroll
   for (int i = 0; i < D / 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
-  float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
+  float m_run[2] = {NO_MAX, NO_MAX}, l_run[2] = {0.f, 0.f};
   const float LOG2E = 1.4426950408889634f;
   const float* bias_h = p.seg_bias ? p.seg_bias + head * p.K : nullptr;
 
@@ -758,7 +758,7 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_small_kernel(const __grid_co
   for (int i = threadIdx.x; i < SM::ROWS * CH; i += GTHREADS) {
     const int row = i / CH, ch = i % CH;
     if (q0 + row >= p.t_q) continue;
-    // every row sees at least one key, so the largest reference is finite; a warp without keys weighs nothing
+    // a warp without keys (reference NO_MAX, sum 0) weighs nothing
     float w[SGROUPS], m = -INFINITY, l = 0.f, acc[8] = {};
 #pragma unroll
     for (int k = 0; k < SGROUPS; ++k) m = fmaxf(m, stat[k * SM::ROWS + row]);

@@ -583,7 +583,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             descs = FULL ? p.full_descs : reinterpret_cast<const int2*>(p.seqs[im.seq].plan + im.desc_begin);
             bias_h = p.seg_bias ? p.seg_bias + im.head * p.K : nullptr;
           }
-          float m_ref = -INFINITY, l_sum = 0.f;
+          float m_ref = NO_MAX, l_sum = 0.f;
           // FULL: the scale whose mass is being collected (warp-uniform; scales arrive in ascending order, each as one
           // run of half-tiles, and every scale up to the step has some) and the masses of the finished ones
           int cur_seg = 0;
@@ -704,7 +704,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
               const float mx1 = fmaxf(fmaxf(mq[4], mq[5]), fmaxf(mq[6], mq[7]));
               const float mx = fmaxf(fmaf(mx0, p.scale_log2, b0), fmaf(mx1, p.scale_log2, b1));
               const float m_new = fmaxf(m_ref, mx);
-              const bool grow = m_new > m_ref + RESCALE_THRESHOLD;   // also true on the first tile (m_ref = -inf)
+              const bool grow = m_new > m_ref + RESCALE_THRESHOLD;   // also true on the first tile (m_ref = NO_MAX)
               if (j > 0 && __any_sync(0xffffffffu, grow)) {
                 // O_x holds tiles < j relative to m_ref: rescale the rows whose reference moves.  O_x is complete:
                 // S_x of this tile was issued after the PV products of tile j - 1 by the same thread, and the

@@ -240,7 +240,7 @@ calib_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Ma
     const int row = (warp & 3) * 32 + lane;             // row inside the tile == TMEM lane
     float* seg_smem = reinterpret_cast<float*>(sgen + SM_SEG) + (x * 2 + g) * (HEATKV_MAX_K * BM);   // [scale][row]
     float* stat_smem = reinterpret_cast<float*>(sgen + SM_STAT) + (x * 2 + g) * (2 * BM);           // [reference | sum][row]
-    float m_ref = -INFINITY, l_sum = 0.f;
+    float m_ref = NO_MAX, l_sum = 0.f;
     int cur_seg = -1;                                   // the scale whose mass is being collected (warp-uniform)
     float cur_sum = 0.f;
     bool ok = true;
@@ -279,9 +279,9 @@ calib_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Ma
         }
         const float mx = fmaf(fmaxf(fmaxf(mq[0], mq[1]), fmaxf(mq[2], mq[3])), p.scale_log2, bg);
         const float m_new = fmaxf(m_ref, mx);
-        const bool grow = m_new > m_ref + RESCALE_THRESHOLD;   // also true on the first tile (m_ref = -inf)
+        const bool grow = m_new > m_ref + RESCALE_THRESHOLD;   // also true on the first tile (m_ref = NO_MAX)
         if (grow) {
-          if (m_ref > -INFINITY) {
+          if (m_ref > NO_MAX) {
             // everything collected so far is relative to m_ref: move it to the new reference
             const float f = exp2f(m_ref - m_new);
             l_sum *= f;
@@ -348,10 +348,10 @@ calib_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Ma
       const float* st0 = reinterpret_cast<const float*>(sgen + SM_STAT) + (x * 2) * (2 * BM);
       const float* st1 = st0 + 2 * BM;
       // Eq. 2: mean over the step's rows of mass(row, scale) / rowsum(row); rows past t_q are padding.  A thread
-      // that saw no valid key keeps the reference -inf and contributes nothing.
+      // that saw no valid key keeps the reference NO_MAX and contributes nothing.
       const float m0 = st0[row], m1 = st1[row];
       const float m = fmaxf(m0, m1);
-      const float w0 = m0 > -INFINITY ? exp2f(m0 - m) : 0.f, w1 = m1 > -INFINITY ? exp2f(m1 - m) : 0.f;
+      const float w0 = m0 > NO_MAX ? exp2f(m0 - m) : 0.f, w1 = m1 > NO_MAX ? exp2f(m1 - m) : 0.f;
       const float l = st0[BM + row] * w0 + st1[BM + row] * w1;
       const bool live = q0 + x * BM + row < t_q;
       const float inv = live ? 1.f / l : 0.f;

@@ -150,6 +150,10 @@ cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, c
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// Where a row's running maximum starts: the lowest finite value, so that keys masked by a bias of -inf (or one that leaves
+// the range when scaled) weigh nothing even where they come first; with -inf here their exponent would be -inf minus -inf.
+constexpr float NO_MAX = -3.402823466e38f;
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }

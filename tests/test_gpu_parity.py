@@ -544,6 +544,32 @@ def test_activations_shared_by_heads_or_sequences(hk, d, q_over, kv_over):
             assert np.all(np.abs(beta - want)[mask] <= RTOL_BETA * want[mask])
 
 
+@pytest.mark.parametrize("value", [-np.inf, -3.4e38], ids=["inf", "lowest"])
+@pytest.mark.parametrize("masked", [(0,), (0, 1), (2, 4), ("own",)], ids=["first", "first_two", "middle", "own"])
+def test_scales_masked_by_the_bias(hk, masked, value):
+    """Source scales taken out by a bias of -inf, or of a value that leaves the range once scaled, wherever their keys come in a
+    kernel's order: every kernel, few units (16-query CTAs) and many (64-query forms), generation and calibration."""
+    for H, n_seq, d in ((3, 2, 64), (24, 4, 128)):
+        sh = W.Shape("masked", L=1, H=H, d=d, sides=(1, 2, 3, 5, 7, 12, 16), n_seq=n_seq, s=2)
+        scores = W.synthetic_scas(sh, 6)
+        ref = O.heatkv_schedule(scores, 0.8, sh.s, sh.sides)
+        bias = W.seg_bias_prior_lognormal(sh, 6)
+        for step in range(sh.K):
+            for m in masked:
+                m = step if m == "own" else m
+                if len([i for i in range(step + 1) if i not in masked and not (masked == ("own",) and i == step)]) > 0:
+                    bias[:, step, :, m] = value
+        heads = None if H < 8 else [(0, 0, 0), (3, 0, H - 1), (1, 0, 7)]
+        for kernel in (hk.KERNEL_AUTO, hk.KERNEL_GENERIC, hk.KERNEL_TCGEN05):
+            _run_full_parity(hk, sh, ref, lambda ses: ses.schedule(scas=scores, b=0.8), hk.LAYOUT_PAGED, bias=bias, kernel=kernel,
+                             check_heads=heads, fused=True)
+            if H < 8:
+                for with_out in (False, True):
+                    beta, _, _, want = _calibrate(hk, sh, seeds=[5], bias=bias, with_out=with_out, kernel=kernel)
+                    mask = want > 1e-5
+                    assert np.all(np.abs(beta - want)[mask] <= RTOL_BETA * want[mask]) and np.all(beta[want == 0] < 1e-30)
+
+
 def test_calibration_tiny_four_samples(hk):
     sh = W.TINY
     beta, scas, cas, ref = _calibrate(hk, sh, seeds=range(4))
