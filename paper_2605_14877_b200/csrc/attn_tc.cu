@@ -84,6 +84,13 @@ constexpr uint32_t BAR_TMEM_PTR = N_BARS * 8;                  // offsets inside
 constexpr uint32_t BAR_ABORT = BAR_TMEM_PTR + 4;
 constexpr uint32_t BAR_RING = 256;                             // 2 entries x int32[16]
 constexpr float SUM_LIMIT = 4294967296.f;                      // 2^RESCALE_THRESHOLD: no term of a sum below it is above it
+// FULL: items of at most so many key tiles (the largest such step of a 1024 x 1024 image has 1024 queries) move the reference
+// with every rise of a maximum.  P is rounded to bf16 relative to it, and the few keys that carry a short row are
+// rounded best just below a power of two: output error against 64 bits, 64 queries 2.31e-3 -> 2.12e-3 of the norm, 1024:
+// 2.36e-3 -> 2.27e-3, a pass of 13 scales 2.177e-3 -> 2.107e-3 (warp-level kernel 2.13e-3, 2.27e-3, 2.094e-3) for 3 % of its
+// time.  In longer rows no few keys matter that much (4096 queries 2.35e-3, 2.30e-3 on the warp-level kernel) and following
+// cost 15 to 20 %.
+constexpr int FOLLOW_TILES = 24;
 enum ItemKind : int { ATTENTION = 0, STOP = 2, NOTHING = 3 };
 // ring entry words
 enum ItemWord : int { W_KIND = 0, W_HEAD, W_SEQ, W_TILES, W_NSPLIT, W_SUB, W_SLOT, W_CTR, W_DESC, W_NDESC };
@@ -164,7 +171,9 @@ __device__ __forceinline__ Item read_item(const volatile int32_t* ring, const At
 
 // FULL: heatkv_calibrate_scores with an attention output.  The softmax warps also keep, for every query row, the
 // probability mass of each source scale (a half-tile lies inside one scale; finished scales are parked in the warp's
-// output staging buffer) and add the step's row of beta (Eq. 2) at the end of the item.
+// output staging buffer) and add the step's row of beta (Eq. 2) at the end of the item.  The masses are fp32 results, so all
+// exponentials are ex2's here: with one pair in four from the cubic beta was off by 3.8e-7 on average (13 scales, against 64
+// bits), with none by 1.0e-7 (warp-level kernel 1.3e-7), for 1 % of the time.
 template <int D, bool FULL>
 __global__ void __launch_bounds__(THREADS, 1)
 attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Maps maps) {
@@ -589,6 +598,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
           int cur_seg = 0;
           float cur_mass = 0.f;
           float* masses = reinterpret_cast<float*>(stage) + lane;      // [scale][32 rows]
+          const bool follow = FULL && n_tiles <= FOLLOW_TILES;
           int j = 0;
           // FULL: a warp whose 32 rows all lie past the last query hands on whatever is there (its rows of O and its masses go
           // nowhere): a calibration pass 1.130 -> 1.115 ms.  Generation measured 0.3 to 0.8 % slower with the branch.
@@ -637,7 +647,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
                 const uint64_t xx = fma2(pack2(__uint_as_float(rc[i]), __uint_as_float(rc[i + 1])), scale2, bb2);
                 float e0, e1, x0, x1;
                 unpack2(xx, x0, x1);
-                if (((i >> 1) & POLY_MASK) == POLY_MASK) {
+                if (!FULL && ((i >> 1) & POLY_MASK) == POLY_MASK) {
                   exp2_poly2(xx, e0, e1);
                   if (SPECULATE) top = fmax3(top, x0, x1);
                 } else {
@@ -658,7 +668,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             // meaningless above 2^127); only the second half's maximum is computed, beside them.
             bool take_max = true;
             uint32_t pk0[16], pk1[16];
-            if (SPECULATE && j > 0) {
+            if (SPECULATE && j > 0 && !follow) {
               const uint64_t bb0 = pack2(b0 - m_ref, b0 - m_ref);
               exps(r0, bb0, pk0);
               exps(r1, bb0, pk1);
@@ -704,7 +714,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
               const float mx1 = fmaxf(fmaxf(mq[4], mq[5]), fmaxf(mq[6], mq[7]));
               const float mx = fmaxf(fmaf(mx0, p.scale_log2, b0), fmaf(mx1, p.scale_log2, b1));
               const float m_new = fmaxf(m_ref, mx);
-              const bool grow = m_new > m_ref + RESCALE_THRESHOLD;   // also true on the first tile (m_ref = NO_MAX)
+              const bool grow = m_new > m_ref + (follow ? 0.f : RESCALE_THRESHOLD);   // also true on the first tile (m_ref = NO_MAX)
               if (j > 0 && __any_sync(0xffffffffu, grow)) {
                 // O_x holds tiles < j relative to m_ref: rescale the rows whose reference moves.  O_x is complete:
                 // S_x of this tile was issued after the PV products of tile j - 1 by the same thread, and the
