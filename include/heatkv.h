@@ -264,8 +264,9 @@ int heatkv_schedule_plan_fp8(const heatkv_schedule* sch, int32_t* words, int64_t
 
 /* Admit / retire one image.  Opening reserves the sequence's rows for its whole life (the
  * schedule is static, so the reservation and every page table are known up front) and, on
- * first use of a schedule, uploads its plan on `stream`.  HEATKV_ERR_OUT_OF_PAGES if the
- * pool or the metadata region cannot hold it.                                            */
+ * first use of a schedule, uploads its plan on `stream`.  A plan keeps its place while a
+ * sequence uses it; plans (or their merged tables) that none uses make way when a region is
+ * full.  HEATKV_ERR_OUT_OF_PAGES if the pool or the metadata region cannot hold it.      */
 int heatkv_seq_open(heatkv_ctx* ctx, const heatkv_schedule* sch, void* stream, int* seq_id);
 int heatkv_seq_close(heatkv_ctx* ctx, int seq_id);
 

@@ -97,11 +97,13 @@ struct PlanEntry {
   uint64_t run_off = 0, run_len = 0;    // merged attention tables on the device (run_len 0: none), both from the arena's start
   int32_t run_shift = 0;                // what takes a word offset inside them from the host's blob to the device
   int refs = 0;
+  uint64_t opened = 0;                  // when a sequence last opened with it (counts openings)
 };
 
 struct Seq {
   bool open = false;
   int plan = -1;
+  bool runs = false;                // its plan had its merged tables when it opened; what others do later changes nothing
   uint64_t base_row = 0, rows = 0;
   std::vector<int16_t> done_step;   // per layer: last step whose post-layer update ran (-1 = none)
   std::vector<int16_t> pre_step;    // per layer: last step whose pre-step eviction ran
@@ -132,7 +134,7 @@ struct heatkv_ctx {
   std::vector<std::unique_ptr<PlanEntry>> plans;
   std::vector<Seq> seqs;
   uint64_t reserved_rows = 0, peak_reserved = 0, meta_used = 0;
-  uint64_t launches = 0;
+  uint64_t launches = 0, openings = 0;
   heatkv_kernel_stats kstats = {};             // launches per kernel
   TcState* tc = nullptr;
   CalibTcState* calib_tc = nullptr;
@@ -146,9 +148,52 @@ struct heatkv_ctx {
 
 namespace {
 
+// Room for the plan's merged attention tables, in a region of their own: a plan that finds none does without them.  Tables of
+// plans that no open sequence uses make way, the longest unused first.
+bool place_runs(heatkv_ctx* ctx, PlanEntry* e) {
+  const uint64_t words = e->plan.blob.size() - (uint64_t)e->plan.header().off_run_desc;
+  const uint64_t len = (words * 4 + META_ALIGN - 1) / META_ALIGN * META_ALIGN;
+  while (!ctx->run_tables.alloc(len, &e->run_off)) {
+    PlanEntry* idle = nullptr;
+    for (auto& pe : ctx->plans)
+      if (pe && pe->refs == 0 && pe->run_len && (!idle || pe->opened < idle->opened)) idle = pe.get();
+    if (!idle) return false;
+    ctx->run_tables.release(idle->run_off, idle->run_len);
+    idle->run_len = 0;
+  }
+  e->run_len = len;
+  e->run_shift = (int32_t)((int64_t)(e->run_off - e->meta_off) / 4 - (int64_t)e->plan.header().off_run_desc);
+  return true;
+}
+
+// Copies the first `words` words of the plan's blob (its header, or all but the merged tables) to the device, and the merged
+// tables if they have room.
+int upload_plan(heatkv_ctx* ctx, PlanEntry* e, uint64_t words, cudaStream_t stream) {
+  PlanHeader& h = *reinterpret_cast<PlanHeader*>(e->plan.blob.data());
+  const uint64_t plain_words = (uint64_t)h.off_run_desc, run_words = e->plan.blob.size() - plain_words;
+  const int32_t shift = e->run_len ? e->run_shift : 0;
+  auto shift_runs = [&](int32_t by) { h.off_run_desc += by; h.off_run_begin += by; h.off_run_cnt += by; h.off_run_src += by; };
+  shift_runs(shift);
+  cudaError_t up = cudaMemcpyAsync(ctx->meta + e->meta_off, e->plan.blob.data(), words * 4, cudaMemcpyHostToDevice, stream);
+  if (up == cudaSuccess && e->run_len)
+    up = cudaMemcpyAsync(ctx->meta + e->run_off, e->plan.blob.data() + plain_words, run_words * 4, cudaMemcpyHostToDevice, stream);
+  // the blob is pageable host memory: wait so the vector may be touched again safely
+  if (up == cudaSuccess) up = cudaStreamSynchronize(stream);
+  shift_runs(-shift);
+  if (up == cudaSuccess) return HEATKV_OK;
+  if (e->run_len) ctx->run_tables.release(e->run_off, e->run_len);
+  e->run_len = 0;
+  return HEATKV_ERR_CUDA;
+}
+
 int find_or_load_plan(heatkv_ctx* ctx, const Schedule& s, cudaStream_t stream, int* idx) {
   for (size_t i = 0; i < ctx->plans.size(); ++i)
-    if (ctx->plans[i] && ctx->plans[i]->uid == s.uid) { *idx = (int)i; return HEATKV_OK; }
+    if (ctx->plans[i] && ctx->plans[i]->uid == s.uid) {
+      *idx = (int)i;
+      PlanEntry* e = ctx->plans[i].get();
+      if (e->run_len || !place_runs(ctx, e)) return HEATKV_OK;
+      return upload_plan(ctx, e, sizeof(PlanHeader) / 4, stream);
+    }
   if (s.L != ctx->cfg.L || s.H != ctx->cfg.H || s.K != ctx->cfg.K || s.s != ctx->cfg.s)
     return HEATKV_ERR_SHAPE_MISMATCH;
   for (int i = 0; i < s.K; ++i)
@@ -176,26 +221,11 @@ int find_or_load_plan(heatkv_ctx* ctx, const Schedule& s, cudaStream_t stream, i
   if (!ok) return HEATKV_ERR_OUT_OF_PAGES;
   e->meta_off = off;
   e->meta_len = bytes;
-  // The merged tables go to a region of their own: a plan that finds no room there does without them.
-  PlanHeader& h = *reinterpret_cast<PlanHeader*>(e->plan.blob.data());
-  const uint64_t run_words = e->plan.blob.size() - plain_words;
-  uint64_t run_len = (run_words * 4 + META_ALIGN - 1) / META_ALIGN * META_ALIGN;
-  if (ctx->run_tables.alloc(run_len, &e->run_off)) {
-    e->run_len = run_len;
-    e->run_shift = (int32_t)((int64_t)(e->run_off - off) / 4 - (int64_t)plain_words);
-  }
-  auto shift_runs = [&](int32_t by) { h.off_run_desc += by; h.off_run_begin += by; h.off_run_cnt += by; h.off_run_src += by; };
-  shift_runs(e->run_shift);
-  cudaError_t up = cudaMemcpyAsync(ctx->meta + off, e->plan.blob.data(), plain_words * 4, cudaMemcpyHostToDevice, stream);
-  if (up == cudaSuccess && e->run_len)
-    up = cudaMemcpyAsync(ctx->meta + e->run_off, e->plan.blob.data() + plain_words, run_words * 4, cudaMemcpyHostToDevice, stream);
-  // the blob is pageable host memory: wait so the vector may be touched again safely
-  if (up == cudaSuccess) up = cudaStreamSynchronize(stream);
-  shift_runs(-e->run_shift);
-  if (up != cudaSuccess) {
+  place_runs(ctx, e.get());
+  rc = upload_plan(ctx, e.get(), plain_words, stream);
+  if (rc != HEATKV_OK) {
     ctx->metas.release(off, bytes);
-    if (e->run_len) ctx->run_tables.release(e->run_off, e->run_len);
-    return HEATKV_ERR_CUDA;
+    return rc;
   }
   ctx->meta_used += bytes;
   size_t slot = ctx->plans.size();
@@ -283,7 +313,7 @@ int gather_seqs(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int layer, int s
 // A call reads the merged attention tables when no bias per scale is given and every sequence's plan has them.
 bool all_have_runs(const heatkv_ctx* ctx, const int* seq_ids, int n_seq) {
   for (int i = 0; i < n_seq; ++i)
-    if (!ctx->plans[ctx->seqs[seq_ids[i]].plan]->run_len) return false;
+    if (!ctx->seqs[seq_ids[i]].runs) return false;
   return true;
 }
 
@@ -652,11 +682,13 @@ int heatkv_seq_open(heatkv_ctx* ctx, const heatkv_schedule* sch, void* stream_, 
   Seq& q = ctx->seqs[id];
   q.open = true;
   q.plan = pi;
+  q.runs = pe.run_len != 0;
   q.base_row = start;
   q.rows = (uint64_t)pe.plan.reserved_rows;
   q.done_step.assign(ctx->cfg.L, -1);
   q.pre_step.assign(ctx->cfg.L, -1);
   pe.refs++;
+  pe.opened = ++ctx->openings;
   ctx->reserved_rows += q.rows;
   ctx->peak_reserved = std::max(ctx->peak_reserved, ctx->reserved_rows);
   *seq_id = id;

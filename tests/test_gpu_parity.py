@@ -437,6 +437,52 @@ def test_merged_tables_are_optional(hk, layout):
     assert torch.equal(outs[1], outs[2])          # one plan without them: the whole call goes without
 
 
+@pytest.mark.parametrize("fp8", [False, True], ids=["bf16", "fp8"])
+def test_merged_tables_make_way_for_plans_in_use(hk, fp8):
+    """Scratch for one plan's merged tables: they belong to the plan opened last, a plan that found none gets them when it is opened
+    again, and a sequence keeps for life what it opened with.  Bit for bit against contexts with room for all and for none."""
+    from paper_2605_14877_b200.sweep import Session
+    sh = W.Shape("mid", L=1, H=6, d=128, sides=W.SIDES_13[:9], n_seq=1, s=3)
+    q, k, v = W.qkv_layer(sh, 0, 0, device="cuda")
+    cfg = hk.Config.make(sh.L, sh.H, sh.d, sh.t, sh.s)
+    sch = hk.heatkv_build_schedule(cfg, scas=W.synthetic_scas(sh, 3), b=0.6)
+    words = hk.heatkv_schedule_plan_fp8(sch)[0] if fp8 else hk.heatkv_schedule_plan(sch, hk.LAYOUT_PAGED)
+    hk.heatkv_schedule_free(sch)
+    one = (len(words) - int(words[18])) * 4
+    assert one > 1280                             # so that what is left of the last KB holds no second one
+    outs = {}
+
+    def run(ses, sid):
+        out = torch.zeros_like(q)
+        ses.generate([sid], lambda l: (q, k, v), lambda l: out)
+        hk.heatkv_seq_close(ses.ctx, sid)
+        return W.bf16_bits(out).copy()
+
+    for name, scratch in (("all", 1 << 26), ("none", 1024), ("one", 8 * ((one + 255) // 256 * 256 + 1023 & ~1023))):
+        with Session(sh.L, sh.H, sh.d, sh.t, sh.s, pool_rows=4 * sh.H * (sh.c[-2] + 64 * sh.K), kernel=hk.KERNEL_GENERIC,
+                     scratch_bytes=scratch, cache_dtype=hk.CACHE_FP8_E4M3 if fp8 else hk.CACHE_BF16) as ses:
+            a, b = (ses.schedule(scas=W.synthetic_scas(sh, seed), b=0.6) for seed in (3, 4))
+            open_ = lambda s: hk.heatkv_seq_open(ses.ctx, s)
+            got = [("a", run(ses, open_(a))), ("b", run(ses, open_(b))), ("a", run(ses, open_(a)))]
+            i, j = open_(a), open_(b)             # room for one: b does without while a is open
+            got += [("a", run(ses, i)), ("b without" if name == "one" else "b", run(ses, j))]
+            j = open_(b)
+            got += [("b", run(ses, j))]
+            i, j = open_(b), open_(a)             # a without; then b leaves, a second a gets them, the first goes on as it was
+            got += [("b", run(ses, i))]
+            n = open_(a)
+            got += [("a without" if name == "one" else "a", run(ses, j)), ("a", run(ses, n))]
+            outs[name] = got
+            assert hk.heatkv_device_status(ses.ctx) == 0
+            for s in (a, b):
+                hk.heatkv_schedule_free(s)
+    want = dict(outs["all"])
+    without = dict(outs["none"])
+    assert not np.array_equal(want["a"], without["a"]) and not np.array_equal(want["b"], without["b"])
+    for which, bits in outs["one"]:
+        assert np.array_equal(bits, (without if "without" in which else want)[which[0]]), which
+
+
 def test_split_heads_are_reproducible_bit_for_bit(hk):
     """Pieces of a cut head are merged in piece order whichever arrives last: the same generation run four
     times gives identical output bits (steps of this workload are cut, see the test above)."""
