@@ -3,6 +3,7 @@
  * small images; from here 5. */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
+#include <limits.h>
 
 #include "heatkv.h"
 
@@ -22,6 +23,10 @@ static int fail(int rc, const char* where) {
 }
 
 static int current_stream(void** out) {
+  if (!hooks.check) {
+    PyErr_SetString(PyExc_RuntimeError, "set_hooks has not been called");
+    return -1;
+  }
   PyObject* dev = PyObject_CallNoArgs(hooks.device);
   if (!dev) return -1;
   PyObject* st = PyObject_CallOneArg(hooks.raw_stream, dev);
@@ -90,45 +95,51 @@ static int layer_step(heatkv_ctx* ctx, const int* ids, int n_seq, int layer, int
   return rc == HEATKV_OK ? 0 : fail(rc, where);
 }
 
-/* sequence ids of a call */
+/* a context handle: None (a closed session) is the library's to refuse */
+static int parse_ctx(PyObject* v, void* out) {
+  void* p = v == Py_None ? NULL : PyLong_AsVoidPtr(v);
+  if (PyErr_Occurred()) return 0;
+  *(heatkv_ctx**)out = (heatkv_ctx*)p;
+  return 1;
+}
+
+/* sequence ids of a call, anything int() takes; a batch past the limit keeps its length and is the library's to refuse */
 static int parse_ids(PyObject* seq, int* ids, int* n) {
   PyObject* f = PySequence_Fast(seq, "seq_ids must be a sequence");
   if (!f) return -1;
   const Py_ssize_t m = PySequence_Fast_GET_SIZE(f);
-  if (m > HEATKV_MAX_BATCH) {                      /* the library's own answer to a batch of that size */
-    Py_DECREF(f);
-    return fail(HEATKV_ERR_INVALID_ARG, "heatkv_attention_append");
-  }
-  for (Py_ssize_t i = 0; i < m; ++i) {
-    ids[i] = (int)PyLong_AsLong(PySequence_Fast_GET_ITEM(f, i));
+  for (Py_ssize_t i = 0; i < m && i < HEATKV_MAX_BATCH; ++i) {
+    PyObject* v = PyNumber_Long(PySequence_Fast_GET_ITEM(f, i));
+    if (!v) break;
+    ids[i] = (int)PyLong_AsLong(v);
+    Py_DECREF(v);
     if (PyErr_Occurred()) break;
   }
   Py_DECREF(f);
-  *n = (int)m;
+  *n = m < INT_MAX ? (int)m : INT_MAX;
   return PyErr_Occurred() ? -1 : 0;
 }
 
 static PyObject* py_run_layer_step(PyObject* self, PyObject* args) {
-  unsigned long long ctx;
+  heatkv_ctx* ctx;
   int layer, step, fused, n;
   long long lo;
   PyObject *seq, *q, *k, *v, *out, *bias;
   int ids[HEATKV_MAX_BATCH];
-  if (!PyArg_ParseTuple(args, "KOiiLOOOOOp", &ctx, &seq, &layer, &step, &lo, &q, &k, &v, &out, &bias, &fused)) return NULL;
-  if (parse_ids(seq, ids, &n) || layer_step((heatkv_ctx*)(uintptr_t)ctx, ids, n, layer, step, lo, q, k, v, out, bias, fused))
+  if (!PyArg_ParseTuple(args, "O&OiiLOOOOOp", parse_ctx, &ctx, &seq, &layer, &step, &lo, &q, &k, &v, &out, &bias, &fused)) return NULL;
+  if (parse_ids(seq, ids, &n) || layer_step(ctx, ids, n, layer, step, lo, q, k, v, out, bias, fused))
     return NULL;
   Py_RETURN_NONE;
 }
 
 static PyObject* py_generate(PyObject* self, PyObject* args) {
-  unsigned long long ctx;
+  heatkv_ctx* c;
   int L, fused, n;
   PyObject *seq, *begins, *qkv_of, *out_of, *bias_of, *after;
   int ids[HEATKV_MAX_BATCH];
-  if (!PyArg_ParseTuple(args, "KOO!iOOOOp", &ctx, &seq, &PyTuple_Type, &begins, &L, &qkv_of, &out_of, &bias_of, &after, &fused))
+  if (!PyArg_ParseTuple(args, "O&OO!iOOOOp", parse_ctx, &c, &seq, &PyTuple_Type, &begins, &L, &qkv_of, &out_of, &bias_of, &after, &fused))
     return NULL;
   if (parse_ids(seq, ids, &n)) return NULL;
-  heatkv_ctx* c = (heatkv_ctx*)(uintptr_t)ctx;
   const int K = (int)PyTuple_GET_SIZE(begins);
   for (int step = 0; step < K; ++step) {
     const int64_t lo = PyLong_AsLongLong(PyTuple_GET_ITEM(begins, step));

@@ -507,6 +507,41 @@ def test_split_heads_are_reproducible_bit_for_bit(hk):
         assert np.array_equal(r, runs[0])
 
 
+@pytest.mark.parametrize("where", ["qkv", "two_tensors", "bias", "out", "after"])
+def test_generation_stops_at_a_callback_that_raises(hk, where):
+    """The exception of a callback comes out of Session.generate as it is; the context stays usable."""
+    from paper_2605_14877_b200.sweep import Session
+    sh = W.TINY
+    q, k, v = W.qkv_layer(sh, 0, 0, device="cuda")
+
+    class Stop(Exception):
+        pass
+
+    def stop(at, value=None):
+        if at == where:
+            raise Stop
+        return value
+
+    with Session(sh.L, sh.H, sh.d, sh.t, sh.s, pool_rows=4096) as ses:
+        sch = ses.schedule(scas=W.synthetic_scas(sh, 1), b=1.0)
+        outs = []
+        for failing in (True, False):
+            sid = hk.heatkv_seq_open(ses.ctx, sch)
+            out = torch.zeros_like(q)
+            outs.append(out)
+            if not failing:
+                ses.generate([sid], lambda l: (q, k, v), lambda l: out)
+            else:
+                with pytest.raises(ValueError if where == "two_tensors" else Stop):
+                    ses.generate([sid], lambda l: stop("qkv", (q, k) if where == "two_tensors" else (q, k, v)),
+                                 lambda l: stop("out", out), lambda l, step: stop("bias"), lambda step, l: stop("after"))
+            hk.heatkv_seq_close(ses.ctx, sid)
+        torch.cuda.synchronize()
+        assert outs[1].abs().sum(dim=-1).min().item() > 0 and hk.heatkv_device_status(ses.ctx) == 0
+        assert (outs[0].abs().sum().item() > 0) == (where == "after")     # it ran after the first step's layer
+        hk.heatkv_schedule_free(sch)
+
+
 def test_full_budget_equals_uncompressed(hk):
     sh = W.Shape("full", L=1, H=2, d=64, sides=W.SIDES_13[:9], n_seq=1, s=2)
     scores = W.synthetic_scas(sh, 1)

@@ -484,3 +484,49 @@ def test_bounded_waits_start_after_the_launch_before():
                 assert "pdl_wait();" in common + part[: first.start()], (name, part.splitlines()[0])
                 roles += 1
     assert roles == 6                                       # copies, products, softmax of either kernel
+
+
+@pytest.fixture
+def native(hk):
+    """The call sequencer with a stream that needs no GPU; without a context every library call is refused."""
+    import torch
+    from paper_2605_14877_b200 import _native, heatkv
+    _native.set_hooks(heatkv._check, lambda: 0, lambda dev: 0)
+    yield _native
+    _native.set_hooks(heatkv._check, torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+
+
+def test_call_sequencer_errors(hk, native):
+    """A closed session (context None) and a batch past the limit are the library's to refuse; ids are whatever int() takes; bad
+    views and ids raise before any call."""
+    import torch
+    x = torch.zeros(1, 2, 4, 64, dtype=torch.bfloat16)
+    one = lambda ctx, ids, q=x, fused=True: native.run_layer_step(ctx, ids, 0, 0, 0, q, x, x, x, None, fused)
+    sweep = lambda ctx, ids: native.generate(ctx, ids, (0, 1), 1, lambda l: (x, x, x), lambda l: x, None, None, True)
+    for ids in ([0], (0.0,), np.zeros(1, dtype=np.int64), torch.zeros(1, dtype=torch.int64), range(200)):
+        for call in (one, sweep, lambda c, i: one(c, i, fused=False)):
+            with pytest.raises(hk.HeatKVError) as e:
+                call(None, ids)
+            assert e.value.status == -1
+    for call in (one, sweep):
+        with pytest.raises(TypeError):
+            call(None, 3)
+        with pytest.raises(ValueError):
+            call(None, ["x"])
+        with pytest.raises(TypeError):
+            call("ctx", [0])
+    with pytest.raises(AssertionError):
+        one(None, [0], q=x.transpose(2, 3))
+    with pytest.raises(AssertionError):
+        one(None, [0], q=x[0])
+
+
+def test_call_sequencer_without_hooks():
+    import subprocess
+    import sys
+    code = ("import importlib.util as u, glob; s = u.spec_from_file_location('_native', glob.glob('paper_2605_14877_b200/_native*.so')[0]);"
+            "m = u.module_from_spec(s); s.loader.exec_module(m)\n"
+            "try: m.generate(0, [0], (0,), 1, None, None, None, None, True)\n"
+            "except RuntimeError as e: print(e)")
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert r.returncode == 0 and "set_hooks" in r.stdout, (r.returncode, r.stderr)
