@@ -145,7 +145,10 @@ static PyObject* py_generate(PyObject* self, PyObject* args) {
     const int64_t lo = PyLong_AsLongLong(PyTuple_GET_ITEM(begins, step));
     void* stream;
     if (PyErr_Occurred() || current_stream(&stream)) return NULL;
-    int rc = heatkv_append_compact(c, ids, n, -1, step, NULL, NULL, NULL, stream);
+    int rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = heatkv_append_compact(c, ids, n, -1, step, NULL, NULL, NULL, stream);
+    Py_END_ALLOW_THREADS
     if (rc != HEATKV_OK) {
       fail(rc, "heatkv_append_compact");
       return NULL;

@@ -530,3 +530,12 @@ def test_call_sequencer_without_hooks():
             "except RuntimeError as e: print(e)")
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
     assert r.returncode == 0 and "set_hooks" in r.stdout, (r.returncode, r.stderr)
+
+
+def test_call_sequencer_lets_other_threads_run():
+    """A launch may block (a full queue, a host callback before it): every library call is made without the interpreter lock."""
+    with open(os.path.join(ROOT, "paper_2605_14877_b200", "csrc", "native_module.c")) as f:
+        code = re.sub(r"/\*.*?\*/|\"[^\"]*\"", "", f.read(), flags=re.S)
+    unlocked = re.findall(r"Py_BEGIN_ALLOW_THREADS(.*?)Py_END_ALLOW_THREADS", code, flags=re.S)
+    calls = re.compile(r"= heatkv_\w+\(")
+    assert len(calls.findall(code)) == sum(len(calls.findall(u)) for u in unlocked) == 4
