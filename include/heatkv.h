@@ -95,8 +95,8 @@ typedef struct {
   uint64_t arena_bytes;          /* metadata region + scratch region + K pool + V pool     */
   uint64_t meta_bytes;           /* bytes of the arena set aside for plans; 0 = default    */
   uint64_t scratch_bytes;        /* bytes of the arena for partial results of heads whose key range is
-                                    split over several CTAs, an eighth of it (at most 32 MiB) for the
-                                    plans' merged tables; 0 = default (1/8 of the arena, at most
+                                    split over several CTAs, 1/32 to 1/8 of it (at most 32 MiB) for
+                                    the plans' merged tables; 0 = default (1/8 of the arena, at most
                                     128 MiB); too little only disables both                         */
   int32_t cache_dtype;           /* heatkv_cache_dtype; FP8_E4M3 needs the paged layout                    */
   int32_t reserved0;
@@ -308,7 +308,7 @@ int heatkv_attention_append(heatkv_ctx* ctx, const int* seq_ids /*HOST*/, int n_
                             const float* seg_bias, void* out, void* stream);
 
 /* How the tensor-memory attention kernel would cut the work of heatkv_scale_attention(seq_ids, layer,
- * step): *split_tiles = longest piece, in 128-key tiles, among the heads whose key range is cut (0: every
+ * step) without seg_bias: *split_tiles = longest piece, in 128-key tiles, among the heads whose key range is cut (0: every
  * work item takes a whole head's key range), *items = work items of the launch (an upper bound when the
  * call mixes schedules).  A cut head's pieces leave partial results in the arena's scratch region, where
  * the last to arrive merges them.  The choice (a piece count per head) minimises an estimate of the launch's

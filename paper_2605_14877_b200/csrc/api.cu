@@ -506,18 +506,23 @@ int heatkv_create(const heatkv_config* cfg, void* stream_, heatkv_ctx** out) {
   {   // scratch region: arrival counters first (kept zero between launches), then the partial-result slots
     const uint64_t ctr_bytes = std::min<uint64_t>(scratch / 4, 256u << 10) / 1024 * 1024;
     const uint64_t slot_bytes = (uint64_t)tc_split_slot_floats(cfg->d) * 4;
-    // ... and at its end the plans' merged attention tables (half a megabyte for 13 scales of 4 layers x 30 heads)
-    const uint64_t run_bytes = std::min<uint64_t>(scratch / 8, 32u << 20) / 1024 * 1024;
+    int dev = 0, n_sm = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n_sm > 0)
+      ctx->n_sm = n_sm;
+    // ... and at its end the plans' merged attention tables (half a megabyte for 13 scales of 4 layers x 30 heads): what lies
+    // beyond three slots per SM (of 968 launches of 130 workloads one wanted more, 448), at least 1/32 and at most 1/8.  With
+    // 1/8 always, a scratch of 16 MiB held 108 slots of 128-wide heads; 112 to 120 is what many steps of 400 to 1024 queries
+    // want.  Too little for 16 slots cuts nothing worth while.
+    const uint64_t beyond = scratch - std::min<uint64_t>(scratch, ctr_bytes + 3ull * ctx->n_sm * slot_bytes);
+    const uint64_t least = scratch - ctr_bytes < 16 * slot_bytes ? scratch / 8 : scratch / 32;
+    const uint64_t run_bytes = std::min<uint64_t>({std::max<uint64_t>(beyond, least), scratch / 8, 32u << 20}) / 1024 * 1024;
     ctx->run_tables.reset(meta + scratch - run_bytes, run_bytes);
     ctx->split_counters = reinterpret_cast<uint32_t*>(ctx->meta + meta);
     ctx->split_ctrs = ctr_bytes / 4;
     ctx->split_partials = reinterpret_cast<float*>(ctx->meta + meta + ctr_bytes);
     ctx->split_slots = (scratch - ctr_bytes - run_bytes) / slot_bytes;
     if (ctr_bytes && cudaMemsetAsync(ctx->split_counters, 0, ctr_bytes, stream) != cudaSuccess) return HEATKV_ERR_CUDA;
-    int dev = 0, n_sm = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n_sm > 0)
-      ctx->n_sm = n_sm;
   }
   const uint64_t bf16_rows = fp8 ? stage_rows : rows;           // rows of the two bf16 arrays the attention kernels read
   ctx->v_pool = ctx->k_pool + bf16_rows * cfg->d;

@@ -483,6 +483,19 @@ def test_merged_tables_make_way_for_plans_in_use(hk, fp8):
         assert np.array_equal(bits, (without if "without" in which else want)[which[0]]), which
 
 
+def test_small_scratch_still_cuts_long_heads(hk):
+    """7 heads x 4 sequences at 400 queries want 112 partial slots; 16 MiB of scratch hold them beside the merged tables."""
+    sh = W.Shape("cut", L=1, H=7, d=128, sides=W.SIDES_13[:8], n_seq=4, s=3)
+    got = []
+    for scratch in (1 << 24, 1 << 26):
+        with _session(hk, sh, 4 * sh.H * (sh.c[-2] + 64 * sh.K), hk.LAYOUT_PAGED, hk.KERNEL_AUTO, scratch_bytes=scratch) as ses:
+            sch = ses.schedule(scas=W.synthetic_scas(sh, 3), b=1.0)
+            ids = [hk.heatkv_seq_open(ses.ctx, sch) for _ in range(sh.n_seq)]
+            got.append(hk.heatkv_attention_split(ses.ctx, ids, 0, 7))
+            hk.heatkv_schedule_free(sch)
+    assert got[0] == got[1] and got[0][0] > 0
+
+
 def test_split_heads_are_reproducible_bit_for_bit(hk):
     """Pieces of a cut head are merged in piece order whichever arrives last: the same generation run four
     times gives identical output bits (steps of this workload are cut, see the test above)."""
