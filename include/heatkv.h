@@ -13,7 +13,8 @@
  *    scale k, so t[step] tokens are generated at `step` and c[step] = t[0]+..+t[step].
  *  - Activations are bf16, shaped [n_seq, H, t_step, d] with d contiguous; the other
  *    three strides are given in elements by heatkv_strides (NULL = densely packed).
- *    Base pointers must be 16-byte aligned and strides multiples of 8 elements.
+ *    Base pointers must be 16-byte aligned and strides multiples of 8 elements.  A head or
+ *    sequence stride of inputs may be 0: one tensor shared by all heads or sequences.
  *  - Every pointer is marked HOST or DEVICE.  Device buffers belong to the caller (the
  *    library never allocates or frees device memory); the library owns only the host
  *    objects behind heatkv_ctx / heatkv_schedule.  Kernels are enqueued on the given
@@ -71,7 +72,8 @@ typedef enum {
 
 typedef enum {
   HEATKV_KERNEL_AUTO = 0,      /* tensor-memory kernel for steps of >= 256 queries (>= 128 once a call holds
-                                  64 (sequence, head) units), generic otherwise */
+                                  64 (sequence, head) units; >= 48 in calibration with an attention output),
+                                  generic otherwise */
   HEATKV_KERNEL_GENERIC = 1,   /* warp-level MMA kernel for every step                    */
   HEATKV_KERNEL_TCGEN05 = 2    /* tcgen05 / TMEM / TMA kernel wherever its shape rules allow */
 } heatkv_kernel_choice;
@@ -162,11 +164,14 @@ int heatkv_destroy(heatkv_ctx* ctx);
  * sequences: attention of the t[step] queries over ALL c[step] keys (no pruning), fused
  * with the per-row probability mass on each source scale; the mean over rows is added to
  * beta_accum[layer][h][step][0..step] for every head (sum over the n_seq sequences; every
- * sequence counts as one data point d).  The attention matrix is never written out.
+ * sequence counts as one data point d).  The attention matrix is never written out.  Against 64 bits the
+ * masses of 13 scales are off by 4e-7 of themselves on average without an output, where one exponential in three
+ * is a cubic, and by 1e-7 with one; 2e-6 was the largest seen.
  *   q       DEVICE bf16 [n_seq,H,t[step],d]   strides q_*
  *   k_full  DEVICE bf16 [n_seq,H,c[step],d]   strides kv_*  (all scales up to `step`)
  *   v_full  DEVICE bf16 like k_full, or NULL when `out` is NULL
- *   seg_bias DEVICE fp32 [H][K] additive logit bias per source scale, or NULL
+ *   seg_bias DEVICE fp32 [H][K] additive logit bias per source scale (-inf takes a scale out; one that a query
+ *           sees must remain), or NULL
  *   beta_accum DEVICE fp32 [L][H][K][K], zero-initialised by the caller before the first call
  *   out     DEVICE bf16 [n_seq,H,t[step],d] strides o_*: the attention output, or NULL
  * Without an output the o_* strides are not read (they may be left zero).                */
@@ -287,7 +292,8 @@ int heatkv_append_compact(heatkv_ctx* ctx, const int* seq_ids /*HOST*/, int n_se
  * scale, raster order inside) followed by the step's own t[step] keys, which always come
  * from k_new / v_new and are all visible.  bf16 operands, fp32 accumulation, probabilities
  * rounded to bf16 before the PV product.
- *   q, k_new, v_new DEVICE bf16 [n_seq,H,t[step],d]; seg_bias DEVICE fp32 [H][K] or NULL;
+ *   q, k_new, v_new DEVICE bf16 [n_seq,H,t[step],d]; seg_bias DEVICE fp32 [H][K] (-inf takes a
+ *   scale out, as in heatkv_calibrate_scores) or NULL;
  *   out DEVICE bf16 [n_seq,H,t[step],d].                                                 */
 int heatkv_scale_attention(heatkv_ctx* ctx, const int* seq_ids /*HOST*/, int n_seq, int layer,
                            int step, const void* q, const void* k_new, const void* v_new,

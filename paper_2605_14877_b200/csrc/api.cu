@@ -897,14 +897,14 @@ int heatkv_calibrate_scores(heatkv_ctx* ctx, int layer, int step, int n_seq, con
   p.layer = layer;
   p.beta_row = beta_accum + (((int64_t)layer * ctx->cfg.H) * ctx->cfg.K + step) * ctx->cfg.K;
   // Large steps run on tensor memory: without an output (256 queries and more) the pass is S = Q K^T plus bookkeeping (the
-  // calibration kernel), with one (48 and more) it is the attention kernel with that bookkeeping beside its softmax (13 scales, 16 heads,
-  // 2 sequences: 1.24 ms a pass against 6.05 ms on the warp-level kernel).
+  // calibration kernel), with one (48 and more) it is the attention kernel with that bookkeeping beside its softmax (13 scales,
+  // 16 heads, 2 sequences: 1.23 ms a pass against 6.0 ms on the warp-level kernel).
   const int choice = ctx->cfg.kernel;
   const int64_t items = (int64_t)ctx->cfg.H * ((p.t_q + 255) / 256);
   bool use_tc = choice != HEATKV_KERNEL_GENERIC && calib_tc_supported(ctx->calib_tc, p, ctx->cfg.d, n_seq) &&
                 (!out || (tc_supported(ctx->tc, p, ctx->cfg.d, n_seq) && items * n_seq <= INT32_MAX));
-  // (with an output the warp-level kernel pays two products per key at mma.sync rate in one CTA per 16 queries and head, so the
-  // line lies lower: 144 queries 13.3 us on tensor memory against 24.9, 64: 10.2 and 13.2, 36: 8.5 and 8.8, 16: 8.3 and 6.9)
+  // (with an output the warp-level kernel pays two products per key at mma.sync rate in one CTA per 64 queries and head, so the
+  // line lies lower: 144 queries 13.3 us on tensor memory against 22.2, 64: 11.0 and 11.2, 36: 8.8 and 8.9, 16: 8.6 and 7.9)
   if (choice == HEATKV_KERNEL_AUTO && p.t_q < (out ? 48 : 256)) use_tc = false;
   cudaError_t e;
   if (use_tc && out) {

@@ -16,6 +16,8 @@
 //               back into the columns S occupied, and rescales O only when the row max grew
 //               by more than 2^32 since the last reference (the sum keeps the same reference,
 //               so the result is exact).  The same warps write the item's result.
+// Times of whole cases in this file's comments are GPU time of short bursts (SM clock 1.6 to 1.9 GHz), both sides in turn on
+// one box; back to back, under the power limit, the same passes take 6 to 14 % longer.
 // TMEM columns: S_A/P_A 0..127, S_B/P_B 128..255, O_A 256..383, O_B 384..511.
 // The MMA order S_A S_B (PV_A S_A' PV_B S_B')* lets the softmax of one tile overlap the
 // tensor work of the other.  The host may cut a head's key range into pieces (a count per head); their
@@ -1110,7 +1112,8 @@ cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int n_seq, cudaStre
   if (full) {
     // Items of calibration are all of one length, so a partly filled last round costs as much as a full one.  Where its single
     // query tiles would still all run at once it is issued as those (a tile alone is quicker per key tile than one of a
-    // pair): 2 sequences x 16 heads, 256 queries 16.7 -> 14.7 us, 400: 24.0 -> 21.7, 1600: 123.2 -> 117.6; a pass 1.105 -> 1.073 ms.
+    // pair): 2 sequences x 16 heads, 256 queries 16.7 -> 14.7 us, 400: 24.0 -> 21.7, 1600: 123.2 -> 117.6; a pass 1.105 -> 1.073 ms
+    // (before short items followed their maximum).
     const int total = q.attn_items, n_qp = (p.t_q + 2 * tc::BM - 1) / (2 * tc::BM), whole = total / st->n_sm * st->n_sm;
     const bool tail_single = p.t_q - (n_qp - 1) * 2 * tc::BM <= tc::BM;
     int singles = 0;

@@ -39,8 +39,9 @@ struct Builder {
   }
   // Merged attention tables.  The sinks of a paged head share a page, and the rows of a ragged head all follow one another, so
   // without a bias per scale there is no reason to start a half-tile (64 keys of work, however few are real) with every
-  // scale.  Measured, generation: eight images
-  // at 10x 3.758 -> 3.619 ms, the largest model 6.607 -> 6.358, the ragged layout 2.593 -> 2.480, a 256 x 256 preview 183 -> 163 us
+  // scale.  Measured, generation: eight images at 10x 3.758 -> 3.619 ms, the largest model 6.607 -> 6.358, the ragged layout
+  // 2.593 -> 2.480, a 256 x 256 preview 183 -> 163 us (GPU time of short bursts; back to back, under the power limit, the
+  // large ones take 6 to 14 % longer)
   void merge_runs() {
     run_begin.assign(attn_begin.size(), 0);
     run_cnt.assign(attn_begin.size(), 0);

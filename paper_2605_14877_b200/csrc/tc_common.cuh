@@ -13,7 +13,7 @@ constexpr uint32_t WAIT_LIMIT = 1u << 18;               // tries per wait; each 
 // How far (log2 units) a row's maximum may rise above the reference of its exponentials before O, sums and masses are moved to a
 // new one.  They are floating-point numbers, so a low reference costs no precision: with terms up to 2^32 a row's sums
 // stay far inside fp32's range (n * 2^32 * |V|).  A move costs a read and a write of O for 32 rows when any of them needs it; with a bias
-// on the current scale's keys a threshold of 8 moved often (a pair generated at 20x 2.323 ms, at 32 2.222; one
+// on the current scale's keys a threshold of 8 moved often (GPU time of short bursts: a pair generated at 20x 2.323 ms, at 32 2.222; one
 // calibration batch of recorded steps 0.728 and 0.710; cases without a bias the same).
 constexpr float RESCALE_THRESHOLD = 32.0f;
 constexpr int POLY_MASK = 3;                            // pairs whose index has these bits set take the polynomial exp2 (3: one pair in four)
