@@ -166,7 +166,7 @@ int heatkv_destroy(heatkv_ctx* ctx);
  * beta_accum[layer][h][step][0..step] for every head (sum over the n_seq sequences; every
  * sequence counts as one data point d).  The attention matrix is never written out.  Against 64 bits the
  * masses of 13 scales are off by 4e-7 of themselves on average without an output, where one exponential in three
- * is a cubic, and by 1e-7 with one; 2e-6 was the largest seen.
+ * is a cubic (5e-6 was the largest seen), and by 1e-7 with one (1e-6).
  *   q       DEVICE bf16 [n_seq,H,t[step],d]   strides q_*
  *   k_full  DEVICE bf16 [n_seq,H,c[step],d]   strides kv_*  (all scales up to `step`)
  *   v_full  DEVICE bf16 like k_full, or NULL when `out` is NULL
