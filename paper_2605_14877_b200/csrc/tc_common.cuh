@@ -54,27 +54,24 @@ __device__ __forceinline__ bool mbar_try_hint(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 // Bounded wait.  Returns false when the CTA is aborting (this wait or another one ran out).
+// Kept to a few instructions: one is compiled in at every hand-over between warps, and what they take of the instruction caches
+// the softmax loop loses (with the loop unrolled, as the compiler does where the abort flag is read every 32nd try, the
+// attention kernel was 96 KB of code, so it is 81).
+template <bool HINT = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag,
                                           uint32_t* status, uint32_t limit = WAIT_LIMIT) {
+#pragma unroll 1
   for (uint32_t it = 0; it < limit; ++it) {
-    if (mbar_try(bar, parity)) return true;
-    if ((it & 31u) == 31u && *abort_flag) return false;
+    if (HINT ? mbar_try_hint(bar, parity) : mbar_try(bar, parity)) return true;
+    if (*abort_flag) return false;
   }
   *abort_flag = 1;
   atomicOr(status, 1u);
   return false;
 }
-
-// Bounded wait built on the hinted test.
-__device__ __forceinline__ bool mbar_wait_hint(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag,
-                                               uint32_t* status, uint32_t limit = WAIT_LIMIT) {
-  for (uint32_t it = 0; it < limit; ++it) {
-    if (mbar_try_hint(bar, parity)) return true;
-    if ((it & 31u) == 31u && *abort_flag) return false;
-  }
-  *abort_flag = 1;
-  atomicOr(status, 1u);
-  return false;
+// ... built on the hinted test.
+__device__ __forceinline__ bool mbar_wait_hint(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t* status) {
+  return mbar_wait<true>(bar, parity, abort_flag, status);
 }
 
 // Tensor maps of [n_seq, H, t, d] views.  A head or sequence stride of 0 (one tensor shared by all heads or sequences) has no
@@ -241,9 +238,10 @@ __device__ __forceinline__ bool elect_one() {
 }
 // The same for a converged warp with the vote inside the loop: one vote per try, and a provably uniform result.
 __device__ __forceinline__ bool warp_wait_vote(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t* status) {
+#pragma unroll 1
   for (uint32_t it = 0; it < WAIT_LIMIT; ++it) {
     if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
-    if ((it & 31u) == 31u && __any_sync(0xffffffffu, *abort_flag)) return false;
+    if (__any_sync(0xffffffffu, *abort_flag)) return false;
   }
   *abort_flag = 1;
   atomicOr(status, 1u);
