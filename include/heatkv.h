@@ -318,7 +318,8 @@ int heatkv_attention_append(heatkv_ctx* ctx, const int* seq_ids /*HOST*/, int n_
  * work item takes a whole head's key range), *items = work items of the launch (an upper bound when the
  * call mixes schedules).  A cut head's pieces leave partial results in the arena's scratch region, where
  * the last to arrive merges them.  The choice (a piece count per head) minimises an estimate of the launch's
- * makespan over the SMs and is cached per (schedule, step, layer, batch size).  Host only. */
+ * makespan over the SMs and is cached per (schedule, step, layer, batch size).  A launch of few and short items (at most one per
+ * two SMs, 20 key tiles) runs uncut on pairs of CTAs instead, so there the figures only say what that saves.  Host only. */
 int heatkv_attention_split(heatkv_ctx* ctx, const int* seq_ids /*HOST*/, int n_seq, int layer, int step,
                            int32_t* split_tiles, int32_t* items);
 

@@ -11,7 +11,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libheatkv.so")
 NATIVE = os.path.join(HERE, "_native" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
-SOURCES = ["schedule.cpp", "plan.cpp", "split.cpp", "api.cu", "attn_generic.cu", "attn_tc.cu", "calib_tc.cu", "cache_kernels.cu"]
+SOURCES = ["schedule.cpp", "plan.cpp", "split.cpp", "api.cu", "attn_generic.cu", "attn_tc.cu", "attn_pair.cu", "calib_tc.cu", "cache_kernels.cu"]
 
 
 def _stale() -> bool:

@@ -25,6 +25,8 @@ void tc_destroy(TcState* st);
 bool tc_ready(const TcState* st);
 bool tc_supported(const TcState* st, const AttnParams& p, int d, int n_seq);
 cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int n_seq, cudaStream_t stream);
+bool tc_pair_wanted(const TcState* st, int t_q, int64_t items, int tiles);
+cudaError_t launch_attn_pair(TcState* st, const AttnParams& p, int n_seq, cudaStream_t stream);
 int tc_split_slot_floats(int d);
 cudaError_t launch_wait_expiry(uint32_t* status, uint32_t* result, cudaStream_t stream);
 struct CalibTcState;
@@ -353,6 +355,22 @@ void fill_head_table(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, i
   p->off_desc = tab.desc + shift;
   p->off_src = tab.src + shift;
   p->table_heads = pe0.sched.H;
+}
+
+// Work items of the call without any cut, if the kernel of CTA pairs takes it; else 0.
+int pair_items(const heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int layer, const AttnParams& p) {
+  const int64_t items = (int64_t)n_seq * ctx->cfg.H * ((p.t_q + 255) / 256);
+  const int own_slots = (p.n_own + HEATKV_PAGE_TOKENS - 1) / HEATKV_PAGE_TOKENS;
+  if (!tc_pair_wanted(ctx->tc, p.t_q, items, 0)) return 0;
+  int tiles = 0;
+  for (int i = 0; i < n_seq; ++i) {                         // the longest head: first in its plan's order
+    const PlanEntry& pe = *ctx->plans[ctx->seqs[seq_ids[i]].plan];
+    const int32_t* blob = pe.plan.blob.data();
+    const size_t u = pe.sched.at(step, layer, 0);
+    const int32_t head = blob[pe.plan.header().off_order + u];
+    tiles = std::max(tiles, (blob[attn_tables(pe.plan.header(), p.runs).cnt + u + head] + own_slots + 1) / 2);
+  }
+  return tc_pair_wanted(ctx->tc, p.t_q, items, tiles) ? (int)items : 0;
 }
 
 // Fills the splitting fields of the launch parameters.  When the whole call follows one schedule the choice
@@ -808,7 +826,14 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
   }
   if (fuse) p.append_tiles = (ctx->cfg.t[step] + HEATKV_PAGE_TOKENS - 1) / HEATKV_PAGE_TOKENS + 1;
   cudaError_t e;
-  if (use_tc) {
+  if (const int items = use_tc ? pair_items(ctx, seq_ids, n_seq, step, layer, p) : 0) {
+    fill_head_table(ctx, seq_ids, n_seq, step, layer, &p);
+    p.n_seq = n_seq;
+    p.items_per_seq = items / n_seq;
+    e = launch_attn_pair(ctx->tc, p, n_seq, stream);
+    ctx->launches += 1;
+    ctx->kstats.attention_tcgen05 += 1;
+  } else if (use_tc) {
     try {
       choose_split(ctx, seq_ids, n_seq, step, layer, &p);
     } catch (const std::bad_alloc&) {

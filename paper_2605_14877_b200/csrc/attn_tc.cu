@@ -26,17 +26,13 @@
 // CTA records a status word, drains its own copies and leaves.
 #include <algorithm>
 
-#include "append_device.cuh"
+#include "attn_items.cuh"
 #include "internal.h"
-#include "tc_common.cuh"
 
 namespace heatkv {
 
 namespace tc {
 
-constexpr int BM = 128;                 // rows per Q tile
-constexpr int BN = 128;                 // keys per tile (two 64-row half-tiles)
-constexpr int HALF = 64;
 constexpr int THREADS = 384;
 constexpr int KV_STAGES = 2;
 // Registers are handed from the four utility warps to the eight softmax warps.  setmaxnreg only moves
@@ -97,42 +93,7 @@ enum ItemKind : int { ATTENTION = 0, STOP = 2, NOTHING = 3 };
 // ring entry words
 enum ItemWord : int { W_KIND = 0, W_HEAD, W_SEQ, W_TILES, W_NSPLIT, W_SUB, W_SLOT, W_CTR, W_DESC, W_NDESC };
 constexpr int WORK_COUNTER_WORD = 16;                          // word of the status region that hands out the attention items
-constexpr int STORE_COUNTER_WORD = 17;                         // ... and the cache-update items
 
-
-struct Maps {
-  CUtensorMap q, k_own, v_own, k_pool, v_pool, out;
-};
-
-// One key half-tile: where it comes from and how many of its 64 rows are real.
-struct Slot {
-  int pool_row;     // >= 0: row in the pool; < 0: own-scale tokens starting at -(pool_row + 1)
-  int n_valid;
-  int seg;
-};
-
-// FULL (calibration with an attention output): every key comes from the caller's tensor, and the descriptors, cut at
-// source-scale borders, number its rows.
-template <bool FULL>
-__device__ __forceinline__ Slot get_slot(int i, const int2* descs, int n_desc, int n_slots, int64_t base_row,
-                                         int t_own, int step) {
-  Slot s;
-  int valid = i < n_slots;
-  if (!valid) i = n_slots - 1;                      // padding half-tile: re-read finite data, mask everything
-  if (i < n_desc) {
-    int2 d = descs[i];
-    s.pool_row = FULL ? -(d.x + 1) : (int)(base_row + d.x);
-    s.n_valid = d.y & 0xff;
-    s.seg = (d.y >> 8) & 0xff;
-  } else {
-    int tok0 = (i - n_desc) * HALF;
-    s.pool_row = -(tok0 + 1);
-    s.n_valid = min(HALF, t_own - tok0);
-    s.seg = step;
-  }
-  if (!valid) s.n_valid = 0;
-  return s;
-}
 
 // What every role derives from a ring entry of kind ATTENTION.
 struct Item {
@@ -535,25 +496,9 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
     }
   } else if (p.store_items > 0) {
     // ------------------------------------------------------------------ cache update (warps 2 and 3)
-    // Each warp takes destination half-tiles of (sequence, head) units from a counter of its own and copies
-    // their rows while the other warps work on attention items.  Every store warp of the launch ends with one
-    // fetch past the end; the last of those store_items + 2 * CTAs fetches resets the counter.
+    // their rows are copied while the other warps work on attention items
     pdl_wait();
-    uint32_t* store_counter = p.status + STORE_COUNTER_WORD;
-    const uint32_t fetches = (uint32_t)p.store_items + 2u * gridDim.x;
-    for (;;) {
-      uint32_t old = 0;
-      if (lane == 0) {
-        old = atomicAdd(store_counter, 1u);
-        if (old == fetches - 1u) *reinterpret_cast<volatile uint32_t*>(store_counter) = 0;
-      }
-      const int a = (int)__shfl_sync(0xffffffffu, old, 0);
-      if (a >= p.store_items) break;
-      const int sq = a % p.n_seq, hd = (a / p.n_seq) % p.H, j = a / (p.n_seq * p.H);
-      const int64_t src = sq * p.kv_seq + hd * p.kv_head;
-      append_half_tile(p.seqs[sq].plan, p.seqs[sq].base_row, u + hd, j, p.k_new + src, p.v_new + src, p.kv_tok,
-                       const_cast<__nv_bfloat16*>(p.k_pool), const_cast<__nv_bfloat16*>(p.v_pool), D, lane, 32);
-    }
+    store_rows_loop<D>(p, 2u * gridDim.x, lane);
   }
   } else {
     reg_alloc<REGS_SOFTMAX>();
@@ -1001,35 +946,42 @@ cudaError_t launch_wait_expiry(uint32_t* status, uint32_t* result, cudaStream_t 
 }
 
 // ---------------------------------------------------------------------------------- host side
+int pair_create(int d, int* n_pairs);
+cudaError_t launch_attn_pair_kernel(int d, const AttnParams& p, const tc::Maps& maps, cudaStream_t stream);
+
 struct TcState {
   PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   CUtensorMap k_pool, v_pool;
+  CUtensorMap v_pool_half;   // as v_pool with boxes of d / 2 columns: what one CTA of a pair keeps of a tile's values
   int n_sm = 148;
+  int n_pairs = 0;           // CTA pairs of attn_pair_kernel the device holds at once
   int d = 0;                 // head dimension of the context (64 or 128)
   bool ready = false;
 };
 
 namespace {
 
-bool encode_2d(TcState* st, CUtensorMap* m, void* base, uint64_t rows) {
+// boxes of `cols` columns (64 or 32), their rows swizzled over their 128 or 64 bytes
+CUtensorMapSwizzle swizzle_of(int cols) { return cols == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B; }
+
+bool encode_2d(TcState* st, CUtensorMap* m, void* base, uint64_t rows, int cols) {
   cuuint64_t dims[2] = {(cuuint64_t)st->d, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)st->d * 2};
-  cuuint32_t box[2] = {64, (cuuint32_t)tc::HALF};
+  cuuint32_t box[2] = {(cuuint32_t)cols, (cuuint32_t)tc::HALF};
   cuuint32_t estr[2] = {1, 1};
   return st->encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(cols), CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // [n_seq, H, t, d] view with element strides -> 4-D map (d, token, head, sequence)
 bool encode_4d(TcState* st, CUtensorMap* m, const void* base, int t, int H, int n_seq, int64_t s_tok, int64_t s_head,
-               int64_t s_seq, bool output = false) {
+               int64_t s_seq, int cols = 64, int rows = tc::HALF) {
   const tc::MapShape g = tc::map_shape(st->d, t, H, n_seq, s_tok, s_head, s_seq);
-  // inputs: 64 x 64 boxes; the output leaves in a warp's 32 rows x 32 columns
-  cuuint32_t box[4] = {output ? 32u : 64u, output ? 32u : (cuuint32_t)tc::HALF, 1, 1};
+  cuuint32_t box[4] = {(cuuint32_t)cols, (cuuint32_t)rows, 1, 1};
   cuuint32_t estr[4] = {1, 1, 1, 1};
   return st->encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), g.dims, g.strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, output ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(cols), CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -1050,7 +1002,8 @@ int tc_create(const heatkv_config& cfg, void* k_pool, void* v_pool, uint64_t poo
     return HEATKV_OK;                                   // no driver entry point: generic kernel only
   }
   st->encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-  if (!encode_2d(st, &st->k_pool, k_pool, pool_rows) || !encode_2d(st, &st->v_pool, v_pool, pool_rows))
+  if (!encode_2d(st, &st->k_pool, k_pool, pool_rows, 64) || !encode_2d(st, &st->v_pool, v_pool, pool_rows, 64) ||
+      !encode_2d(st, &st->v_pool_half, v_pool, pool_rows, cfg.d / 2))
     return HEATKV_OK;
   const int smem = cfg.d == 128 ? (int)tc::Layout<128>::SM_ALLOC : (int)tc::Layout<64>::SM_ALLOC;
   const void* kernels[2] = {cfg.d == 128 ? (const void*)tc::attn_tc_kernel<128, false> : (const void*)tc::attn_tc_kernel<64, false>,
@@ -1072,6 +1025,8 @@ int tc_create(const heatkv_config& cfg, void* k_pool, void* v_pool, uint64_t poo
   if (cudaGetDevice(&dev) == cudaSuccess &&
       cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n_sm > 0)
     st->n_sm = n_sm;
+  const int rc = pair_create(cfg.d, &st->n_pairs);
+  if (rc != HEATKV_OK) return rc;
   st->ready = true;
   return HEATKV_OK;
 }
@@ -1091,17 +1046,42 @@ bool tc_supported(const TcState* st, const AttnParams& p, int d, int n_seq) {
   return true;
 }
 
+namespace {
+bool encode_call(TcState* st, tc::Maps* maps, const AttnParams& p, int n_seq, int v_cols) {
+  maps->k_pool = st->k_pool;
+  maps->v_pool = v_cols == 64 ? st->v_pool : st->v_pool_half;
+  // inputs: boxes of 64 rows; the output leaves in a warp's 32 rows x 32 columns
+  return encode_4d(st, &maps->q, p.q, p.t_q, p.H, n_seq, p.q_tok, p.q_head, p.q_seq) &&
+         encode_4d(st, &maps->k_own, p.k_new, p.n_own, p.H, n_seq, p.kv_tok, p.kv_head, p.kv_seq) &&
+         encode_4d(st, &maps->v_own, p.v_new, p.n_own, p.H, n_seq, p.kv_tok, p.kv_head, p.kv_seq, v_cols) &&
+         encode_4d(st, &maps->out, p.out, p.t_q, p.H, n_seq, p.o_tok, p.o_head, p.o_seq, 32, 32);
+}
+}  // namespace
+
+// Does a launch of `items` (sequence, head, 256 queries) with at most `tiles` key tiles go to attn_pair_kernel?  Where all its pairs
+// run at once, and not past PAIR_TILES: attn_tc_kernel would cut longer heads into pieces, which pays from there on.  Back
+// to back, attn_tc_kernel against attn_pair_kernel: 32 items, 256 queries 13.0 and 10.5 us; 64 items, 400 queries 19.5 and 14.5;
+// 4 heads x 1024 queries, 16 items of 20 tiles, 27.9 and 24.2; past the lines 4 heads x 1600 queries (28 items of 32 tiles)
+// 30.0 and 36.1, 28 heads x 576 queries (84 items) 25.4 and 35.5.  A tile of 128 queries is left to one CTA.
+constexpr int PAIR_TILES = 20;
+bool tc_pair_wanted(const TcState* st, int t_q, int64_t items, int tiles) {
+  return t_q > tc::BM && items <= st->n_pairs && tiles <= PAIR_TILES;
+}
+
+cudaError_t launch_attn_pair(TcState* st, const AttnParams& p, int n_seq, cudaStream_t stream) {
+  tc::Maps maps;
+  AttnParams q = p;
+  q.attn_items = p.items_per_seq * n_seq;
+  q.store_items = p.append_tiles * p.H * n_seq;
+  if (p.n_seq != n_seq || q.attn_items < 1 || !encode_call(st, &maps, p, n_seq, st->d / 2)) return cudaErrorInvalidValue;
+  return launch_attn_pair_kernel(st->d, q, maps, stream);
+}
+
 // Attention of a scale step (p.items_per_seq work items per sequence) or, with p.full_slots > 0, calibration with an
 // attention output over all p.n_own keys of p.k_new / p.v_new.
 cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int n_seq, cudaStream_t stream) {
   tc::Maps maps;
-  maps.k_pool = st->k_pool;
-  maps.v_pool = st->v_pool;
-  if (!encode_4d(st, &maps.q, p.q, p.t_q, p.H, n_seq, p.q_tok, p.q_head, p.q_seq) ||
-      !encode_4d(st, &maps.k_own, p.k_new, p.n_own, p.H, n_seq, p.kv_tok, p.kv_head, p.kv_seq) ||
-      !encode_4d(st, &maps.v_own, p.v_new, p.n_own, p.H, n_seq, p.kv_tok, p.kv_head, p.kv_seq) ||
-      !encode_4d(st, &maps.out, p.out, p.t_q, p.H, n_seq, p.o_tok, p.o_head, p.o_seq, true))
-    return cudaErrorInvalidValue;
+  if (!encode_call(st, &maps, p, n_seq, 64)) return cudaErrorInvalidValue;
   if (p.n_seq != n_seq || p.items_per_seq < 1) return cudaErrorInvalidValue;
   // one resident CTA per SM takes the attention items in turn; its two spare warps take the cache-update items
   AttnParams q = p;

@@ -301,6 +301,46 @@ def test_tensor_memory_kernel_rows_survive_an_item_without_rows(hk, d, calibrate
     assert (out[:, :, 1:].double() - p @ v.double()).abs().max().item() <= ATOL_MAX
 
 
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+@pytest.mark.parametrize("H,n_seq,with_bias", [(37, 2, False), (25, 3, True)], ids=["every_pair", "one_more"])
+def test_cta_pair_kernel_line(hk, d, H, n_seq, with_bias):
+    """Launches of 74 (one per CTA pair of the device) and 75 items of up to 256 queries: 144 queries leave the second CTA 16
+    rows, 289 are a second item of 33 rows of which the second CTA has none."""
+    sh = W.Shape("pairs", L=1, H=H, d=d, sides=(4, 12, 16, 17), n_seq=n_seq, s=1)
+    scores = W.synthetic_scas(sh, 2)
+    ref = O.heatkv_schedule(scores, 0.6, sh.s, sh.sides)
+    heads = [(i % n_seq, 0, h) for i, h in enumerate((0, 1, 7, H // 2, H - 1))]
+    _run_full_parity(hk, sh, ref, lambda ses: ses.schedule(scas=scores, b=0.6), hk.LAYOUT_PAGED, kernel=hk.KERNEL_TCGEN05,
+                     bias=W.seg_bias_prior_lognormal(sh, 5) if with_bias else None, check_heads=heads, fused=True)
+
+
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+def test_cta_pair_kernel_mixed_schedules(hk, d):
+    """Sequences of different schedules in one call (no head table in the launch parameters), around the longest head that goes to
+    CTA pairs: at 1024 queries 20 key tiles of 128 when everything is kept, at 1600 queries 32."""
+    from paper_2605_14877_b200.sweep import Session
+    sh = W.Shape("mixed", L=1, H=2, d=d, sides=W.SIDES_13[:11], n_seq=3, s=1)
+    fractions = [np.array([[1.0, 0.0]]), np.array([[0.5, 1.0]]), np.array([[0.0, 0.25]])]
+    q, k, v = W.qkv_layer(sh, 0, 0, device="cuda")
+    host = [_f64(x) for x in (q, k, v)]
+    out = torch.zeros_like(q)
+    with Session(sh.L, sh.H, sh.d, sh.t, sh.s, pool_rows=3 * sh.H * (sh.c[-2] + 64 * sh.K), kernel=hk.KERNEL_TCGEN05) as ses:
+        schedules = [ses.schedule(policy=hk.POLICY_EXPLICIT, fraction=f) for f in fractions]
+        ids = [hk.heatkv_seq_open(ses.ctx, s) for s in schedules]
+        ses.generate(ids, lambda l: (q, k, v), lambda l: out, fused=True)
+        torch.cuda.synchronize()
+        assert hk.heatkv_device_status(ses.ctx) == 0
+        for s in schedules:
+            hk.heatkv_schedule_free(s)
+    for i, f in enumerate(fractions):
+        ref = O.explicit_schedule(f, sh.s, sh.sides)
+        for h in range(sh.H):
+            for step in range(4, sh.K + 1):
+                lo, hi = sh.c[step - 2], sh.c[step - 1]
+                want = O.scale_attention(host[0][i, h, lo:hi], host[1][i, h], host[2][i, h], ref, step, 0, h, 1.0 / math.sqrt(d))
+                _check_attention(out[i, h, lo:hi], want, (i, h, step))
+
+
 def test_tensor_memory_kernel_full_cache(hk):
     """b = 1: long page tables (up to 4121 prior keys), tcgen05 kernel, no bias."""
     sh = W.Shape("full128", L=1, H=2, d=128, sides=W.SIDES_13[:12], n_seq=1, s=3)
