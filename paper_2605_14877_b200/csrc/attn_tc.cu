@@ -1060,7 +1060,7 @@ bool encode_call(TcState* st, tc::Maps* maps, const AttnParams& p, int n_seq, in
 
 // Does a launch of `items` (sequence, head, 256 queries) with at most `tiles` key tiles go to attn_pair_kernel?  Where all its pairs
 // run at once, and not past PAIR_TILES: attn_tc_kernel would cut longer heads into pieces, which pays from there on.  Back
-// to back, attn_tc_kernel against attn_pair_kernel: 32 items, 256 queries 13.0 and 10.5 us; 64 items, 400 queries 19.5 and 14.5;
+// to back, attn_tc_kernel against attn_pair_kernel: 32 items, 256 queries 13.0 and 10.0 us; 64 items, 400 queries 19.5 and 14.0;
 // 4 heads x 1024 queries, 16 items of 20 tiles, 27.9 and 24.2; past the lines 4 heads x 1600 queries (28 items of 32 tiles)
 // 30.0 and 36.1, 28 heads x 576 queries (84 items) 25.4 and 35.5.  A tile of 128 queries is left to one CTA.
 constexpr int PAIR_TILES = 20;
