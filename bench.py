@@ -39,11 +39,14 @@ DATA_SEED = 0
 METRIC = "images_per_sec_scale_step_attention_2b_class_20x"
 N_LAYERS = 32            # layers of the 2B-class model: one step replays the layer sweep this many times
 UNIT = "images/s"
-# dram__bytes_read.sum + dram__bytes_write.sum of the dominant kernel's seven launches of one layer sweep, from
-# the ncu capture summarised in profiles/attn_tc_kernel_config2.md, with the sources the captured kernel was
-# built from (first 16 hex digits of their SHA-256); reported as null once either file has changed
-TRAFFIC_CAPTURE = {"bytes_per_layer_sweep": 308.6e6,
-                   "sources": {"attn_tc.cu": "71cef66cb59cb29b", "tc_common.cuh": "bc9aa7583e1ed4b3"}}
+# dram__bytes_read.sum + dram__bytes_write.sum of the seven tensor-memory launches of one layer sweep, from
+# the ncu capture summarised in profiles/attn_tc_kernel_config2.md, with the sources the captured kernels were
+# built from (first 16 hex digits of their SHA-256); reported as null once one of them has changed
+TRAFFIC_CAPTURE = {"bytes_per_layer_sweep": 309.4e6,
+                   "sources": {"attn_tc.cu": "129be9b38d2076b0",
+                               "attn_pair.cu": "205f8e095cdb6582",
+                               "attn_items.cuh": "5ab8d6e646201b2e",
+                               "tc_common.cuh": "43837b557b2ec231"}}
 
 
 def captured_traffic():
