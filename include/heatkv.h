@@ -362,6 +362,8 @@ int heatkv_allocator_stats(heatkv_ctx* ctx, heatkv_alloc_stats* out);
 int heatkv_launch_count(heatkv_ctx* ctx, uint64_t* n);
 /* The same per kernel, with the state of the tensor-memory kernels' set-up. */
 int heatkv_kernel_launches(heatkv_ctx* ctx, heatkv_kernel_stats* out);
+/* How many of the attention_tcgen05 launches ran uncut on pairs of CTAs (attn_pair_kernel; see heatkv_attention_split). */
+int heatkv_pair_launches(heatkv_ctx* ctx, uint64_t* n);
 /* Appendix on S-CAS stability -- how much the head ordering moves between calibration sets.  scas_runs HOST
  * [n_runs][L][H][K]: S-CAS of n_runs independent calibration sets (heatkv_finalize_scores).  For every prunable
  * source scale k (s <= k <= K-2, 0-based) each run ranks the L*H heads by ascending S-CAS (ties by ascending

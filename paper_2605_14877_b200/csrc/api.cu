@@ -138,6 +138,7 @@ struct heatkv_ctx {
   uint64_t reserved_rows = 0, peak_reserved = 0, meta_used = 0;
   uint64_t launches = 0, openings = 0;
   heatkv_kernel_stats kstats = {};             // launches per kernel
+  uint64_t pair_launches = 0;                  // of kstats.attention_tcgen05: on pairs of CTAs
   TcState* tc = nullptr;
   CalibTcState* calib_tc = nullptr;
   // key-range splitting of the tensor-memory attention kernel
@@ -833,6 +834,7 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
     e = launch_attn_pair(ctx->tc, p, n_seq, stream);
     ctx->launches += 1;
     ctx->kstats.attention_tcgen05 += 1;
+    ctx->pair_launches += 1;
   } else if (use_tc) {
     try {
       choose_split(ctx, seq_ids, n_seq, step, layer, &p);
@@ -1338,6 +1340,12 @@ int heatkv_kernel_launches(heatkv_ctx* ctx, heatkv_kernel_stats* out) {
   *out = ctx->kstats;
   out->tcgen05_attention_ready = tc_ready(ctx->tc) ? 1u : 0u;
   out->tcgen05_calibration_ready = calib_tc_ready(ctx->calib_tc) ? 1u : 0u;
+  return HEATKV_OK;
+}
+
+int heatkv_pair_launches(heatkv_ctx* ctx, uint64_t* n) {
+  if (!ctx || !n) return HEATKV_ERR_INVALID_ARG;
+  *n = ctx->pair_launches;
   return HEATKV_OK;
 }
 

@@ -60,9 +60,10 @@ def _check_attention(got_bf16, ref_f64, what, stats=None):
 
 
 def _run_full_parity(hk, sh, ref, make_schedule, layout, seed=0, bias=None, kernel=None, n_seq=None,
-                     check_heads=None, check_cache=True, fused=False, mutate=None, want_kernels=None):
+                     check_heads=None, check_cache=True, fused=False, mutate=None, want_kernels=None, want_pairs=None):
     """Whole generation of one batch; compares every (seq, layer, head, step) unless check_heads
-    restricts the oracle work to a list of (seq, layer, head)."""
+    restricts the oracle work to a list of (seq, layer, head).  `want_pairs`: the 0-based steps whose attention has to run on
+    pairs of CTAs."""
     n_seq = sh.n_seq if n_seq is None else n_seq
     sm = 1.0 / math.sqrt(sh.d)
     with _session(hk, sh, pool_rows=n_seq * (sh.L * sh.H * (sh.c[-2] + 64 * sh.K) + 64), layout=layout,
@@ -78,7 +79,10 @@ def _run_full_parity(hk, sh, ref, make_schedule, layout, seed=0, bias=None, kern
         bias_dev = None if bias is None else torch.from_numpy(bias).cuda()
         heads = check_heads or [(s_, l, h) for s_ in range(n_seq) for l in range(sh.L) for h in range(sh.H)]
 
+        pairs = [0]                                         # launches on CTA pairs up to each (step, layer)
+
         def after(step, layer):
+            pairs.append(hk.heatkv_pair_launches(ses.ctx))
             if not check_cache or step + 1 >= sh.K:
                 return
             for (s_, l, h) in heads:
@@ -127,6 +131,9 @@ def _run_full_parity(hk, sh, ref, make_schedule, layout, seed=0, bias=None, kern
             assert ks.attention_generic == sh.L * (len(big) - sum(big))
         if want_kernels is not None:
             assert (ks.attention_tcgen05, ks.attention_generic) == want_kernels
+        if want_pairs is not None:
+            ran = np.diff(pairs).reshape(sh.K, sh.L)
+            assert np.array_equal(ran, np.isin(np.arange(sh.K), want_pairs)[:, None] * np.ones(sh.L)), ran
         hk.heatkv_schedule_free(sch)
     return launches
 
@@ -302,16 +309,17 @@ def test_tensor_memory_kernel_rows_survive_an_item_without_rows(hk, d, calibrate
 
 
 @pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
-@pytest.mark.parametrize("H,n_seq,with_bias", [(37, 2, False), (25, 3, True)], ids=["every_pair", "one_more"])
-def test_cta_pair_kernel_line(hk, d, H, n_seq, with_bias):
-    """Launches of 74 (one per CTA pair of the device) and 75 items of up to 256 queries: 144 queries leave the second CTA 16
-    rows, 289 are a second item of 33 rows of which the second CTA has none."""
+@pytest.mark.parametrize("H,n_seq,with_bias,pairs", [(37, 2, False, (1, 2)), (25, 3, True, ()), (9, 4, False, (1, 2, 3))],
+                         ids=["every_pair", "one_more", "odd_tail"])
+def test_cta_pair_kernel_line(hk, d, H, n_seq, with_bias, pairs):
+    """Launches of 74 (one per CTA pair of the device) and 75 items of up to 256 queries; 144 queries leave the second CTA 16 rows.
+    289 queries are a second item of 33 rows of which the second CTA has none: on pairs where they make 72 items."""
     sh = W.Shape("pairs", L=1, H=H, d=d, sides=(4, 12, 16, 17), n_seq=n_seq, s=1)
     scores = W.synthetic_scas(sh, 2)
     ref = O.heatkv_schedule(scores, 0.6, sh.s, sh.sides)
     heads = [(i % n_seq, 0, h) for i, h in enumerate((0, 1, 7, H // 2, H - 1))]
     _run_full_parity(hk, sh, ref, lambda ses: ses.schedule(scas=scores, b=0.6), hk.LAYOUT_PAGED, kernel=hk.KERNEL_TCGEN05,
-                     bias=W.seg_bias_prior_lognormal(sh, 5) if with_bias else None, check_heads=heads, fused=True)
+                     bias=W.seg_bias_prior_lognormal(sh, 5) if with_bias else None, check_heads=heads, fused=True, want_pairs=pairs)
 
 
 @pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
