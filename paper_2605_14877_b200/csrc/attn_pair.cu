@@ -63,7 +63,7 @@ enum Bar : uint32_t {
   P_EMPTY = 25,                       // + tile & 1   the tile's PV product is done
   REF = 27,                           // + 4 warpgroup + warp   the reference after a tile of that warpgroup is published
   SUMS = 35,                          // + warp
-  DRAIN = 39,                         // + issuer
+  DRAIN = 39,                         // + issuer   its last product is done
   N_BARS = 41
 };
 constexpr uint32_t BAR_TMEM_PTR = N_BARS * 8, BAR_ABORT = BAR_TMEM_PTR + 4;
@@ -267,6 +267,12 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
         drain(V_FULL, min(max(j - 1, 0), n_tiles));
         drain(Q_FULL, 1);
       }
+      // The products read and signal both CTAs: neither leaves before the last of either issuer, complete run or not.  (Whoever
+      // gave up has left its reason in the status word.)
+#pragma unroll 1
+      for (int i = 0; i < 2; ++i)
+#pragma unroll 1
+        for (uint32_t t = 0; t < WAIT_LIMIT && !mbar_try_hint(bar(DRAIN + i), 0); ++t) {}
     } else if (warp == 1 && rank == 1) {
       // ------------------------------------------------------------------ word of CTA 1's copies for the issuers, in their order
       pdl_wait();
@@ -301,7 +307,7 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
             mma_ss_pair(lead, tmem + b * BN, qa + (((ks >> 2) * (BM * 128) + (ks & 3) * 32) >> 4),
                         ka + (((ks >> 2) * (HALF * 128) + (ks & 3) * 32) >> 4), DESC_HI_128, IDESC, ks > 0);
           tc_commit_pair(lead, bar(S_FULL + b));
-          tc_commit_pair(lead, bar(K_EMPTY + st));
+          tc_commit_pair(lead && j + STAGES < n_tiles, bar(K_EMPTY + st));   // a stage nobody fills again has no one waiting
         }
       } else {
         constexpr uint32_t IDESC = instr_desc(2 * BM, D, 0, 1);      // P from TMEM, V MN-major
@@ -322,15 +328,10 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
           }
           if (!ok) break;
           tc_commit_pair(lead, bar(P_EMPTY + b));
-          tc_commit_pair(lead, bar(V_EMPTY + st));
+          tc_commit_pair(lead && j + STAGES < n_tiles, bar(V_EMPTY + st));
         }
       }
-      if (!ok) {
-        // leaving early: the products in flight read both CTAs' memory
-        tc_commit_pair(lead, bar(DRAIN + warp - 1));
-#pragma unroll 1
-        for (uint32_t t = 0; t < WAIT_LIMIT && !mbar_try(bar(DRAIN + warp - 1), 0); ++t) {}
-      }
+      tc_commit_pair(lead, bar(DRAIN + warp - 1));
     } else if (p.store_items > 0) {
       // ------------------------------------------------------------------ cache update (three warps of a pair)
       pdl_wait();
@@ -496,14 +497,17 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
     }
     // ---- the two warpgroups' row sums meet; the one with the last tile writes the result
     volatile float2* sums = reinterpret_cast<volatile float2*>(sgen + L::SM_SUM) + row;
-    if (ok && !no_rows && ((n_tiles - 1) & 1) != w) {          // (a warpgroup without a tile: 0 and NO_MAX)
+    const bool writes = ((n_tiles - 1) & 1) == w;
+    if (ok && !no_rows && !writes) {                           // (a warpgroup without a tile: 0 and NO_MAX)
       sums->x = l_sum;
       sums->y = m_ref;
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(SUMS + wr));
-    } else if (ok && !no_rows) {
+    }
+    // with rows or without: the product of this warpgroup's last tile signals its barrier in both CTAs
+    if (ok && n_tiles > w) ok = warp_wait(bar(P_EMPTY + w), ((n_tiles - 1 - w) >> 1) & 1);
+    if (ok && !no_rows && writes) {
       ok = warp_wait(bar(SUMS + wr), 0);
-      if (ok) ok = warp_wait(bar(P_EMPTY + w), ((n_tiles - 1) >> 1) & 1);
       if (ok) {
         tc_fence_after();
         l_sum = fmaf(sums->x, exp2f(sums->y - m_ref), l_sum);  // (references only rise, so this one is the higher)
@@ -545,7 +549,7 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
 
   tc_fence_before();
   __syncthreads();
-  cluster_sync();                                              // nobody signals or reads this CTA any more
+  cluster_sync();      // nobody reads or signals this CTA any more: what the products signal was waited for in both
   if (warp == 0) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");

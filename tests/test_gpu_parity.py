@@ -349,6 +349,45 @@ def test_cta_pair_kernel_mixed_schedules(hk, d):
                 _check_attention(out[i, h, lo:hi], want, (i, h, step))
 
 
+def _pair_steps(hk, t, H, d, n_seq=1, bias=None, kernel=None, **schedule):
+    """One generation of a single layer over scales of t tokens, every output against attention in 64 bits over what the schedule
+    keeps; returns the steps whose attention ran on pairs of CTAs.  |V| / 4 stays below 1.1, so that the bf16 roundings of P and O
+    (2^-9 relative each) stay within 0.0041 of the 1e-2 bar."""
+    from paper_2605_14877_b200.sweep import Session
+    K, c = len(t), np.cumsum([0] + list(t))
+    gen = torch.Generator(device="cuda").manual_seed(sum(t) + H)
+    q, k, v = (torch.randn(n_seq, H, c[-1], d, generator=gen, device="cuda").mul_(f).bfloat16() for f in (1, 1, 0.25))
+    out, pairs = torch.zeros_like(q), [0]
+    with Session(1, H, d, t, 0, pool_rows=n_seq * H * (c[-2] + 64 * K), kernel=hk.KERNEL_TCGEN05 if kernel is None else kernel) as ses:
+        sch = ses.schedule(**(schedule or {"policy": hk.POLICY_EXPLICIT, "fraction": np.ones((1, H))}))
+        mask = hk.heatkv_schedule_masks(sch, K, 1, H)[0][:, 0]
+        ids = [hk.heatkv_seq_open(ses.ctx, sch) for _ in range(n_seq)]
+        ses.generate(ids, lambda l: (q, k, v), lambda l: out, None if bias is None else lambda l, step: bias[step],
+                     lambda step, l: pairs.append(hk.heatkv_pair_launches(ses.ctx)), fused=True)
+        torch.cuda.synchronize()
+        assert hk.heatkv_device_status(ses.ctx) == 0
+        hk.heatkv_schedule_free(sch)
+    scale_of = np.repeat(np.arange(K), t)
+    for step in range(K):
+        lo, hi = c[step], c[step + 1]
+        x = q[:, :, lo:hi].double() @ k[:, :, :hi].double().transpose(2, 3) / math.sqrt(d)
+        own = scale_of[:hi] == step
+        for h in range(H):
+            x[:, h, :, torch.from_numpy(~(own | ((mask[step, h] >> scale_of[:hi]) & 1 == 1))).cuda()] = -math.inf
+        if bias is not None:
+            x += bias[step].double()[:, torch.from_numpy(scale_of[:hi]).cuda()][:, None]
+        want = torch.softmax(x, dim=-1) @ v[:, :, :hi].double()
+        assert (out[:, :, lo:hi].double() - want).abs().max().item() <= ATOL_MAX, step
+    return [step for step in range(K) if pairs[step + 1] > pairs[step]]
+
+
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+def test_cta_pair_kernel_ends_after_any_tile(hk, d):
+    """Two to thirteen key tiles, so that a launch ends in every stage of K and V and on either softmax warpgroup, where the second CTA
+    has one row (129 queries) or none (the second item of 257)."""
+    assert _pair_steps(hk, [129, 257] * 4, 3, d, n_seq=2) == list(range(8))
+
+
 def test_tensor_memory_kernel_full_cache(hk):
     """b = 1: long page tables (up to 4121 prior keys), tcgen05 kernel, no bias."""
     sh = W.Shape("full128", L=1, H=2, d=128, sides=W.SIDES_13[:12], n_seq=1, s=3)
