@@ -9,11 +9,12 @@
 // per key tile.  Launches that do fill the GPU are better off with attn_tc_kernel: there two pairs of these take 12 % longer
 // than one CTA with two query tiles (both softmax warpgroups are then busy throughout and share their sub-partition's issue slots).
 // Warp roles:
-//   warp 0      copies: the CTA's queries, its 64 keys of every tile and its D / 2 columns of the tile's values.
-//   warp 1      CTA 0: issues S = Q K^T for the pair.  CTA 1: passes on to CTA 0 that its own copies have landed.
+//   warp 0      copies: the CTA's queries, its 64 keys of every tile and its D / 2 columns of the tile's values.  They complete on
+//               barriers of CTA 0, where the issuers wait for both CTAs' at once.
+//   warp 1      CTA 0: issues S = Q K^T for the pair.
 //   warp 2      CTA 0: issues O += P V for the pair (an issuer of its own: with one for both, its waits alone took 2500 cycles per
-//               tile).  CTA 1: cache update.
-//   warp 3      cache update (only when the call carries it).
+//               tile).
+//   warp 3 and warps 1 to 3 of CTA 1   cache update (only when the call carries it).
 //   warps 4-7   softmax of even key tiles, warps 8-11 of odd ones, one thread per query row.  A row's reference is common to
 //               both and handed from tile to tile through shared memory; the sums meet at the end, where the warpgroup of the
 //               last tile writes the result.
@@ -56,7 +57,7 @@ struct Layout {
 };
 
 enum Bar : uint32_t {
-  Q_FULL = 0,
+  Q_FULL = 0,                         // Q_FULL, K_FULL, V_FULL: in CTA 0, for the copies of both
   K_FULL = 1, K_EMPTY = 5, V_FULL = 9, V_EMPTY = 13,  // + stage
   S_FULL = 17, S_READ = 19,           // + tile & 1
   P_FULL = 21,                        // + 2 (tile & 1) + half
@@ -83,8 +84,25 @@ __device__ __forceinline__ uint32_t in_cta0(uint32_t addr) {
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// A hand-over of tensor memory to an issuer in CTA 0, which waits with mbar_try_cluster.  Relaxed: tcgen05.fence on either side orders
+// the tensor memory, nothing else is handed over.  (With release and acquire here and for CTA 1's copies, passed on by a warp of
+// it, a preview pair took 161 us, with them for the copies alone 156; so 150.)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
-  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+}
+// Copies into this CTA's shared memory that complete on a barrier of either CTA of the pair.
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t cluster_bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+      ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(cluster_bar)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
+                                                 uint32_t cluster_bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+      ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(cluster_bar)
+      : "memory");
 }
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
   uint32_t ok;
@@ -171,9 +189,8 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
   // cluster barrier, a launch took 0.3 to 0.6 us more: 256 queries, 32 items 10.5, now 10.0 us.)
   if (threadIdx.x - 32u < N_BARS) {
     const uint32_t i = threadIdx.x - 32u;
-    const bool landed = i < K_EMPTY || (i >= V_FULL && i < V_EMPTY);   // Q_FULL, K_FULL, V_FULL: CTA 0 hears of both CTAs' copies
     const bool warps = i >= S_READ && i < P_EMPTY;     // S_READ, P_FULL (used in CTA 0): a warpgroup's warps in both CTAs
-    mbar_init(bar(i), warps ? 8 : landed && rank == 0 ? 2 : 1);
+    mbar_init(bar(i), warps ? 8 : 1);
     if (i == 0) *abort_flag = *reinterpret_cast<volatile uint32_t*>(p.status) != 0;   // an earlier CTA gave up: do not wait again
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -193,6 +210,10 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
   auto slot_of = [&](int i, int64_t base_row) { return get_slot<false>(i, descs, n_desc, n_slots, base_row, p.n_own, p.step); };
 
   auto warp_wait = [&](uint32_t b, uint32_t parity) { return tc::warp_wait(b, parity, abort_flag, p.status); };
+  // for the issuers: both CTAs' softmax warps arrive there
+  auto warp_wait_cluster = [&](uint32_t b, uint32_t parity) {
+    return (bool)__all_sync(0xffffffffu, mbar_wait<Try::CLUSTER>(b, parity, abort_flag, p.status));
+  };
   // for roles that have time: a suspended warp leaves its issue slots to the softmax
   auto warp_wait_idle = [&](uint32_t b, uint32_t parity) {
     return (bool)__all_sync(0xffffffffu, mbar_wait_hint(b, parity, abort_flag, p.status));
@@ -205,18 +226,22 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
       const bool leader = elect_one();
       const int64_t base_row = p.seqs[seq].base_row;
       const int kv_head = head & p.kv_head_mask, kv_seq = seq & p.kv_seq_mask;
+      auto landed = [&](uint32_t which, uint32_t bytes) {     // the barrier in CTA 0, which expects as much from CTA 1
+        if (rank == 0) mbar_expect_tx(bar(which), 2 * bytes);
+        return in_cta0(bar(which));
+      };
       auto load_k = [&](int j) {                       // this CTA's 64 keys of tile j
         const uint32_t st = j % STAGES, use = j / STAGES;
         const Slot sl = slot_of(2 * j + (int)rank, base_row);
         if (j == 0) pdl_wait();                        // the first descriptors are read while the launch before may still run
         if (use > 0) ok = warp_wait_idle(bar(K_EMPTY + st), (use - 1) & 1);
         if (ok && leader) {
-          mbar_expect_tx(bar(K_FULL + st), L::K_BYTES);
+          const uint32_t full = landed(K_FULL + st, L::K_BYTES);
 #pragma unroll
           for (int ch = 0; ch < NCH; ++ch) {
             const uint32_t dst = sbase + L::SM_K + st * L::K_BYTES + ch * (HALF * 128);
-            if (sl.pool_row >= 0) tma_load_2d(dst, &maps.k_pool, ch * 64, sl.pool_row, bar(K_FULL + st));
-            else tma_load_4d(dst, &maps.k_own, ch * 64, -sl.pool_row - 1, kv_head, kv_seq, bar(K_FULL + st));
+            if (sl.pool_row >= 0) tma_load_2d_pair(dst, &maps.k_pool, ch * 64, sl.pool_row, full);
+            else tma_load_4d_pair(dst, &maps.k_own, ch * 64, -sl.pool_row - 1, kv_head, kv_seq, full);
           }
         }
         __syncwarp();
@@ -226,13 +251,13 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
         const Slot sl[2] = {slot_of(2 * j, base_row), slot_of(2 * j + 1, base_row)};
         if (use > 0) ok = warp_wait_idle(bar(V_EMPTY + st), (use - 1) & 1);
         if (ok && leader) {
-          mbar_expect_tx(bar(V_FULL + st), L::V_BYTES);
+          const uint32_t full = landed(V_FULL + st, L::V_BYTES);
           const int col = (int)rank * (D / 2);
 #pragma unroll
           for (int hf = 0; hf < 2; ++hf) {
             const uint32_t dst = sbase + L::SM_V + st * L::V_BYTES + hf * (HALF * D);
-            if (sl[hf].pool_row >= 0) tma_load_2d(dst, &maps.v_pool, col, sl[hf].pool_row, bar(V_FULL + st));
-            else tma_load_4d(dst, &maps.v_own, col, -sl[hf].pool_row - 1, kv_head, kv_seq, bar(V_FULL + st));
+            if (sl[hf].pool_row >= 0) tma_load_2d_pair(dst, &maps.v_pool, col, sl[hf].pool_row, full);
+            else tma_load_4d_pair(dst, &maps.v_own, col, -sl[hf].pool_row - 1, kv_head, kv_seq, full);
           }
         }
         __syncwarp();
@@ -245,18 +270,25 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
         if (!ok) break;
         if (j == 0) {
           if (leader) {
-            mbar_expect_tx(bar(Q_FULL), L::Q_BYTES);
+            const uint32_t full = landed(Q_FULL, L::Q_BYTES);
             for (int i = 0; i < 2 * NCH; ++i)          // 64-column half i / 2, rows 64 (i & 1) ..
-              tma_load_4d(sbase + L::SM_Q + i * (HALF * 128), &maps.q, (i >> 1) * 64, q_row0 + (i & 1) * HALF, head & p.q_head_mask,
-                          seq & p.q_seq_mask, bar(Q_FULL));
+              tma_load_4d_pair(sbase + L::SM_Q + i * (HALF * 128), &maps.q, (i >> 1) * 64, q_row0 + (i & 1) * HALF,
+                               head & p.q_head_mask, seq & p.q_seq_mask, full);
           }
           __syncwarp();
         }
         if (j >= 2) load_v(j - 2);
         if (!ok) break;
       }
-      if (!ok || *abort_flag) {
-        // leaving early: let every copy this warp started land before the CTA exits (tiles 0 .. j of K and 0 .. j - 2 of V at most)
+      // The products read and signal both CTAs: neither leaves before the last of either issuer, complete run or not.  (Whoever
+      // gave up has left its reason in the status word.)
+#pragma unroll 1
+      for (int i = 0; i < 2; ++i)
+#pragma unroll 1
+        for (uint32_t t = 0; t < WAIT_LIMIT && !mbar_try_hint(bar(DRAIN + i), 0); ++t) {}
+      if (rank == 0 && (!ok || *abort_flag)) {
+        // leaving early: let every copy of either CTA land before they exit (tiles 0 .. j of K and 0 .. j - 2 of V at most).  What
+        // CTA 1 still lacks runs into the bound; an issuer that gives up over it sets this CTA's flag before its last commit.
         auto drain = [&](uint32_t first, int tiles) {
 #pragma unroll 1
           for (int i = max(0, tiles - STAGES); i < tiles; ++i)
@@ -266,25 +298,6 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
         drain(K_FULL, min(j + 1, n_tiles));
         drain(V_FULL, min(max(j - 1, 0), n_tiles));
         drain(Q_FULL, 1);
-      }
-      // The products read and signal both CTAs: neither leaves before the last of either issuer, complete run or not.  (Whoever
-      // gave up has left its reason in the status word.)
-#pragma unroll 1
-      for (int i = 0; i < 2; ++i)
-#pragma unroll 1
-        for (uint32_t t = 0; t < WAIT_LIMIT && !mbar_try_hint(bar(DRAIN + i), 0); ++t) {}
-    } else if (warp == 1 && rank == 1) {
-      // ------------------------------------------------------------------ word of CTA 1's copies for the issuers, in their order
-      pdl_wait();
-      auto forward = [&](uint32_t which, uint32_t parity) {
-        ok = ok && warp_wait_idle(bar(which), parity);
-        if (ok && lane == 0) mbar_arrive_cluster(in_cta0(bar(which)));
-      };
-#pragma unroll 1
-      for (int j = 0; j < n_tiles + 2 && ok; ++j) {
-        if (j < n_tiles) forward(K_FULL + j % STAGES, (j / STAGES) & 1);
-        if (j == 0) forward(Q_FULL, 0);
-        if (j >= 2) forward(V_FULL + (j - 2) % STAGES, ((j - 2) / STAGES) & 1);
       }
     } else if (warp < 3 && rank == 0) {
       // ------------------------------------------------------------------ MMA issuers (CTA 0, for the pair)
@@ -297,7 +310,7 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
 #pragma unroll 1
         for (int j = 0; j < n_tiles && ok; ++j) {
           const uint32_t b = j & 1, st = j % STAGES;
-          if (j >= 2) ok = warp_wait(bar(S_READ + b), ((j >> 1) - 1) & 1);
+          if (j >= 2) ok = warp_wait_cluster(bar(S_READ + b), ((j >> 1) - 1) & 1);
           if (ok) ok = warp_wait(bar(K_FULL + st), (j / STAGES) & 1);
           if (!ok) break;
           tc_fence_after();
@@ -319,7 +332,7 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
           const uint32_t va = desc_lo(sbase + L::SM_V + st * L::V_BYTES), pa = tmem + T_P + b * 64;
 #pragma unroll
           for (int h = 0; h < 2; ++h) {                // keys 64 h .. 64 h + 63
-            if (ok) ok = warp_wait(bar(P_FULL + 2 * b + h), (j >> 1) & 1);
+            if (ok) ok = warp_wait_cluster(bar(P_FULL + 2 * b + h), (j >> 1) & 1);
             if (!ok) break;
             tc_fence_after();
 #pragma unroll
@@ -333,9 +346,9 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
       }
       tc_commit_pair(lead, bar(DRAIN + warp - 1));
     } else if (p.store_items > 0) {
-      // ------------------------------------------------------------------ cache update (three warps of a pair)
+      // ------------------------------------------------------------------ cache update (four warps of a pair)
       pdl_wait();
-      store_rows_loop<D>(p, 3u * (gridDim.x >> 1), lane);
+      store_rows_loop<D>(p, 2u * gridDim.x, lane);
     }
   } else {
     reg_alloc<REGS_SOFTMAX>();

@@ -53,16 +53,33 @@ __device__ __forceinline__ bool mbar_try_hint(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// The same for a barrier that threads of the cluster's other CTA arrive at.  Relaxed: it orders execution, which is what
+// hand-overs of tensor memory need beside the tcgen05.fence on either side.
+__device__ __forceinline__ bool mbar_try_cluster(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+enum class Try { PLAIN, HINT, CLUSTER };
 // Bounded wait.  Returns false when the CTA is aborting (this wait or another one ran out).
 // Kept to a few instructions: one is compiled in at every hand-over between warps, and what they take of the instruction caches
 // the softmax loop loses (with the loop unrolled, as the compiler does where the abort flag is read every 32nd try, the
 // attention kernel was 96 KB of code, so it is 81).
-template <bool HINT = false>
+template <Try HOW = Try::PLAIN>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag,
                                           uint32_t* status, uint32_t limit = WAIT_LIMIT) {
 #pragma unroll 1
   for (uint32_t it = 0; it < limit; ++it) {
-    if (HINT ? mbar_try_hint(bar, parity) : mbar_try(bar, parity)) return true;
+    if (HOW == Try::HINT      ? mbar_try_hint(bar, parity)
+        : HOW == Try::CLUSTER ? mbar_try_cluster(bar, parity)
+                              : mbar_try(bar, parity))
+      return true;
     if (*abort_flag) return false;
   }
   *abort_flag = 1;
@@ -71,7 +88,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 }
 // ... built on the hinted test.
 __device__ __forceinline__ bool mbar_wait_hint(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t* status) {
-  return mbar_wait<true>(bar, parity, abort_flag, status);
+  return mbar_wait<Try::HINT>(bar, parity, abort_flag, status);
 }
 
 // Tensor maps of [n_seq, H, t, d] views.  A head or sequence stride of 0 (one tensor shared by all heads or sequences) has no
