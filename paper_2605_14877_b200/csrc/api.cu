@@ -363,13 +363,11 @@ int pair_items(const heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, i
   const int64_t items = (int64_t)n_seq * ctx->cfg.H * ((p.t_q + 255) / 256);
   const int own_slots = (p.n_own + HEATKV_PAGE_TOKENS - 1) / HEATKV_PAGE_TOKENS;
   if (!tc_pair_wanted(ctx->tc, p.t_q, items, 0)) return 0;
-  int tiles = 0;
-  for (int i = 0; i < n_seq; ++i) {                         // the longest head: first in its plan's order
+  int tiles = 0;                                            // of the longest head (the plan's order is by tokens, not by half-tiles)
+  for (int i = 0; i < n_seq; ++i) {
     const PlanEntry& pe = *ctx->plans[ctx->seqs[seq_ids[i]].plan];
-    const int32_t* blob = pe.plan.blob.data();
-    const size_t u = pe.sched.at(step, layer, 0);
-    const int32_t head = blob[pe.plan.header().off_order + u];
-    tiles = std::max(tiles, (blob[attn_tables(pe.plan.header(), p.runs).cnt + u + head] + own_slots + 1) / 2);
+    const int32_t* cnt = pe.plan.blob.data() + attn_tables(pe.plan.header(), p.runs).cnt + pe.sched.at(step, layer, 0);
+    tiles = std::max(tiles, (*std::max_element(cnt, cnt + ctx->cfg.H) + own_slots + 1) / 2);
   }
   return tc_pair_wanted(ctx->tc, p.t_q, items, tiles) ? (int)items : 0;
 }

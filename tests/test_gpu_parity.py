@@ -388,6 +388,16 @@ def test_cta_pair_kernel_ends_after_any_tile(hk, d):
     assert _pair_steps(hk, [129, 257] * 4, 3, d, n_seq=2) == list(range(8))
 
 
+def test_cta_pair_kernel_line_counts_half_tiles(hk):
+    """Of two heads at the last step one sees 896 tokens in 14 half-tiles, the other 845 in 26 (thirteen scales of 65): with 16 of the
+    step's own that is 21 key tiles, one past the line, although the first comes first by tokens.  A step before, 20."""
+    t = [65] * 13 + [896, 1024]
+    scas = np.full((1, 2, len(t)), 0.1)
+    scas[0, 1] = 0.9
+    scas[0, :, 13] = 0.9, 0.1
+    assert _pair_steps(hk, t, 2, 128, scas=scas, b=0.5) == [13]
+
+
 def test_tensor_memory_kernel_full_cache(hk):
     """b = 1: long page tables (up to 4121 prior keys), tcgen05 kernel, no bias."""
     sh = W.Shape("full128", L=1, H=2, d=128, sides=W.SIDES_13[:12], n_seq=1, s=3)
