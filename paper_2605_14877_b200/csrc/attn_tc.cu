@@ -1067,6 +1067,16 @@ constexpr int PAIR_TILES = 20;
 bool tc_pair_wanted(const TcState* st, int t_q, int64_t items, int tiles) {
   return t_q > tc::BM && items <= st->n_pairs && tiles <= PAIR_TILES;
 }
+// ... where attn_tc_kernel would take `cut_items` items of at most `run` tiles instead?  With 128-wide heads in any case.  A pair takes
+// 0.79 us per tile for either width, but a tile of 64-wide heads takes attn_tc_kernel 1.2 us instead of 1.7, a piece more to merge
+// 0.8 and a full GPU 1.8 us more than an empty one.  64-wide heads x 256 queries, attn_tc_kernel against attn_pair_kernel: 1 item of 14
+// tiles 14.8 and 14.6, of 20 tiles (5 pieces) 16.7 and 19.4; 24 items of 15 tiles 16.5 and 15.7, of 20 tiles 18.5 and 19.7; 64 items of 20
+// tiles (2 pieces) 23.6 and 21.3.  Of 568 launches of 1 to 72 items this picks none that is more than 2.5 % slower than the other.
+bool tc_pair_beats_cut(const TcState* st, int tiles, int run, int cut_items) {
+  return st->d == 128 || 64 * tiles <= 96 * run + 64 * ((tiles + run - 1) / run) + 256 + cut_items;
+}
+// Up to here that holds for any cut into pieces of SPLIT_MIN_PIECE tiles and more.
+bool tc_pair_sure(const TcState* st, int tiles) { return st->d == 128 || tiles <= 13; }
 
 cudaError_t launch_attn_pair(TcState* st, const AttnParams& p, int n_seq, cudaStream_t stream) {
   tc::Maps maps;

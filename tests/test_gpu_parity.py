@@ -388,6 +388,14 @@ def test_cta_pair_kernel_ends_after_any_tile(hk, d):
     assert _pair_steps(hk, [129, 257] * 4, 3, d, n_seq=2) == list(range(8))
 
 
+@pytest.mark.parametrize("d,H,tiles,pairs", [(64, 8, 13, True), (64, 8, 20, False), (64, 72, 20, True), (64, 72, 21, False),
+                                             (128, 8, 20, True), (128, 8, 21, False)])
+def test_cta_pair_kernel_against_cuts(hk, d, H, tiles, pairs):
+    """256 queries over `tiles` key tiles go to CTA pairs where that is faster than cutting the heads: with 64-wide heads the cut
+    into pieces of 4 wins for 8 heads of 20 tiles, not where 72 heads leave room for two pieces each."""
+    assert (1 in _pair_steps(hk, [tiles * 128 - 256, 256], H, d)) == pairs
+
+
 def test_cta_pair_kernel_line_counts_half_tiles(hk):
     """Of two heads at the last step one sees 896 tokens in 14 half-tiles, the other 845 in 26 (thirteen scales of 65): with 16 of the
     step's own that is 21 key tiles, one past the line, although the first comes first by tokens.  A step before, 20."""
