@@ -383,9 +383,9 @@ def _pair_steps(hk, t, H, d, n_seq=1, bias=None, kernel=None, **schedule):
 
 @pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
 def test_cta_pair_kernel_ends_after_any_tile(hk, d):
-    """Two to thirteen key tiles, so that a launch ends in every stage of K and V and on either softmax warpgroup, where the second CTA
-    has one row (129 queries) or none (the second item of 257)."""
-    assert _pair_steps(hk, [129, 257] * 4, 3, d, n_seq=2) == list(range(8))
+    """2, 3, 6, 8, 11 and 13 key tiles, so that a launch ends in every stage of K and V and on either softmax warpgroup, where the
+    second CTA has one row (129 queries) or none (the second item of 257)."""
+    assert _pair_steps(hk, [129, 129, 257, 257, 64, 257, 129], 3, d, n_seq=2) == [0, 1, 2, 3, 5, 6]
 
 
 @pytest.mark.parametrize("d,H,tiles,pairs", [(64, 8, 13, True), (64, 8, 20, False), (64, 72, 20, True), (64, 72, 21, False),
