@@ -572,28 +572,28 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
 }  // namespace pair
 
 // ---------------------------------------------------------------------------------- host side
-// Sets the kernel up on the current device; *n_pairs = pairs of CTAs it holds at once (0: it cannot run them).
-int pair_create(int d, int* n_pairs) {
-  *n_pairs = 0;
+// Sets the kernel up on the current device: the pairs of CTAs it holds at once.  0: it cannot run them, attn_tc_kernel takes all.
+int pair_create(int d) {
   const void* kern = d == 128 ? (const void*)pair::attn_pair_kernel<128> : (const void*)pair::attn_pair_kernel<64>;
   const int smem = d == 128 ? (int)pair::Layout<128>::SM_ALLOC : (int)pair::Layout<64>::SM_ALLOC;
   cudaFuncAttributes attr;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaFuncGetAttributes(&attr, kern) != cudaSuccess) {
     cudaGetLastError();
-    return HEATKV_OK;
+    return 0;
   }
   // the register hand-over inside the kernel must fit in what the launch really allocates
-  if (attr.numRegs * pair::THREADS < 128 * pair::REGS_SMALL + 256 * pair::REGS_SOFTMAX) return HEATKV_ERR_CUDA;
+  if (attr.numRegs * pair::THREADS < 128 * pair::REGS_SMALL + 256 * pair::REGS_SOFTMAX) return 0;
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3(2);
   lc.blockDim = dim3(pair::THREADS);
   lc.dynamicSmemBytes = smem;
-  if (cudaOccupancyMaxActiveClusters(n_pairs, kern, &lc) != cudaSuccess) {
+  int n_pairs = 0;
+  if (cudaOccupancyMaxActiveClusters(&n_pairs, kern, &lc) != cudaSuccess) {
     cudaGetLastError();
-    *n_pairs = 0;
+    return 0;
   }
-  return HEATKV_OK;
+  return n_pairs;
 }
 
 cudaError_t launch_attn_pair_kernel(int d, const AttnParams& p, const tc::Maps& maps, cudaStream_t stream) {

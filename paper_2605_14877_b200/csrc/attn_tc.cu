@@ -946,7 +946,7 @@ cudaError_t launch_wait_expiry(uint32_t* status, uint32_t* result, cudaStream_t 
 }
 
 // ---------------------------------------------------------------------------------- host side
-int pair_create(int d, int* n_pairs);
+int pair_create(int d);
 cudaError_t launch_attn_pair_kernel(int d, const AttnParams& p, const tc::Maps& maps, cudaStream_t stream);
 
 struct TcState {
@@ -1025,8 +1025,7 @@ int tc_create(const heatkv_config& cfg, void* k_pool, void* v_pool, uint64_t poo
   if (cudaGetDevice(&dev) == cudaSuccess &&
       cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n_sm > 0)
     st->n_sm = n_sm;
-  const int rc = pair_create(cfg.d, &st->n_pairs);
-  if (rc != HEATKV_OK) return rc;
+  st->n_pairs = pair_create(cfg.d);
   st->ready = true;
   return HEATKV_OK;
 }
