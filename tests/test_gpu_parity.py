@@ -191,12 +191,20 @@ def test_tensor_memory_kernel_head_dim_64(hk, layout):
                          kernel=hk.KERNEL_AUTO, check_cache=False)
 
 
+# Steps of more than 128 queries with few units run on CTA pairs; 40 heads x 2 sequences are past the 74 items of that kernel, on
+# attn_tc_kernel (no step on pairs; heads from both 32-lane chunks of its item lookup and from both sequences are compared).
+BOTH_KERNELS = pytest.mark.parametrize("H,n_sides,heads,want_pairs",
+                                       [(2, 11, None, None), (40, 9, [(0, 0, 0), (1, 0, 17), (0, 0, 31), (1, 0, 39)], ())],
+                                       ids=["pairs", "past_pairs"])
+
+
+@BOTH_KERNELS
 @pytest.mark.parametrize("where", ["first_half", "second_half", "everywhere"])
-def test_tensor_memory_kernel_outlier_keys(hk, where):
+def test_tensor_memory_kernel_outlier_keys(hk, where, H, n_sides, heads, want_pairs):
     """Sparse keys scaled by 16 (logits of +-40 and more) that first show up in later key tiles, in the first 64
     keys of a tile, in the last 64, or in both: the running reference of the online softmax has to move by tens
     of units in the middle of a head (rescaling O and the row sum), and the result must still match the oracle."""
-    sh = W.Shape("outlier", L=1, H=2, d=128, sides=W.SIDES_13[:11], n_seq=2, s=3)
+    sh = W.Shape("outlier", L=1, H=H, d=128, sides=W.SIDES_13[:n_sides], n_seq=2, s=3)
     scores = W.synthetic_scas(sh, 2)
     ref = O.heatkv_schedule(scores, 0.5, sh.s, sh.sides)
 
@@ -214,15 +222,16 @@ def test_tensor_memory_kernel_outlier_keys(hk, where):
         # output format itself resolves 1e-2
         return q, k, v * 0.25
 
-    _run_full_parity(hk, sh, ref, lambda ses: ses.schedule(scas=scores, b=0.5), hk.LAYOUT_PAGED,
-                     kernel=hk.KERNEL_TCGEN05, check_cache=False, fused=True, mutate=mutate)
+    _run_full_parity(hk, sh, ref, lambda ses: ses.schedule(scas=scores, b=0.5), hk.LAYOUT_PAGED, check_heads=heads,
+                     kernel=hk.KERNEL_TCGEN05, check_cache=False, fused=True, mutate=mutate, want_pairs=want_pairs)
 
 
+@BOTH_KERNELS
 @pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
-def test_tensor_memory_kernel_lagging_reference(hk, d):
+def test_tensor_memory_kernel_lagging_reference(hk, d, H, n_sides, heads, want_pairs):
     """Sparse keys scaled by 6 in later key tiles: row maxima rise by some 5 to 30 log2 units, less than what moves the online
     softmax's reference, so P and the row sums hold terms far above 1."""
-    sh = W.Shape("lagging", L=1, H=2, d=d, sides=W.SIDES_13[:11], n_seq=2, s=3)
+    sh = W.Shape("lagging", L=1, H=H, d=d, sides=W.SIDES_13[:n_sides], n_seq=2, s=3)
     scores = W.synthetic_scas(sh, 2)
     ref = O.heatkv_schedule(scores, 0.5, sh.s, sh.sides)
 
@@ -234,15 +243,16 @@ def test_tensor_memory_kernel_lagging_reference(hk, d):
         # allow 4.2 * 2^-8 = 0.0165; V scaled by 1/4 (exact) brings that bound to 0.0041, inside the 1e-2 bar
         return q, k, v * 0.25
 
-    _run_full_parity(hk, sh, ref, lambda ses: ses.schedule(scas=scores, b=0.5), hk.LAYOUT_PAGED,
-                     kernel=hk.KERNEL_TCGEN05, check_cache=False, fused=True, mutate=mutate)
+    _run_full_parity(hk, sh, ref, lambda ses: ses.schedule(scas=scores, b=0.5), hk.LAYOUT_PAGED, check_heads=heads,
+                     kernel=hk.KERNEL_TCGEN05, check_cache=False, fused=True, mutate=mutate, want_pairs=want_pairs)
 
 
+@BOTH_KERNELS
 @pytest.mark.parametrize("where", ["first_half", "second_half"])
-def test_tensor_memory_kernel_outlier_keys_head_dim_64(hk, where):
-    """64-wide heads take a tile's exponentials before its maximum is known: keys scaled by 40 (logits of +-100 and more, past the
+def test_tensor_memory_kernel_outlier_keys_head_dim_64(hk, where, H, n_sides, heads, want_pairs):
+    """attn_tc_kernel takes the exponentials of 64-wide heads before a tile's maximum is known: keys scaled by 40 (logits of +-100 and more, past the
     polynomial's range) in either half of later tiles, at positions of both exponential forms, must still move the reference."""
-    sh = W.Shape("outlier64", L=1, H=2, d=64, sides=W.SIDES_13[:11], n_seq=2, s=3)
+    sh = W.Shape("outlier64", L=1, H=H, d=64, sides=W.SIDES_13[:n_sides], n_seq=2, s=3)
     scores = W.synthetic_scas(sh, 2)
     ref = O.heatkv_schedule(scores, 0.5, sh.s, sh.sides)
 
@@ -253,17 +263,18 @@ def test_tensor_memory_kernel_outlier_keys_head_dim_64(hk, where):
         k[:, :, pick] *= 40
         return q, k, v * 0.25                      # |O| below 1.1, so the two bf16 roundings stay within 0.0041 (bar 1e-2)
 
-    _run_full_parity(hk, sh, ref, lambda ses: ses.schedule(scas=scores, b=0.5), hk.LAYOUT_PAGED,
-                     kernel=hk.KERNEL_TCGEN05, check_cache=False, fused=True, mutate=mutate)
+    _run_full_parity(hk, sh, ref, lambda ses: ses.schedule(scas=scores, b=0.5), hk.LAYOUT_PAGED, check_heads=heads,
+                     kernel=hk.KERNEL_TCGEN05, check_cache=False, fused=True, mutate=mutate, want_pairs=want_pairs)
 
 
 @pytest.mark.parametrize("token_major", [False, True], ids=["head_major", "token_major"])
 @pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
-def test_tensor_memory_kernel_writes_its_own_rows_only(hk, d, token_major):
+@pytest.mark.parametrize("H", [3, 40], ids=["pairs", "past_pairs"])
+def test_tensor_memory_kernel_writes_its_own_rows_only(hk, H, d, token_major):
     """The output leaves in boxes of 32 rows: at token counts around multiples of 32 and 128 a step fills its rows of every head
     and sequence and leaves the rows behind them alone."""
     from paper_2605_14877_b200.sweep import Session
-    sh = W.Shape("guard", L=1, H=3, d=d, sides=(1, 5, 6, 8, 11, 12, 16, 17), n_seq=2, s=1)
+    sh = W.Shape("guard", L=1, H=H, d=d, sides=(1, 5, 6, 8, 11, 12, 16, 17), n_seq=2, s=1)
     q, k, v = W.qkv_layer(sh, 0, 0, device="cuda")
     shape = (sh.n_seq, sh.c[-1] + 64, sh.H, d) if token_major else (sh.n_seq, sh.H, sh.c[-1] + 64, d)
     buf = torch.full(shape, 7.0, dtype=torch.bfloat16, device="cuda")
@@ -280,6 +291,7 @@ def test_tensor_memory_kernel_writes_its_own_rows_only(hk, d, token_major):
 
         ses.generate(ids, lambda l: (q, k, v), lambda l: out, None, after)
         assert hk.heatkv_device_status(ses.ctx) == 0
+        assert hk.heatkv_pair_launches(ses.ctx) == (3 if H == 3 else 0)       # the steps of 144, 256 and 289 tokens
         hk.heatkv_schedule_free(sch)
 
 
@@ -349,7 +361,7 @@ def test_cta_pair_kernel_mixed_schedules(hk, d):
                 _check_attention(out[i, h, lo:hi], want, (i, h, step))
 
 
-def _pair_steps(hk, t, H, d, n_seq=1, bias=None, kernel=None, **schedule):
+def _pair_steps(hk, t, H, d, n_seq=1, bias=None, kernel=None, scratch_bytes=1 << 26, **schedule):
     """One generation of a single layer over scales of t tokens, every output against attention in 64 bits over what the schedule
     keeps; returns the steps whose attention ran on pairs of CTAs.  |V| / 4 stays below 1.1, so that the bf16 roundings of P and O
     (2^-9 relative each) stay within 0.0041 of the 1e-2 bar."""
@@ -358,7 +370,8 @@ def _pair_steps(hk, t, H, d, n_seq=1, bias=None, kernel=None, **schedule):
     gen = torch.Generator(device="cuda").manual_seed(sum(t) + H)
     q, k, v = (torch.randn(n_seq, H, c[-1], d, generator=gen, device="cuda").mul_(f).bfloat16() for f in (1, 1, 0.25))
     out, pairs = torch.zeros_like(q), [0]
-    with Session(1, H, d, t, 0, pool_rows=n_seq * H * (c[-2] + 64 * K), kernel=hk.KERNEL_TCGEN05 if kernel is None else kernel) as ses:
+    with Session(1, H, d, t, 0, pool_rows=n_seq * H * (c[-2] + 64 * K), kernel=hk.KERNEL_TCGEN05 if kernel is None else kernel,
+                 scratch_bytes=scratch_bytes) as ses:
         sch = ses.schedule(**(schedule or {"policy": hk.POLICY_EXPLICIT, "fraction": np.ones((1, H))}))
         mask = hk.heatkv_schedule_masks(sch, K, 1, H)[0][:, 0]
         ids = [hk.heatkv_seq_open(ses.ctx, sch) for _ in range(n_seq)]
@@ -601,6 +614,20 @@ def test_small_scratch_still_cuts_long_heads(hk):
     assert got[0] == got[1] and got[0][0] > 0
 
 
+def test_small_scratch_cuts_are_launched(hk):
+    """The same 56 items with 24 key tiles, past the line of the CTA pairs: the cut that both sizes of scratch hold is what runs."""
+    t, got = [256, 2304, 400], []
+    for scratch in (1 << 24, 1 << 26):
+        assert 2 not in _pair_steps(hk, t, 7, 128, n_seq=4, scratch_bytes=scratch)
+        sh = W.Shape("cut", L=1, H=7, d=128, sides=(16, 48, 20), n_seq=4, s=0)
+        with _session(hk, sh, 4 * sh.H * (sh.c[-2] + 64 * sh.K), hk.LAYOUT_PAGED, hk.KERNEL_AUTO, scratch_bytes=scratch) as ses:
+            sch = ses.schedule(policy=hk.POLICY_EXPLICIT, fraction=np.ones((1, 7)))
+            ids = [hk.heatkv_seq_open(ses.ctx, sch) for _ in range(sh.n_seq)]
+            got.append(hk.heatkv_attention_split(ses.ctx, ids, 0, 2))
+            hk.heatkv_schedule_free(sch)
+    assert got[0] == got[1] and got[0][0] > 0
+
+
 def test_split_heads_are_reproducible_bit_for_bit(hk):
     """Pieces of a cut head are merged in piece order whichever arrives last: the same generation run four
     times gives identical output bits (steps of this workload are cut, see the test above)."""
@@ -741,6 +768,18 @@ def test_activations_shared_by_heads_or_sequences(hk, d, q_over, kv_over):
                                              torch.from_numpy(bias).cuda()[0].contiguous(), acc)
             beta = hk.heatkv_finalize_scores(ses.ctx, acc, sh.n_seq, sh.L, sh.H, sh.K)[0]
             assert np.all(np.abs(beta - want)[mask] <= RTOL_BETA * want[mask])
+
+
+@pytest.mark.parametrize("q_over,kv_over", [((), (1,)), ((0,), (0, 1)), ((0, 1), (0,))], ids=["kv_heads", "all_seqs", "q_both"])
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+def test_activations_shared_past_the_pair_line(hk, d, q_over, kv_over):
+    """The same strides on attn_tc_kernel with a second query tile, partly filled (144 and 289 queries) and full (256)."""
+    sh = W.Shape("shared", L=1, H=40, d=d, sides=(1, 4, 12, 16, 17), n_seq=2, s=1)
+    scores = W.synthetic_scas(sh, 6)
+    ref = O.heatkv_schedule(scores, 0.6, sh.s, sh.sides)
+    _run_full_parity(hk, sh, ref, lambda ses: ses.schedule(scas=scores, b=0.6), hk.LAYOUT_PAGED, kernel=hk.KERNEL_TCGEN05,
+                     check_heads=[(0, 0, 0), (1, 0, 17), (1, 0, 39)], fused=True, want_pairs=(),
+                     mutate=lambda l, q, k, v: (_shared(q, q_over), _shared(k, kv_over), _shared(v, kv_over)))
 
 
 @pytest.mark.parametrize("value", [-np.inf, -3.4e38], ids=["inf", "lowest"])
