@@ -40,7 +40,7 @@ METRIC = "images_per_sec_scale_step_attention_2b_class_20x"
 N_LAYERS = 32            # layers of the 2B-class model: one step replays the layer sweep this many times
 UNIT = "images/s"
 # dram__bytes_read.sum + dram__bytes_write.sum of the seven tensor-memory launches of one layer sweep, from
-# the ncu capture summarised in profiles/attn_tc_kernel_config2.md, with the sources the captured kernels were
+# an ncu capture of them, with the sources the captured kernels were
 # built from (first 16 hex digits of their SHA-256); reported as null once one of them has changed
 TRAFFIC_CAPTURE = {"bytes_per_layer_sweep": 309.4e6,
                    "sources": {"attn_tc.cu": "129be9b38d2076b0",
@@ -366,6 +366,7 @@ def run_few_heads_workload(args):
             ses = Session(sh.L, sh.H, sh.d, sh.t, sh.s, pool_rows=2 * sh.H * (sh.c[-2] + 64 * sh.K), scratch_bytes=scratch)
             sch = ses.schedule(scas=scores, b=b)
             ms, reps = np.zeros(sh.K), max(3, min(args.steps, 20))
+            on_pairs = set()                             # steps whose launch runs uncut on CTA pairs
             for rep in range(reps + 2):
                 ids = [hk.heatkv_seq_open(ses.ctx, sch)]
                 if rep == 0 and scratch > 1024:
@@ -373,16 +374,23 @@ def run_few_heads_workload(args):
                     res["ctas_per_scale"] = [hk.heatkv_attention_split(ses.ctx, ids, 0, st)[1] for st in range(sh.K)]
                 for step in range(sh.K):
                     ses.pre_step(ids, step)
+                    before = hk.heatkv_pair_launches(ses.ctx)
                     flush.fill_(1)
                     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
                     e0.record()
                     hk.heatkv_scale_attention(ses.ctx, ids, 0, step, qs[step], ks[step], vs[step], None, None, outs[step])
                     e1.record()
+                    if hk.heatkv_pair_launches(ses.ctx) > before:
+                        on_pairs.add(step)
                     hk.heatkv_append_compact(ses.ctx, ids, 0, step, ks[step], vs[step], None)
                     torch.cuda.synchronize()
                     if rep >= 2:
                         ms[step] += e0.elapsed_time(e1) / reps
                 hk.heatkv_seq_close(ses.ctx, ids[0])
+            res[name.replace("_ms", "_pair_scales")] = sorted(step + 1 for step in on_pairs)
+            if scratch > 1024:
+                for step in on_pairs:
+                    res["split_tiles_per_scale"][step], res["ctas_per_scale"][step] = 0, 2 * sh.H * -(-sh.t[step] // 256)
             res[name] = [round(float(x), 4) for x in ms]
             res[name.replace("_ms", "_sum_ms")] = round(float(ms.sum()), 4)
             assert hk.heatkv_device_status(ses.ctx) == 0
@@ -810,7 +818,7 @@ def main():
     qs_, ks_, vs_, os_ = layer_bufs[0]
     flush = torch.empty(256 << 20, dtype=torch.uint8, device=dev)
 
-    def sweep(events=None, bufs=None):
+    def sweep(events=None, bufs=None, after_attention=None):
         """One image pair through one layer: 13 x (pre-step eviction, attention, append/compaction)."""
         stream = torch.cuda.current_stream()
         bq, bk, bv, bo = bufs or (qs_, ks_, vs_, os_)
@@ -825,6 +833,8 @@ def main():
                 hk.heatkv_scale_attention(ses.ctx, ids, 0, step, bq[step], bk[step], bv[step], None, bias[0, step], bo[step])
             if events is not None and step in events:
                 events[step][1].record(stream)
+            if after_attention is not None:
+                after_attention()
             if args.calls != "fused":
                 hk.heatkv_append_compact(ses.ctx, ids, 0, step, bk[step], bv[step], None)
         for i in ids:
@@ -897,11 +907,17 @@ def main():
     clocks = sampler.stop()
     per_step_ms = np.array([[ke[kk][0].elapsed_time(ke[kk][1]) for kk in range(shape.K)] for ke in kern_events])
     assert hk.heatkv_device_status(ses.ctx) == 0
-    # how the tensor-memory launches cut their work (host-side report of the library's choice)
+    # how the tensor-memory launches cut their work (host-side report of the library's choice), and which of them ran uncut on CTA
+    # pairs (the library's count, per scale of one more sweep)
+    seen = [hk.heatkv_pair_launches(ses.ctx)]
+    sweep(after_attention=lambda: seen.append(hk.heatkv_pair_launches(ses.ctx)))
+    barrier()
+    on_pairs = np.diff(seen) > 0
     ids_ = [hk.heatkv_seq_open(ses.ctx, sch) for _ in range(n_seq)]
     cuts = [hk.heatkv_attention_split(ses.ctx, ids_, 0, kk) for kk in range(shape.K)]
     for i in ids_:
         hk.heatkv_seq_close(ses.ctx, i)
+    cuts = [(0, n_seq * shape.H * -(-shape.t[kk] // 256)) if on_pairs[kk] else cuts[kk] for kk in range(shape.K)]
 
     # ---- end to end: the same step from pinned host buffers, copies inside the timed region.  Every layer's
     # Q/K/V go up and its output comes down (one pinned set serves all layers: the bytes moved are what counts).
@@ -966,7 +982,9 @@ def main():
     ks1 = hk.heatkv_kernel_launches(ses.ctx)
     if args.kernel != "generic":
         assert ks1.tcgen05_attention_ready == 1 and per_step_kernels["attention_tcgen05"] == N_LAYERS * len(tc_steps), per_step_kernels
-    dominant = ("tc::attn_tc_kernel<%d> (tcgen05.mma, TMEM accumulators, TMA gathers)" % shape.d
+    pair_scales = [kk + 1 for kk in range(shape.K) if on_pairs[kk]]
+    dominant = ("tc::attn_tc_kernel<%d>%s (tcgen05.mma, TMEM accumulators, TMA gathers)"
+                % (shape.d, ", at scales %s pair::attn_pair_kernel<%d>" % (pair_scales, shape.d) if pair_scales else "")
                 if per_step_kernels["attention_tcgen05"] else "attn_generic_kernel<%d> (mma.sync)" % shape.d)
     cache_update = None
     if rank == 0 and world == 1 and args.layout == "paged":
@@ -1003,6 +1021,7 @@ def main():
         "attention_ms_per_scale": [round(float(x), 5) for x in attn_ms],
         "work_items_per_scale": [int(c[1]) for c in cuts],
         "longest_piece_tiles_per_scale": [int(c[0]) for c in cuts],
+        "cta_pair_scales": pair_scales,
         "attention_tflops_per_scale": [round(flops[kk] / (float(attn_ms[kk]) * 1e-3) / 1e12, 1) for kk in range(shape.K)],
         "attention_algorithmic_gb_per_s_per_scale": [round(by[kk] / (float(attn_ms[kk]) * 1e-3) / 1e9, 1) for kk in range(shape.K)],
         "attention_tflops_all_scales": sum(flops) / (float(attn_ms.sum()) * 1e-3) / 1e12,
@@ -1011,7 +1030,7 @@ def main():
                         "call": "heatkv_calibrate_scores_steps (all 13 steps of a batch in one call)",
                         "ms_per_sample_batch_step_calls": calib_ms_step_calls / len(CALIB_SEEDS)},
         "kernels_per_step": per_step_kernels,
-        "roofline": {"bound": "tensor", "kernel": f"{dominant}: its {len(tc_steps)} launches per layer sweep (scales with t_k >= 256), "
+        "roofline": {"bound": "tensor", "kernel": f"{dominant}: {len(tc_steps)} launches per layer sweep (scales with t_k >= 256), "
                                                   f"{per_step_kernels['attention_tcgen05']} per step",
                      "timing": "CUDA events around each launch, call by call, mean over layer sweeps",
                      "achieved": achieved, "peak": pk["bf16_tflops"], "unit": "TFLOP/s",
