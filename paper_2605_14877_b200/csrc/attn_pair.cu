@@ -32,7 +32,9 @@ using namespace tc;
 
 constexpr int THREADS = 384;
 constexpr int STAGES = 4;               // of K and of V
-constexpr int REGS_LAUNCH = 168;        // what ptxas assigns under __launch_bounds__(384, 1)
+// What ptxas assigns under __launch_bounds__(384, 1), for either head size; 44 bytes a thread spilled (11 stores, 32 loads), in all
+// roles together.
+constexpr int REGS_LAUNCH = 168;
 constexpr int REGS_SMALL = 72, REGS_SOFTMAX = 216;
 static_assert(128 * REGS_SMALL + 256 * REGS_SOFTMAX <= THREADS * REGS_LAUNCH, "register hand-over exceeds the CTA's allocation");
 constexpr uint32_t OUT_BYTES = 4096;    // per softmax warp: two buffers of 32 rows x 64 B for the output rows
