@@ -319,8 +319,8 @@ int heatkv_attention_append(heatkv_ctx* ctx, const int* seq_ids /*HOST*/, int n_
  * call mixes schedules).  A cut head's pieces leave partial results in the arena's scratch region, where
  * the last to arrive merges them.  The choice (a piece count per head) minimises an estimate of the launch's
  * makespan over the SMs and is cached per (schedule, step, layer, batch size).  A launch of few and short items (at most one per
- * two SMs, 20 key tiles; of 64-wide heads past 13 tiles only where the cut would take longer) runs uncut on pairs of CTAs
- * instead, so there the figures only say what that saves; heatkv_pair_launches tells.  Host only. */
+ * two SMs, 16 key tiles, of 64-wide heads 12) runs uncut on pairs of CTAs instead, so there the figures only say what that saves;
+ * heatkv_pair_launches tells.  Host only. */
 int heatkv_attention_split(heatkv_ctx* ctx, const int* seq_ids /*HOST*/, int n_seq, int layer, int step,
                            int32_t* split_tiles, int32_t* items);
 

@@ -26,8 +26,6 @@ bool tc_ready(const TcState* st);
 bool tc_supported(const TcState* st, const AttnParams& p, int d, int n_seq);
 cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int n_seq, cudaStream_t stream);
 bool tc_pair_wanted(const TcState* st, int t_q, int64_t items, int tiles);
-bool tc_pair_beats_cut(const TcState* st, int tiles, int run, int cut_items);
-bool tc_pair_sure(const TcState* st, int tiles);
 cudaError_t launch_attn_pair(TcState* st, const AttnParams& p, int n_seq, cudaStream_t stream);
 int tc_split_slot_floats(int d);
 cudaError_t launch_wait_expiry(uint32_t* status, uint32_t* result, cudaStream_t stream);
@@ -360,8 +358,8 @@ void fill_head_table(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, i
   p->table_heads = pe0.sched.H;
 }
 
-// Work items of the call without any cut, if the kernel of CTA pairs can take it; else 0.  *longest = key tiles of its longest head.
-int pair_items(const heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int layer, const AttnParams& p, int* longest) {
+// Work items of the call without any cut, if the kernel of CTA pairs takes it; else 0.  *longest = key tiles of its longest head.
+int pair_items(const heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int layer, const AttnParams& p, int32_t* longest) {
   const int64_t items = (int64_t)n_seq * ctx->cfg.H * ((p.t_q + 255) / 256);
   const int own_slots = (p.n_own + HEATKV_PAGE_TOKENS - 1) / HEATKV_PAGE_TOKENS;
   if (!tc_pair_wanted(ctx->tc, p.t_q, items, 0)) return 0;
@@ -378,9 +376,8 @@ int pair_items(const heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, i
 // Fills the splitting fields of the launch parameters.  When the whole call follows one schedule the choice
 // is a piece count per head: long heads are cut to a common longest run, and the heads dispatched last may be
 // cut further so that the last round of items fills the SMs.  It is cached per (schedule, step, layer, batch
-// size).  Calls that mix schedules use one longest run for all of them.  Returns the longest run of tiles any item takes (0: whole
-// heads of several schedules).
-int choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int layer, AttnParams* p) {
+// size).  Calls that mix schedules use one longest run for all of them.
+void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int layer, AttnParams* p) {
   const int n_qp = (p->t_q + 255) / 256, own_slots = (p->n_own + HEATKV_PAGE_TOKENS - 1) / HEATKV_PAGE_TOKENS;
   const PlanEntry& pe0 = *ctx->plans[ctx->seqs[seq_ids[0]].plan];
   bool one_plan = pe0.sched.H <= 64;
@@ -427,7 +424,6 @@ int choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int l
   // one plan for the whole call (the usual case): its heads, by descending key count, travel in the parameters
   p->table_heads = 0;
   p->longest_piece = 0;
-  int run = one_plan ? 0 : lmax;
   if (one_plan) {
     const PlanHeader& hdr = pe0.plan.header();
     const int32_t* blob = pe0.plan.blob.data();
@@ -440,9 +436,7 @@ int choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int l
       p->table_head[i] = (int16_t)order[i];
       p->table_tiles[i] = (int16_t)tiles[i];
       p->table_split[i] = (int16_t)ch.ns[i];
-      const int piece = (tiles[i] + ch.ns[i] - 1) / ch.ns[i];
-      if (ch.ns[i] > 1) p->longest_piece = std::max(p->longest_piece, piece);
-      run = std::max(run, piece);
+      if (ch.ns[i] > 1) p->longest_piece = std::max(p->longest_piece, (tiles[i] + ch.ns[i] - 1) / ch.ns[i]);
     }
     p->table_heads = H;
   } else {
@@ -455,7 +449,6 @@ int choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int l
   p->ctrs_per_seq = m.ctrs;
   p->split_partials = ctx->split_partials;
   p->split_counters = ctx->split_counters;
-  return run;
 }
 
 }  // namespace
@@ -833,24 +826,22 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
   }
   if (fuse) p.append_tiles = (ctx->cfg.t[step] + HEATKV_PAGE_TOKENS - 1) / HEATKV_PAGE_TOKENS + 1;
   cudaError_t e;
-  int tiles = 0, pairs = use_tc ? pair_items(ctx, seq_ids, n_seq, step, layer, p, &tiles) : 0;
-  if (use_tc && (!pairs || !tc_pair_sure(ctx->tc, tiles))) {
-    try {
-      const int run = choose_split(ctx, seq_ids, n_seq, step, layer, &p);
-      if (pairs && !tc_pair_beats_cut(ctx->tc, tiles, run > 0 ? std::min(run, tiles) : tiles, p.items_per_seq * n_seq)) pairs = 0;
-    } catch (const std::bad_alloc&) {
-      return HEATKV_ERR_HOST_MEMORY;
-    }
-  }
-  if (pairs) {
+  int32_t longest = 0;
+  if (const int items = use_tc ? pair_items(ctx, seq_ids, n_seq, step, layer, p, &longest) : 0) {
     fill_head_table(ctx, seq_ids, n_seq, step, layer, &p);
     p.n_seq = n_seq;
-    p.items_per_seq = pairs / n_seq;
+    p.items_per_seq = items / n_seq;
+    p.longest_piece = longest;
     e = launch_attn_pair(ctx->tc, p, n_seq, stream);
     ctx->launches += 1;
     ctx->kstats.attention_tcgen05 += 1;
     ctx->pair_launches += 1;
   } else if (use_tc) {
+    try {
+      choose_split(ctx, seq_ids, n_seq, step, layer, &p);
+    } catch (const std::bad_alloc&) {
+      return HEATKV_ERR_HOST_MEMORY;
+    }
     e = launch_attn_tc(ctx->tc, p, n_seq, stream);
     ctx->launches += 1;
     ctx->kstats.attention_tcgen05 += 1;

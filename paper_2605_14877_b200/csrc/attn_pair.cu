@@ -365,6 +365,12 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
     // where the issuers are told (CTA 0)
     const uint32_t s_read = in_cta0(bar(S_READ + w)), p_full = in_cta0(bar(P_FULL + 2 * w));
     const bool no_rows = q_row0 + wr * 32 >= p.t_q;     // nothing below the last query: hand on whatever is there
+    // The reference follows the maximum in the first two tiles and in every fourth, where the pieces of a cut head would start, if
+    // attn_tc_kernel would cut any of the launch's heads: a row's largest weight rounds to bf16 without error where it is its reference,
+    // and a cut head has a reference per piece.  Error of the output against 64 bits, of its norm, x 1e-3, cut / on pairs / on pairs
+    // with the first tile's reference throughout: 48 heads x 256 queries, 7 tiles 2.298 / 2.287 / 2.326, 10 tiles
+    // 2.290 / 2.287 / 2.329, 13 tiles 2.308 / 2.300 / 2.336; the same as times: 400 queries x 32 heads, 8 tiles 18.5 / 13.9 / 12.6 us.
+    const bool follows = p.longest_piece >= 2 * SPLIT_MIN_PIECE - 1;
     float m_ref = NO_MAX, l_sum = 0.f;
     int j = w;
     pdl_wait();
@@ -433,7 +439,7 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
         ref = *ref_smem;
       }
       float m_new = fmaxf(ref, mx);
-      const bool grow = m_new > ref + RESCALE_THRESHOLD;       // also true on the first tile (ref = NO_MAX)
+      const bool grow = m_new > ref + (follows && (j < 2 || (j & 3) == 0) ? 0.f : RESCALE_THRESHOLD);   // (true on the first tile: NO_MAX)
       if (!grow) m_new = ref;
       if (grow || j == 0) *ref_smem = m_new;
       __syncwarp();

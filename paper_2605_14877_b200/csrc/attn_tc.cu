@@ -1058,24 +1058,16 @@ bool encode_call(TcState* st, tc::Maps* maps, const AttnParams& p, int n_seq, in
 }  // namespace
 
 // Does a launch of `items` (sequence, head, 256 queries) with at most `tiles` key tiles go to attn_pair_kernel?  Where all its pairs
-// run at once, and not past PAIR_TILES: attn_tc_kernel would cut longer heads into pieces, which pays from there on.  Back
-// to back, attn_tc_kernel against attn_pair_kernel: 32 items, 256 queries 13.0 and 10.0 us; 64 items, 400 queries 19.5 and 14.0;
-// 4 heads x 1024 queries, 16 items of 20 tiles, 27.9 and 24.2; past the lines 4 heads x 1600 queries (28 items of 32 tiles)
-// 30.0 and 36.1, 28 heads x 576 queries (84 items) 25.4 and 35.5.  A tile of 128 queries is left to one CTA.
-constexpr int PAIR_TILES = 20;
+// run at once, and not past the line where attn_tc_kernel's pieces of longer heads are quicker for some number of items (a pair takes
+// 0.8 us per tile and 0.6 more for one where references follow the maximum; a tile of 64-wide heads takes attn_tc_kernel 1.2 us instead
+// of 1.7).  Back to back, attn_tc_kernel against attn_pair_kernel: 32 items of 256 queries and 3 tiles 13.0 and 10.0 us; 64 items, 400
+// queries, 8 tiles 18.5 and 13.9; 256 queries, 16 tiles, 1 item 19.0 and 19.3, 24 items 21.3 and 19.6; 64-wide heads, 12 tiles, 1 item
+// 14.1 and 14.4, 24 items 15.0 and 14.7.  Of 475 launches up to the lines none is more than 2.6 % slower on pairs, those at the lines
+// are 5.7 and 2.1 % faster in the mean; at 20 tiles of 128-wide heads up to 4.9 % slower, 0.9 % faster in the mean; 28 heads x 576
+// queries (84 items) 25.4 and 35.5 us.  A tile of 128 queries is left to one CTA.
 bool tc_pair_wanted(const TcState* st, int t_q, int64_t items, int tiles) {
-  return t_q > tc::BM && items <= st->n_pairs && tiles <= PAIR_TILES;
+  return t_q > tc::BM && items <= st->n_pairs && tiles <= (st->d == 128 ? 16 : 12);
 }
-// ... where attn_tc_kernel would take `cut_items` items of at most `run` tiles instead?  With 128-wide heads in any case.  A pair takes
-// 0.79 us per tile for either width, but a tile of 64-wide heads takes attn_tc_kernel 1.2 us instead of 1.7, a piece more to merge
-// 0.8 and a full GPU 1.8 us more than an empty one.  64-wide heads x 256 queries, attn_tc_kernel against attn_pair_kernel: 1 item of 14
-// tiles 14.8 and 14.6, of 20 tiles (5 pieces) 16.7 and 19.4; 24 items of 15 tiles 16.5 and 15.7, of 20 tiles 18.5 and 19.7; 64 items of 20
-// tiles (2 pieces) 23.6 and 21.3.  Of 568 launches of 1 to 72 items this picks none that is more than 2.5 % slower than the other.
-bool tc_pair_beats_cut(const TcState* st, int tiles, int run, int cut_items) {
-  return st->d == 128 || 64 * tiles <= 96 * run + 64 * ((tiles + run - 1) / run) + 256 + cut_items;
-}
-// Up to here that holds for any cut into pieces of SPLIT_MIN_PIECE tiles and more.
-bool tc_pair_sure(const TcState* st, int tiles) { return st->d == 128 || tiles <= 13; }
 
 cudaError_t launch_attn_pair(TcState* st, const AttnParams& p, int n_seq, cudaStream_t stream) {
   tc::Maps maps;

@@ -46,7 +46,7 @@ struct AttnParams {
   int16_t table_head[64];
   int16_t table_tiles[64];
   int16_t table_split[64];        // pieces the head's key range is cut into (1: whole head)
-  int32_t longest_piece;          // host report: longest piece among the heads that are cut (0: none is)
+  int32_t longest_piece;          // longest piece among the heads that are cut (0: none is; host report); CTA pairs: longest head
   int32_t append_tiles;           // > 0: the launch also stores the step's K/V (paged layout): that many destination
                                   // half-tile slots per (sequence, head) follow the attention work
   // tensor-memory kernel, calibration with an attention output (full_slots > 0): the step's key half-tiles, cut at
