@@ -393,7 +393,11 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
     // This warp's instruction stream is part of every key tile's chain (P handed over -> PV, next S -> softmax), so it is kept
     // short: item words and the TMEM base come through a shuffle and are provably uniform, and the products are predicated on
     // one lane instead of branched around.  Measured: a pair generated at 20x 2.395 -> 2.339 ms of GPU time, the largest
-    // model's batch 7.025 -> 6.763 ms, 64-wide heads unchanged (1.66 ms); one thread running the whole role lost 5 %.
+    // model's batch 7.025 -> 6.763 ms, 64-wide heads unchanged (1.66 ms); one thread running the whole role lost 5 %.  The lane is
+    // elected anew for every tile and the descriptors are a base and a constant: 65 instructions less per tile, 1024 queries x 296
+    // heads x 24 tiles 369.4 -> 363.5 us (64-wide heads 306.7 -> 302.7).  What matters is that the compiler knows the warp to be
+    // converged: where it does not (a `continue` past the __syncwarp at the loop's end, a lane mask that a failed wait may clear) it
+    // branches around every product, 33 branches and 350 instructions more per tile, and the kernel is 6 % slower.
     const uint32_t lead = elect_one();
     constexpr uint32_t IDESC_S = instr_desc(BM, BN, 0, 0);     // Q, K both K-major
     constexpr uint32_t IDESC_PV = instr_desc(BM, D, 0, 1);     // P from TMEM, V MN-major
@@ -403,21 +407,21 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
     auto mma_wait = [&](uint32_t b, uint32_t parity) {
       return D == 64 ? warp_wait_vote(b, parity, abort_flag, p.status) : warp_wait(b, parity, abort_flag, p.status);
     };
-    auto issue_s = [&](int x, int st) {
-      const uint32_t qa = sbase + SM_Q + x * TILE_BYTES, ka = sbase + SM_K + st * TILE_BYTES;
+    const uint32_t q_lo = desc_lo(sbase + SM_Q, 16), k_lo = desc_lo(sbase + SM_K, 16), v_lo = desc_lo(sbase + SM_V, HALF_COLS_BYTES);
+    auto issue_s = [&](uint32_t lead, int x, int st) {
+      const uint32_t qa = q_lo + x * (TILE_BYTES >> 4), ka = k_lo + st * (TILE_BYTES >> 4);
 #pragma unroll
       for (int ks = 0; ks < D / 16; ++ks) {
-        const uint32_t off = (ks >> 2) * HALF_COLS_BYTES + (ks & 3) * 32;
-        mma_ss(lead, tmem + x * 128, smem_desc(qa + off, 16, 1024), smem_desc(ka + off, 16, 1024), IDESC_S, ks > 0);
+        const uint32_t off = ((ks >> 2) * HALF_COLS_BYTES + (ks & 3) * 32) >> 4;
+        mma_ss(lead, tmem + x * 128, qa + off, ka + off, IDESC_S, ks > 0);
       }
     };
     // keys 64h .. 64h+63 of the tile: four K=16 steps
-    auto issue_pv = [&](int x, int st, int h, bool first) {
-      const uint32_t va = sbase + SM_V + st * TILE_BYTES;
+    auto issue_pv = [&](uint32_t lead, int x, int st, int h, bool first) {
+      const uint32_t va = v_lo + st * (TILE_BYTES >> 4);
 #pragma unroll
       for (int ks = 4 * h; ks < 4 * h + 4; ++ks)
-        mma_ts(lead, tmem + 256 + x * 128, tmem + x * 128 + ks * 8, smem_desc(va + ks * 2048, HALF_COLS_BYTES, 1024),
-               IDESC_PV, !(first && ks == 0));
+        mma_ts(lead, tmem + 256 + x * 128, tmem + x * 128 + ks * 8, va + ks * (2048 >> 4), IDESC_PV, !(first && ks == 0));
     };
     uint32_t g = 0;                                    // key tiles consumed so far (all items)
     uint32_t cx[2] = {0, 0};                           // key tiles of query tile x so far
@@ -440,7 +444,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
         if (ok) {
           tc_fence_after();
           for (int x = 0; x < nq; ++x) {
-            issue_s(x, st0);
+            issue_s(lead, x, st0);
             tc_commit(lead, bar(S_FULL + x));
             if (n_tiles == 1) tc_commit(lead, bar(Q_EMPTY + x));
           }
@@ -454,6 +458,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
           const uint32_t st = (g + j) % KV_STAGES, stn = (g + j + 1) % KV_STAGES;
           const uint32_t parn = ((g + j + 1) / KV_STAGES) & 1;
           const bool more = j + 1 < n_tiles;
+          const uint32_t lead = elect_one();
 #pragma unroll
           for (int x = 0; x < 2; ++x) {
             if (x >= nq || !ok) continue;
@@ -461,16 +466,16 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             ok = mma_wait(bar(P_FULL + 2 * x), ph);
             if (!ok) continue;
             tc_fence_after();
-            issue_pv(x, st, 0, j == 0);
+            issue_pv(lead, x, st, 0, j == 0);
             // the next tile's keys are waited for here, off the path between the last half of P and the next S
             if (more && x == 0) ok = mma_wait(bar(K_FULL + stn), parn);
             if (!ok) continue;
             ok = mma_wait(bar(P_FULL + 2 * x + 1), ph);
             if (!ok) continue;
             tc_fence_after();
-            issue_pv(x, st, 1, false);
+            issue_pv(lead, x, st, 1, false);
             if (more) {
-              issue_s(x, stn);
+              issue_s(lead, x, stn);
               tc_commit(lead, bar(S_FULL + x));
               if (j + 2 == n_tiles) tc_commit(lead, bar(Q_EMPTY + x));     // the item's last product that reads Q_x
             } else {

@@ -222,7 +222,7 @@ calib_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Ma
 #pragma unroll
             for (int ks = 0; ks < D / 16; ++ks) {
               const uint32_t off = (ks >> 2) * HALF_COLS_BYTES + (ks & 3) * 32;
-              mma_ss(1u, tmem + x * 128, smem_desc(qa + off, 16, 1024), smem_desc(ka + off, 16, 1024), IDESC_S, ks > 0);
+              mma_ss(1u, tmem + x * 128, desc_lo(qa + off, 16), desc_lo(ka + off, 16), IDESC_S, ks > 0);
             }
             tc_commit(1u, bar(S_FULL + x));
           }
