@@ -320,7 +320,8 @@ int heatkv_attention_append(heatkv_ctx* ctx, const int* seq_ids /*HOST*/, int n_
  * the last to arrive merges them.  The choice (a piece count per head) minimises an estimate of the launch's
  * makespan over the SMs and is cached per (schedule, step, layer, batch size).  A launch of few and short items (at most one per
  * two SMs, 16 key tiles, of 64-wide heads 12) runs uncut on pairs of CTAs instead, so there the figures only say what that saves;
- * heatkv_pair_launches tells.  Host only. */
+ * heatkv_pair_launches tells.  One whose items would leave SMs idle may also take query tiles of 128 one by one, with whole key
+ * ranges, instead of in pairs (its own items are not counted here; heatkv_lone_launches tells).  Host only. */
 int heatkv_attention_split(heatkv_ctx* ctx, const int* seq_ids /*HOST*/, int n_seq, int layer, int step,
                            int32_t* split_tiles, int32_t* items);
 
@@ -365,6 +366,8 @@ int heatkv_launch_count(heatkv_ctx* ctx, uint64_t* n);
 int heatkv_kernel_launches(heatkv_ctx* ctx, heatkv_kernel_stats* out);
 /* How many of the attention_tcgen05 launches ran uncut on pairs of CTAs (attn_pair_kernel; see heatkv_attention_split). */
 int heatkv_pair_launches(heatkv_ctx* ctx, uint64_t* n);
+/* ... and of them those in which some work items are one query tile of 128 instead of two. */
+int heatkv_lone_launches(heatkv_ctx* ctx, uint64_t* n);
 /* Appendix on S-CAS stability -- how much the head ordering moves between calibration sets.  scas_runs HOST
  * [n_runs][L][H][K]: S-CAS of n_runs independent calibration sets (heatkv_finalize_scores).  For every prunable
  * source scale k (s <= k <= K-2, 0-based) each run ranks the L*H heads by ascending S-CAS (ties by ascending

@@ -139,6 +139,7 @@ struct heatkv_ctx {
   uint64_t launches = 0, openings = 0;
   heatkv_kernel_stats kstats = {};             // launches per kernel
   uint64_t pair_launches = 0;                  // of kstats.attention_tcgen05: on pairs of CTAs
+  uint64_t lone_launches = 0;                  // ... with query tiles by themselves
   TcState* tc = nullptr;
   CalibTcState* calib_tc = nullptr;
   // key-range splitting of the tensor-memory attention kernel
@@ -376,8 +377,9 @@ int pair_items(const heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, i
 // Fills the splitting fields of the launch parameters.  When the whole call follows one schedule the choice
 // is a piece count per head: long heads are cut to a common longest run, and the heads dispatched last may be
 // cut further so that the last round of items fills the SMs.  It is cached per (schedule, step, layer, batch
-// size).  Calls that mix schedules use one longest run for all of them.
-void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int layer, AttnParams* p) {
+// size).  Calls that mix schedules use one longest run for all of them.  Where it is quicker the launch takes query tiles one by one
+// instead of cutting anything (unless `cuts_only`).
+void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int layer, bool cuts_only, AttnParams* p) {
   const int n_qp = (p->t_q + 255) / 256, own_slots = (p->n_own + HEATKV_PAGE_TOKENS - 1) / HEATKV_PAGE_TOKENS;
   const PlanEntry& pe0 = *ctx->plans[ctx->seqs[seq_ids[0]].plan];
   bool one_plan = pe0.sched.H <= 64;
@@ -392,12 +394,17 @@ void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int 
            (uint64_t)sh.ctrs * n_seq * SPLIT_CTRS_PER_GROUP <= ctx->split_ctrs;
   };
   auto it = ctx->split_choice.find(key);
-  if (it == ctx->split_choice.end())
-    it = ctx->split_choice.emplace(key, split_search(tiles, n_qp, n_seq, ctx->n_sm, one_plan, ctx->split_slots,
-                                                     ctx->split_ctrs)).first;
+  if (it == ctx->split_choice.end()) {
+    SplitChoice made = split_search(tiles, n_qp, n_seq, ctx->n_sm, one_plan, ctx->split_slots, ctx->split_ctrs);
+    single_search(tiles, p->t_q, n_seq, ctx->n_sm, one_plan, &made);
+    it = ctx->split_choice.emplace(key, std::move(made)).first;
+  }
   const SplitChoice& ch = it->second;
-  SplitShape m = split_shape(tiles, ch.ns, n_qp);
-  int lmax = ch.lmax > 0 ? ch.lmax : 0;
+  const bool lone = !cuts_only && !ch.lone.empty(), all_lone = lone && ch.lone[0] == 0 && ch.lone[H - 1] == 0;
+  const std::vector<int>& pieces = lone ? ch.lone : ch.ns;
+  const int n_qt = (p->t_q + 127) / 128;
+  SplitShape m = split_shape(tiles, pieces, n_qp, n_qt);
+  int lmax = !lone && ch.lmax > 0 ? ch.lmax : 0;
   if (!one_plan) {
     // other schedules in the batch follow the same longest run; the per-sequence bounds cover all of them
     auto bounds = [&](int lm) {
@@ -409,8 +416,8 @@ void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int 
         last_plan = pi;
         const std::vector<int> t = ordered_tiles(*ctx->plans[pi], step, layer, own_slots, p->runs);
         std::vector<int> ns(t.size());
-        for (size_t k = 0; k < t.size(); ++k) ns[k] = split_pieces_for(t[k], lm);
-        const SplitShape sh = split_shape(t, ns, n_qp);
+        for (size_t k = 0; k < t.size(); ++k) ns[k] = all_lone ? 0 : split_pieces_for(t[k], lm);
+        const SplitShape sh = split_shape(t, ns, n_qp, n_qt);
         b.items = std::max(b.items, sh.items); b.slots = std::max(b.slots, sh.slots); b.ctrs = std::max(b.ctrs, sh.ctrs);
       }
       return b;
@@ -435,8 +442,8 @@ void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int 
       p->table_desc_begin[i] = tab.desc + (p->runs ? pe0.run_shift : 0) + 2 * begin[order[i]];
       p->table_head[i] = (int16_t)order[i];
       p->table_tiles[i] = (int16_t)tiles[i];
-      p->table_split[i] = (int16_t)ch.ns[i];
-      if (ch.ns[i] > 1) p->longest_piece = std::max(p->longest_piece, (tiles[i] + ch.ns[i] - 1) / ch.ns[i]);
+      p->table_split[i] = (int16_t)pieces[i];
+      if (pieces[i] > 1) p->longest_piece = std::max(p->longest_piece, (tiles[i] + pieces[i] - 1) / pieces[i]);
     }
     p->table_heads = H;
   } else {
@@ -445,6 +452,7 @@ void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int 
   p->n_seq = n_seq;
   p->split_tiles = lmax;
   p->items_per_seq = m.items;
+  p->lone = !lone ? 0 : one_plan || !all_lone ? 1 : 2;
   p->slots_per_seq = m.slots;
   p->ctrs_per_seq = m.ctrs;
   p->split_partials = ctx->split_partials;
@@ -838,13 +846,14 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
     ctx->pair_launches += 1;
   } else if (use_tc) {
     try {
-      choose_split(ctx, seq_ids, n_seq, step, layer, &p);
+      choose_split(ctx, seq_ids, n_seq, step, layer, false, &p);
     } catch (const std::bad_alloc&) {
       return HEATKV_ERR_HOST_MEMORY;
     }
     e = launch_attn_tc(ctx->tc, p, n_seq, stream);
     ctx->launches += 1;
     ctx->kstats.attention_tcgen05 += 1;
+    ctx->lone_launches += p.lone != 0;
   } else {
     fill_head_table(ctx, seq_ids, n_seq, step, layer, &p);
     e = launch_attn_generic(p, ctx->cfg.d, n_seq, false, ctx->n_sm, stream);
@@ -883,7 +892,7 @@ int heatkv_attention_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int l
   p.t_q = p.n_own = ctx->cfg.t[step];
   p.runs = all_have_runs(ctx, seq_ids, n_seq);                  // (a call without a per-scale bias)
   try {
-    choose_split(ctx, seq_ids, n_seq, step, layer, &p);
+    choose_split(ctx, seq_ids, n_seq, step, layer, true, &p);
   } catch (const std::bad_alloc&) {
     return HEATKV_ERR_HOST_MEMORY;
   }
@@ -1347,6 +1356,12 @@ int heatkv_kernel_launches(heatkv_ctx* ctx, heatkv_kernel_stats* out) {
 int heatkv_pair_launches(heatkv_ctx* ctx, uint64_t* n) {
   if (!ctx || !n) return HEATKV_ERR_INVALID_ARG;
   *n = ctx->pair_launches;
+  return HEATKV_OK;
+}
+
+int heatkv_lone_launches(heatkv_ctx* ctx, uint64_t* n) {
+  if (!ctx || !n) return HEATKV_ERR_INVALID_ARG;
+  *n = ctx->lone_launches;
   return HEATKV_OK;
 }
 

@@ -22,7 +22,9 @@
 // The MMA order S_A S_B (PV_A S_A' PV_B S_B')* lets the softmax of one tile overlap the
 // tensor work of the other.  The host may cut a head's key range into pieces (a count per head); their
 // unnormalised results meet in a scratch region, where, for every group of 32 rows, the warp that arrives
-// last adds them up in piece order.  All barrier phases run on across items.  Every wait is bounded; on expiry the
+// last adds them up in piece order.  An item may also be a single query tile (the host's choice for launches that leave SMs idle, and the
+// odd last tile of a head beside those): then A and B are its even and its odd key tiles, so that one's softmax runs under the
+// other's products as it does for two query tiles, and the two results meet in the CTA.  All barrier phases run on across items.  Every wait is bounded; on expiry the
 // CTA records a status word, drains its own copies and leaves.
 #include <algorithm>
 
@@ -76,7 +78,8 @@ enum Bar : uint32_t {
   P_FULL = 14,                  // +2x+h  half h (keys 64h..64h+63) of P_x of the tile is in TMEM (128 arrivals)
   PV_DONE = 18,                 // +x  O_x includes the item's last tile (one completion per item)
   ITEM_FULL = 20, ITEM_EMPTY = 22,  // +ring entry; EMPTY takes one arrival from the MMA warp and each softmax warp
-  N_BARS = 24
+  MEET = 24,                    // +w  the two softmax warps of 32 rows in an item of one query tile: two phases per item
+  N_BARS = 28
 };
 constexpr uint32_t BAR_TMEM_PTR = N_BARS * 8;                  // offsets inside the barrier region
 constexpr uint32_t BAR_ABORT = BAR_TMEM_PTR + 4;
@@ -92,18 +95,21 @@ constexpr int FOLLOW_TILES = 24;
 enum ItemKind : int { ATTENTION = 0, STOP = 2, NOTHING = 3 };
 // ring entry words
 enum ItemWord : int { W_KIND = 0, W_HEAD, W_SEQ, W_TILES, W_NSPLIT, W_SUB, W_SLOT, W_CTR, W_DESC, W_NDESC };
+
 constexpr int WORK_COUNTER_WORD = 16;                          // word of the status region that hands out the attention items
 
 
 // What every role derives from a ring entry of kind ATTENTION.
 struct Item {
   int head, seq, n_split, sub, piece, qp, q0, nq, j0, n_tiles, slot_base, ctr_base, n_desc, n_slots, desc_begin;
+  // One query tile, its key tiles taken by the two softmax warpgroups in turn (S_A, O_A: tiles 0, 2, ..; S_B, O_B: 1, 3, ..)
+  bool shared;
 };
 // (the shuffle makes a word provably warp-uniform)
 __device__ __forceinline__ int ring_word(const volatile int32_t* ring, int word) {
   return __shfl_sync(0xffffffffu, ring[word], 0);
 }
-template <bool FULL>
+template <bool FULL, bool LONE>
 __device__ __forceinline__ Item read_item(const volatile int32_t* ring, const AttnParams& p, int n_qp) {
   Item it;
   it.head = ring_word(ring, W_HEAD);
@@ -115,10 +121,12 @@ __device__ __forceinline__ Item read_item(const volatile int32_t* ring, const At
   it.desc_begin = ring_word(ring, W_DESC);
   it.n_desc = ring_word(ring, W_NDESC);
   const int tiles = ring_word(ring, W_TILES);
-  it.piece = it.sub / n_qp;
-  it.qp = it.sub % n_qp;
-  it.q0 = it.qp * (2 * BM);
-  it.nq = (it.q0 + BM < p.t_q) ? 2 : 1;             // does tile B hold any query?
+  const bool one = LONE && it.n_split == 0;         // the head's items are single query tiles
+  it.piece = LONE ? 0 : it.sub / n_qp;
+  it.qp = LONE ? it.sub : it.sub % n_qp;
+  it.q0 = it.qp * (one ? BM : 2 * BM);
+  it.nq = (!one && it.q0 + BM < p.t_q) ? 2 : 1;     // does tile B hold any query?
+  it.shared = LONE && it.nq == 1;
   if (FULL) {                                       // one query tile of the pair (W_SLOT: 0 both, 1 the first, 2 the second)
     const int single = ring_word(ring, W_SLOT);
     if (single > 0) it.nq = 1;
@@ -126,18 +134,23 @@ __device__ __forceinline__ Item read_item(const volatile int32_t* ring, const At
   }
   it.n_slots = FULL ? it.n_desc : it.n_desc + (p.n_own + HALF - 1) / HALF;
   // this item's run of key tiles: [j0, j0 + n_tiles) of the head's ceil(n_slots / 2)
-  const int piece_tiles = (tiles + it.n_split - 1) / it.n_split;
+  const int piece_tiles = LONE ? tiles : (tiles + it.n_split - 1) / it.n_split;
   it.j0 = it.piece * piece_tiles;
   it.n_tiles = min(tiles, it.j0 + piece_tiles) - it.j0;
   return it;
 }
 
+// LONE: some of the launch's items are a single query tile, none is a piece of a head.  An instantiation of its own, because
+// each way of ending an item costs the others: with the pieces' code beside it a launch took 1.5 us more (from the second
+// kind of item in a launch on, the instruction caches hold neither), and one kernel for everything 0.3 to 1.5 us more everywhere.
+// What bounds such an item is what bounds a pair: 28 heads x 576 queries, 0.80 us per key tile where a pair takes 1.52; filled SMs
+// 1.02 and 1.83.  Keys come one tile ahead of the values here, a step is half as long (in the pair's order 1.35 us).
 // FULL: heatkv_calibrate_scores with an attention output.  The softmax warps also keep, for every query row, the
 // probability mass of each source scale (a half-tile lies inside one scale; finished scales are parked in the warp's
 // output staging buffer) and add the step's row of beta (Eq. 2) at the end of the item.  The masses are fp32 results, so all
 // exponentials are ex2's here: with one pair in four from the cubic beta was off by 3.8e-7 on average (13 scales, against 64
 // bits), with none by 1.0e-7 (warp-level kernel 1.3e-7), for 1 % of the time.
-template <int D, bool FULL>
+template <int D, bool FULL, bool LONE>
 __global__ void __launch_bounds__(THREADS, 1)
 attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Maps maps) {
   using L = Layout<D>;
@@ -177,6 +190,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
       mbar_init(bar(ITEM_FULL + x), 1);
       mbar_init(bar(ITEM_EMPTY + x), 9);
     }
+    for (int w = 0; w < 4; ++w) mbar_init(bar(MEET + w), 2);
     for (int s = 0; s < KV_STAGES; ++s) {
       mbar_init(bar(K_FULL + s), 1);
       mbar_init(bar(K_EMPTY + s), 1);
@@ -274,9 +288,9 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             } else {
               h = pv.order()[u + i];
               tiles = (pv.attn_cnt(p.runs)[u + h] + own_slots + 1) >> 1;
-              ns = p.split_tiles > 0 ? (tiles + p.split_tiles - 1) / p.split_tiles : 1;
+              ns = LONE && p.lone == 2 ? 0 : p.split_tiles > 0 ? (tiles + p.split_tiles - 1) / p.split_tiles : 1;
             }
-            cnt = n_qp * ns;
+            cnt = ns > 0 ? n_qp * ns : (p.t_q + BM - 1) / BM;   // 0: the head's query tiles one by one
           }
           const int scnt = ns > 1 ? cnt : 0, ccnt = ns > 1 ? n_qp : 0;
           int inc = cnt, sinc = scnt, cinc = ccnt;
@@ -293,7 +307,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             ring[W_SEQ] = seq;
             ring[W_TILES] = tiles;
             ring[W_NSPLIT] = ns;
-            ring[W_SUB] = item - excl;                        // piece * n_qp + query tile pair
+            ring[W_SUB] = item - excl;                        // piece * n_qp + query tile pair, or (no pieces) query tile
             ring[W_SLOT] = slots_before + sinc - scnt;        // first partial slot of this head
             ring[W_CTR] = ctrs_before + cinc - ccnt;          // first arrival counter group of this head
             ring[W_DESC] = p.table_heads > 0 ? p.table_desc_begin[i] : pv.w[p.runs ? 18 : 4] + 2 * pv.attn_begin(p.runs)[u + h];
@@ -310,7 +324,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
       }
       const bool is_attn = ring_word(ring, W_KIND) == ATTENTION;
       Item im;
-      if (is_attn) im = read_item<FULL>(ring, p, n_qp);
+      if (is_attn) im = read_item<FULL, LONE>(ring, p, n_qp);
       __syncwarp();
       if (leader) mbar_arrive(bar(ITEM_FULL + slot));
       if (!is_attn) continue;
@@ -318,63 +332,132 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
       const int64_t base_row = FULL ? 0 : p.seqs[seq].base_row;
       const int q_head = im.head & p.q_head_mask, q_seq = seq & p.q_seq_mask;
       const int kv_head = im.head & p.kv_head_mask, kv_seq = seq & p.kv_seq_mask;
-      for (int j = 0; j < im.n_tiles && ok; ++j, ++g) {
-        const uint32_t st = g % KV_STAGES;
-        const uint32_t use = g / KV_STAGES;
-        Slot sl[2];
-        for (int hf = 0; hf < 2; ++hf)
-          sl[hf] = get_slot<FULL>(2 * (im.j0 + j) + hf, descs, im.n_desc, im.n_slots, base_row, p.n_own, p.step);
-        // the first item is decoded and its descriptors are read while the launch before may still run
-        if (g == 0) pdl_wait();
-        // K first: the S product of the next tile needs it earliest
-        if (use > 0) ok = warp_wait(bar(K_EMPTY + st), (use - 1) & 1, abort_flag, p.status);
-        if (!ok) break;
-        armed_k |= 1u << st;
-        par_k = (par_k & ~(1u << st)) | ((use & 1) << st);
-        if (leader) {
-          mbar_expect_tx(bar(K_FULL + st), TILE_BYTES);
+      if (LONE && im.shared) {
+        // Pool rows of 32 half-tiles at a time, one per lane (a look-up per tile would be a chain of its own).
+        const int first_slot = 2 * im.j0;
+        int rows = 0, rows_at = -32;
+        auto half_tile = [&](int i) {
+          if (i >= rows_at + 32) {
+            rows_at = i;
+            rows = get_slot<FULL>(first_slot + i + lane, descs, im.n_desc, im.n_slots, base_row, p.n_own, p.step).pool_row;
+          }
+          return __shfl_sync(0xffffffffu, rows, i - rows_at);
+        };
+        auto load = [&](uint32_t smem, const CUtensorMap* pool, const CUtensorMap* own, int row0, int row1, uint32_t full) {
+          if (!leader) return;
+          mbar_expect_tx(full, TILE_BYTES);
           for (int hf = 0; hf < 2; ++hf)
             for (int ch = 0; ch < NCH; ++ch) {
-              uint32_t dst = sbase + SM_K + st * TILE_BYTES + ch * HALF_COLS_BYTES + hf * SLOT_BYTES;
-              if (sl[hf].pool_row >= 0) tma_load_2d(dst, &maps.k_pool, ch * 64, sl[hf].pool_row, bar(K_FULL + st));
-              else tma_load_4d(dst, &maps.k_own, ch * 64, -sl[hf].pool_row - 1, kv_head, kv_seq, bar(K_FULL + st));
+              const int row = hf == 0 ? row0 : row1;
+              const uint32_t dst = smem + ch * HALF_COLS_BYTES + hf * SLOT_BYTES;
+              if (row >= 0) tma_load_2d(dst, pool, ch * 64, row, full);
+              else tma_load_4d(dst, own, ch * 64, -row - 1, kv_head, kv_seq, full);
             }
-        }
-        if (j == 0) {
-          // the item's query tiles, once the last S product of the previous item has read the old ones
-#pragma unroll
-          for (int x = 0; x < 2; ++x) {
-            if (x >= im.nq || !ok) continue;
-            if (iq[x] > 0) ok = warp_wait(bar(Q_EMPTY + x), (iq[x] - 1) & 1, abort_flag, p.status);
-            if (!ok) continue;
-            armed_q |= 1u << x;
-            par_q = (par_q & ~(1u << x)) | ((iq[x] & 1) << x);
-            ++iq[x];
+        };
+        auto load_k = [&](uint32_t t, int row0, int row1) {             // t: key tiles before it, over all items
+          const uint32_t st = t % KV_STAGES, use = t / KV_STAGES;
+          if (use > 0) ok = warp_wait(bar(K_EMPTY + st), (use - 1) & 1, abort_flag, p.status);
+          if (!ok) return;
+          armed_k |= 1u << st;
+          par_k = (par_k & ~(1u << st)) | ((use & 1) << st);
+          load(sbase + SM_K + st * TILE_BYTES, &maps.k_pool, &maps.k_own, row0, row1, bar(K_FULL + st));
+        };
+        int next0 = 0, next1 = 0;                                       // half-tiles of the tile whose keys came ahead
+        for (int j = 0; j < im.n_tiles && ok; ++j, ++g) {
+          const int row0 = j > 0 ? next0 : half_tile(0), row1 = j > 0 ? next1 : half_tile(1);
+          // the first item is decoded and its descriptors are read while the launch before may still run
+          if (g == 0) pdl_wait();
+          // K first: the S product of the next tile needs it earliest
+          if (j == 0) load_k(g, row0, row1);
+          if (!ok) break;
+          if (j == 0) {
+            if (iq[0] > 0) ok = warp_wait(bar(Q_EMPTY), (iq[0] - 1) & 1, abort_flag, p.status);
+            if (!ok) break;
+            armed_q |= 1u;
+            par_q = (par_q & ~1u) | (iq[0] & 1);
+            ++iq[0];
             if (leader) {
-              mbar_expect_tx(bar(Q_FULL + x), TILE_BYTES);
+              mbar_expect_tx(bar(Q_FULL), TILE_BYTES);
               for (int ch = 0; ch < NCH; ++ch)
                 for (int hf = 0; hf < 2; ++hf)
-                  tma_load_4d(sbase + SM_Q + x * TILE_BYTES + ch * HALF_COLS_BYTES + hf * SLOT_BYTES, &maps.q, ch * 64,
-                              im.q0 + x * BM + hf * HALF, q_head, q_seq, bar(Q_FULL + x));
+                  tma_load_4d(sbase + SM_Q + ch * HALF_COLS_BYTES + hf * SLOT_BYTES, &maps.q, ch * 64, im.q0 + hf * HALF, q_head, q_seq,
+                              bar(Q_FULL));
             }
           }
+          if (j + 1 < im.n_tiles) {             // the step is half as long: the next keys do not wait behind these values
+            next0 = half_tile(2 * j + 2);
+            next1 = half_tile(2 * j + 3);
+            load_k(g + 1, next0, next1);
+            if (!ok) break;
+          }
+          const uint32_t st = g % KV_STAGES, use = g / KV_STAGES;
+          if (use > 0) ok = warp_wait(bar(V_EMPTY + st), (use - 1) & 1, abort_flag, p.status);
           if (!ok) break;
+          armed_v |= 1u << st;
+          par_v = (par_v & ~(1u << st)) | ((use & 1) << st);
+          load(sbase + SM_V + st * TILE_BYTES, &maps.v_pool, &maps.v_own, row0, row1, bar(V_FULL + st));
+          __syncwarp();
         }
-        if (use > 0) ok = warp_wait(bar(V_EMPTY + st), (use - 1) & 1, abort_flag, p.status);
-        if (!ok) break;
-        armed_v |= 1u << st;
-        par_v = (par_v & ~(1u << st)) | ((use & 1) << st);
-        if (leader) {
-          mbar_expect_tx(bar(V_FULL + st), TILE_BYTES);
+      } else {
+        for (int j = 0; j < im.n_tiles && ok; ++j, ++g) {
+          const uint32_t st = g % KV_STAGES;
+          const uint32_t use = g / KV_STAGES;
+          Slot sl[2];
           for (int hf = 0; hf < 2; ++hf)
-            for (int ch = 0; ch < NCH; ++ch) {
-              uint32_t dst = sbase + SM_V + st * TILE_BYTES + ch * HALF_COLS_BYTES + hf * SLOT_BYTES;
-              if (sl[hf].pool_row >= 0) tma_load_2d(dst, &maps.v_pool, ch * 64, sl[hf].pool_row, bar(V_FULL + st));
-              else tma_load_4d(dst, &maps.v_own, ch * 64, -sl[hf].pool_row - 1, kv_head, kv_seq, bar(V_FULL + st));
+            sl[hf] = get_slot<FULL>(2 * (im.j0 + j) + hf, descs, im.n_desc, im.n_slots, base_row, p.n_own, p.step);
+          // the first item is decoded and its descriptors are read while the launch before may still run
+          if (g == 0) pdl_wait();
+          // K first: the S product of the next tile needs it earliest
+          if (use > 0) ok = warp_wait(bar(K_EMPTY + st), (use - 1) & 1, abort_flag, p.status);
+          if (!ok) break;
+          armed_k |= 1u << st;
+          par_k = (par_k & ~(1u << st)) | ((use & 1) << st);
+          if (leader) {
+            mbar_expect_tx(bar(K_FULL + st), TILE_BYTES);
+            for (int hf = 0; hf < 2; ++hf)
+              for (int ch = 0; ch < NCH; ++ch) {
+                uint32_t dst = sbase + SM_K + st * TILE_BYTES + ch * HALF_COLS_BYTES + hf * SLOT_BYTES;
+                if (sl[hf].pool_row >= 0) tma_load_2d(dst, &maps.k_pool, ch * 64, sl[hf].pool_row, bar(K_FULL + st));
+                else tma_load_4d(dst, &maps.k_own, ch * 64, -sl[hf].pool_row - 1, kv_head, kv_seq, bar(K_FULL + st));
+              }
+          }
+          if (j == 0) {
+            // the item's query tiles, once the last S product of the previous item has read the old ones
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+              if (x >= im.nq || !ok) continue;
+              if (iq[x] > 0) ok = warp_wait(bar(Q_EMPTY + x), (iq[x] - 1) & 1, abort_flag, p.status);
+              if (!ok) continue;
+              armed_q |= 1u << x;
+              par_q = (par_q & ~(1u << x)) | ((iq[x] & 1) << x);
+              ++iq[x];
+              if (leader) {
+                mbar_expect_tx(bar(Q_FULL + x), TILE_BYTES);
+                for (int ch = 0; ch < NCH; ++ch)
+                  for (int hf = 0; hf < 2; ++hf)
+                    tma_load_4d(sbase + SM_Q + x * TILE_BYTES + ch * HALF_COLS_BYTES + hf * SLOT_BYTES, &maps.q, ch * 64,
+                                im.q0 + x * BM + hf * HALF, q_head, q_seq, bar(Q_FULL + x));
+              }
             }
+            if (!ok) break;
+          }
+          if (use > 0) ok = warp_wait(bar(V_EMPTY + st), (use - 1) & 1, abort_flag, p.status);
+          if (!ok) break;
+          armed_v |= 1u << st;
+          par_v = (par_v & ~(1u << st)) | ((use & 1) << st);
+          if (leader) {
+            mbar_expect_tx(bar(V_FULL + st), TILE_BYTES);
+            for (int hf = 0; hf < 2; ++hf)
+              for (int ch = 0; ch < NCH; ++ch) {
+                uint32_t dst = sbase + SM_V + st * TILE_BYTES + ch * HALF_COLS_BYTES + hf * SLOT_BYTES;
+                if (sl[hf].pool_row >= 0) tma_load_2d(dst, &maps.v_pool, ch * 64, sl[hf].pool_row, bar(V_FULL + st));
+                else tma_load_4d(dst, &maps.v_own, ch * 64, -sl[hf].pool_row - 1, kv_head, kv_seq, bar(V_FULL + st));
+              }
+          }
+          __syncwarp();
         }
-        __syncwarp();
       }
+      __syncwarp();
     }
     if (!ok || *abort_flag) {
       // leaving early: let every copy this warp started land before the CTA exits
@@ -408,8 +491,8 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
       return D == 64 ? warp_wait_vote(b, parity, abort_flag, p.status) : warp_wait(b, parity, abort_flag, p.status);
     };
     const uint32_t q_lo = desc_lo(sbase + SM_Q, 16), k_lo = desc_lo(sbase + SM_K, 16), v_lo = desc_lo(sbase + SM_V, HALF_COLS_BYTES);
-    auto issue_s = [&](uint32_t lead, int x, int st) {
-      const uint32_t qa = q_lo + x * (TILE_BYTES >> 4), ka = k_lo + st * (TILE_BYTES >> 4);
+    auto issue_s = [&](uint32_t lead, int qx, int x, int st) {                // S_x = Q_qx K^T
+      const uint32_t qa = q_lo + qx * (TILE_BYTES >> 4), ka = k_lo + st * (TILE_BYTES >> 4);
 #pragma unroll
       for (int ks = 0; ks < D / 16; ++ks) {
         const uint32_t off = ((ks >> 2) * HALF_COLS_BYTES + (ks & 3) * 32) >> 4;
@@ -434,9 +517,56 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
       const int kind = ring_word(ring, W_KIND);
       if (kind == STOP) break;
       if (kind == ATTENTION) {
-        const Item im = read_item<FULL>(ring, p, n_qp);
+        const Item im = read_item<FULL, LONE>(ring, p, n_qp);
         const int nq = im.nq, n_tiles = im.n_tiles;
         const uint32_t st0 = g % KV_STAGES, par0 = (g / KV_STAGES) & 1;
+        if (LONE && im.shared) {
+          // One query tile: key tile t goes through S, P and O number t & 1, so that the softmax of one tile overlaps the
+          // products of the next as it does with two query tiles.
+          static_assert(KV_STAGES == 2, "tile t + 2 takes the stage of tile t");
+          ok = mma_wait(bar(Q_FULL), iq[0] & 1);
+          for (int t = 0; t < min(n_tiles, 2) && ok; ++t) {
+            const uint32_t st = (g + t) % KV_STAGES;
+            ok = mma_wait(bar(K_FULL + st), ((g + t) / KV_STAGES) & 1);
+            if (!ok) break;
+            tc_fence_after();
+            issue_s(lead, 0, t, st);
+            tc_commit(lead, bar(S_FULL + t));
+            tc_commit(lead, bar(K_EMPTY + st));
+            if (t + 1 == n_tiles) tc_commit(lead, bar(Q_EMPTY));
+          }
+#pragma unroll 1
+          for (int t = 0; t < n_tiles && ok; ++t) {
+            const uint32_t x = t & 1, st = (g + t) % KV_STAGES, par = ((g + t) / KV_STAGES) & 1;
+            const uint32_t ph = ((x ? cx[1] : cx[0]) + (t >> 1)) & 1;
+            const bool more = t + 2 < n_tiles;
+            ok = mma_wait(bar(V_FULL + st), par);
+            if (ok) ok = mma_wait(bar(P_FULL + 2 * x), ph);
+            if (!ok) break;
+            tc_fence_after();
+            issue_pv(lead, x, st, 0, t < 2);
+            if (more) ok = mma_wait(bar(K_FULL + st), par ^ 1);
+            if (ok) ok = mma_wait(bar(P_FULL + 2 * x + 1), ph);
+            if (!ok) break;
+            tc_fence_after();
+            issue_pv(lead, x, st, 1, false);
+            tc_commit(lead, bar(V_EMPTY + st));
+            if (more) {
+              issue_s(lead, 0, x, st);
+              tc_commit(lead, bar(S_FULL + x));
+              tc_commit(lead, bar(K_EMPTY + st));
+              if (t + 3 == n_tiles) tc_commit(lead, bar(Q_EMPTY));
+            }
+          }
+          if (ok) {
+            tc_commit(lead, bar(PV_DONE));
+            tc_commit(lead, bar(PV_DONE + 1));
+          }
+          g += n_tiles;
+          cx[0] += (n_tiles + 1) >> 1;
+          cx[1] += n_tiles >> 1;
+          ++iq[0];
+        } else {
 #pragma unroll
         for (int x = 0; x < 2; ++x)
           if (x < nq && ok) ok = mma_wait(bar(Q_FULL + x), iq[x] & 1);
@@ -444,7 +574,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
         if (ok) {
           tc_fence_after();
           for (int x = 0; x < nq; ++x) {
-            issue_s(lead, x, st0);
+            issue_s(lead, x, x, st0);
             tc_commit(lead, bar(S_FULL + x));
             if (n_tiles == 1) tc_commit(lead, bar(Q_EMPTY + x));
           }
@@ -475,7 +605,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             tc_fence_after();
             issue_pv(lead, x, st, 1, false);
             if (more) {
-              issue_s(lead, x, stn);
+              issue_s(lead, x, x, stn);
               tc_commit(lead, bar(S_FULL + x));
               if (j + 2 == n_tiles) tc_commit(lead, bar(Q_EMPTY + x));     // the item's last product that reads Q_x
             } else {
@@ -495,6 +625,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             cx[x] += n_tiles;
             ++iq[x];
           }
+        }
       }
       __syncwarp();
       if (ok && lead) mbar_arrive(bar(ITEM_EMPTY + slot));
@@ -530,17 +661,18 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
         // Only what the tile loop needs stays in registers; the epilogue reads the ring entry again.
         int n_tiles, nq;
         {
-          const Item im = read_item<FULL>(ring, p, n_qp);
-          n_tiles = im.n_tiles;
-          nq = im.nq;
+          const Item im = read_item<FULL, LONE>(ring, p, n_qp);
+          n_tiles = im.shared ? (im.n_tiles + 1 - x) >> 1 : im.n_tiles;      // those this warpgroup takes
+          nq = im.shared ? 2 : im.nq;
         }
         if (x < nq) {
-          int j0, n_desc, n_slots, q0;
+          int j0, n_desc, n_slots, q0, stride;
           const int2* descs;
           const float* bias_h;
           {
-            const Item im = read_item<FULL>(ring, p, n_qp);
-            j0 = im.j0; n_desc = im.n_desc; n_slots = im.n_slots; q0 = im.q0;
+            const Item im = read_item<FULL, LONE>(ring, p, n_qp);
+            stride = im.shared ? 2 : 1;
+            j0 = im.shared ? x : im.j0; n_desc = im.n_desc; n_slots = im.n_slots; q0 = im.q0;
             descs = FULL ? p.full_descs : reinterpret_cast<const int2*>(p.seqs[im.seq].plan + im.desc_begin);
             bias_h = p.seg_bias ? p.seg_bias + im.head * p.K : nullptr;
           }
@@ -562,8 +694,9 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
           }
           for (; j < n_tiles && ok; ++j) {
             const uint32_t ph = (cx + j) & 1;
-            Slot s0 = get_slot<FULL>(2 * (j0 + j), descs, n_desc, n_slots, 0, p.n_own, p.step);       // row numbers unused here
-            Slot s1 = get_slot<FULL>(2 * (j0 + j) + 1, descs, n_desc, n_slots, 0, p.n_own, p.step);
+            Slot s0 = get_slot<FULL>(2 * j0, descs, n_desc, n_slots, 0, p.n_own, p.step);       // row numbers unused here
+            Slot s1 = get_slot<FULL>(2 * j0 + 1, descs, n_desc, n_slots, 0, p.n_own, p.step);
+            j0 += LONE ? stride : 1;
             const float b0 = bias_h ? bias_h[s0.seg] * LOG2E : 0.f;
             const float b1 = bias_h ? bias_h[s1.seg] * LOG2E : 0.f;
             ok = __all_sync(0xffffffffu, mbar_wait(bar(S_FULL + x), ph, abort_flag, p.status));
@@ -733,9 +866,9 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
           if (ok) ok = __all_sync(0xffffffffu, mbar_wait(bar(PV_DONE + x), items_x & 1, abort_flag, p.status));
           ++items_x;
           cx += n_tiles;
-          const Item im = read_item<FULL>(ring, p, n_qp);
+          const Item im = read_item<FULL, LONE>(ring, p, n_qp);
           const int seq = im.seq;
-          const int q_row0 = im.q0 + x * BM;
+          const int q_row0 = im.shared ? im.q0 : im.q0 + x * BM;
           if (FULL && ok && !no_rows) {
             // Eq. 2: mean over the step's rows of mass(row, scale) / rowsum(row); rows past t_q are padding
             const float inv_t = 1.f / (float)p.t_q;
@@ -757,9 +890,9 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
           // A warp without a row below the last query writes nothing, the buffer included: its last store may still be reading one
           // half, and only a store of its own for every group would make the wait for all but the newest one cover that half.
           const bool any_row = q_row0 + (warp & 3) * 32 < p.t_q;
-          auto store_rows = [&](const float (&acc)[32], float inv, int c) {
+          auto store_rows = [&](const float (&acc)[32], float inv, int c, int half) {
             if (!any_row) return;
-            unsigned char* buf = stage + (c & 1) * 2048;
+            unsigned char* buf = stage + half * 2048;
             if (lane == 0) bulk_wait_read<1>();                 // the store before the last has read this half
             __syncwarp();
 #pragma unroll
@@ -780,7 +913,53 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
               bulk_commit();
             }
           };
-          if (ok && im.n_split == 1) {
+          if (LONE && ok && im.shared) {
+            // The two warps of these 32 rows meet: each leaves its reference and row sum in its staging buffer, then takes half
+            // of the columns of both results.  The half of the buffer that is not written first holds them; with one group of
+            // columns that group takes the other half, so that here as after other items the newest store reads half 1.
+            constexpr int NG = D / 64, EX = NG > 1 ? 1 : 0;
+            if (lane == 0) bulk_wait_read<0>();
+            __syncwarp();
+            reinterpret_cast<float2*>(stage + EX * 2048)[lane] = make_float2(m_ref, l_sum);
+            __syncwarp();
+            const uint32_t meet = bar(MEET + (warp & 3));
+            if (lane == 0) mbar_arrive(meet);
+            ok = __all_sync(0xffffffffu, mbar_wait(meet, 0, abort_flag, p.status));
+            if (ok) {
+              tc_fence_after();
+              const unsigned char* other = sgen + SM_OUT + (warp < 8 ? warp : warp - 8) * STAGE_BYTES;
+              const float2 ml = reinterpret_cast<const float2*>(other + EX * 2048)[lane];
+              const bool both = im.n_tiles > 1;                 // else the second warpgroup had no key tile
+              const float m_all = fmaxf(m_ref, ml.x);
+              float w_own = exp2f(m_ref - m_all), w_other = exp2f(ml.x - m_all);
+              const float inv = 1.f / (l_sum * w_own + ml.y * w_other);
+              uint32_t a[NG][32], b[NG][32];
+#pragma unroll
+              for (int c = 0; c < NG; ++c) {
+                tmem_ld32(tmem + lane_base + 256 + (x * NG + c) * 32, a[c]);
+                tmem_ld32(tmem + lane_base + 384 + (x * NG + c) * 32, b[c]);
+              }
+              tmem_wait_ld();
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(meet);                 // the other warp's results and its two words have been read
+              const float wa = x == 0 ? w_own : w_other, wb = x == 0 ? w_other : w_own;
+#pragma unroll
+              for (int c = 0; c < NG; ++c) {
+                float acc[32];
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                  acc[i] = __uint_as_float(a[c][i]) * wa;
+                  if (both) acc[i] = fmaf(__uint_as_float(b[c][i]), wb, acc[i]);
+                }
+                if (c == NG - 1) {
+                  ok = __all_sync(0xffffffffu, mbar_wait(meet, 1, abort_flag, p.status));
+                  tc_fence_after();
+                }
+                if (ok) store_rows(acc, inv, x * NG + c, NG > 1 ? c : 1);
+              }
+            }
+          } else if (ok && (LONE || im.n_split == 1)) {
             tc_fence_after();
             const float inv = 1.f / l_sum;
             // the whole row of O in one go, so the four groups' conversions and stores overlap
@@ -792,11 +971,11 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
               float acc[32];
 #pragma unroll
               for (int i = 0; i < 32; ++i) acc[i] = __uint_as_float(r[i]);
-              store_rows(acc, inv, c);
+              store_rows(acc, inv, c, c & 1);
             };
 #pragma unroll
             for (int c = 0; c < D / 32; ++c) out_group(o[c], c);
-          } else if (ok) {
+          } else if (!LONE && ok) {
             // A piece of a split head: publish the unnormalised O of this row with its reference and row
             // sum; the warp that arrives last at the counter of these 32 rows merges
             // sum over pieces of 2^(m_piece - m) * (O_piece, l_piece).
@@ -903,7 +1082,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
                     acc[4 * i + 3] = fmaf(v.w, w, acc[4 * i + 3]);
                   }
                 }
-                store_rows(acc, inv, c);
+                store_rows(acc, inv, c, c & 1);
               }
             }
           }
@@ -1011,8 +1190,10 @@ int tc_create(const heatkv_config& cfg, void* k_pool, void* v_pool, uint64_t poo
       !encode_2d(st, &st->v_pool_half, v_pool, pool_rows, cfg.d / 2))
     return HEATKV_OK;
   const int smem = cfg.d == 128 ? (int)tc::Layout<128>::SM_ALLOC : (int)tc::Layout<64>::SM_ALLOC;
-  const void* kernels[2] = {cfg.d == 128 ? (const void*)tc::attn_tc_kernel<128, false> : (const void*)tc::attn_tc_kernel<64, false>,
-                            cfg.d == 128 ? (const void*)tc::attn_tc_kernel<128, true> : (const void*)tc::attn_tc_kernel<64, true>};
+  const bool wide = cfg.d == 128;
+  const void* kernels[3] = {wide ? (const void*)tc::attn_tc_kernel<128, false, false> : (const void*)tc::attn_tc_kernel<64, false, false>,
+                            wide ? (const void*)tc::attn_tc_kernel<128, false, true> : (const void*)tc::attn_tc_kernel<64, false, true>,
+                            wide ? (const void*)tc::attn_tc_kernel<128, true, false> : (const void*)tc::attn_tc_kernel<64, true, false>};
   for (const void* kern : kernels) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
       cudaGetLastError();
@@ -1094,7 +1275,7 @@ cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int n_seq, cudaStre
   q.attn_items = p.items_per_seq * n_seq;
   q.store_items = p.append_tiles * p.H * n_seq;
   dim3 grid((unsigned)std::min(q.attn_items, st->n_sm));
-  const bool full = p.full_slots > 0;
+  const bool full = p.full_slots > 0, lone = p.lone != 0;
   if (full) {
     // Items of calibration are all of one length, so a partly filled last round costs as much as a full one.  Where its single
     // query tiles would still all run at once it is issued as those (a tile alone is quicker per key tile than one of a
@@ -1110,9 +1291,9 @@ cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int n_seq, cudaStre
     grid = dim3((unsigned)std::min(q.attn_items, st->n_sm));
   }
   if (st->d == 128)
-    return launch_pdl(full ? tc::attn_tc_kernel<128, true> : tc::attn_tc_kernel<128, false>, grid, tc::THREADS,
+    return launch_pdl(full ? tc::attn_tc_kernel<128, true, false> : lone ? tc::attn_tc_kernel<128, false, true> : tc::attn_tc_kernel<128, false, false>, grid, tc::THREADS,
                       tc::Layout<128>::SM_ALLOC, stream, q, maps);
-  return launch_pdl(full ? tc::attn_tc_kernel<64, true> : tc::attn_tc_kernel<64, false>, grid, tc::THREADS,
+  return launch_pdl(full ? tc::attn_tc_kernel<64, true, false> : lone ? tc::attn_tc_kernel<64, false, true> : tc::attn_tc_kernel<64, false, false>, grid, tc::THREADS,
                     tc::Layout<64>::SM_ALLOC, stream, q, maps);
 }
 

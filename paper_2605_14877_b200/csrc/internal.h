@@ -93,6 +93,8 @@ constexpr int SPLIT_CTRS_PER_GROUP = 8;   // arrival counters per (head, query t
 struct SplitChoice {
   std::vector<int> ns;
   int lmax = 0;
+  // What the launch does instead, if not empty: whole heads in pairs of query tiles (1; an odd last tile by itself) or one by one (0).
+  std::vector<int> lone;
 };
 // Items of one sequence: count, partial slots, counter groups.
 struct SplitShape {
@@ -102,10 +104,11 @@ struct SplitShape {
 inline int split_pieces_for(int tiles, int lmax) { return lmax > 0 ? (tiles + lmax - 1) / lmax : 1; }
 // Every piece of an equal cut must hold at least one tile.
 inline bool split_cut_ok(int tiles, int ns) { return ns >= 1 && (ns - 1) * ((tiles + ns - 1) / ns) < tiles; }
-SplitShape split_shape(const std::vector<int>& tiles, const std::vector<int>& ns, int n_qp);
+SplitShape split_shape(const std::vector<int>& tiles, const std::vector<int>& ns, int n_qp, int n_qt);
 double split_makespan(const std::vector<int>& tiles, const std::vector<int>& ns, int n_qp, int n_seq, int n_sm);
 SplitChoice split_search(const std::vector<int>& tiles, int n_qp, int n_seq, int n_sm, bool per_head, uint64_t max_slots,
                          uint64_t max_ctrs);
+void single_search(const std::vector<int>& tiles, int t_q, int n_seq, int n_sm, bool per_head, SplitChoice* choice);
 
 int build_schedule(const heatkv_config& cfg, const double* scas, const double* cas, int policy,
                    int accounting, double b, const double* fraction, Schedule* out);

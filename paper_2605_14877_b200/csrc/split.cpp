@@ -9,10 +9,10 @@
 
 namespace heatkv {
 
-SplitShape split_shape(const std::vector<int>& tiles, const std::vector<int>& ns, int n_qp) {
+SplitShape split_shape(const std::vector<int>& tiles, const std::vector<int>& ns, int n_qp, int n_qt) {
   SplitShape r;
   for (size_t i = 0; i < tiles.size(); ++i) {
-    r.items += n_qp * ns[i];
+    r.items += ns[i] > 0 ? n_qp * ns[i] : n_qt;
     if (ns[i] > 1) { r.slots += n_qp * ns[i]; r.ctrs += n_qp; }
   }
   return r;
@@ -27,22 +27,22 @@ SplitShape split_shape(const std::vector<int>& tiles, const std::vector<int>& ns
 // as many items at once as it has SMs: the search on a new context (a thousand launches of hundreds of items, on the way
 // of a model's first image) takes 1.3 ms where a heap of single SMs took 75 (32 heads, 2 layers, 13 scales).
 // `give_up`: any value at or above it may be returned as soon as the launch cannot end before it.
-static double makespan(const std::vector<int>& tiles, const std::vector<int>& ns, int n_qp, int n_seq, int n_sm, double give_up) {
-  constexpr double FIXED = 2.0, PUBLISH = 1.0, MERGE_PER_PIECE = 1.5;
+struct ItemRun {
+  double cost;
+  int n;                                                   // items of that cost, per sequence
+};
+static void add(std::vector<ItemRun>& items, double cost, int n) {
+  if (!items.empty() && items.back().cost == cost) items.back().n += n;       // neighbours that are alike
+  else items.push_back({cost, n});
+}
+constexpr double FIXED = 2.0, PUBLISH = 1.0, MERGE_PER_PIECE = 1.5;
+static double finish(const std::vector<ItemRun>& items, int n_seq, int n_sm, double give_up) {
   double total = 0.0, longest = 0.0;
   size_t n_items = 0;
-  auto cost = [&](size_t i, int pc) {
-    const int piece = (tiles[i] + ns[i] - 1) / ns[i];
-    const int len = std::min(tiles[i], (pc + 1) * piece) - pc * piece;
-    return len + FIXED + (ns[i] > 1 ? PUBLISH + MERGE_PER_PIECE * (ns[i] - 1) / ns[i] : 0.0);
-  };
-  for (size_t i = 0; i < tiles.size(); ++i) {
-    for (int pc = 0; pc < ns[i]; ++pc) {
-      const double c = cost(i, pc);
-      total += c * n_qp;
-      longest = std::max(longest, c);
-    }
-    n_items += (size_t)n_qp * ns[i];
+  for (const ItemRun& it : items) {
+    total += it.cost * it.n;
+    longest = std::max(longest, it.cost);
+    n_items += it.n;
   }
   n_items *= (size_t)n_seq;
   if (n_items > 8192) return total * n_seq / n_sm + longest;
@@ -52,30 +52,41 @@ static double makespan(const std::vector<int>& tiles, const std::vector<int>& ns
     double t;                                              // finish time
     int sms;                                               // SMs that share it
   };
-  std::vector<Run> runs = {{0.0, n_sm}};                   // binary min-heap
+  std::vector<Run> runs;                                   // binary min-heap
+  runs.reserve(2 * items.size() + 2);
+  runs.push_back({0.0, n_sm});
   auto later = [](const Run& a, const Run& b) { return a.t > b.t; };
   double end = 0.0;
-  for (size_t i = 0; i < tiles.size(); ++i)
-    for (int pc = 0; pc < ns[i]; ++pc) {
-      const double c = cost(i, pc);
-      for (int left = n_qp * n_seq; left > 0;) {
-        std::pop_heap(runs.begin(), runs.end(), later);
-        Run& r = runs.back();
-        const int n = std::min(left, r.sms);
-        const double t = r.t + c;
-        left -= n;
-        end = std::max(end, t);
-        if (n < r.sms) {
-          r.sms -= n;
-          std::push_heap(runs.begin(), runs.end(), later);
-          runs.push_back({t, n});
-        } else {
-          r.t = t;
-        }
+  for (const ItemRun& it : items)
+    for (int left = it.n * n_seq; left > 0;) {
+      std::pop_heap(runs.begin(), runs.end(), later);
+      Run& r = runs.back();
+      const int n = std::min(left, r.sms);
+      const double t = r.t + it.cost;
+      left -= n;
+      end = std::max(end, t);
+      if (n < r.sms) {
+        r.sms -= n;
         std::push_heap(runs.begin(), runs.end(), later);
+        runs.push_back({t, n});
+      } else {
+        r.t = t;
       }
+      std::push_heap(runs.begin(), runs.end(), later);
     }
   return end;
+}
+
+static double makespan(const std::vector<int>& tiles, const std::vector<int>& ns, int n_qp, int n_seq, int n_sm, double give_up) {
+  std::vector<ItemRun> items;
+  items.reserve(2 * tiles.size());
+  for (size_t i = 0; i < tiles.size(); ++i)
+    for (int pc = 0; pc < ns[i]; ++pc) {
+      const int piece = (tiles[i] + ns[i] - 1) / ns[i];
+      const int len = std::min(tiles[i], (pc + 1) * piece) - pc * piece;
+      add(items, len + FIXED + (ns[i] > 1 ? PUBLISH + MERGE_PER_PIECE * (ns[i] - 1) / ns[i] : 0.0), n_qp);
+    }
+  return finish(items, n_seq, n_sm, give_up);
 }
 
 double split_makespan(const std::vector<int>& tiles, const std::vector<int>& ns, int n_qp, int n_seq, int n_sm) {
@@ -121,13 +132,68 @@ SplitChoice split_search(const std::vector<int>& tiles, int n_qp, int n_seq, int
         }
         for (int i = 0; i < H; ++i) ok = ok && split_cut_ok(tiles[i], ns[i]);
         if (!ok || (lmax == 0 && tail == 0)) continue;
-        if (!fits(split_shape(tiles, ns, n_qp))) continue;
+        if (!fits(split_shape(tiles, ns, n_qp, 0))) continue;
         const double take = std::min(BETTER * best_t, WORTH * whole_t);
         const double t = makespan(tiles, ns, n_qp, n_seq, n_sm, take);
         if (t < take) { best_t = t; best.ns = ns; best.lmax = tail == 0 ? lmax : -1; }
       }
   }
   return best;
+}
+
+// Should the launch take query tiles one by one instead (SplitChoice::lone)?  Such an item takes its key tiles two at a time, so it is
+// half as long as a pair's without the partial results of a cut, at the price of keys and values read once per tile instead of once
+// per pair: per key tile 1.02 us where a pair takes 1.83 (1024 queries, 12 to 40 key tiles, 296 heads) and 0.80 where a pair takes 1.52
+// (28 heads x 576 queries).  Candidates: the longest heads, the ones dispatched last, both, all, or none but the odd last tiles.  Back
+// to back: 32 heads x 576 queries, two of 12 and thirty of 5 to 7 tiles, 22.5 -> 16.8 us; 28 x 576, 12 tiles, 25.9 -> 18.5; 28 x 1024,
+// 20 tiles, all by themselves 44 against 39 (not taken); 128 x 1600 queries, last tiles alone, 224.5 -> 218.8.  A cut's estimate is known
+// to within 5 %, that of whole heads better: by as much this one has to be ahead.
+constexpr double TILE_SINGLE = 0.55;        // a key tile of such an item
+constexpr double TILE_PADDED = 0.81;        // of a lone query tile run as the first of a pair
+constexpr double LONE_LAUNCH = 0.8;         // more code to fetch, the meeting of the two results
+void single_search(const std::vector<int>& tiles, int t_q, int n_seq, int n_sm, bool per_head, SplitChoice* choice) {
+  const int H = (int)tiles.size(), n_qp = (t_q + 255) / 256, n_qt = (t_q + 127) / 128, odd = n_qt & 1;
+  if (H == 0) return;
+  std::vector<ItemRun> items;
+  auto list = [&](const std::vector<int>& ns, bool lone) {
+    items.clear();
+    for (int i = 0, m; i < H; i += m) {
+      for (m = 1; i + m < H && tiles[i + m] == tiles[i] && ns[i + m] == ns[i];) ++m;       // heads that are alike
+      if (ns[i] == 0) {
+        add(items, TILE_SINGLE * tiles[i] + FIXED, m * n_qt);
+        continue;
+      }
+      const int k = ns[i], piece = (tiles[i] + k - 1) / k;
+      const double fixed = FIXED + (k > 1 ? PUBLISH + MERGE_PER_PIECE * (k - 1) / k : 0.0);
+      for (int pc = 0; pc < k; ++pc) {
+        const int len = std::min(tiles[i], (pc + 1) * piece) - pc * piece;
+        if (n_qp > odd) add(items, len + fixed, m * (n_qp - odd));
+        if (odd) add(items, (lone ? TILE_SINGLE : TILE_PADDED) * len + fixed, m);
+      }
+    }
+  };
+  list(choice->ns, false);
+  const bool is_cut = std::any_of(choice->ns.begin(), choice->ns.end(), [](int n) { return n > 1; });
+  double take = (is_cut ? WORTH : BETTER) * finish(items, n_seq, n_sm, HUGE_VAL) - LONE_LAUNCH;
+  std::vector<int> ns(H);
+  auto attempt = [&](int first, int last) {
+    ns.assign(H, 1);
+    std::fill(ns.begin(), ns.begin() + first, 0);
+    std::fill(ns.end() - last, ns.end(), 0);
+    list(ns, true);
+    const double t = finish(items, n_seq, n_sm, take);
+    if (t >= take) return;
+    take = BETTER * t;
+    choice->lone = ns;
+  };
+  attempt(H, 0);
+  if (odd) attempt(0, 0);
+  if (!per_head) return;
+  for (int first = 0, tried = 0; first < H && tried < 4; ++tried) {
+    for (int last = first == 0 ? 1 : 0; first + last < H; last = last ? 2 * last : 1) attempt(first, last);
+    const int longest = tiles[first];
+    while (first < H && tiles[first] == longest) ++first;
+  }
 }
 
 }  // namespace heatkv

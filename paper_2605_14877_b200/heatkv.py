@@ -23,7 +23,7 @@ __all__ = [
     "heatkv_schedule_plan", "heatkv_schedule_plan_fp8", "heatkv_seq_open", "heatkv_seq_close", "heatkv_append_compact", "heatkv_scale_attention",
     "heatkv_attention_append", "heatkv_split_plan",
     "heatkv_cache_bytes", "heatkv_retained_indices", "heatkv_export_head", "heatkv_export_head_fp8", "heatkv_allocator_stats",
-    "CACHE_BF16", "CACHE_FP8_E4M3", "heatkv_launch_count", "heatkv_kernel_launches", "heatkv_pair_launches", "heatkv_rank_dispersion", "heatkv_seq_reservation",
+    "CACHE_BF16", "CACHE_FP8_E4M3", "heatkv_launch_count", "heatkv_kernel_launches", "heatkv_pair_launches", "heatkv_lone_launches", "heatkv_rank_dispersion", "heatkv_seq_reservation",
     "KernelStats",
     "heatkv_selftest_wait_expiry", "heatkv_device_status", "heatkv_strerror", "heatkv_attention_split", "arena_bytes_for",
 ]
@@ -106,7 +106,7 @@ def exported_symbols():
             "heatkv_scale_attention", "heatkv_attention_append", "heatkv_cache_bytes", "heatkv_seq_reservation",
             "heatkv_retained_indices", "heatkv_export_head", "heatkv_export_head_fp8",
             "heatkv_attention_split", "heatkv_split_plan", "heatkv_allocator_stats", "heatkv_launch_count",
-            "heatkv_kernel_launches", "heatkv_pair_launches", "heatkv_rank_dispersion", "heatkv_selftest_wait_expiry", "heatkv_device_status",
+            "heatkv_kernel_launches", "heatkv_pair_launches", "heatkv_lone_launches", "heatkv_rank_dispersion", "heatkv_selftest_wait_expiry", "heatkv_device_status",
             "heatkv_strerror"]
 
 
@@ -152,6 +152,7 @@ _lib.heatkv_export_head_fp8.argtypes = [_P, C.c_int, C.c_int, C.c_int, _P, _P, _
 _lib.heatkv_allocator_stats.argtypes = [_P, C.POINTER(AllocStats)]
 _lib.heatkv_launch_count.argtypes = [_P, C.POINTER(C.c_uint64)]
 _lib.heatkv_pair_launches.argtypes = [_P, C.POINTER(C.c_uint64)]
+_lib.heatkv_lone_launches.argtypes = [_P, C.POINTER(C.c_uint64)]
 _lib.heatkv_device_status.argtypes = [_P, _P]
 _lib.heatkv_selftest_wait_expiry.argtypes = [_P, _P]
 _lib.heatkv_kernel_launches.argtypes = [_P, C.POINTER(KernelStats)]
@@ -402,6 +403,12 @@ def heatkv_kernel_launches(ctx: int) -> KernelStats:
 def heatkv_pair_launches(ctx: int) -> int:
     n = C.c_uint64()
     _check(_lib.heatkv_pair_launches(ctx, C.byref(n)), "heatkv_pair_launches")
+    return n.value
+
+
+def heatkv_lone_launches(ctx: int) -> int:
+    n = C.c_uint64()
+    _check(_lib.heatkv_lone_launches(ctx, C.byref(n)), "heatkv_lone_launches")
     return n.value
 
 

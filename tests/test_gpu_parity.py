@@ -447,6 +447,44 @@ def test_cta_pair_kernel_line_counts_half_tiles(hk):
     assert _pair_steps(hk, t, 2, 128, scas=scas, b=0.5) == [9]
 
 
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+@pytest.mark.parametrize("H,n_seq,t,fractions,lone", [
+    (28, 1, [128, 576], None, [1]),                     # all query tiles one by one, 6 key tiles, the last with 64 rows
+    (4, 1, [128, 256, 128, 100], [1, 0.5, 0.25, 0], [2, 3]),   # one query tile, of 128 and 100 rows; 1 to 5 key tiles
+    (34, 2, [640, 576], [1] * 4 + [0] * 30, [0, 1]),    # the first and last heads' tiles, the odd last tiles and pairs in one launch
+    (30, 5, [768, 384], None, [0, 1]),                  # pairs and odd last tiles only, 9 key tiles
+], ids=["all", "few_tiles", "some_heads", "last_tiles"])
+def test_lone_query_tiles(hk, monkeypatch, d, H, n_seq, t, fractions, lone):
+    """Work items of one query tile, whose key tiles the two softmax warpgroups take in turn: odd and even counts, none for the second
+    warpgroup, beside items of two query tiles.  Every output against attention in 64 bits."""
+    monkeypatch.setattr(hk, "heatkv_pair_launches", hk.heatkv_lone_launches)        # the steps to be returned
+    f = np.ones((1, H)) if fractions is None else np.array([fractions])
+    assert _pair_steps(hk, t, H, d, n_seq=n_seq, policy=hk.POLICY_EXPLICIT, fraction=f) == lone
+
+
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+def test_lone_query_tiles_mixed_schedules(hk, d):
+    """The same in a call of two schedules (no head table in the launch parameters): 28 units of 12 or 5 key tiles, 576 queries."""
+    from paper_2605_14877_b200.sweep import Session
+    H, t = 14, [960, 576]
+    fractions = [np.ones((1, H)), np.arange(H)[None] % 2.0]
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    q, k, v = (torch.randn(2, H, sum(t), d, generator=gen, device="cuda").mul_(f).bfloat16() for f in (1, 1, 0.25))
+    out = torch.zeros_like(q)
+    with Session(1, H, d, t, 0, pool_rows=2 * H * (sum(t) + 128), kernel=hk.KERNEL_TCGEN05) as ses:
+        schedules = [ses.schedule(policy=hk.POLICY_EXPLICIT, fraction=f) for f in fractions]
+        ids = [hk.heatkv_seq_open(ses.ctx, s) for s in schedules]
+        ses.generate(ids, lambda l: (q, k, v), lambda l: out)
+        torch.cuda.synchronize()
+        assert hk.heatkv_device_status(ses.ctx) == 0 and hk.heatkv_lone_launches(ses.ctx) == 1
+        for s in schedules:
+            hk.heatkv_schedule_free(s)
+    x = q[:, :, t[0]:].double() @ k.double().transpose(2, 3) / math.sqrt(d)
+    x[1, ::2, :, : t[0]] = -math.inf
+    want = torch.softmax(x, dim=-1) @ v.double()
+    assert (out[:, :, t[0]:].double() - want).abs().max().item() <= ATOL_MAX
+
+
 def test_tensor_memory_kernel_full_cache(hk):
     """b = 1: long page tables (up to 4121 prior keys), tcgen05 kernel, no bias."""
     sh = W.Shape("full128", L=1, H=2, d=128, sides=W.SIDES_13[:12], n_seq=1, s=3)
