@@ -9,23 +9,32 @@
 
 namespace heatkv {
 
-// `u` = (step * L + layer) * H + head.  Returns at once when the head does not store half-tile `j`.
+// What half-tile `j` of a head's update is, from the plan alone: `n` rows (0: the head does not store it), the first of them token
+// `tok0` of the step, to pool rows `row` and up.  `u` = (step * L + layer) * H + head; `base_row` is the sequence's first row.
+struct AppendPlace {
+  int n, tok0;
+  int64_t row;
+};
+__device__ __forceinline__ AppendPlace append_place(const int32_t* plan, int64_t base_row, int u, int j) {
+  PlanView pv(plan);
+  AppendPlace a = {0, 0, 0};
+  if (j >= pv.app_cnt()[u]) return a;
+  const int2* descs = pv.descs() + pv.app_begin()[u];
+  for (int i = 0; i < j; ++i) a.tok0 += descs[i].y & 0xff;
+  const int2 dsc = descs[j];
+  a.n = dsc.y & 0xff;
+  a.row = base_row + dsc.x;
+  return a;
+}
+
 // All `nthreads` threads of the CTA call it with their `tid`; rows are copied verbatim in 16-byte words.
-__device__ __forceinline__ void append_half_tile(const int32_t* plan, int64_t base_row, int u, int j,
-                                                 const __nv_bfloat16* __restrict__ k_src,
+__device__ __forceinline__ void append_half_tile(const AppendPlace& a, const __nv_bfloat16* __restrict__ k_src,
                                                  const __nv_bfloat16* __restrict__ v_src, int64_t kv_tok,
                                                  __nv_bfloat16* __restrict__ k_pool, __nv_bfloat16* __restrict__ v_pool,
                                                  int d, int tid, int nthreads) {
   constexpr int UNROLL = 4;
-  PlanView pv(plan);
-  const int cnt = pv.app_cnt()[u];
-  if (j >= cnt) return;
-  const int2* descs = pv.descs() + pv.app_begin()[u];
-  int tok0 = 0;
-  for (int i = 0; i < j; ++i) tok0 += descs[i].y & 0xff;
-  const int2 dsc = descs[j];
-  const int n = dsc.y & 0xff;
-  const int64_t row = base_row + dsc.x;
+  const int n = a.n, tok0 = a.tok0;
+  const int64_t row = a.row;
   const int ch_per_row = d / 8;
   const int total = n * ch_per_row;                      // 16-byte chunks per tensor
   const int64_t src_off = (int64_t)tok0 * kv_tok;
@@ -104,22 +113,15 @@ __device__ __forceinline__ uint2 chunk_to_codes(const int4& v, float scale) {
 // The same for the fp8 cache: destination half-tile `j` of the head's new K and V, quantised row by row on the way.
 // The d / 8 lanes that hold one row (consecutive lanes of one warp) agree on the row's largest magnitude by
 // shuffles, then every lane converts its own 8 values of K and of V.  `nthreads` must be a multiple of 32 and
-// every thread of the calling warps must take part (the shuffles name the whole warp); `base_row` is the
-// sequence's first row in the code pools.
-__device__ __forceinline__ void append_half_tile_fp8(const int32_t* plan, int64_t base_row, int u, int j,
-                                                     const __nv_bfloat16* __restrict__ k_src,
+// every thread of the calling warps must take part (the shuffles name the whole warp); the place's rows are
+// those of the code pools.
+__device__ __forceinline__ void append_half_tile_fp8(const AppendPlace& a, const __nv_bfloat16* __restrict__ k_src,
                                                      const __nv_bfloat16* __restrict__ v_src, int64_t kv_tok,
                                                      uint8_t* __restrict__ k8_pool, uint8_t* __restrict__ v8_pool,
                                                      int8_t* __restrict__ k_exp, int8_t* __restrict__ v_exp, int d, int tid,
                                                      int nthreads) {
-  PlanView pv(plan);
-  if (j >= pv.app_cnt()[u]) return;
-  const int2* descs = pv.descs() + pv.app_begin()[u];
-  int tok0 = 0;
-  for (int i = 0; i < j; ++i) tok0 += descs[i].y & 0xff;
-  const int2 dsc = descs[j];
-  const int n = dsc.y & 0xff;
-  const int64_t row0 = base_row + dsc.x;
+  const int n = a.n, tok0 = a.tok0;
+  const int64_t row0 = a.row;
   const int ch_per_row = d / 8;                          // 16 or 8: a power of two that divides the warp
   const int total = n * ch_per_row;
   const int64_t src_off = (int64_t)tok0 * kv_tok;
@@ -150,6 +152,25 @@ __device__ __forceinline__ void append_half_tile_fp8(const int32_t* plan, int64_
       }
     }
   }
+}
+
+// One CTA of an attention launch that carries the cache update: half-tile `j` of (sequence, head).  The plan is read and the rows
+// are sent for while the launch before may still run: behind pdl_wait the look-up's three dependent loads outlasted the attention of
+// the smallest steps (7 steps x 32 layers of 256 x 256 pairs 1205 -> 1180 us).
+template <int D>
+__device__ __forceinline__ void append_cta(const AttnParams& p, int seq, int head, int j, int tid, int nthreads) {
+  const int64_t src = seq * p.kv_seq + head * p.kv_head;
+  const bool fp8 = p.k8_pool != nullptr;
+  const AppendPlace a =
+      append_place(p.seqs[seq].plan, fp8 ? p.pool_base[seq] : p.seqs[seq].base_row, (p.step * p.L + p.layer) * p.H + head, j);
+  prefetch_rows(p.k_new + src + a.tok0 * p.kv_tok, 2 * p.kv_tok, a.n, 2 * D, tid, nthreads);
+  prefetch_rows(p.v_new + src + a.tok0 * p.kv_tok, 2 * p.kv_tok, a.n, 2 * D, tid, nthreads);
+  pdl_wait();
+  if (fp8)
+    append_half_tile_fp8(a, p.k_new + src, p.v_new + src, p.kv_tok, p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, D, tid, nthreads);
+  else
+    append_half_tile(a, p.k_new + src, p.v_new + src, p.kv_tok, const_cast<__nv_bfloat16*>(p.k_pool),
+                     const_cast<__nv_bfloat16*>(p.v_pool), D, tid, nthreads);
 }
 
 }  // namespace heatkv

@@ -87,16 +87,7 @@ __global__ void __launch_bounds__(GTHREADS * GROUPS, 2 / GROUPS) attn_generic_ke
   // every sequence are dispatched first; calibration: grid = (query tiles, heads, sequences)
   if (!CALIB && (int)blockIdx.x >= (p.t_q + GM - 1) / GM) {
     // cache update riding on this launch: one CTA per (destination half-tile, sequence, head)
-    const int sq = blockIdx.y, hd = blockIdx.z, j = blockIdx.x - (p.t_q + GM - 1) / GM;
-    const int64_t src = sq * p.kv_seq + hd * p.kv_head;
-    pdl_wait();
-    if (p.k8_pool)
-      append_half_tile_fp8(p.seqs[sq].plan, p.pool_base[sq], (p.step * p.L + p.layer) * p.H + hd, j, p.k_new + src,
-                           p.v_new + src, p.kv_tok, p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, D, threadIdx.x, GTHREADS * GROUPS);
-    else
-      append_half_tile(p.seqs[sq].plan, p.seqs[sq].base_row, (p.step * p.L + p.layer) * p.H + hd, j, p.k_new + src,
-                       p.v_new + src, p.kv_tok, const_cast<__nv_bfloat16*>(p.k_pool), const_cast<__nv_bfloat16*>(p.v_pool),
-                       D, threadIdx.x, GTHREADS * GROUPS);
+    append_cta<D>(p, blockIdx.y, blockIdx.z, blockIdx.x - (p.t_q + GM - 1) / GM, threadIdx.x, GTHREADS * GROUPS);
     return;
   }
   const int seq = CALIB ? blockIdx.z : blockIdx.y;
@@ -501,16 +492,7 @@ __global__ void __launch_bounds__(GTHREADS, 2) attn_small_kernel(const __grid_co
   const int q_tiles = (p.t_q + SM::ROWS - 1) / SM::ROWS;
   if ((int)blockIdx.x >= q_tiles) {
     // cache update riding on this launch: one CTA per (destination half-tile, sequence, head)
-    const int sq = blockIdx.y, hd = blockIdx.z, j = blockIdx.x - q_tiles;
-    const int64_t src = sq * p.kv_seq + hd * p.kv_head;
-    pdl_wait();
-    if (p.k8_pool)
-      append_half_tile_fp8(p.seqs[sq].plan, p.pool_base[sq], (p.step * p.L + p.layer) * p.H + hd, j, p.k_new + src,
-                           p.v_new + src, p.kv_tok, p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, D, threadIdx.x, GTHREADS);
-    else
-      append_half_tile(p.seqs[sq].plan, p.seqs[sq].base_row, (p.step * p.L + p.layer) * p.H + hd, j, p.k_new + src,
-                       p.v_new + src, p.kv_tok, const_cast<__nv_bfloat16*>(p.k_pool), const_cast<__nv_bfloat16*>(p.v_pool),
-                       D, threadIdx.x, GTHREADS);
+    append_cta<D>(p, blockIdx.y, blockIdx.z, blockIdx.x - q_tiles, threadIdx.x, GTHREADS);
     return;
   }
   const int grp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;

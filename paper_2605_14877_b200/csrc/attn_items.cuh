@@ -62,7 +62,7 @@ __device__ __forceinline__ void store_rows_loop(const AttnParams& p, uint32_t n_
     if (a >= p.store_items) break;
     const int sq = a % p.n_seq, hd = (a / p.n_seq) % p.H, j = a / (p.n_seq * p.H);
     const int64_t src = sq * p.kv_seq + hd * p.kv_head;
-    append_half_tile(p.seqs[sq].plan, p.seqs[sq].base_row, u + hd, j, p.k_new + src, p.v_new + src, p.kv_tok,
+    append_half_tile(append_place(p.seqs[sq].plan, p.seqs[sq].base_row, u + hd, j), p.k_new + src, p.v_new + src, p.kv_tok,
                      const_cast<__nv_bfloat16*>(p.k_pool), const_cast<__nv_bfloat16*>(p.v_pool), D, lane, 32);
   }
 }

@@ -21,7 +21,7 @@ __global__ void __launch_bounds__(CP_THREADS) append_kernel(const __grid_constan
   const int seq = blockIdx.z, head = blockIdx.y, j = blockIdx.x;
   const int u = (p.step * p.L + p.layer) * p.H + head;
   const int64_t src = seq * p.kv_seq + head * p.kv_head;
-  append_half_tile(p.seqs[seq].plan, p.seqs[seq].base_row, u, j, p.k_new + src, p.v_new + src, p.kv_tok, p.k_pool,
+  append_half_tile(append_place(p.seqs[seq].plan, p.seqs[seq].base_row, u, j), p.k_new + src, p.v_new + src, p.kv_tok, p.k_pool,
                    p.v_pool, p.d, threadIdx.x, CP_THREADS);
 }
 
@@ -78,8 +78,8 @@ __global__ void __launch_bounds__(CP_THREADS) append_fp8_kernel(const __grid_con
   const int seq = blockIdx.z, head = blockIdx.y, j = blockIdx.x;
   const int u = (p.step * p.L + p.layer) * p.H + head;
   const int64_t src = seq * p.kv_seq + head * p.kv_head;
-  append_half_tile_fp8(p.seqs[seq].plan, p.seqs[seq].base_row, u, j, p.k_new + src, p.v_new + src, p.kv_tok, p.k8_pool,
-                       p.v8_pool, p.k_exp, p.v_exp, p.d, threadIdx.x, CP_THREADS);
+  append_half_tile_fp8(append_place(p.seqs[seq].plan, p.seqs[seq].base_row, u, j), p.k_new + src, p.v_new + src, p.kv_tok,
+                       p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, p.d, threadIdx.x, CP_THREADS);
 }
 
 // Expansion of the visible head-scales of one (step, layer) into the bf16 staging rows the attention kernels
@@ -95,8 +95,9 @@ __global__ void __launch_bounds__(CP_THREADS) stage_fp8_kernel(const __grid_cons
   if ((int)blockIdx.x >= expand) {
     const int a = blockIdx.x - expand, seq = a % n_seq, head = (a / n_seq) % p.H, j = a / (n_seq * p.H);
     const int64_t src = seq * p.kv_seq + head * p.kv_head;
-    append_half_tile_fp8(p.seqs[seq].plan, p.seqs[seq].base_row, (p.step * p.L + p.layer) * p.H + head, j, p.k_new + src,
-                         p.v_new + src, p.kv_tok, p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, p.d, threadIdx.x, CP_THREADS);
+    append_half_tile_fp8(append_place(p.seqs[seq].plan, p.seqs[seq].base_row, (p.step * p.L + p.layer) * p.H + head, j),
+                         p.k_new + src, p.v_new + src, p.kv_tok, p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, p.d, threadIdx.x,
+                         CP_THREADS);
     return;
   }
   const bool is_v = blockIdx.x & 1;
