@@ -126,12 +126,12 @@ __device__ __forceinline__ Item read_item(const volatile int32_t* ring, const At
   it.qp = LONE ? it.sub : it.sub % n_qp;
   it.q0 = it.qp * (one ? BM : 2 * BM);
   it.nq = (!one && it.q0 + BM < p.t_q) ? 2 : 1;     // does tile B hold any query?
-  it.shared = LONE && it.nq == 1;
   if (FULL) {                                       // one query tile of the pair (W_SLOT: 0 both, 1 the first, 2 the second)
     const int single = ring_word(ring, W_SLOT);
     if (single > 0) it.nq = 1;
     if (single == 2) it.q0 += BM;
   }
+  it.shared = LONE && it.nq == 1;
   it.n_slots = FULL ? it.n_desc : it.n_desc + (p.n_own + HALF - 1) / HALF;
   // this item's run of key tiles: [j0, j0 + n_tiles) of the head's ceil(n_slots / 2)
   const int piece_tiles = LONE ? tiles : (tiles + it.n_split - 1) / it.n_split;
@@ -701,11 +701,13 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
           int cur_seg = 0;
           float cur_mass = 0.f;
           float* masses = reinterpret_cast<float*>(stage) + lane;      // [scale][32 rows]
-          const bool follow = FULL && n_tiles <= FOLLOW_TILES;
+          if (FULL && LONE)                                            // a scale may lie in the other warpgroup's tiles alone
+            for (int s = 0; s <= p.step; ++s) masses[s * 32] = 0.f;
+          const bool follow = FULL && (n_slots + 1) / 2 <= FOLLOW_TILES;
           int j = 0;
           // FULL: a warp whose 32 rows all lie past the last query hands on whatever is there (its rows of O and its masses go
           // nowhere): a calibration pass 1.130 -> 1.115 ms.  Generation measured 0.3 to 0.8 % slower with the branch.
-          const bool no_rows = FULL && q0 + x * BM + (warp & 3) * 32 >= p.t_q;
+          const bool no_rows = FULL && q0 + (stride == 2 ? 0 : x * BM) + (warp & 3) * 32 >= p.t_q;
           for (; no_rows && j < n_tiles && ok; ++j) {
             ok = __all_sync(0xffffffffu, mbar_wait(bar(S_FULL + x), (cx + j) & 1, abort_flag, p.status));
             mbar_arrive(bar(P_FULL + 2 * x));
@@ -888,10 +890,10 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
           const Item im = read_item<FULL, LONE>(ring, p, n_qp);
           const int seq = im.seq;
           const int q_row0 = im.shared ? im.q0 : im.q0 + x * BM;
-          if (FULL && ok && !no_rows) {
-            // Eq. 2: mean over the step's rows of mass(row, scale) / rowsum(row); rows past t_q are padding
-            const float inv_t = 1.f / (float)p.t_q;
-            const float w = q_row0 + row < p.t_q ? inv_t / l_sum : 0.f;
+          // Eq. 2: mean over the step's rows of mass(row, scale) / rowsum(row), `inv_l` = this row's 1 / rowsum relative to its
+          // reference; rows past t_q are padding
+          auto add_beta = [&](float inv_l) {
+            const float w = q_row0 + row < p.t_q ? inv_l / (float)p.t_q : 0.f;
             float* beta = p.beta_row + (int64_t)im.head * p.K * p.K;
             for (int s = 0; s <= p.step; ++s) {
               float v = (s == cur_seg ? cur_mass : masses[s * 32]) * w;
@@ -900,7 +902,8 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
               if (lane == 0) atomicAdd(beta + s, v);
             }
             __syncwarp();                                   // the buffer now takes output rows
-          }
+          };
+          if (FULL && ok && !no_rows && !im.shared) add_beta(1.f / l_sum);
           // Normalised rows leave through this warp's staging buffer: per group of 32 columns every thread parks its 64 bytes
           // (16-byte chunks, chunk ^ (row / 2 mod 4): the copy engine's 64-byte swizzle, free of bank conflicts) and one bulk
           // store writes the 32 rows, clipping those past the last query.  The halves of the buffer alternate.  Loads from the
@@ -936,7 +939,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             // The two warps of these 32 rows meet: each leaves its reference and row sum in its staging buffer, then takes half
             // of the columns of both results.  The half of the buffer that is not written first holds them; with one group of
             // columns that group takes the other half, so that here as after other items the newest store reads half 1.
-            constexpr int NG = D / 64, EX = NG > 1 ? 1 : 0;
+            constexpr int NG = D / 64, EX = NG > 1 || FULL ? 1 : 0;          // (FULL: the masses lie in half 0)
             if (lane == 0) bulk_wait_read<0>();
             __syncwarp();
             reinterpret_cast<float2*>(stage + EX * 2048)[lane] = make_float2(m_ref, l_sum);
@@ -952,6 +955,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
               const float m_all = fmaxf(m_ref, ml.x);
               float w_own = exp2f(m_ref - m_all), w_other = exp2f(ml.x - m_all);
               const float inv = 1.f / (l_sum * w_own + ml.y * w_other);
+              if (FULL && !no_rows) add_beta(w_own * inv);
               uint32_t a[NG][32], b[NG][32];
 #pragma unroll
               for (int c = 0; c < NG; ++c) {
@@ -1209,10 +1213,16 @@ int tc_create(const heatkv_config& cfg, void* k_pool, void* v_pool, uint64_t poo
       !encode_2d(st, &st->v_pool_half, v_pool, pool_rows, cfg.d / 2))
     return HEATKV_OK;
   const int smem = cfg.d == 128 ? (int)tc::Layout<128>::SM_ALLOC : (int)tc::Layout<64>::SM_ALLOC;
-  const bool wide = cfg.d == 128;
-  const void* kernels[3] = {wide ? (const void*)tc::attn_tc_kernel<128, false, false> : (const void*)tc::attn_tc_kernel<64, false, false>,
-                            wide ? (const void*)tc::attn_tc_kernel<128, false, true> : (const void*)tc::attn_tc_kernel<64, false, true>,
-                            wide ? (const void*)tc::attn_tc_kernel<128, true, false> : (const void*)tc::attn_tc_kernel<64, true, false>};
+  const void* kernels[4];
+  for (int i = 0; i < 4; ++i)
+    kernels[i] = cfg.d == 128 ? (i == 0   ? (const void*)tc::attn_tc_kernel<128, false, false>
+                                 : i == 1 ? (const void*)tc::attn_tc_kernel<128, false, true>
+                                 : i == 2 ? (const void*)tc::attn_tc_kernel<128, true, false>
+                                          : (const void*)tc::attn_tc_kernel<128, true, true>)
+                              : (i == 0   ? (const void*)tc::attn_tc_kernel<64, false, false>
+                                 : i == 1 ? (const void*)tc::attn_tc_kernel<64, false, true>
+                                 : i == 2 ? (const void*)tc::attn_tc_kernel<64, true, false>
+                                          : (const void*)tc::attn_tc_kernel<64, true, true>);
   for (const void* kern : kernels) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
       cudaGetLastError();
@@ -1294,12 +1304,15 @@ cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int n_seq, cudaStre
   q.attn_items = p.items_per_seq * n_seq;
   q.store_items = p.append_tiles * p.H * n_seq;
   dim3 grid((unsigned)std::min(q.attn_items, st->n_sm));
-  const bool full = p.full_slots > 0, lone = p.lone != 0;
+  const bool full = p.full_slots > 0;
+  bool lone = p.lone != 0;
   if (full) {
     // Items of calibration are all of one length, so a partly filled last round costs as much as a full one.  Where its single
-    // query tiles would still all run at once it is issued as those (a tile alone is quicker per key tile than one of a
-    // pair): 2 sequences x 16 heads, 256 queries 16.7 -> 14.7 us, 400: 24.0 -> 21.7, 1600: 123.2 -> 117.6; a pass 1.105 -> 1.073 ms
-    // (before short items followed their maximum).
+    // query tiles would still all run at once it is issued as those, half as long.  Odd last tiles are single items from the second
+    // round on; one round is as long as its pairs, and the kernel without single items is the quicker one for those (1024 queries 55.3
+    // against 56.3 us, 2304: 193.4 and 195.5; 576 with an odd tile 37.6 and 39.5).  2 sequences x 16 heads, with single tiles run as the
+    // first of a pair before: 144 queries 12.9 -> 11.2 us, 256: 16.7 -> 13.4, 400: 24.9 -> 18.9, 1600: 117 -> 103, 4096: 586 -> 554; 8
+    // sequences, 576 queries: 103.5 -> 93.5, 1024: 203 -> 190.
     const int total = q.attn_items, n_qp = (p.t_q + 2 * tc::BM - 1) / (2 * tc::BM), whole = total / st->n_sm * st->n_sm;
     const bool tail_single = p.t_q - (n_qp - 1) * 2 * tc::BM <= tc::BM;
     int singles = 0;
@@ -1307,13 +1320,18 @@ cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int n_seq, cudaStre
     const bool cut = singles <= st->n_sm && total < INT32_MAX - 2 * st->n_sm;
     q.full_whole = cut ? whole : total;
     if (cut) q.attn_items = whole + 2 * (total - whole);
+    lone = (cut && whole < total) || (tail_single && total > st->n_sm);
     grid = dim3((unsigned)std::min(q.attn_items, st->n_sm));
   }
-  if (st->d == 128)
-    return launch_pdl(full ? tc::attn_tc_kernel<128, true, false> : lone ? tc::attn_tc_kernel<128, false, true> : tc::attn_tc_kernel<128, false, false>, grid, tc::THREADS,
-                      tc::Layout<128>::SM_ALLOC, stream, q, maps);
-  return launch_pdl(full ? tc::attn_tc_kernel<64, true, false> : lone ? tc::attn_tc_kernel<64, false, true> : tc::attn_tc_kernel<64, false, false>, grid, tc::THREADS,
-                    tc::Layout<64>::SM_ALLOC, stream, q, maps);
+  auto launch = [&](auto kernel, uint32_t smem) { return launch_pdl(kernel, grid, tc::THREADS, smem, stream, q, maps); };
+  if (st->d == 128) {
+    constexpr uint32_t smem = tc::Layout<128>::SM_ALLOC;
+    if (full) return lone ? launch(tc::attn_tc_kernel<128, true, true>, smem) : launch(tc::attn_tc_kernel<128, true, false>, smem);
+    return lone ? launch(tc::attn_tc_kernel<128, false, true>, smem) : launch(tc::attn_tc_kernel<128, false, false>, smem);
+  }
+  constexpr uint32_t smem = tc::Layout<64>::SM_ALLOC;
+  if (full) return lone ? launch(tc::attn_tc_kernel<64, true, true>, smem) : launch(tc::attn_tc_kernel<64, true, false>, smem);
+  return lone ? launch(tc::attn_tc_kernel<64, false, true>, smem) : launch(tc::attn_tc_kernel<64, false, false>, smem);
 }
 
 }  // namespace heatkv

@@ -1047,6 +1047,32 @@ def test_calibration_with_output_is_as_exact_as_the_warp_level_kernel(hk, d):
     assert all(t <= 1.02 * g for g, t in zip(*err_out)), err_out
 
 
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+@pytest.mark.parametrize("H,t", [(3, [128, 128, 64, 64, 128, 200]), (2, [1, 130]), (150, [100, 300])],
+                         ids=["scales_of_one_warpgroup", "one_tile_and_a_row", "odd_tails_of_two_rounds"])
+def test_calibration_with_output_lone_query_tiles(hk, d, H, t):
+    """Work items of one query tile, whose key tiles the two softmax warpgroups take in turn: a scale may lie in one's tiles alone.
+    Masses are fp32 sums of exponentials that are off by at most 2^-22 of themselves; a bias of up to 4 spreads them."""
+    from paper_2605_14877_b200.sweep import Session
+    K, c = len(t), np.cumsum([0] + list(t))
+    gen = torch.Generator(device="cuda").manual_seed(H)
+    q, k, v = (torch.randn(1, H, c[-1], d, generator=gen, device="cuda").mul_(f).bfloat16() for f in (1, 1, 0.25))
+    bias = 4 * torch.rand(H, K, generator=gen, device="cuda")
+    beta = torch.zeros(1, H, K, K, device="cuda")
+    lo = int(c[-2])
+    out = torch.zeros_like(q[:, :, lo:])
+    with Session(1, H, d, t, 0, pool_rows=64, kernel=hk.KERNEL_TCGEN05) as ses:
+        qs = q[:, :, lo:]
+        hk.heatkv_calibrate_scores(ses.ctx, 0, K - 1, 1, qs, k, v, hk.Strides.of(qs, k, out), bias, beta, out)
+        torch.cuda.synchronize()
+        assert hk.heatkv_device_status(ses.ctx) == 0
+    scale_of = torch.from_numpy(np.repeat(np.arange(K), t)).cuda()
+    p = torch.softmax(qs.double() @ k.double().transpose(2, 3) / math.sqrt(d) + bias.double()[None, :, None, scale_of], dim=-1)
+    assert (out.double() - p @ v.double()).abs().max().item() <= ATOL_MAX
+    want = torch.stack([p[..., scale_of == s].sum(-1).mean(-1)[0] for s in range(K)], -1)
+    assert ((beta[0, :, K - 1].double() - want).abs() / want).max().item() <= 2.0 ** -20
+
+
 def test_config2_calibration_full_size(hk):
     """Sec. 3.1, Eq. 2 and Eq. 4 at the size the bench calibrates at: 13 scales, 2 sequences x 16 heads, bias on
     the current scale, automatic kernel choice (tensor-memory kernel for the seven steps of 256 tokens and more:
