@@ -114,7 +114,9 @@ __device__ __forceinline__ uint2 chunk_to_codes(const int4& v, float scale) {
 // The d / 8 lanes that hold one row (consecutive lanes of one warp) agree on the row's largest magnitude by
 // shuffles, then every lane converts its own 8 values of K and of V.  `nthreads` must be a multiple of 32 and
 // every thread of the calling warps must take part (the shuffles name the whole warp); the place's rows are
-// those of the code pools.
+// those of the code pools.  UNROLL rounds of loads are in flight at once: 4 where a launch is bound by latency, 1 where it
+// is bound by memory (there 2 or 4 are 7 % slower).
+template <int UNROLL>
 __device__ __forceinline__ void append_half_tile_fp8(const AppendPlace& a, const __nv_bfloat16* __restrict__ k_src,
                                                      const __nv_bfloat16* __restrict__ v_src, int64_t kv_tok,
                                                      uint8_t* __restrict__ k8_pool, uint8_t* __restrict__ v8_pool,
@@ -126,29 +128,36 @@ __device__ __forceinline__ void append_half_tile_fp8(const AppendPlace& a, const
   const int total = n * ch_per_row;
   const int64_t src_off = (int64_t)tok0 * kv_tok;
   const int rounds = (total + nthreads - 1) / nthreads;
-  for (int it = 0; it < rounds; ++it) {                  // every thread runs every round: the shuffles need whole warps
-    const int i = it * nthreads + tid;
-    const bool live = i < total;                         // whole rows are live or not (ch_per_row divides 32)
-    const int r = i / ch_per_row, ch = i % ch_per_row;
-    int4 kv = make_int4(0, 0, 0, 0), vv = make_int4(0, 0, 0, 0);
-    if (live) {
-      const int64_t off = src_off + (int64_t)r * kv_tok + ch * 8;
-      kv = __ldg(reinterpret_cast<const int4*>(k_src + off));
-      vv = __ldg(reinterpret_cast<const int4*>(v_src + off));
+  for (int it = 0; it < rounds; it += UNROLL) {          // every thread runs every round: the shuffles need whole warps
+    int4 kv[UNROLL], vv[UNROLL];
+#pragma unroll
+    for (int uu = 0; uu < UNROLL; ++uu) {
+      const int i = (it + uu) * nthreads + tid;
+      kv[uu] = vv[uu] = make_int4(0, 0, 0, 0);
+      if (i < total) {                                   // whole rows are live or not (ch_per_row divides 32)
+        const int64_t off = src_off + (int64_t)(i / ch_per_row) * kv_tok + i % ch_per_row * 8;
+        kv[uu] = __ldg(reinterpret_cast<const int4*>(k_src + off));
+        vv[uu] = __ldg(reinterpret_cast<const int4*>(v_src + off));
+      }
     }
-    uint32_t ka = chunk_amax_bits(kv), va = chunk_amax_bits(vv);
-    for (int o = 1; o < ch_per_row; o <<= 1) {
-      ka = max(ka, __shfl_xor_sync(0xffffffffu, ka, o));
-      va = max(va, __shfl_xor_sync(0xffffffffu, va, o));
-    }
-    if (live) {
-      const int ke = fp8_row_exponent(ka), ve = fp8_row_exponent(va);
-      const int64_t row = row0 + r;
-      *reinterpret_cast<uint2*>(k8_pool + row * d + ch * 8) = chunk_to_codes(kv, pow2f(-ke));
-      *reinterpret_cast<uint2*>(v8_pool + row * d + ch * 8) = chunk_to_codes(vv, pow2f(-ve));
-      if (ch == 0) {
-        k_exp[row] = (int8_t)ke;
-        v_exp[row] = (int8_t)ve;
+#pragma unroll
+    for (int uu = 0; uu < UNROLL; ++uu) {
+      const int i = (it + uu) * nthreads + tid;
+      const int r = i / ch_per_row, ch = i % ch_per_row;
+      uint32_t ka = chunk_amax_bits(kv[uu]), va = chunk_amax_bits(vv[uu]);
+      for (int o = 1; o < ch_per_row; o <<= 1) {
+        ka = max(ka, __shfl_xor_sync(0xffffffffu, ka, o));
+        va = max(va, __shfl_xor_sync(0xffffffffu, va, o));
+      }
+      if (i < total) {
+        const int ke = fp8_row_exponent(ka), ve = fp8_row_exponent(va);
+        const int64_t row = row0 + r;
+        *reinterpret_cast<uint2*>(k8_pool + row * d + ch * 8) = chunk_to_codes(kv[uu], pow2f(-ke));
+        *reinterpret_cast<uint2*>(v8_pool + row * d + ch * 8) = chunk_to_codes(vv[uu], pow2f(-ve));
+        if (ch == 0) {
+          k_exp[row] = (int8_t)ke;
+          v_exp[row] = (int8_t)ve;
+        }
       }
     }
   }
@@ -167,7 +176,7 @@ __device__ __forceinline__ void append_cta(const AttnParams& p, int seq, int hea
   prefetch_rows(p.v_new + src + a.tok0 * p.kv_tok, 2 * p.kv_tok, a.n, 2 * D, tid, nthreads);
   pdl_wait();
   if (fp8)
-    append_half_tile_fp8(a, p.k_new + src, p.v_new + src, p.kv_tok, p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, D, tid, nthreads);
+    append_half_tile_fp8<4>(a, p.k_new + src, p.v_new + src, p.kv_tok, p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, D, tid, nthreads);
   else
     append_half_tile(a, p.k_new + src, p.v_new + src, p.kv_tok, const_cast<__nv_bfloat16*>(p.k_pool),
                      const_cast<__nv_bfloat16*>(p.v_pool), D, tid, nthreads);

@@ -197,3 +197,34 @@ def test_fp8_cache_config2_full_size(hk):
     ref = O.heatkv_schedule(scores, 0.05, sh.s, sh.sides)
     bias = W.seg_bias_current_scale(sh, 0)
     _run_fp8(hk, sh, ref, lambda ses: ses.schedule(scas=scores, b=0.05), hk.KERNEL_AUTO, bias=bias, fused=True)
+
+
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+@pytest.mark.parametrize("H,n_seq", [(3, 2), (40, 8)], ids=["few_ctas", "many_ctas"])
+def test_update_beside_the_expansion_stores_what_the_update_alone_stores(hk, H, n_seq, d):
+    """The cache update on the expansion's launch (in its form for few CTAs and for many: 54 and 2 240 at 130 queries) against the
+    update as a launch of its own: the same codes and exponent bytes, over half-tiles of 1 to 64 rows."""
+    from paper_2605_14877_b200.sweep import Session
+    t = [1, 63, 65, 130, 20]
+    gen = torch.Generator(device="cuda").manual_seed(H)
+    q, k, v = (torch.randn(n_seq, H, sum(t), d, generator=gen, device="cuda") for _ in range(3))
+    q, k, v = (x.mul_(torch.exp(3 * torch.randn(n_seq, H, sum(t), 1, generator=gen, device="cuda"))).bfloat16() for x in (q, k, v))
+    got = []
+    for fused in (True, False):
+        out = torch.zeros_like(q)
+        with Session(1, H, d, t, 0, pool_rows=n_seq * H * (sum(t) + 64 * len(t)), kernel=hk.KERNEL_TCGEN05,
+                     cache_dtype=hk.CACHE_FP8_E4M3, stage_bytes=256 << 20) as ses:
+            sch = ses.schedule(policy=hk.POLICY_EXPLICIT, fraction=np.ones((1, H)))
+            ids = [hk.heatkv_seq_open(ses.ctx, sch) for _ in range(n_seq)]
+            ses.generate(ids, lambda l: (q, k, v), lambda l: out, fused=fused)
+            n = sum(t[:-1])
+            for s, h in ((0, 0), (n_seq - 1, H - 1), (n_seq // 2, H // 2)):
+                codes = [torch.zeros(n, d, dtype=torch.uint8, device="cuda") for _ in range(2)]
+                exps = [torch.zeros(n, dtype=torch.int8, device="cuda") for _ in range(2)]
+                hk.heatkv_export_head_fp8(ses.ctx, ids[s], 0, h, *codes, *exps)
+                got.append([x.cpu() for x in codes + exps])
+            torch.cuda.synchronize()
+            assert hk.heatkv_device_status(ses.ctx) == 0
+            hk.heatkv_schedule_free(sch)
+    for a, b in zip(got[:3], got[3:]):
+        assert all(torch.equal(x, y) for x, y in zip(a, b)) and a[0].any()
