@@ -146,11 +146,14 @@ SplitChoice split_search(const std::vector<int>& tiles, int n_qp, int n_seq, int
 // per pair: per key tile 1.02 us where a pair takes 1.83 (1024 queries, 12 to 40 key tiles, 296 heads) and 0.80 where a pair takes 1.52
 // (28 heads x 576 queries).  Candidates: the longest heads, the ones dispatched last, both, all, or none but the odd last tiles.  Back
 // to back: 32 heads x 576 queries, two of 12 and thirty of 5 to 7 tiles, 22.5 -> 16.8 us; 28 x 576, 12 tiles, 25.9 -> 18.5; 28 x 1024,
-// 20 tiles, all by themselves 44 against 39 (not taken); 128 x 1600 queries, last tiles alone, 224.5 -> 218.8.  A cut's estimate is known
-// to within 5 %, that of whole heads better: by as much this one has to be ahead.
+// 20 tiles, all by themselves 44 against 39 (not taken); 128 x 1600 queries, last tiles alone, 224.5 -> 218.8.  Launches with cuts are
+// longer than their estimate by what the last piece's way through memory takes and no other item hides (14 launches of 80 to
+// 288 items: whole heads and lone tiles 1.58 us per unit and 2.3, cuts 3.4 to 5.8 us more): 102 items of 256 queries, 30 of 12 tiles, cut
+// in three 20.6 us, lone 15.9; 32 heads x 1024 queries, 4 of 19 tiles, cut in two 27.4, lone 22.6.
 constexpr double TILE_SINGLE = 0.55;        // a key tile of such an item
 constexpr double TILE_PADDED = 0.81;        // of a lone query tile run as the first of a pair
-constexpr double LONE_LAUNCH = 0.8;         // more code to fetch, the meeting of the two results
+constexpr double LONE_LAUNCH = 0.8;         // a kernel of its own: its code is fetched anew between launches of the other
+constexpr double CUT_LAUNCH = 3.0;
 void single_search(const std::vector<int>& tiles, int t_q, int n_seq, int n_sm, bool per_head, SplitChoice* choice) {
   const int H = (int)tiles.size(), n_qp = (t_q + 255) / 256, n_qt = (t_q + 127) / 128, odd = n_qt & 1;
   if (H == 0) return;
@@ -174,7 +177,7 @@ void single_search(const std::vector<int>& tiles, int t_q, int n_seq, int n_sm, 
   };
   list(choice->ns, false);
   const bool is_cut = std::any_of(choice->ns.begin(), choice->ns.end(), [](int n) { return n > 1; });
-  double take = (is_cut ? WORTH : BETTER) * finish(items, n_seq, n_sm, HUGE_VAL) - LONE_LAUNCH;
+  double take = BETTER * (finish(items, n_seq, n_sm, HUGE_VAL) + (is_cut ? CUT_LAUNCH : 0.0)) - LONE_LAUNCH;
   std::vector<int> ns(H);
   auto attempt = [&](int first, int last) {
     ns.assign(H, 1);
