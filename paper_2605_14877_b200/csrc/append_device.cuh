@@ -114,9 +114,7 @@ __device__ __forceinline__ uint2 chunk_to_codes(const int4& v, float scale) {
 // The d / 8 lanes that hold one row (consecutive lanes of one warp) agree on the row's largest magnitude by
 // shuffles, then every lane converts its own 8 values of K and of V.  `nthreads` must be a multiple of 32 and
 // every thread of the calling warps must take part (the shuffles name the whole warp); the place's rows are
-// those of the code pools.  UNROLL rounds of loads are in flight at once: 4 where a launch is bound by latency, 1 where it
-// is bound by memory (there 2 or 4 are 7 % slower).
-template <int UNROLL>
+// those of the code pools.
 __device__ __forceinline__ void append_half_tile_fp8(const AppendPlace& a, const __nv_bfloat16* __restrict__ k_src,
                                                      const __nv_bfloat16* __restrict__ v_src, int64_t kv_tok,
                                                      uint8_t* __restrict__ k8_pool, uint8_t* __restrict__ v8_pool,
@@ -127,6 +125,48 @@ __device__ __forceinline__ void append_half_tile_fp8(const AppendPlace& a, const
   const int ch_per_row = d / 8;                          // 16 or 8: a power of two that divides the warp
   const int total = n * ch_per_row;
   const int64_t src_off = (int64_t)tok0 * kv_tok;
+  const int rounds = (total + nthreads - 1) / nthreads;
+  for (int it = 0; it < rounds; ++it) {                  // every thread runs every round: the shuffles need whole warps
+    const int i = it * nthreads + tid;
+    const bool live = i < total;                         // whole rows are live or not (ch_per_row divides 32)
+    const int r = i / ch_per_row, ch = i % ch_per_row;
+    int4 kv = make_int4(0, 0, 0, 0), vv = make_int4(0, 0, 0, 0);
+    if (live) {
+      const int64_t off = src_off + (int64_t)r * kv_tok + ch * 8;
+      kv = __ldg(reinterpret_cast<const int4*>(k_src + off));
+      vv = __ldg(reinterpret_cast<const int4*>(v_src + off));
+    }
+    uint32_t ka = chunk_amax_bits(kv), va = chunk_amax_bits(vv);
+    for (int o = 1; o < ch_per_row; o <<= 1) {
+      ka = max(ka, __shfl_xor_sync(0xffffffffu, ka, o));
+      va = max(va, __shfl_xor_sync(0xffffffffu, va, o));
+    }
+    if (live) {
+      const int ke = fp8_row_exponent(ka), ve = fp8_row_exponent(va);
+      const int64_t row = row0 + r;
+      *reinterpret_cast<uint2*>(k8_pool + row * d + ch * 8) = chunk_to_codes(kv, pow2f(-ke));
+      *reinterpret_cast<uint2*>(v8_pool + row * d + ch * 8) = chunk_to_codes(vv, pow2f(-ve));
+      if (ch == 0) {
+        k_exp[row] = (int8_t)ke;
+        v_exp[row] = (int8_t)ve;
+      }
+    }
+  }
+}
+
+// The same with four rounds of loads in flight, for launches that are bound by latency (where one is bound by memory, 2 or 4 rounds
+// are 7 % slower; in the attention kernels of small steps their registers cost 1 to 2 % of a pass).
+__device__ __forceinline__ void append_half_tile_fp8_ahead(const AppendPlace& a, const __nv_bfloat16* __restrict__ k_src,
+                                                           const __nv_bfloat16* __restrict__ v_src, int64_t kv_tok,
+                                                           uint8_t* __restrict__ k8_pool, uint8_t* __restrict__ v8_pool,
+                                                           int8_t* __restrict__ k_exp, int8_t* __restrict__ v_exp, int d, int tid,
+                                                           int nthreads) {
+  const int n = a.n, tok0 = a.tok0;
+  const int64_t row0 = a.row;
+  const int ch_per_row = d / 8;                          // 16 or 8: a power of two that divides the warp
+  const int total = n * ch_per_row;
+  const int64_t src_off = (int64_t)tok0 * kv_tok;
+  constexpr int UNROLL = 4;
   const int rounds = (total + nthreads - 1) / nthreads;
   for (int it = 0; it < rounds; it += UNROLL) {          // every thread runs every round: the shuffles need whole warps
     int4 kv[UNROLL], vv[UNROLL];
@@ -176,7 +216,7 @@ __device__ __forceinline__ void append_cta(const AttnParams& p, int seq, int hea
   prefetch_rows(p.v_new + src + a.tok0 * p.kv_tok, 2 * p.kv_tok, a.n, 2 * D, tid, nthreads);
   pdl_wait();
   if (fp8)
-    append_half_tile_fp8<4>(a, p.k_new + src, p.v_new + src, p.kv_tok, p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, D, tid, nthreads);
+    append_half_tile_fp8(a, p.k_new + src, p.v_new + src, p.kv_tok, p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, D, tid, nthreads);
   else
     append_half_tile(a, p.k_new + src, p.v_new + src, p.kv_tok, const_cast<__nv_bfloat16*>(p.k_pool),
                      const_cast<__nv_bfloat16*>(p.v_pool), D, tid, nthreads);

@@ -266,15 +266,18 @@ attn_pair_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ M
       };
       // what the first copies will fetch, sent for while the launch before may still run
       if (leader) {
+        const bool pool = !p.k8_pool;                    // (staging rows: the launch before is writing them)
         const Slot k0 = slot_of((int)rank, base_row);
         for (int ch = 0; ch < NCH; ++ch)
-          if (k0.pool_row >= 0) tma_prefetch_2d(&maps.k_pool, ch * 64, k0.pool_row);
+          if (k0.pool_row >= 0 && !pool) continue;
+          else if (k0.pool_row >= 0) tma_prefetch_2d(&maps.k_pool, ch * 64, k0.pool_row);
           else tma_prefetch_4d(&maps.k_own, ch * 64, -k0.pool_row - 1, kv_head, kv_seq);
         for (int i = 0; i < 2 * NCH; ++i)
           tma_prefetch_4d(&maps.q, (i >> 1) * 64, q_row0 + (i & 1) * HALF, head & p.q_head_mask, seq & p.q_seq_mask);
         for (int hf = 0; hf < 2; ++hf) {
           const Slot v0 = slot_of(hf, base_row);
-          if (v0.pool_row >= 0) tma_prefetch_2d(&maps.v_pool, (int)rank * (D / 2), v0.pool_row);
+          if (v0.pool_row >= 0 && !pool) continue;
+          else if (v0.pool_row >= 0) tma_prefetch_2d(&maps.v_pool, (int)rank * (D / 2), v0.pool_row);
           else tma_prefetch_4d(&maps.v_own, (int)rank * (D / 2), -v0.pool_row - 1, kv_head, kv_seq);
         }
       }

@@ -338,7 +338,8 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
         for (int hf = 0; hf < 2; ++hf) {
           const int row = get_slot<FULL>(2 * im.j0 + hf, descs, im.n_desc, im.n_slots, base_row, p.n_own, p.step).pool_row;
           for (int ch = 0; ch < NCH; ++ch) {
-            if (row >= 0) {
+            if (row >= 0 && p.k8_pool) {                      // staging rows: the launch before is writing them
+            } else if (row >= 0) {
               tma_prefetch_2d(&maps.k_pool, ch * 64, row);
               tma_prefetch_2d(&maps.v_pool, ch * 64, row);
             } else {

@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(CP_THREADS) append_fp8_kernel(const __grid_con
   const int seq = blockIdx.z, head = blockIdx.y, j = blockIdx.x;
   const int u = (p.step * p.L + p.layer) * p.H + head;
   const int64_t src = seq * p.kv_seq + head * p.kv_head;
-  append_half_tile_fp8<1>(append_place(p.seqs[seq].plan, p.seqs[seq].base_row, u, j), p.k_new + src, p.v_new + src, p.kv_tok,
+  append_half_tile_fp8(append_place(p.seqs[seq].plan, p.seqs[seq].base_row, u, j), p.k_new + src, p.v_new + src, p.kv_tok,
                        p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, p.d, threadIdx.x, CP_THREADS);
 }
 
@@ -89,19 +89,23 @@ __global__ void __launch_bounds__(CP_THREADS) append_fp8_kernel(const __grid_con
 // after those quantise them into the code pools: the plan releases no page that this step still reads before the update,
 // so the two need no order between them, and the update costs no launch of its own (4 sequences x 16 heads, 2 layers, 13
 // scales at budget 1/10: 2.43 -> 2.32 ms a pass, the small steps' direct reading included).
-// UNROLL: rounds of the update's loads in flight.  A launch of up to ten CTAs per SM is a chain of them (4 rounds: 640 CTAs 12.7 -> 10.5 us,
+// AHEAD: four rounds of the update's loads in flight.  A launch of up to ten CTAs per SM is a chain of them (640 CTAs 12.7 -> 10.5 us,
 // 1088: 13.0 -> 11.0; one sequence x 16 heads x 4 layers at budget 1/5 1 809 -> 1 731 us a pass); more CTAs fill the SMs, and the registers
 // cost some of them (1792 CTAs 15.3 -> 16.8, 3096 to 4008: 18.3 -> 19.0).
-template <int UNROLL>
+template <bool AHEAD>
 __global__ void __launch_bounds__(CP_THREADS) stage_fp8_kernel(const __grid_constant__ CopyParams p, int slots, int n_seq) {
   pdl_trigger();
   const int expand = slots * n_seq * 2;
   if ((int)blockIdx.x >= expand) {
     const int a = blockIdx.x - expand, seq = a % n_seq, head = (a / n_seq) % p.H, j = a / (n_seq * p.H);
     const int64_t src = seq * p.kv_seq + head * p.kv_head;
-    append_half_tile_fp8<UNROLL>(append_place(p.seqs[seq].plan, p.seqs[seq].base_row, (p.step * p.L + p.layer) * p.H + head, j),
-                         p.k_new + src, p.v_new + src, p.kv_tok, p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, p.d, threadIdx.x,
-                         CP_THREADS);
+    const AppendPlace to = append_place(p.seqs[seq].plan, p.seqs[seq].base_row, (p.step * p.L + p.layer) * p.H + head, j);
+    if (AHEAD)
+      append_half_tile_fp8_ahead(to, p.k_new + src, p.v_new + src, p.kv_tok, p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, p.d,
+                                 threadIdx.x, CP_THREADS);
+    else
+      append_half_tile_fp8(to, p.k_new + src, p.v_new + src, p.kv_tok, p.k8_pool, p.v8_pool, p.k_exp, p.v_exp, p.d, threadIdx.x,
+                           CP_THREADS);
     return;
   }
   const bool is_v = blockIdx.x & 1;
@@ -147,8 +151,8 @@ cudaError_t launch_stage_fp8(const CopyParams& p, int n_seq, int slots, bool upd
   const int64_t ctas = (int64_t)slots * n_seq * 2 + tiles * p.H * n_seq;
   if (ctas < 1) return cudaSuccess;
   if (ctas > INT32_MAX) return cudaErrorInvalidValue;
-  if (ctas <= 1480) stage_fp8_kernel<4><<<(unsigned)ctas, CP_THREADS, 0, stream>>>(p, slots, n_seq);
-  else stage_fp8_kernel<1><<<(unsigned)ctas, CP_THREADS, 0, stream>>>(p, slots, n_seq);
+  if (ctas <= 1480) stage_fp8_kernel<true><<<(unsigned)ctas, CP_THREADS, 0, stream>>>(p, slots, n_seq);
+  else stage_fp8_kernel<false><<<(unsigned)ctas, CP_THREADS, 0, stream>>>(p, slots, n_seq);
   return cudaGetLastError();
 }
 
