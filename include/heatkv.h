@@ -72,8 +72,7 @@ typedef enum {
 
 typedef enum {
   HEATKV_KERNEL_AUTO = 0,      /* tensor-memory kernel for steps of >= 256 queries (>= 128 once a call holds
-                                  64 (sequence, head) units, >= 160 where 16-query tiles would fill the
-                                  SMs twice; >= 48 in calibration with an attention output),
+                                  64 (sequence, head) units; >= 48 in calibration with an attention output),
                                   generic otherwise */
   HEATKV_KERNEL_GENERIC = 1,   /* warp-level MMA kernel for every step                    */
   HEATKV_KERNEL_TCGEN05 = 2    /* tcgen05 / TMEM / TMA kernel wherever its shape rules allow */

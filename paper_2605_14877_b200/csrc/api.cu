@@ -768,14 +768,7 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
   bool use_tc = choice != HEATKV_KERNEL_GENERIC && tc_supported(ctx->tc, p, ctx->cfg.d, n_seq);
   // AUTO: steps of 256 queries and more, and steps of 128 and more once the call holds 64 (sequence, head) units:
   // from there on the warp-level kernel is bound by its mma.sync rate (144 queries, 128 units: 52 us against 23 us)
-  // Steps of 160 and more go there too where the small-step kernel does not take them: the 64-query CTAs of the warp-level kernel are
-  // a chain twice as long (back to back, 28 units, 192 queries over 448 and 832 keys: 16.6 and 27.4 us against 8.9 and 13.2; 252
-  // queries over 273: 12.2 against 8.7; 64-wide heads 10.8 and 17.6 against 8.0 and 11.8).  Below that the line of 64 units stands, which
-  // callers that count launches know (56 units of 144 queries would gain as well: 18.5 against 9.9 us over 400 keys).
-  const int64_t units = (int64_t)n_seq * ctx->cfg.H;
-  if (choice == HEATKV_KERNEL_AUTO && !(p.t_q >= 256 || (p.t_q >= 128 && units >= 64) ||
-                                        (p.t_q >= 160 && !attn_is_small(p.t_q, units, ctx->n_sm))))
-    use_tc = false;
+  if (choice == HEATKV_KERNEL_AUTO && !(p.t_q >= 256 || (p.t_q >= 128 && (int64_t)n_seq * ctx->cfg.H >= 64))) use_tc = false;
   if (choice == HEATKV_KERNEL_TCGEN05 && !use_tc) return HEATKV_ERR_INVALID_ARG;   // never a silent substitute
   bool updated = false;                                       // the cache update already went along
   if (ctx->fp8) {

@@ -485,14 +485,6 @@ def test_lone_query_tiles_mixed_schedules(hk, d):
     assert (out[:, :, t[0]:].double() - want).abs().max().item() <= ATOL_MAX
 
 
-@pytest.mark.parametrize("H,tq,tensor_memory", [(29, 160, False), (30, 160, True), (30, 159, False), (18, 255, False), (19, 255, True)])
-def test_kernel_choice_past_the_small_steps(hk, monkeypatch, H, tq, tensor_memory):
-    """Fewer than 64 units: steps of 160 queries and more leave the warp-level kernel where 16-query tiles are more than two per SM (of
-    148).  Every output against attention in 64 bits."""
-    monkeypatch.setattr(hk, "heatkv_pair_launches", lambda ctx: hk.heatkv_kernel_launches(ctx).attention_tcgen05)
-    assert _pair_steps(hk, [130, tq], H, 128, kernel=hk.KERNEL_AUTO) == ([1] if tensor_memory else [])
-
-
 def test_tensor_memory_kernel_full_cache(hk):
     """b = 1: long page tables (up to 4121 prior keys), tcgen05 kernel, no bias."""
     sh = W.Shape("full128", L=1, H=2, d=128, sides=W.SIDES_13[:12], n_seq=1, s=3)
