@@ -453,6 +453,9 @@ void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int 
   p->split_tiles = lmax;
   p->items_per_seq = m.items;
   p->lone = !lone ? 0 : one_plan || !all_lone ? 1 : 2;
+  // Where the heads would be cut, every piece has a reference of its own, which rounds the largest weight of its rows least; a second
+  // look at the maximum gives the two halves of a lone tile as much.
+  p->lone_follow = lone && std::any_of(ch.ns.begin(), ch.ns.end(), [](int n) { return n > 1; });
   p->slots_per_seq = m.slots;
   p->ctrs_per_seq = m.ctrs;
   p->split_partials = ctx->split_partials;

@@ -82,6 +82,7 @@ struct AttnParams {
   int32_t direct8, off_desc, off_src;
   int32_t runs;                   // no per-scale bias: the plan's merged attention tables (PlanView)
   int32_t lone;                   // tensor-memory kernel: items may be one query tile (1), without a head table all are (2)
+  int32_t lone_follow;            // ... and references follow the maximum in an item's second tile, too
   int32_t full_whole;             // calibration with output: work items before this one hold a pair of query tiles, later ones one
 };
 

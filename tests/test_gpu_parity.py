@@ -485,6 +485,35 @@ def test_lone_query_tiles_mixed_schedules(hk, d):
     assert (out[:, :, t[0]:].double() - want).abs().max().item() <= ATOL_MAX
 
 
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+@pytest.mark.parametrize("tile", [1, 2, 3])
+def test_lone_query_tiles_references_follow(hk, d, tile):
+    """Heads of 18 key tiles that would be cut into pieces if their query tiles did not run one by one.  As in the test of the CTA
+    pairs above: two keys have weight, one in the first tile and a larger one (by 2^1 to 2^2) in the first or second tile that one of
+    the warpgroups takes; its weight has to be the reference, exact in bf16, so what is left is the rounding of the output."""
+    from paper_2605_14877_b200.sweep import Session
+    H, t = 30, [1792, 512]
+    q, k, v = (torch.zeros(1, H, sum(t), d, device="cuda") for _ in range(3))
+    q[..., 0] = 1 + torch.arange(sum(t), device="cuda") % 128 / 128
+    k[..., 0] = -2.0 ** 10
+    c = 0.6875 * math.sqrt(d)
+    k[:, :, 0, 0], k[:, :, 128 * tile, 0], v[:, :, 128 * tile] = c, 2 * c, 1
+    q, k, v = (x.bfloat16() for x in (q, k, v))
+    out = torch.zeros_like(q)
+    with Session(1, H, d, t, 0, pool_rows=H * (sum(t) + 128), kernel=hk.KERNEL_TCGEN05) as ses:
+        sch = ses.schedule(policy=hk.POLICY_EXPLICIT, fraction=np.ones((1, H)))
+        sid = hk.heatkv_seq_open(ses.ctx, sch)
+        assert hk.heatkv_attention_split(ses.ctx, [sid], 0, 1)[0] > 0
+        before = []
+        ses.generate([sid], lambda l: (q, k, v), lambda l: out, None, lambda step, l: before.append(hk.heatkv_lone_launches(ses.ctx)))
+        torch.cuda.synchronize()
+        assert hk.heatkv_device_status(ses.ctx) == 0 and before[1] == before[0] + 1
+        hk.heatkv_schedule_free(sch)
+    x = q[:, :, t[0]:].double() @ k.double().transpose(2, 3) / math.sqrt(d)
+    want = torch.softmax(x, dim=-1) @ v.double()
+    assert want.min().item() > 0.5 and (out[:, :, t[0]:].double() - want).abs().max().item() <= 2.0 ** -9 + 2.0 ** -13
+
+
 def test_tensor_memory_kernel_full_cache(hk):
     """b = 1: long page tables (up to 4121 prior keys), tcgen05 kernel, no bias."""
     sh = W.Shape("full128", L=1, H=2, d=128, sides=W.SIDES_13[:12], n_seq=1, s=3)
