@@ -404,10 +404,10 @@ void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int 
   const std::vector<int>& pieces = lone ? ch.lone : ch.ns;
   const int n_qt = (p->t_q + 127) / 128;
   SplitShape m = split_shape(tiles, pieces, n_qp, n_qt);
-  int lmax = !lone && ch.lmax > 0 ? ch.lmax : 0;
+  int lmax = ch.lmax > 0 ? ch.lmax : 0;
   if (!one_plan) {
     // other schedules in the batch follow the same longest run; the per-sequence bounds cover all of them
-    auto bounds = [&](int lm) {
+    auto bounds = [&](int lm, bool uncut) {
       SplitShape b;
       int last_plan = -1;
       for (int i = 0; i < n_seq; ++i) {
@@ -416,17 +416,18 @@ void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int 
         last_plan = pi;
         const std::vector<int> t = ordered_tiles(*ctx->plans[pi], step, layer, own_slots, p->runs);
         std::vector<int> ns(t.size());
-        for (size_t k = 0; k < t.size(); ++k) ns[k] = all_lone ? 0 : split_pieces_for(t[k], lm);
+        for (size_t k = 0; k < t.size(); ++k) ns[k] = uncut ? !all_lone : split_pieces_for(t[k], lm);
         const SplitShape sh = split_shape(t, ns, n_qp, n_qt);
         b.items = std::max(b.items, sh.items); b.slots = std::max(b.slots, sh.slots); b.ctrs = std::max(b.ctrs, sh.ctrs);
       }
       return b;
     };
-    m = bounds(lmax);
+    m = bounds(lmax, false);
     if (lmax > 0 && !fits(m)) {
       lmax = 0;                                             // another schedule in the batch needs more scratch: whole heads
-      m = bounds(0);
+      m = bounds(0, false);
     }
+    if (lone) m = bounds(lmax, true);
   }
   // one plan for the whole call (the usual case): its heads, by descending key count, travel in the parameters
   p->table_heads = 0;
@@ -442,20 +443,17 @@ void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int 
       p->table_desc_begin[i] = tab.desc + (p->runs ? pe0.run_shift : 0) + 2 * begin[order[i]];
       p->table_head[i] = (int16_t)order[i];
       p->table_tiles[i] = (int16_t)tiles[i];
-      p->table_split[i] = (int16_t)pieces[i];
+      p->table_split[i] = (int16_t)(lone && pieces[i] == 0 ? -ch.ns[i] : ch.ns[i]);
       if (pieces[i] > 1) p->longest_piece = std::max(p->longest_piece, (tiles[i] + pieces[i] - 1) / pieces[i]);
     }
     p->table_heads = H;
   } else {
-    p->longest_piece = lmax;
+    p->longest_piece = lone ? 0 : lmax;
   }
   p->n_seq = n_seq;
   p->split_tiles = lmax;
   p->items_per_seq = m.items;
   p->lone = !lone ? 0 : one_plan || !all_lone ? 1 : 2;
-  // Where the heads would be cut, every piece has a reference of its own, which rounds the largest weight of its rows least; a second
-  // look at the maximum gives the two halves of a lone tile as much.
-  p->lone_follow = lone && std::any_of(ch.ns.begin(), ch.ns.end(), [](int n) { return n > 1; });
   p->slots_per_seq = m.slots;
   p->ctrs_per_seq = m.ctrs;
   p->split_partials = ctx->split_partials;

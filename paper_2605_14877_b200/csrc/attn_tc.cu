@@ -27,6 +27,7 @@
 // other's products as it does for two query tiles, and the two results meet in the CTA.  All barrier phases run on across items.  Every wait is bounded; on expiry the
 // CTA records a status word, drains its own copies and leaves.
 #include <algorithm>
+#include <climits>
 
 #include "attn_items.cuh"
 #include "internal.h"
@@ -121,7 +122,7 @@ __device__ __forceinline__ Item read_item(const volatile int32_t* ring, const At
   it.desc_begin = ring_word(ring, W_DESC);
   it.n_desc = ring_word(ring, W_NDESC);
   const int tiles = ring_word(ring, W_TILES);
-  const bool one = LONE && it.n_split == 0;         // the head's items are single query tiles
+  const bool one = LONE && it.n_split < 0;          // the head's items are single query tiles
   it.piece = LONE ? 0 : it.sub / n_qp;
   it.qp = LONE ? it.sub : it.sub % n_qp;
   it.q0 = it.qp * (one ? BM : 2 * BM);
@@ -288,11 +289,12 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             } else {
               h = pv.order()[u + i];
               tiles = (pv.attn_cnt(p.runs)[u + h] + own_slots + 1) >> 1;
-              ns = LONE && p.lone == 2 ? 0 : p.split_tiles > 0 ? (tiles + p.split_tiles - 1) / p.split_tiles : 1;
+              ns = p.split_tiles > 0 ? (tiles + p.split_tiles - 1) / p.split_tiles : 1;
+              if (LONE && p.lone == 2) ns = -ns;
             }
-            cnt = ns > 0 ? n_qp * ns : (p.t_q + BM - 1) / BM;   // 0: the head's query tiles one by one
+            cnt = !LONE ? n_qp * ns : ns > 0 ? n_qp : (p.t_q + BM - 1) / BM;    // below 0: the head's query tiles one by one
           }
-          const int scnt = ns > 1 ? cnt : 0, ccnt = ns > 1 ? n_qp : 0;
+          const int scnt = !LONE && ns > 1 ? cnt : 0, ccnt = !LONE && ns > 1 ? n_qp : 0;
           int inc = cnt, sinc = scnt, cinc = ccnt;
 #pragma unroll
           for (int o = 1; o < 32; o <<= 1) {
@@ -686,13 +688,18 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
           nq = im.shared ? 2 : im.nq;
         }
         if (x < nq) {
-          int j0, n_desc, n_slots, q0, stride;
+          int j0, n_desc, n_slots, q0, stride, piece = INT_MAX, in_piece = 2, first_looks = 1;
           const int2* descs;
           const float* bias_h;
           {
             const Item im = read_item<FULL, LONE>(ring, p, n_qp);
             stride = im.shared ? 2 : 1;
             j0 = im.shared ? x : im.j0; n_desc = im.n_desc; n_slots = im.n_slots; q0 = im.q0;
+            if (!FULL && LONE && abs(im.n_split) > 1) {                        // the pieces the head would be cut into (`look` below)
+              piece = (im.n_tiles + abs(im.n_split) - 1) / abs(im.n_split);
+              in_piece = j0;
+              first_looks = stride;
+            }
             descs = FULL ? p.full_descs : reinterpret_cast<const int2*>(p.seqs[im.seq].plan + im.desc_begin);
             bias_h = p.seg_bias ? p.seg_bias + im.head * p.K : nullptr;
           }
@@ -775,11 +782,15 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
             // meaningless above 2^127); only the second half's maximum is computed, beside them.
             bool take_max = true;
             uint32_t pk0[16], pk1[16];
-            // Lone tiles of a launch that would be cut: the second tile, too, sets the reference.  Against 64 bits, relative to the cut
-            // heads they replace, outputs are then 0.1 to 0.8 % closer (without it up to 0.7 % further off; 1024 queries of an image
-            // pair 2.331e-3 of the norm cut, 2.342e-3 without, 2.325e-3 with it), for 0.7 to 1.3 % of a pass.
-            const bool second = !FULL && LONE && p.lone_follow != 0 && j == 1;
-            if (SPECULATE && j > 0 && !follow && !second) {
+            // A head that would be cut had a reference, and an exact weight for it, in every piece.  Here its references follow the
+            // maximum in the first two tiles of every such piece (and in a lone warpgroup's first two), heads that would stay whole
+            // keep the first tile's.  Against 64 bits no launch measured is then further off than the cuts it replaces (second tiles
+            // alone, in all heads of such a launch: single heads up to 1.3 % further off, those left as pairs of query tiles; with a bias
+            // that raises the last tiles an emulation has them 4 % further off).  An image pair at 20x: 576 queries 19.5 -> 18.5 us.
+            const bool look = !FULL && LONE && (in_piece < 2 || j < first_looks);
+            if (LONE) in_piece += stride;
+            if (LONE && in_piece >= piece) in_piece -= piece;
+            if (SPECULATE && j > 0 && !follow && !look) {
               const uint64_t bb0 = pack2(b0 - m_ref, b0 - m_ref);
               exps(r0, bb0, pk0);
               exps(r1, bb0, pk1);
@@ -825,7 +836,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
               const float mx1 = fmaxf(fmaxf(mq[4], mq[5]), fmaxf(mq[6], mq[7]));
               const float mx = fmaxf(fmaf(mx0, p.scale_log2, b0), fmaf(mx1, p.scale_log2, b1));
               const float m_new = fmaxf(m_ref, mx);
-              const bool grow = m_new > m_ref + (follow || second ? 0.f : RESCALE_THRESHOLD);   // also true on the first tile (m_ref = NO_MAX)
+              const bool grow = m_new > m_ref + (follow || look ? 0.f : RESCALE_THRESHOLD);   // also true on the first tile (m_ref = NO_MAX)
               if (j > 0 && __any_sync(0xffffffffu, grow)) {
                 // O_x holds tiles < j relative to m_ref: rescale the rows whose reference moves.  O_x is complete:
                 // S_x of this tile was issued after the PV products of tile j - 1 by the same thread, and the

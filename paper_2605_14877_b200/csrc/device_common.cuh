@@ -45,7 +45,8 @@ struct AttnParams {
                                   // its heads by descending key count, the head index, its key tiles and its pieces
   int16_t table_head[64];
   int16_t table_tiles[64];
-  int16_t table_split[64];        // pieces the head's key range is cut into (1: whole head; 0: whole, its query tiles one by one)
+  int16_t table_split[64];        // pieces the head's key range is cut into (1: whole head); with `lone`, those it would be cut into,
+                                  // negative where its query tiles go one by one
   int32_t longest_piece;          // longest piece among the heads that are cut (0: none is; host report); CTA pairs: longest head
   int32_t append_tiles;           // > 0: the launch also stores the step's K/V (paged layout): that many destination
                                   // half-tile slots per (sequence, head) follow the attention work
@@ -81,8 +82,8 @@ struct AttnParams {
   // offsets of the descriptors and of the pool rows behind them
   int32_t direct8, off_desc, off_src;
   int32_t runs;                   // no per-scale bias: the plan's merged attention tables (PlanView)
-  int32_t lone;                   // tensor-memory kernel: items may be one query tile (1), without a head table all are (2)
-  int32_t lone_follow;            // ... and references follow the maximum in an item's second tile, too
+  int32_t lone;                   // tensor-memory kernel: items may be one query tile (1), without a head table all are (2), and
+                                  // nothing is cut (split_tiles: the longest run there would be otherwise)
   int32_t full_whole;             // calibration with output: work items before this one hold a pair of query tiles, later ones one
 };
 

@@ -514,6 +514,36 @@ def test_lone_query_tiles_references_follow(hk, d, tile):
     assert want.min().item() > 0.5 and (out[:, :, t[0]:].double() - want).abs().max().item() <= 2.0 ** -9 + 2.0 ** -13
 
 
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+@pytest.mark.parametrize("tile", [1, 10, 11])
+def test_lone_launch_references_follow_in_pairs(hk, d, tile):
+    """The same for heads that stay pairs of query tiles beside odd last ones: 19 key tiles that would be cut into pieces of 10 and 9, so
+    that a key at the start of the second piece (the first of tile 10 or, for the other warpgroup of a lone tile, of 11) was its
+    reference.  Heads of 3 tiles, which would not be cut, run beside them."""
+    from paper_2605_14877_b200.sweep import Session
+    H, n_seq, t = 30, 5, [2048, 384]
+    q, k, v = (torch.zeros(1, H, sum(t), d, device="cuda") for _ in range(3))
+    q[..., 0] = 1 + torch.arange(sum(t), device="cuda") % 128 / 128
+    k[..., 0] = -2.0 ** 10
+    c = 0.6875 * math.sqrt(d)
+    k[:, :, 0, 0], k[:, :, 128 * tile, 0], v[:, :, 128 * tile] = c, 2 * c, 1
+    q, k, v = (x.bfloat16().expand(n_seq, -1, -1, -1) for x in (q, k, v))
+    out = torch.zeros(n_seq, H, sum(t), d, dtype=torch.bfloat16, device="cuda")
+    with Session(1, H, d, t, 0, pool_rows=n_seq * H * (sum(t) + 128), kernel=hk.KERNEL_TCGEN05) as ses:
+        sch = ses.schedule(policy=hk.POLICY_EXPLICIT, fraction=np.arange(H)[None] < H / 2)
+        ids = [hk.heatkv_seq_open(ses.ctx, sch) for _ in range(n_seq)]
+        assert hk.heatkv_attention_split(ses.ctx, ids, 0, 1)[0] == 10
+        before = []
+        ses.generate(ids, lambda l: (q, k, v), lambda l: out, None, lambda step, l: before.append(hk.heatkv_lone_launches(ses.ctx)))
+        torch.cuda.synchronize()
+        assert hk.heatkv_device_status(ses.ctx) == 0 and before[1] == before[0] + 1
+        hk.heatkv_schedule_free(sch)
+    x = q[0, : H // 2, t[0]:].double() @ k[0, : H // 2].double().transpose(1, 2) / math.sqrt(d)
+    want = torch.softmax(x, dim=-1) @ v[0, : H // 2].double()
+    got = out[:, : H // 2, t[0]:].double()
+    assert want.min().item() > 0.5 and (got - want).abs().max().item() <= 2.0 ** -9 + 2.0 ** -13
+
+
 def test_tensor_memory_kernel_full_cache(hk):
     """b = 1: long page tables (up to 4121 prior keys), tcgen05 kernel, no bias."""
     sh = W.Shape("full128", L=1, H=2, d=128, sides=W.SIDES_13[:12], n_seq=1, s=3)
