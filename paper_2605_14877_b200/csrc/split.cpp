@@ -24,73 +24,105 @@ SplitShape split_shape(const std::vector<int>& tiles, const std::vector<int>& ns
 // to clock stamps of the kernel: an item costs its tiles plus the result's way out and the next item's start;
 // a piece writes fp32 partials instead, and the piece that arrives last reads the others.
 // The items of a piece are all alike and the SMs that finish at the same moment are kept as one entry, so an entry takes
-// as many items at once as it has SMs: the search on a new context (a thousand launches of hundreds of items, on the way
-// of a model's first image) takes 1.3 ms where a heap of single SMs took 75 (32 heads, 2 layers, 13 scales).
-// `give_up`: any value at or above it may be returned as soon as the launch cannot end before it.
+// as many items at once as it has SMs.  The searches look at a thousand launches of hundreds of items on the way of a model's first
+// image, so a candidate's total and longest item come from sums per head, and its items are only listed and simulated (in buffers that
+// the whole search shares) where that bound is below the best so far: both searches for every step and layer of a pair of images at 20x
+// (16 heads, 4 layers) take 0.32 ms where listing every candidate took 1.4, with 32 heads of 64 (2 layers) 0.26 and 1.9.
+constexpr double FIXED = 2.0, PUBLISH = 1.0, MERGE_PER_PIECE = 1.5;
+constexpr size_t SIMULATED_ITEMS = 8192;
 struct ItemRun {
   double cost;
   int n;                                                   // items of that cost, per sequence
 };
-static void add(std::vector<ItemRun>& items, double cost, int n) {
-  if (!items.empty() && items.back().cost == cost) items.back().n += n;       // neighbours that are alike
-  else items.push_back({cost, n});
-}
-constexpr double FIXED = 2.0, PUBLISH = 1.0, MERGE_PER_PIECE = 1.5;
-static double finish(const std::vector<ItemRun>& items, int n_seq, int n_sm, double give_up) {
+// What every estimate needs of a number of heads.
+struct Load {
   double total = 0.0, longest = 0.0;
-  size_t n_items = 0;
-  for (const ItemRun& it : items) {
-    total += it.cost * it.n;
-    longest = std::max(longest, it.cost);
-    n_items += it.n;
+  size_t items = 0;
+  uint64_t slots = 0, ctrs = 0;
+  Load operator+(const Load& o) const {
+    return {total + o.total, std::max(longest, o.longest), items + o.items, slots + o.slots, ctrs + o.ctrs};
   }
-  n_items *= (size_t)n_seq;
-  if (n_items > 8192) return total * n_seq / n_sm + longest;
-  const double at_least = std::max(total * n_seq / n_sm, longest);
-  if (at_least >= give_up) return at_least;
+  Load items_of(double cost, int n) const { return *this + Load{cost * n, n > 0 ? cost : 0.0, (size_t)n, 0, 0}; }
+};
+struct Launch {
+  int n_seq, n_sm;
+  std::vector<ItemRun> items;
   struct Run {
     double t;                                              // finish time
     int sms;                                               // SMs that share it
   };
   std::vector<Run> runs;                                   // binary min-heap
-  runs.reserve(2 * items.size() + 2);
-  runs.push_back({0.0, n_sm});
-  auto later = [](const Run& a, const Run& b) { return a.t > b.t; };
-  double end = 0.0;
-  for (const ItemRun& it : items)
-    for (int left = it.n * n_seq; left > 0;) {
-      std::pop_heap(runs.begin(), runs.end(), later);
-      Run& r = runs.back();
-      const int n = std::min(left, r.sms);
-      const double t = r.t + it.cost;
-      left -= n;
-      end = std::max(end, t);
-      if (n < r.sms) {
-        r.sms -= n;
-        std::push_heap(runs.begin(), runs.end(), later);
-        runs.push_back({t, n});
-      } else {
-        r.t = t;
-      }
-      std::push_heap(runs.begin(), runs.end(), later);
-    }
-  return end;
-}
 
-static double makespan(const std::vector<int>& tiles, const std::vector<int>& ns, int n_qp, int n_seq, int n_sm, double give_up) {
-  std::vector<ItemRun> items;
-  items.reserve(2 * tiles.size());
-  for (size_t i = 0; i < tiles.size(); ++i)
-    for (int pc = 0; pc < ns[i]; ++pc) {
-      const int piece = (tiles[i] + ns[i] - 1) / ns[i];
-      const int len = std::min(tiles[i], (pc + 1) * piece) - pc * piece;
-      add(items, len + FIXED + (ns[i] > 1 ? PUBLISH + MERGE_PER_PIECE * (ns[i] - 1) / ns[i] : 0.0), n_qp);
-    }
-  return finish(items, n_seq, n_sm, give_up);
+  void add(double cost, int n) {
+    if (!items.empty() && items.back().cost == cost) items.back().n += n;     // neighbours that are alike
+    else items.push_back({cost, n});
+  }
+  // The estimate of a launch whose items `list` adds; any value at or above `give_up` if it cannot end before that.
+  template <typename F>
+  double estimate(const Load& sum, double give_up, F list) {
+    if (sum.items * n_seq > SIMULATED_ITEMS) return sum.total * n_seq / n_sm + sum.longest;
+    const double at_least = std::max(sum.total * n_seq / n_sm, sum.longest);
+    if (at_least >= give_up) return at_least;
+    items.clear();
+    list();
+    return finish(give_up);
+  }
+  double finish(double give_up) {
+    runs.clear();
+    runs.push_back({0.0, n_sm});
+    auto later = [](const Run& a, const Run& b) { return a.t > b.t; };
+    double end = 0.0;
+    for (const ItemRun& it : items)
+      for (int left = it.n * n_seq; left > 0;) {
+        const double t = runs[0].t + it.cost;
+        const int n = std::min(left, runs[0].sms);
+        left -= n;
+        end = std::max(end, t);
+        if (end >= give_up) return end;
+        if (n < runs[0].sms) {
+          runs[0].sms -= n;                                // (it stays the earliest)
+          runs.push_back({t, n});
+          std::push_heap(runs.begin(), runs.end(), later);
+          continue;
+        }
+        size_t at = 0;                                     // the earliest entry ends at t now: down to its place
+        for (size_t below; (below = 2 * at + 1) < runs.size(); at = below) {
+          if (below + 1 < runs.size() && runs[below + 1].t < runs[below].t) ++below;
+          if (runs[below].t >= t) break;
+          runs[at] = runs[below];
+        }
+        runs[at] = {t, n};
+      }
+    return end;
+  }
+};
+
+// Pieces of a head: all but the last as long as the first.
+struct Cut {
+  int full, last;
+  double fixed;
+  Cut(int tiles, int ns) : full((tiles + ns - 1) / ns), last(tiles - (ns - 1) * full),
+                           fixed(FIXED + (ns > 1 ? PUBLISH + MERGE_PER_PIECE * (ns - 1) / ns : 0.0)) {}
+};
+static Load head_load(int tiles, int ns, int n_qp) {
+  const Cut c(tiles, ns);
+  Load r = Load().items_of(c.full + c.fixed, n_qp * (ns - 1)).items_of(c.last + c.fixed, n_qp);
+  if (ns > 1) { r.slots = (uint64_t)n_qp * ns; r.ctrs = n_qp; }
+  return r;
+}
+static void add_head(Launch& launch, int tiles, int ns, int n_qp) {
+  const Cut c(tiles, ns);
+  if (ns > 1) launch.add(c.full + c.fixed, n_qp * (ns - 1));
+  launch.add(c.last + c.fixed, n_qp);
 }
 
 double split_makespan(const std::vector<int>& tiles, const std::vector<int>& ns, int n_qp, int n_seq, int n_sm) {
-  return makespan(tiles, ns, n_qp, n_seq, n_sm, HUGE_VAL);
+  Launch launch{n_seq, n_sm};
+  Load sum;
+  for (size_t i = 0; i < tiles.size(); ++i) sum = sum + head_load(tiles[i], ns[i], n_qp);
+  return launch.estimate(sum, HUGE_VAL, [&] {
+    for (size_t i = 0; i < tiles.size(); ++i) add_head(launch, tiles[i], ns[i], n_qp);
+  });
 }
 
 // The search.  Long heads are cut to a common longest run (candidates: the longest head divided by 2..16), and,
@@ -107,11 +139,9 @@ SplitChoice split_search(const std::vector<int>& tiles, int n_qp, int n_seq, int
   SplitChoice best;
   best.ns.assign(H, 1);
   if (H == 0) return best;
+  Launch launch{n_seq, n_sm};
   double best_t = split_makespan(tiles, best.ns, n_qp, n_seq, n_sm);
   const double whole_t = best_t;
-  auto fits = [&](const SplitShape& sh) {
-    return (uint64_t)sh.slots * n_seq <= max_slots && (uint64_t)sh.ctrs * n_seq * SPLIT_CTRS_PER_GROUP <= max_ctrs;
-  };
   const int max_tiles = *std::max_element(tiles.begin(), tiles.end());
   std::vector<int> lmaxes = {0};
   for (int div : {2, 3, 4, 6, 8, 12, 16}) {
@@ -119,24 +149,38 @@ SplitChoice split_search(const std::vector<int>& tiles, int n_qp, int n_seq, int
     if (cand < SPLIT_MIN_PIECE) break;
     lmaxes.push_back(cand);
   }
+  std::vector<int> base(H);
+  std::vector<Load> before(H + 1);                         // of the heads before this one
   for (int lmax : lmaxes) {
-    std::vector<int> base(H);
-    for (int i = 0; i < H; ++i) base[i] = split_pieces_for(tiles[i], lmax);
-    for (int extra = 1; extra <= (per_head ? 3 : 1); ++extra)
-      for (int tail = (extra == 1 ? 0 : 1); tail <= (extra == 1 ? 0 : H); ++tail) {
-        std::vector<int> ns = base;
-        bool ok = true;
-        for (int i = H - tail; i < H; ++i) {
-          ns[i] = base[i] * extra;
-          ok = ok && (tiles[i] + ns[i] - 1) / ns[i] >= SPLIT_MIN_PIECE;
-        }
-        for (int i = 0; i < H; ++i) ok = ok && split_cut_ok(tiles[i], ns[i]);
-        if (!ok || (lmax == 0 && tail == 0)) continue;
-        if (!fits(split_shape(tiles, ns, n_qp, 0))) continue;
-        const double take = std::min(BETTER * best_t, WORTH * whole_t);
-        const double t = makespan(tiles, ns, n_qp, n_seq, n_sm, take);
-        if (t < take) { best_t = t; best.ns = ns; best.lmax = tail == 0 ? lmax : -1; }
+    int base_ok = 0;                                       // heads before the first whose equal cut would leave a piece empty
+    for (int i = 0; i < H; ++i) {
+      base[i] = split_pieces_for(tiles[i], lmax);
+      before[i + 1] = before[i] + head_load(tiles[i], base[i], n_qp);
+      if (base_ok == i && split_cut_ok(tiles[i], base[i])) ++base_ok;
+    }
+    // the last `tail` heads in `extra` times as many pieces
+    auto attempt = [&](int extra, int tail, const Load& sum) {
+      if (sum.slots * n_seq > max_slots || sum.ctrs * n_seq * SPLIT_CTRS_PER_GROUP > max_ctrs) return;
+      const double take = std::min(BETTER * best_t, WORTH * whole_t);
+      const double t = launch.estimate(sum, take, [&] {
+        for (int i = 0; i < H; ++i) add_head(launch, tiles[i], i < H - tail ? base[i] : base[i] * extra, n_qp);
+      });
+      if (t >= take) return;
+      best_t = t;
+      best.lmax = tail == 0 ? lmax : -1;
+      best.ns = base;
+      for (int i = H - tail; i < H; ++i) best.ns[i] *= extra;
+    };
+    if (lmax > 0 && base_ok == H) attempt(1, 0, before[H]);
+    for (int extra = 2; extra <= (per_head ? 3 : 1); ++extra) {
+      Load finer;
+      for (int i = H - 1; i >= 0; --i) {
+        const int ns = base[i] * extra;
+        if ((tiles[i] + ns - 1) / ns < SPLIT_MIN_PIECE || !split_cut_ok(tiles[i], ns)) break;
+        finer = finer + head_load(tiles[i], ns, n_qp);
+        if (base_ok >= i) attempt(extra, H - i, before[i] + finer);
       }
+    }
   }
   return best;
 }
@@ -157,37 +201,60 @@ constexpr double CUT_LAUNCH = 3.0;
 void single_search(const std::vector<int>& tiles, int t_q, int n_seq, int n_sm, bool per_head, SplitChoice* choice) {
   const int H = (int)tiles.size(), n_qp = (t_q + 255) / 256, n_qt = (t_q + 127) / 128, odd = n_qt & 1;
   if (H == 0) return;
-  std::vector<ItemRun> items;
-  auto list = [&](const std::vector<int>& ns, bool lone) {
-    items.clear();
+  Launch launch{n_seq, n_sm};
+  std::vector<Load> pairs(H + 1), singles(H + 1);          // of the heads before this one: whole, and with their query tiles one by one
+  Load as_chosen;
+  for (int i = 0; i < H; ++i) {
+    const double one = TILE_SINGLE * tiles[i] + FIXED;
+    singles[i + 1] = singles[i].items_of(one, n_qt);
+    pairs[i + 1] = pairs[i].items_of(tiles[i] + FIXED, n_qp - odd).items_of(one, odd);
+    const int ns = choice->ns[i];
+    const Cut c(tiles[i], ns);
+    as_chosen = as_chosen.items_of(c.full + c.fixed, (ns - 1) * (n_qp - odd)).items_of(c.last + c.fixed, n_qp - odd);
+    if (odd)
+      as_chosen = as_chosen.items_of(TILE_PADDED * c.full + c.fixed, ns - 1).items_of(TILE_PADDED * c.last + c.fixed, 1);
+  }
+  const double chosen_t = launch.estimate(as_chosen, HUGE_VAL, [&] {
     for (int i = 0, m; i < H; i += m) {
-      for (m = 1; i + m < H && tiles[i + m] == tiles[i] && ns[i + m] == ns[i];) ++m;       // heads that are alike
-      if (ns[i] == 0) {
-        add(items, TILE_SINGLE * tiles[i] + FIXED, m * n_qt);
-        continue;
-      }
-      const int k = ns[i], piece = (tiles[i] + k - 1) / k;
-      const double fixed = FIXED + (k > 1 ? PUBLISH + MERGE_PER_PIECE * (k - 1) / k : 0.0);
-      for (int pc = 0; pc < k; ++pc) {
-        const int len = std::min(tiles[i], (pc + 1) * piece) - pc * piece;
-        if (n_qp > odd) add(items, len + fixed, m * (n_qp - odd));
-        if (odd) add(items, (lone ? TILE_SINGLE : TILE_PADDED) * len + fixed, m);
+      const int ns = choice->ns[i];
+      for (m = 1; i + m < H && tiles[i + m] == tiles[i] && choice->ns[i + m] == ns;) ++m;  // heads that are alike
+      const Cut c(tiles[i], ns);
+      for (int pc = 0; pc < ns; ++pc) {
+        const int len = pc + 1 < ns ? c.full : c.last;
+        if (n_qp > odd) launch.add(len + c.fixed, m * (n_qp - odd));
+        if (odd) launch.add(TILE_PADDED * len + c.fixed, m);
       }
     }
-  };
-  list(choice->ns, false);
+  });
   const bool is_cut = std::any_of(choice->ns.begin(), choice->ns.end(), [](int n) { return n > 1; });
-  double take = BETTER * (finish(items, n_seq, n_sm, HUGE_VAL) + (is_cut ? CUT_LAUNCH : 0.0)) - LONE_LAUNCH;
-  std::vector<int> ns(H);
+  double take = BETTER * (chosen_t + (is_cut ? CUT_LAUNCH : 0.0)) - LONE_LAUNCH;
   auto attempt = [&](int first, int last) {
-    ns.assign(H, 1);
-    std::fill(ns.begin(), ns.begin() + first, 0);
-    std::fill(ns.end() - last, ns.end(), 0);
-    list(ns, true);
-    const double t = finish(items, n_seq, n_sm, take);
+    // (a sum of differences: the bound it gives may be an ulp off, the simulation decides)
+    Load sum = singles[first];
+    const Load &mid0 = pairs[first], &mid1 = pairs[H - last], &end0 = singles[H - last], &end1 = singles[H];
+    sum.total += mid1.total - mid0.total + end1.total - end0.total;
+    sum.items += mid1.items - mid0.items + end1.items - end0.items;
+    // (heads by descending tiles: the first of each kind is the longest)
+    if (first < H - last) sum.longest = std::max(sum.longest, n_qp > odd ? tiles[first] + FIXED : TILE_SINGLE * tiles[first] + FIXED);
+    if (last > 0) sum.longest = std::max(sum.longest, TILE_SINGLE * tiles[H - last] + FIXED);
+    const double t = launch.estimate(sum, take, [&] {
+      for (int i = 0, m; i < H; i += m) {
+        const bool single = i < first || i >= H - last;
+        const int until = i < first ? first : single ? H : H - last;
+        for (m = 1; i + m < until && tiles[i + m] == tiles[i];) ++m;
+        if (single) {
+          launch.add(TILE_SINGLE * tiles[i] + FIXED, m * n_qt);
+          continue;
+        }
+        if (n_qp > odd) launch.add(tiles[i] + FIXED, m * (n_qp - odd));
+        if (odd) launch.add(TILE_SINGLE * tiles[i] + FIXED, m);
+      }
+    });
     if (t >= take) return;
     take = BETTER * t;
-    choice->lone = ns;
+    choice->lone.assign(H, 1);
+    std::fill(choice->lone.begin(), choice->lone.begin() + first, 0);
+    std::fill(choice->lone.end() - last, choice->lone.end(), 0);
   };
   attempt(H, 0);
   if (odd) attempt(0, 0);
@@ -201,18 +268,41 @@ void single_search(const std::vector<int>& tiles, int t_q, int n_seq, int n_sm, 
 
 }  // namespace heatkv
 
+static bool valid(const int32_t* tiles, int n_heads, int queries, int n_seq, int n_sm) {
+  if (!tiles || n_heads < 1 || queries < 1 || n_seq < 1 || n_sm < 1) return false;
+  for (int i = 0; i < n_heads; ++i)
+    if (tiles[i] < 1 || (i > 0 && tiles[i] > tiles[i - 1])) return false;
+  return true;
+}
+
 extern "C" int heatkv_split_plan(const int32_t* tiles, int n_heads, int n_qp, int n_seq, int n_sm, int per_head,
                                  uint64_t max_slots, uint64_t max_ctrs, int32_t* pieces, double* makespan_whole,
                                  double* makespan_cut) {
-  if (!tiles || !pieces || n_heads < 1 || n_qp < 1 || n_seq < 1 || n_sm < 1) return HEATKV_ERR_INVALID_ARG;
-  for (int i = 0; i < n_heads; ++i)
-    if (tiles[i] < 1 || (i > 0 && tiles[i] > tiles[i - 1])) return HEATKV_ERR_INVALID_ARG;
+  if (!pieces || !valid(tiles, n_heads, n_qp, n_seq, n_sm)) return HEATKV_ERR_INVALID_ARG;
   try {
     const std::vector<int> t(tiles, tiles + n_heads);
     const heatkv::SplitChoice ch = heatkv::split_search(t, n_qp, n_seq, n_sm, per_head != 0, max_slots, max_ctrs);
     for (int i = 0; i < n_heads; ++i) pieces[i] = ch.ns[i];
     if (makespan_whole) *makespan_whole = heatkv::split_makespan(t, std::vector<int>(n_heads, 1), n_qp, n_seq, n_sm);
     if (makespan_cut) *makespan_cut = heatkv::split_makespan(t, ch.ns, n_qp, n_seq, n_sm);
+  } catch (const std::bad_alloc&) {
+    return HEATKV_ERR_HOST_MEMORY;
+  }
+  return HEATKV_OK;
+}
+
+extern "C" int heatkv_lone_plan(const int32_t* tiles, int n_heads, int t_q, int n_seq, int n_sm, int per_head, uint64_t max_slots,
+                                uint64_t max_ctrs, int32_t* pieces, int32_t* singles, int32_t* lone) {
+  if (!pieces || !singles || !lone || !valid(tiles, n_heads, t_q, n_seq, n_sm)) return HEATKV_ERR_INVALID_ARG;
+  try {
+    const std::vector<int> t(tiles, tiles + n_heads);
+    heatkv::SplitChoice ch = heatkv::split_search(t, (t_q + 255) / 256, n_seq, n_sm, per_head != 0, max_slots, max_ctrs);
+    heatkv::single_search(t, t_q, n_seq, n_sm, per_head != 0, &ch);
+    *lone = !ch.lone.empty();
+    for (int i = 0; i < n_heads; ++i) {
+      pieces[i] = ch.ns[i];
+      singles[i] = *lone && ch.lone[i] == 0;
+    }
   } catch (const std::bad_alloc&) {
     return HEATKV_ERR_HOST_MEMORY;
   }

@@ -21,7 +21,7 @@ __all__ = [
     "heatkv_create", "heatkv_destroy", "heatkv_calibrate_scores", "heatkv_calibrate_scores_steps", "heatkv_calibrate_scores_static",
     "heatkv_finalize_scores", "heatkv_build_schedule", "heatkv_schedule_free", "heatkv_schedule_masks", "heatkv_schedule_footprint",
     "heatkv_schedule_plan", "heatkv_schedule_plan_fp8", "heatkv_seq_open", "heatkv_seq_close", "heatkv_append_compact", "heatkv_scale_attention",
-    "heatkv_attention_append", "heatkv_split_plan",
+    "heatkv_attention_append", "heatkv_split_plan", "heatkv_lone_plan",
     "heatkv_cache_bytes", "heatkv_retained_indices", "heatkv_export_head", "heatkv_export_head_fp8", "heatkv_allocator_stats",
     "CACHE_BF16", "CACHE_FP8_E4M3", "heatkv_launch_count", "heatkv_kernel_launches", "heatkv_pair_launches", "heatkv_lone_launches", "heatkv_rank_dispersion", "heatkv_seq_reservation",
     "KernelStats",
@@ -105,7 +105,7 @@ def exported_symbols():
             "heatkv_schedule_footprint", "heatkv_schedule_plan", "heatkv_schedule_plan_fp8", "heatkv_seq_open", "heatkv_seq_close", "heatkv_append_compact",
             "heatkv_scale_attention", "heatkv_attention_append", "heatkv_cache_bytes", "heatkv_seq_reservation",
             "heatkv_retained_indices", "heatkv_export_head", "heatkv_export_head_fp8",
-            "heatkv_attention_split", "heatkv_split_plan", "heatkv_allocator_stats", "heatkv_launch_count",
+            "heatkv_attention_split", "heatkv_split_plan", "heatkv_lone_plan", "heatkv_allocator_stats", "heatkv_launch_count",
             "heatkv_kernel_launches", "heatkv_pair_launches", "heatkv_lone_launches", "heatkv_rank_dispersion", "heatkv_selftest_wait_expiry", "heatkv_device_status",
             "heatkv_strerror"]
 
@@ -143,6 +143,8 @@ _lib.heatkv_attention_append.argtypes = [_P, C.POINTER(C.c_int), C.c_int, C.c_in
                                          C.POINTER(Strides), _P, _P, _P]
 _lib.heatkv_split_plan.argtypes = [C.POINTER(C.c_int32), C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_uint64, C.c_uint64,
                                    C.POINTER(C.c_int32), C.POINTER(C.c_double), C.POINTER(C.c_double)]
+_lib.heatkv_lone_plan.argtypes = [C.POINTER(C.c_int32), C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_uint64, C.c_uint64,
+                                  C.POINTER(C.c_int32), C.POINTER(C.c_int32), C.POINTER(C.c_int32)]
 _lib.heatkv_attention_split.argtypes = [_P, C.POINTER(C.c_int), C.c_int, C.c_int, C.c_int, C.POINTER(C.c_int32),
                                         C.POINTER(C.c_int32)]
 _lib.heatkv_cache_bytes.argtypes = [_P, C.c_int, C.POINTER(C.c_uint64), C.POINTER(C.c_uint64)]
@@ -349,6 +351,17 @@ def heatkv_split_plan(tiles, n_qp: int, n_seq: int, n_sm: int = 148, per_head: b
     _check(_lib.heatkv_split_plan(t, n, n_qp, n_seq, n_sm, int(per_head), max_slots, max_ctrs, out, C.byref(a), C.byref(b)),
            "heatkv_split_plan")
     return [int(x) for x in out], a.value, b.value
+
+
+def heatkv_lone_plan(tiles, t_q: int, n_seq: int, n_sm: int = 148, per_head: bool = True,
+                     max_slots: int = 1 << 40, max_ctrs: int = 1 << 40):
+    """(pieces per head, heads whose query tiles go one by one, does the launch take query tiles by themselves instead of cuts)."""
+    n = len(tiles)
+    t = (C.c_int32 * n)(*[int(x) for x in tiles])
+    pieces, singles, lone = (C.c_int32 * n)(), (C.c_int32 * n)(), C.c_int32()
+    _check(_lib.heatkv_lone_plan(t, n, t_q, n_seq, n_sm, int(per_head), max_slots, max_ctrs, pieces, singles, C.byref(lone)),
+           "heatkv_lone_plan")
+    return [int(x) for x in pieces], [bool(x) for x in singles], bool(lone.value)
 
 
 def heatkv_cache_bytes(ctx: int, seq_id: int):

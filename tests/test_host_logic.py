@@ -2,8 +2,10 @@
 symbols, the C++ schedule builder agrees with the oracle on identical scores, and the static
 cache plan (page tables, append targets, ragged moves) replays to exactly the cache the
 oracle defines.  No CUDA call is made."""
+import heapq
 import os
 import re
+import time
 
 import numpy as np
 import pytest
@@ -379,6 +381,91 @@ def test_split_plan_rejects_bad_input():
         hk.heatkv_split_plan([3, 5], n_qp=1, n_seq=1)       # not in dispatch (descending) order
     with pytest.raises(hk.HeatKVError):
         hk.heatkv_split_plan([4, 0], n_qp=1, n_seq=1)
+
+
+def _finish(items, n_sm):
+    """List scheduling of (cost, count) items in order: every item goes to the SM that is free first."""
+    free, end = [0.0] * n_sm, 0.0
+    for cost, n in items:
+        for _ in range(n):
+            t = heapq.heappop(free) + cost
+            heapq.heappush(free, t)
+            end = max(end, t)
+    return end
+
+
+@pytest.mark.parametrize("t_q", [1, 128, 129, 256, 257, 576, 1024, 1600])
+@pytest.mark.parametrize("per_head", [True, False])
+def test_lone_plan_follows_its_estimates(t_q, per_head):
+    """Pairs of query tiles and lone ones against a simulation of single SMs: a lone launch beats the estimate of the cut by what it has to, and
+    where the cut runs, neither all query tiles one by one nor only the odd last ones would have."""
+    import paper_2605_14877_b200 as hk
+    n_qp, n_qt = (t_q + 255) // 256, (t_q + 127) // 128
+    odd = n_qt % 2
+    rng = np.random.default_rng(t_q)
+    taken = 0
+    for _ in range(25):
+        H, n_seq = int(rng.integers(1, 20)), int(rng.integers(1, 5))
+        tiles = sorted((int(x) for x in rng.choice([4, 8, 12, 19, 34], size=H)), reverse=True)
+        pieces, singles, lone = hk.heatkv_lone_plan(tiles, t_q, n_seq, per_head=per_head)
+        assert pieces == hk.heatkv_split_plan(tiles, n_qp, n_seq, per_head=per_head)[0]
+        _pieces_valid(tiles, pieces)
+        assert lone or not any(singles)
+        assert per_head or len(set(singles)) == 1
+
+        def lone_estimate(single):
+            items = []
+            for n, one in zip(tiles, single):                       # heads that are alike lie side by side: their order is immaterial
+                if one:
+                    items.append((0.55 * n + 2, n_qt * n_seq))
+                else:
+                    items += [(n + 2.0, (n_qp - odd) * n_seq), (0.55 * n + 2, odd * n_seq)]
+            return _finish(items, 148)
+        cut = []
+        for n, k in zip(tiles, pieces):
+            full = -(-n // k)
+            for pc in range(k):
+                size, fixed = min(n, (pc + 1) * full) - pc * full, 2 + (1 + 1.5 * (k - 1) / k if k > 1 else 0.0)
+                cut += [(size + fixed, (n_qp - odd) * n_seq), (0.81 * size + fixed, odd * n_seq)]
+        bar = 0.98 * (_finish(cut, 148) + 3.0 * (max(pieces) > 1)) - 0.8
+        # (heads of one length are listed with the odd tiles behind all their pairs: the last round may come out an item longer)
+        slack = 0.55 * max(tiles) + 2 if odd else 1e-9
+        if lone:
+            taken += 1
+            assert lone_estimate(singles) < bar + slack
+        else:
+            assert lone_estimate([True] * H) >= bar - slack
+            assert not odd or lone_estimate([False] * H) >= bar - slack
+    assert taken > 0 or t_q <= 128
+
+
+def test_lone_plan_rejects_bad_input():
+    import paper_2605_14877_b200 as hk
+    for tiles, t_q in (([3, 5], 300), ([4, 0], 300), ([4, 4], 0)):
+        with pytest.raises(hk.HeatKVError):
+            hk.heatkv_lone_plan(tiles, t_q, n_seq=1)
+
+
+def test_choosing_a_launch_form_simulates_few_candidates():
+    """A new batch shape's first pass makes this choice for every step and layer.  All of it -- finer cuts per head, lone query tiles -- against
+    the few cuts of a call that mixes schedules: listing every candidate takes 1.8 to 2.8 times as long as those, listing those that a sum of
+    costs does not rule out 1.05 to 1.25 times."""
+    import paper_2605_14877_b200 as hk
+    rng = np.random.default_rng(3)
+    ratios = []
+    for t_q, top in ((400, 8), (576, 12), (1024, 18), (1600, 24)):
+        tiles = sorted((int(x) for x in rng.integers(4, top + 1, size=60)), reverse=True)
+
+        def best(per_head):
+            times = []
+            for _ in range(30):
+                t0 = time.perf_counter()
+                for _ in range(5):
+                    hk.heatkv_lone_plan(tiles, t_q, 2, per_head=per_head)
+                times.append(time.perf_counter() - t0)
+            return min(times)
+        ratios.append(best(True) / best(False))
+    assert np.mean(ratios) < 1.6, ratios
 
 
 @pytest.mark.parametrize("layout", [0, 1], ids=["ragged", "paged"])
