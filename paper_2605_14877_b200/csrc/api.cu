@@ -378,7 +378,8 @@ int pair_items(const heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, i
 // is a piece count per head: long heads are cut to a common longest run, and the heads dispatched last may be
 // cut further so that the last round of items fills the SMs.  It is cached per (schedule, step, layer, batch
 // size).  Calls that mix schedules use one longest run for all of them.  Where it is quicker the launch takes query tiles one by one
-// instead of cutting anything (unless `cuts_only`).
+// instead of cutting anything (unless `cuts_only`); a call that mixes schedules where that holds, in the same way, for as many
+// sequences of each of them, so that neither the order of a batch decides nor the shortest heads for the longest.
 void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int layer, bool cuts_only, AttnParams* p) {
   const int n_qp = (p->t_q + 255) / 256, own_slots = (p->n_own + HEATKV_PAGE_TOKENS - 1) / HEATKV_PAGE_TOKENS;
   const PlanEntry& pe0 = *ctx->plans[ctx->seqs[seq_ids[0]].plan];
@@ -387,20 +388,31 @@ void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int 
   const std::vector<int> tiles = ordered_tiles(pe0, step, layer, own_slots, p->runs);
   const int H = (int)tiles.size();
   for (int t : tiles) one_plan = one_plan && t <= 16383;          // half-tile counts travel as 16 bits
-  const uint64_t key = (pe0.uid << 24) ^ ((uint64_t)step << 20) ^ ((uint64_t)layer << 8) ^ (uint64_t)n_seq ^
-                       (one_plan ? 0ull : 1ull << 63) ^ (p->runs ? 1ull << 62 : 0ull);
   auto fits = [&](const SplitShape& sh) {
     return (uint64_t)sh.slots * n_seq <= ctx->split_slots &&
            (uint64_t)sh.ctrs * n_seq * SPLIT_CTRS_PER_GROUP <= ctx->split_ctrs;
   };
-  auto it = ctx->split_choice.find(key);
-  if (it == ctx->split_choice.end()) {
-    SplitChoice made = split_search(tiles, n_qp, n_seq, ctx->n_sm, one_plan, ctx->split_slots, ctx->split_ctrs);
-    single_search(tiles, p->t_q, n_seq, ctx->n_sm, one_plan, &made);
-    it = ctx->split_choice.emplace(key, std::move(made)).first;
+  auto choice = [&](const PlanEntry& pe) -> const SplitChoice& {
+    const uint64_t key = (pe.uid << 24) ^ ((uint64_t)step << 20) ^ ((uint64_t)layer << 8) ^ (uint64_t)n_seq ^
+                         (one_plan ? 0ull : 1ull << 63) ^ (p->runs ? 1ull << 62 : 0ull);
+    auto it = ctx->split_choice.find(key);
+    if (it == ctx->split_choice.end()) {
+      const std::vector<int> t = ordered_tiles(pe, step, layer, own_slots, p->runs);
+      SplitChoice made = split_search(t, n_qp, n_seq, ctx->n_sm, one_plan, ctx->split_slots, ctx->split_ctrs);
+      single_search(t, p->t_q, n_seq, ctx->n_sm, one_plan, &made);
+      it = ctx->split_choice.emplace(key, std::move(made)).first;
+    }
+    return it->second;
+  };
+  const SplitChoice& ch = choice(pe0);
+  bool lone = !cuts_only && !ch.lone.empty();
+  const bool all_lone = lone && ch.lone[0] == 0 && ch.lone[H - 1] == 0;
+  for (int i = 1; i < n_seq && lone && !one_plan; ++i) {
+    const int pi = ctx->seqs[seq_ids[i]].plan;
+    if (pi == ctx->seqs[seq_ids[i - 1]].plan) continue;
+    const SplitChoice& other = choice(*ctx->plans[pi]);
+    lone = !other.lone.empty() && (other.lone[0] == 0) == all_lone;
   }
-  const SplitChoice& ch = it->second;
-  const bool lone = !cuts_only && !ch.lone.empty(), all_lone = lone && ch.lone[0] == 0 && ch.lone[H - 1] == 0;
   const std::vector<int>& pieces = lone ? ch.lone : ch.ns;
   const int n_qt = (p->t_q + 127) / 128;
   SplitShape m = split_shape(tiles, pieces, n_qp, n_qt);

@@ -486,6 +486,32 @@ def test_lone_query_tiles_mixed_schedules(hk, d):
 
 
 @pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+@pytest.mark.parametrize("order", [[0, 1], [1, 0]], ids=["long_first", "short_first"])
+def test_mixed_schedules_choose_one_form_in_any_order(hk, d, order):
+    """48 units of 1024 queries: two sequences of 12 key tiles a head would run on lone query tiles, two of 8 on pairs; one of each runs on
+    pairs whichever comes first."""
+    from paper_2605_14877_b200.sweep import Session
+    H, t = 24, [512, 1024]
+    assert hk.heatkv_lone_plan([12] * H, t[1], 2, per_head=False)[2] and not hk.heatkv_lone_plan([8] * H, t[1], 2, per_head=False)[2]
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    q, k, v = (torch.randn(2, H, sum(t), d, generator=gen, device="cuda").mul_(f).bfloat16() for f in (1, 1, 0.25))
+    out = torch.zeros_like(q)
+    before = []
+    with Session(1, H, d, t, 0, pool_rows=2 * H * (sum(t) + 128), kernel=hk.KERNEL_TCGEN05) as ses:
+        schedules = [ses.schedule(policy=hk.POLICY_EXPLICIT, fraction=np.full((1, H), f)) for f in (1.0, 0.0)]
+        ids = [hk.heatkv_seq_open(ses.ctx, schedules[i]) for i in order]
+        ses.generate(ids, lambda l: (q, k, v), lambda l: out, None, lambda step, l: before.append(hk.heatkv_lone_launches(ses.ctx)))
+        torch.cuda.synchronize()
+        assert hk.heatkv_device_status(ses.ctx) == 0 and before[1] == before[0]
+        for s in schedules:
+            hk.heatkv_schedule_free(s)
+    x = q[:, :, t[0]:].double() @ k.double().transpose(2, 3) / math.sqrt(d)
+    x[order.index(1), :, :, : t[0]] = -math.inf
+    want = torch.softmax(x, dim=-1) @ v.double()
+    assert (out[:, :, t[0]:].double() - want).abs().max().item() <= ATOL_MAX
+
+
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
 @pytest.mark.parametrize("tile", [1, 2, 3])
 def test_lone_query_tiles_references_follow(hk, d, tile):
     """Heads of 18 key tiles that would be cut into pieces if their query tiles did not run one by one.  As in the test of the CTA
