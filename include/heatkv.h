@@ -373,7 +373,8 @@ int heatkv_launch_count(heatkv_ctx* ctx, uint64_t* n);
 int heatkv_kernel_launches(heatkv_ctx* ctx, heatkv_kernel_stats* out);
 /* How many of the attention_tcgen05 launches ran uncut on pairs of CTAs (attn_pair_kernel; see heatkv_attention_split). */
 int heatkv_pair_launches(heatkv_ctx* ctx, uint64_t* n);
-/* ... and of them those in which some work items are one query tile of 128 instead of two. */
+/* How many of the attention_tcgen05 launches, and of the calibration_tcgen05 launches with an attention output, had work items of one
+ * query tile of 128 instead of two (attn_tc_kernel, nothing cut).  None of them counts as a launch on pairs of CTAs. */
 int heatkv_lone_launches(heatkv_ctx* ctx, uint64_t* n);
 /* Appendix on S-CAS stability -- how much the head ordering moves between calibration sets.  scas_runs HOST
  * [n_runs][L][H][K]: S-CAS of n_runs independent calibration sets (heatkv_finalize_scores).  For every prunable

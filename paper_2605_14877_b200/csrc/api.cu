@@ -24,7 +24,7 @@ int tc_create(const heatkv_config& cfg, void* k_pool, void* v_pool, uint64_t poo
 void tc_destroy(TcState* st);
 bool tc_ready(const TcState* st);
 bool tc_supported(const TcState* st, const AttnParams& p, int d, int n_seq);
-cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int n_seq, cudaStream_t stream);
+cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int n_seq, cudaStream_t stream, bool* lone);
 bool tc_pair_wanted(const TcState* st, int t_q, int64_t items, int tiles);
 cudaError_t launch_attn_pair(TcState* st, const AttnParams& p, int n_seq, cudaStream_t stream);
 int tc_split_slot_floats(int d);
@@ -139,7 +139,7 @@ struct heatkv_ctx {
   uint64_t launches = 0, openings = 0;
   heatkv_kernel_stats kstats = {};             // launches per kernel
   uint64_t pair_launches = 0;                  // of kstats.attention_tcgen05: on pairs of CTAs
-  uint64_t lone_launches = 0;                  // ... with query tiles by themselves
+  uint64_t lone_launches = 0;                  // of attention_tcgen05 and calibration_tcgen05: with query tiles by themselves
   TcState* tc = nullptr;
   CalibTcState* calib_tc = nullptr;
   // key-range splitting of the tensor-memory attention kernel
@@ -863,10 +863,11 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
     } catch (const std::bad_alloc&) {
       return HEATKV_ERR_HOST_MEMORY;
     }
-    e = launch_attn_tc(ctx->tc, p, n_seq, stream);
+    bool lone = false;
+    e = launch_attn_tc(ctx->tc, p, n_seq, stream, &lone);
     ctx->launches += 1;
     ctx->kstats.attention_tcgen05 += 1;
-    ctx->lone_launches += p.lone != 0;
+    ctx->lone_launches += lone;
   } else {
     fill_head_table(ctx, seq_ids, n_seq, step, layer, &p);
     e = launch_attn_generic(p, ctx->cfg.d, n_seq, false, ctx->n_sm, stream);
@@ -961,7 +962,9 @@ int heatkv_calibrate_scores(heatkv_ctx* ctx, int layer, int step, int n_seq, con
     calib_tc_step_descs(ctx->calib_tc, step, &p.full_descs, &p.full_slots);
     p.n_seq = n_seq;
     p.items_per_seq = (int)items;
-    e = launch_attn_tc(ctx->tc, p, n_seq, stream);
+    bool lone = false;
+    e = launch_attn_tc(ctx->tc, p, n_seq, stream, &lone);
+    ctx->lone_launches += lone;
   } else {
     e = use_tc ? launch_calib_tc(ctx->calib_tc, p, n_seq, stream) : launch_attn_generic(p, ctx->cfg.d, n_seq, true, ctx->n_sm, stream);
   }

@@ -1311,7 +1311,7 @@ cudaError_t launch_attn_pair(TcState* st, const AttnParams& p, int n_seq, cudaSt
 
 // Attention of a scale step (p.items_per_seq work items per sequence) or, with p.full_slots > 0, calibration with an
 // attention output over all p.n_own keys of p.k_new / p.v_new.
-cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int n_seq, cudaStream_t stream) {
+cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int n_seq, cudaStream_t stream, bool* ran_lone) {
   tc::Maps maps;
   if (!encode_call(st, &maps, p, n_seq, 64)) return cudaErrorInvalidValue;
   if (p.n_seq != n_seq || p.items_per_seq < 1) return cudaErrorInvalidValue;
@@ -1339,6 +1339,7 @@ cudaError_t launch_attn_tc(TcState* st, const AttnParams& p, int n_seq, cudaStre
     lone = (cut && whole < total) || (tail_single && total > st->n_sm);
     grid = dim3((unsigned)std::min(q.attn_items, st->n_sm));
   }
+  *ran_lone = lone;
   auto launch = [&](auto kernel, uint32_t smem) { return launch_pdl(kernel, grid, tc::THREADS, smem, stream, q, maps); };
   if (st->d == 128) {
     constexpr uint32_t smem = tc::Layout<128>::SM_ALLOC;

@@ -1150,6 +1150,20 @@ def test_calibration_with_output_lone_query_tiles(hk, d, H, t):
     assert ((beta[0, :, K - 1].double() - want).abs() / want).max().item() <= 2.0 ** -20
 
 
+def test_calibration_lone_launches_are_counted(hk):
+    """Launches of calibration with an output: items of one query tile where they all run at once, pairs where those fill the SMs exactly."""
+    from paper_2605_14877_b200.sweep import Session
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    for n_seq, H, t, lone in ((1, 4, 576, 1), (n_sm, 1, 256, 0)):
+        q, k = (torch.randn(n_seq, H, t, 128, device="cuda").bfloat16() for _ in range(2))
+        out, beta = torch.zeros_like(q), torch.zeros(1, H, 1, 1, device="cuda")
+        with Session(1, H, 128, [t], 0, pool_rows=64, kernel=hk.KERNEL_TCGEN05) as ses:
+            hk.heatkv_calibrate_scores(ses.ctx, 0, 0, n_seq, q, k, k, hk.Strides.of(q, k, out), None, beta, out)
+            torch.cuda.synchronize()
+            assert hk.heatkv_device_status(ses.ctx) == 0 and hk.heatkv_kernel_launches(ses.ctx).calibration_tcgen05 == 1
+            assert hk.heatkv_lone_launches(ses.ctx) == lone and hk.heatkv_pair_launches(ses.ctx) == 0
+
+
 def test_config2_calibration_full_size(hk):
     """Sec. 3.1, Eq. 2 and Eq. 4 at the size the bench calibrates at: 13 scales, 2 sequences x 16 heads, bias on
     the current scale, automatic kernel choice (tensor-memory kernel for the seven steps of 256 tokens and more:
