@@ -348,7 +348,8 @@ def run_cache_workload(args):
 def run_few_heads_workload(args):
     """Key-range splitting on launches that cannot fill the GPU with whole heads (not the headline line):
     one sequence, 2 or 8 heads, d=128, 13 scales, full or half budget.  Every sweep is timed call by call
-    with the scratch region present (splitting allowed) and absent (whole heads only)."""
+    with the scratch region present (splitting allowed) and absent (whole heads only).  In either arm a step may take its query tiles
+    one by one or run on CTA pairs instead, which need no scratch: the scales that do are listed beside the times."""
     import paper_2605_14877_b200 as hk
     from paper_2605_14877_b200.sweep import Session
     torch.cuda.set_device(0)
@@ -366,31 +367,27 @@ def run_few_heads_workload(args):
             ses = Session(sh.L, sh.H, sh.d, sh.t, sh.s, pool_rows=2 * sh.H * (sh.c[-2] + 64 * sh.K), scratch_bytes=scratch)
             sch = ses.schedule(scas=scores, b=b)
             ms, reps = np.zeros(sh.K), max(3, min(args.steps, 20))
-            on_pairs = set()                             # steps whose launch runs uncut on CTA pairs
+            forms = [None] * sh.K                        # what each step launched
             for rep in range(reps + 2):
                 ids = [hk.heatkv_seq_open(ses.ctx, sch)]
-                if rep == 0 and scratch > 1024:
-                    res["split_tiles_per_scale"] = [hk.heatkv_attention_split(ses.ctx, ids, 0, st)[0] for st in range(sh.K)]
-                    res["ctas_per_scale"] = [hk.heatkv_attention_split(ses.ctx, ids, 0, st)[1] for st in range(sh.K)]
                 for step in range(sh.K):
                     ses.pre_step(ids, step)
-                    before = hk.heatkv_pair_launches(ses.ctx)
                     flush.fill_(1)
                     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
                     e0.record()
                     hk.heatkv_scale_attention(ses.ctx, ids, 0, step, qs[step], ks[step], vs[step], None, None, outs[step])
                     e1.record()
-                    if hk.heatkv_pair_launches(ses.ctx) > before:
-                        on_pairs.add(step)
+                    forms[step] = hk.heatkv_last_attention(ses.ctx)
                     hk.heatkv_append_compact(ses.ctx, ids, 0, step, ks[step], vs[step], None)
                     torch.cuda.synchronize()
                     if rep >= 2:
                         ms[step] += e0.elapsed_time(e1) / reps
                 hk.heatkv_seq_close(ses.ctx, ids[0])
-            res[name.replace("_ms", "_pair_scales")] = sorted(step + 1 for step in on_pairs)
+            res[name.replace("_ms", "_pair_scales")] = [i + 1 for i, f in enumerate(forms) if f.kernel == hk.ATTENTION_CTA_PAIRS]
+            res[name.replace("_ms", "_lone_scales")] = [i + 1 for i, f in enumerate(forms) if f.lone]
             if scratch > 1024:
-                for step in on_pairs:
-                    res["split_tiles_per_scale"][step], res["ctas_per_scale"][step] = 0, 2 * sh.H * -(-sh.t[step] // 256)
+                res["split_tiles_per_scale"] = [int(f.longest_piece) for f in forms]
+                res["work_items_per_scale"] = [int(f.items) for f in forms]
             res[name] = [round(float(x), 4) for x in ms]
             res[name.replace("_ms", "_sum_ms")] = round(float(ms.sum()), 4)
             assert hk.heatkv_device_status(ses.ctx) == 0
@@ -907,17 +904,10 @@ def main():
     clocks = sampler.stop()
     per_step_ms = np.array([[ke[kk][0].elapsed_time(ke[kk][1]) for kk in range(shape.K)] for ke in kern_events])
     assert hk.heatkv_device_status(ses.ctx) == 0
-    # how the tensor-memory launches cut their work (host-side report of the library's choice), and which of them ran uncut on CTA
-    # pairs (the library's count, per scale of one more sweep)
-    seen = [hk.heatkv_pair_launches(ses.ctx)]
-    sweep(after_attention=lambda: seen.append(hk.heatkv_pair_launches(ses.ctx)))
+    # the form of every scale's attention launch (the library's record, per scale of one more sweep)
+    forms = []
+    sweep(after_attention=lambda: forms.append(hk.heatkv_last_attention(ses.ctx)))
     barrier()
-    on_pairs = np.diff(seen) > 0
-    ids_ = [hk.heatkv_seq_open(ses.ctx, sch) for _ in range(n_seq)]
-    cuts = [hk.heatkv_attention_split(ses.ctx, ids_, 0, kk) for kk in range(shape.K)]
-    for i in ids_:
-        hk.heatkv_seq_close(ses.ctx, i)
-    cuts = [(0, n_seq * shape.H * -(-shape.t[kk] // 256)) if on_pairs[kk] else cuts[kk] for kk in range(shape.K)]
 
     # ---- end to end: the same step from pinned host buffers, copies inside the timed region.  Every layer's
     # Q/K/V go up and its output comes down (one pinned set serves all layers: the bytes moved are what counts).
@@ -982,9 +972,11 @@ def main():
     ks1 = hk.heatkv_kernel_launches(ses.ctx)
     if args.kernel != "generic":
         assert ks1.tcgen05_attention_ready == 1 and per_step_kernels["attention_tcgen05"] == N_LAYERS * len(tc_steps), per_step_kernels
-    pair_scales = [kk + 1 for kk in range(shape.K) if on_pairs[kk]]
-    dominant = ("tc::attn_tc_kernel<%d>%s (tcgen05.mma, TMEM accumulators, TMA gathers)"
-                % (shape.d, ", at scales %s pair::attn_pair_kernel<%d>" % (pair_scales, shape.d) if pair_scales else "")
+    pair_scales = [kk + 1 for kk in range(shape.K) if forms[kk].kernel == hk.ATTENTION_CTA_PAIRS]
+    lone_scales = [kk + 1 for kk in range(shape.K) if forms[kk].lone]
+    dominant = ("tc::attn_tc_kernel<%d>%s%s (tcgen05.mma, TMEM accumulators, TMA gathers)"
+                % (shape.d, ", at scales %s its form with single query tiles" % lone_scales if lone_scales else "",
+                   ", at scales %s pair::attn_pair_kernel<%d>" % (pair_scales, shape.d) if pair_scales else "")
                 if per_step_kernels["attention_tcgen05"] else "attn_generic_kernel<%d> (mma.sync)" % shape.d)
     cache_update = None
     if rank == 0 and world == 1 and args.layout == "paged":
@@ -1019,9 +1011,10 @@ def main():
         "image_pairs_per_s_one_layer": value * N_LAYERS,
         "effective_kv_tb_per_s": uncompressed_kv_bytes / (float(attn_ms.sum()) * 1e-3) / 1e12,
         "attention_ms_per_scale": [round(float(x), 5) for x in attn_ms],
-        "work_items_per_scale": [int(c[1]) for c in cuts],
-        "longest_piece_tiles_per_scale": [int(c[0]) for c in cuts],
+        "work_items_per_scale": [int(f.items) for f in forms],            # 0: warp-level kernel
+        "longest_piece_tiles_per_scale": [int(f.longest_piece) for f in forms],
         "cta_pair_scales": pair_scales,
+        "lone_tile_scales": lone_scales,
         "attention_tflops_per_scale": [round(flops[kk] / (float(attn_ms[kk]) * 1e-3) / 1e12, 1) for kk in range(shape.K)],
         "attention_algorithmic_gb_per_s_per_scale": [round(by[kk] / (float(attn_ms[kk]) * 1e-3) / 1e9, 1) for kk in range(shape.K)],
         "attention_tflops_all_scales": sum(flops) / (float(attn_ms.sum()) * 1e-3) / 1e12,

@@ -123,6 +123,21 @@ typedef struct {                 /* which kernels a context has launched so far 
   uint64_t other;                /* small helper kernels (fixed-order reduction of the static-scratch call) */
 } heatkv_kernel_stats;
 
+/* The form in which an attention call was launched (heatkv_last_attention). */
+typedef enum heatkv_attention_kernel {
+  HEATKV_ATTENTION_NONE = 0,           /* no attention call has been launched yet                               */
+  HEATKV_ATTENTION_GENERIC = 1,        /* warp-level kernels; the other fields are 0                            */
+  HEATKV_ATTENTION_TCGEN05 = 2,        /* attn_tc_kernel                                                        */
+  HEATKV_ATTENTION_CTA_PAIRS = 3       /* attn_pair_kernel: whole heads, 256 queries an item                    */
+} heatkv_attention_kernel;
+typedef struct heatkv_attention_form {
+  int32_t kernel;          /* heatkv_attention_kernel                                                               */
+  int32_t items;           /* work items of the launch (an upper bound where the call mixes schedules)              */
+  int32_t longest_piece;   /* key tiles of the longest piece of a head that was cut (0: none was; where the call
+                              mixes schedules the longest run a piece may have)                                     */
+  int32_t lone;            /* 1: some items are one query tile of 128, the others a pair of them, and nothing is cut */
+} heatkv_attention_form;
+
 typedef struct {
   uint64_t pool_rows;            /* rows (tokens) the K pool and the V pool can hold        */
   uint64_t reserved_rows;        /* rows reserved by open sequences                         */
@@ -319,9 +334,9 @@ int heatkv_attention_append(heatkv_ctx* ctx, const int* seq_ids /*HOST*/, int n_
  * call mixes schedules).  A cut head's pieces leave partial results in the arena's scratch region, where
  * the last to arrive merges them.  The choice (a piece count per head) minimises an estimate of the launch's
  * makespan over the SMs and is cached per (schedule, step, layer, batch size).  A launch of few and short items (at most one per
- * two SMs, 16 key tiles, of 64-wide heads 12) runs uncut on pairs of CTAs instead, so there the figures only say what that saves;
- * heatkv_pair_launches tells.  One whose items would leave SMs idle may also take query tiles of 128 one by one, with whole key
- * ranges, instead of in pairs (its own items are not counted here; heatkv_lone_launches tells).  Host only. */
+ * two SMs, 16 key tiles, of 64-wide heads 12) runs uncut on pairs of CTAs instead, so there the figures only say what that saves.
+ * One whose items would leave SMs idle may also take query tiles of 128 one by one, with whole key
+ * ranges, instead of in pairs (its own items are not counted here).  heatkv_last_attention has what a launch did.  Host only. */
 int heatkv_attention_split(heatkv_ctx* ctx, const int* seq_ids /*HOST*/, int n_seq, int layer, int step,
                            int32_t* split_tiles, int32_t* items);
 
@@ -376,6 +391,8 @@ int heatkv_pair_launches(heatkv_ctx* ctx, uint64_t* n);
 /* How many of the attention_tcgen05 launches, and of the calibration_tcgen05 launches with an attention output, had work items of one
  * query tile of 128 instead of two (attn_tc_kernel, nothing cut).  None of them counts as a launch on pairs of CTAs. */
 int heatkv_lone_launches(heatkv_ctx* ctx, uint64_t* n);
+/* What the context's last attention call (heatkv_scale_attention, heatkv_attention_append) launched. */
+int heatkv_last_attention(heatkv_ctx* ctx, heatkv_attention_form* out);
 /* Appendix on S-CAS stability -- how much the head ordering moves between calibration sets.  scas_runs HOST
  * [n_runs][L][H][K]: S-CAS of n_runs independent calibration sets (heatkv_finalize_scores).  For every prunable
  * source scale k (s <= k <= K-2, 0-based) each run ranks the L*H heads by ascending S-CAS (ties by ascending

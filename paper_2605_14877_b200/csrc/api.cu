@@ -140,6 +140,7 @@ struct heatkv_ctx {
   heatkv_kernel_stats kstats = {};             // launches per kernel
   uint64_t pair_launches = 0;                  // of kstats.attention_tcgen05: on pairs of CTAs
   uint64_t lone_launches = 0;                  // of attention_tcgen05 and calibration_tcgen05: with query tiles by themselves
+  heatkv_attention_form last_attention = {};   // of the call before
   TcState* tc = nullptr;
   CalibTcState* calib_tc = nullptr;
   // key-range splitting of the tensor-memory attention kernel
@@ -857,6 +858,7 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
     ctx->launches += 1;
     ctx->kstats.attention_tcgen05 += 1;
     ctx->pair_launches += 1;
+    ctx->last_attention = {HEATKV_ATTENTION_CTA_PAIRS, items, 0, 0};
   } else if (use_tc) {
     try {
       choose_split(ctx, seq_ids, n_seq, step, layer, false, &p);
@@ -868,11 +870,13 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
     ctx->launches += 1;
     ctx->kstats.attention_tcgen05 += 1;
     ctx->lone_launches += lone;
+    ctx->last_attention = {HEATKV_ATTENTION_TCGEN05, p.items_per_seq * n_seq, p.longest_piece, lone};
   } else {
     fill_head_table(ctx, seq_ids, n_seq, step, layer, &p);
     e = launch_attn_generic(p, ctx->cfg.d, n_seq, false, ctx->n_sm, stream);
     ctx->launches += 1;
     ctx->kstats.attention_generic += 1;
+    ctx->last_attention = {HEATKV_ATTENTION_GENERIC, 0, 0, 0};
   }
   if (e != cudaSuccess) return HEATKV_ERR_CUDA;
   if (!with_update) return HEATKV_OK;
@@ -1378,6 +1382,12 @@ int heatkv_pair_launches(heatkv_ctx* ctx, uint64_t* n) {
 int heatkv_lone_launches(heatkv_ctx* ctx, uint64_t* n) {
   if (!ctx || !n) return HEATKV_ERR_INVALID_ARG;
   *n = ctx->lone_launches;
+  return HEATKV_OK;
+}
+
+int heatkv_last_attention(heatkv_ctx* ctx, heatkv_attention_form* out) {
+  if (!ctx || !out) return HEATKV_ERR_INVALID_ARG;
+  *out = ctx->last_attention;
   return HEATKV_OK;
 }
 

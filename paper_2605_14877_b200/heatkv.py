@@ -23,8 +23,8 @@ __all__ = [
     "heatkv_schedule_plan", "heatkv_schedule_plan_fp8", "heatkv_seq_open", "heatkv_seq_close", "heatkv_append_compact", "heatkv_scale_attention",
     "heatkv_attention_append", "heatkv_split_plan", "heatkv_lone_plan",
     "heatkv_cache_bytes", "heatkv_retained_indices", "heatkv_export_head", "heatkv_export_head_fp8", "heatkv_allocator_stats",
-    "CACHE_BF16", "CACHE_FP8_E4M3", "heatkv_launch_count", "heatkv_kernel_launches", "heatkv_pair_launches", "heatkv_lone_launches", "heatkv_rank_dispersion", "heatkv_seq_reservation",
-    "KernelStats",
+    "CACHE_BF16", "CACHE_FP8_E4M3", "heatkv_launch_count", "heatkv_kernel_launches", "heatkv_pair_launches", "heatkv_lone_launches", "heatkv_last_attention", "heatkv_rank_dispersion", "heatkv_seq_reservation",
+    "KernelStats", "AttentionForm", "ATTENTION_NONE", "ATTENTION_GENERIC", "ATTENTION_TCGEN05", "ATTENTION_CTA_PAIRS",
     "heatkv_selftest_wait_expiry", "heatkv_device_status", "heatkv_strerror", "heatkv_attention_split", "arena_bytes_for",
 ]
 
@@ -93,6 +93,13 @@ class KernelStats(C.Structure):
                 ("append", C.c_uint64), ("compact", C.c_uint64), ("other", C.c_uint64)]
 
 
+ATTENTION_NONE, ATTENTION_GENERIC, ATTENTION_TCGEN05, ATTENTION_CTA_PAIRS = 0, 1, 2, 3
+
+
+class AttentionForm(C.Structure):
+    _fields_ = [("kernel", C.c_int32), ("items", C.c_int32), ("longest_piece", C.c_int32), ("lone", C.c_int32)]
+
+
 def lib_path() -> str:
     return os.path.join(os.path.dirname(os.path.abspath(__file__)), "libheatkv.so")
 
@@ -106,7 +113,7 @@ def exported_symbols():
             "heatkv_scale_attention", "heatkv_attention_append", "heatkv_cache_bytes", "heatkv_seq_reservation",
             "heatkv_retained_indices", "heatkv_export_head", "heatkv_export_head_fp8",
             "heatkv_attention_split", "heatkv_split_plan", "heatkv_lone_plan", "heatkv_allocator_stats", "heatkv_launch_count",
-            "heatkv_kernel_launches", "heatkv_pair_launches", "heatkv_lone_launches", "heatkv_rank_dispersion", "heatkv_selftest_wait_expiry", "heatkv_device_status",
+            "heatkv_kernel_launches", "heatkv_pair_launches", "heatkv_lone_launches", "heatkv_last_attention", "heatkv_rank_dispersion", "heatkv_selftest_wait_expiry", "heatkv_device_status",
             "heatkv_strerror"]
 
 
@@ -155,6 +162,7 @@ _lib.heatkv_allocator_stats.argtypes = [_P, C.POINTER(AllocStats)]
 _lib.heatkv_launch_count.argtypes = [_P, C.POINTER(C.c_uint64)]
 _lib.heatkv_pair_launches.argtypes = [_P, C.POINTER(C.c_uint64)]
 _lib.heatkv_lone_launches.argtypes = [_P, C.POINTER(C.c_uint64)]
+_lib.heatkv_last_attention.argtypes = [_P, C.POINTER(AttentionForm)]
 _lib.heatkv_device_status.argtypes = [_P, _P]
 _lib.heatkv_selftest_wait_expiry.argtypes = [_P, _P]
 _lib.heatkv_kernel_launches.argtypes = [_P, C.POINTER(KernelStats)]
@@ -423,6 +431,13 @@ def heatkv_lone_launches(ctx: int) -> int:
     n = C.c_uint64()
     _check(_lib.heatkv_lone_launches(ctx, C.byref(n)), "heatkv_lone_launches")
     return n.value
+
+
+def heatkv_last_attention(ctx: int) -> AttentionForm:
+    """The form in which the context's last attention call was launched."""
+    f = AttentionForm()
+    _check(_lib.heatkv_last_attention(ctx, C.byref(f)), "heatkv_last_attention")
+    return f
 
 
 def heatkv_rank_dispersion(scas_runs, s: int) -> np.ndarray:

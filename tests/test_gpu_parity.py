@@ -779,6 +779,66 @@ def test_small_scratch_cuts_are_launched(hk):
     assert got[0] == got[1] and got[0][0] > 0
 
 
+def _launch_forms(hk, t, H, d, n_seq=1, bias=None, fractions=None, cache="bf16", layout="paged", token_major=False, shared=False,
+                  scratch_bytes=1 << 26, fused=True):
+    """One generation of a single layer over scales of t tokens on the tensor-memory kernels, every output against attention in 64 bits
+    (fp8 cache: over the rows as the oracle's quantiser gives them back); returns how each step was launched, and the outputs."""
+    from paper_2605_14877_b200.sweep import Session
+    K, c = len(t), np.cumsum([0] + list(t))
+    gen = torch.Generator(device="cuda").manual_seed(sum(t) + H)
+
+    def rows(f):
+        n = 1 if shared else n_seq
+        x = torch.randn((n, c[-1], H, d) if token_major else (n, H, c[-1], d), generator=gen, device="cuda").mul_(f).bfloat16()
+        x = x.transpose(1, 2) if token_major else x
+        return x.expand(n_seq, -1, -1, -1) if shared else x
+    q, k, v = (rows(f) for f in (1, 1, 0.25))
+    out, forms = torch.zeros(n_seq, H, c[-1], d, dtype=torch.bfloat16, device="cuda"), []
+    with Session(1, H, d, t, 0, pool_rows=n_seq * H * (c[-2] + 64 * K), kernel=hk.KERNEL_TCGEN05, scratch_bytes=scratch_bytes,
+                 layout=hk.LAYOUT_RAGGED if layout == "ragged" else hk.LAYOUT_PAGED,
+                 cache_dtype=hk.CACHE_FP8_E4M3 if cache == "fp8" else hk.CACHE_BF16) as ses:
+        sch = ses.schedule(policy=hk.POLICY_EXPLICIT, fraction=np.ones((1, H)) if fractions is None else np.array([fractions]))
+        mask = hk.heatkv_schedule_masks(sch, K, 1, H)[0][:, 0]
+        ids = [hk.heatkv_seq_open(ses.ctx, sch) for _ in range(n_seq)]
+        ses.generate(ids, lambda l: (q, k, v), lambda l: out, None if bias is None else lambda l, step: bias[step],
+                     lambda step, l: forms.append(hk.heatkv_last_attention(ses.ctx)), fused=fused)
+        torch.cuda.synchronize()
+        assert hk.heatkv_device_status(ses.ctx) == 0
+        hk.heatkv_schedule_free(sch)
+    kept = [k.double(), v.double()]
+    if cache == "fp8":
+        flat = lambda x: x.reshape(-1, d).cpu().numpy()
+        kept = [torch.from_numpy(O.dequantize_rows_e4m3(*O.quantize_rows_e4m3(flat(x)))).cuda().reshape(x.shape) for x in kept]
+    scale_of = torch.from_numpy(np.repeat(np.arange(K), t)).cuda()
+    for step in range(K):
+        lo, hi = c[step], c[step + 1]
+        ks, vs = (torch.cat([x[:, :, :lo], y[:, :, lo:hi].double()], 2) for x, y in zip(kept, (k, v)))
+        x = q[:, :, lo:hi].double() @ ks.transpose(2, 3) / math.sqrt(d)
+        if bias is not None:
+            x += bias[step].double()[:, scale_of[:hi]][:, None]
+        for h in range(H):
+            seen = torch.tensor([s == step or bool(mask[step, h] >> s & 1) for s in range(K)], device="cuda")
+            x[:, h, :, ~seen[scale_of[:hi]]] = -math.inf
+        want = torch.softmax(x, dim=-1) @ vs
+        assert (out[:, :, lo:hi].double() - want).abs().max().item() <= ATOL_MAX, step
+    return forms, out
+
+
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+@pytest.mark.parametrize("H,n_seq,t", [(2, 1, [1280, 1024]), (4, 1, [640, 1600]), (3, 2, [1280, 1600])])
+def test_cut_heads_are_launched_cut(hk, d, H, n_seq, t):
+    """Launches whose heads do run in pieces (a reported cut may give way to CTA pairs or to lone query tiles): with much scratch and
+    with little, the same pieces and the same bits each time."""
+    outs = []
+    for scratch in (1 << 26, 1 << 26, 1 << 25):
+        forms, out = _launch_forms(hk, t, H, d, n_seq=n_seq, scratch_bytes=scratch)
+        f, tiles = forms[1], -(-sum(t) // 128)
+        assert f.kernel == hk.ATTENTION_TCGEN05 and not f.lone
+        assert 0 < f.longest_piece < tiles and f.items > n_seq * H * -(-t[1] // 256)
+        outs.append(out)
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+
+
 def test_split_heads_are_reproducible_bit_for_bit(hk):
     """Pieces of a cut head are merged in piece order whichever arrives last: the same generation run four
     times gives identical output bits (steps of this workload are cut, see the test above)."""
