@@ -839,6 +839,36 @@ def test_cut_heads_are_launched_cut(hk, d, H, n_seq, t):
     assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
 
 
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+@pytest.mark.parametrize("case", ["bias", "fp8", "fp8_bias", "ragged", "token_major", "shared", "last_tiles_bias", "last_tiles_fp8"])
+def test_lone_query_tiles_in_every_form_of_call(hk, d, case):
+    """Launches on single query tiles (28 heads of 11 key tiles) and on pairs beside odd last ones (150 of 9 key tiles): with a bias per scale, from
+    the fp8 cache's staging rows, in the ragged layout, for activations as [token, head] and for sequences that share theirs."""
+    H, n_seq, t = (30, 5, [256, 512, 384]) if "last" in case else (14, 2, [256, 512, 576])
+    bias = None
+    if "bias" in case:
+        gen = torch.Generator(device="cuda").manual_seed(7)
+        bias = 4 * torch.rand(3, H, 3, generator=gen, device="cuda")
+    forms, _ = _launch_forms(hk, t, H, d, n_seq=n_seq, bias=bias, cache="fp8" if "fp8" in case else "bf16",
+                             layout="ragged" if case == "ragged" else "paged", token_major=case == "token_major",
+                             shared=case == "shared", fused=case != "ragged")
+    assert forms[2].kernel == hk.ATTENTION_TCGEN05 and forms[2].lone and forms[2].longest_piece == 0
+    assert forms[2].items == n_seq * H * (2 if "last" in case else 5)
+
+
+@pytest.mark.parametrize("d", [128, 64], ids=["d128", "d64"])
+@pytest.mark.parametrize("first", [0, 1], ids=["first_warpgroup", "second_warpgroup"])
+def test_lone_query_tiles_with_one_warpgroups_keys_masked(hk, d, first):
+    """One query tile of 100 rows over key tiles of one scale each: a bias of minus infinity on every second one leaves one of the two
+    warpgroups without a key, the step's own rows are the other's.  The last head sees all."""
+    H, t = 4, [128] * (3 + first) + [100]
+    K = len(t)
+    bias = torch.zeros(K, H, K, device="cuda")
+    bias[-1, : H - 1, first: K - 1: 2] = -math.inf
+    forms, _ = _launch_forms(hk, t, H, d, bias=bias)
+    assert forms[-1].lone and forms[-1].items == H
+
+
 def test_split_heads_are_reproducible_bit_for_bit(hk):
     """Pieces of a cut head are merged in piece order whichever arrives last: the same generation run four
     times gives identical output bits (steps of this workload are cut, see the test above)."""
