@@ -17,7 +17,7 @@ cudaError_t launch_calibrate_static(const AttnParams& p, int d, int n_seq, cudaS
 cudaError_t launch_append(const CopyParams& p, int n_seq, cudaStream_t stream);
 cudaError_t launch_compact(const CopyParams& p, int n_seq, cudaStream_t stream);
 cudaError_t launch_append_fp8(const CopyParams& p, int n_seq, cudaStream_t stream);
-cudaError_t launch_stage_fp8(const CopyParams& p, int n_seq, int slots, bool update, cudaStream_t stream);
+cudaError_t launch_stage_fp8(const CopyParams& p, int n_seq, int slots, bool update, int n_sm, cudaStream_t stream);
 bool attn_is_small(int t_q, int64_t units, int n_sm);
 struct TcState;
 int tc_create(const heatkv_config& cfg, void* k_pool, void* v_pool, uint64_t pool_rows, TcState** out);
@@ -820,7 +820,7 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
       cp.t_k = ctx->cfg.t[step];
     }
     if (!p.direct8 && (slots > 0 || updated)) {
-      if (launch_stage_fp8(cp, n_seq, slots, updated, stream) != cudaSuccess) return HEATKV_ERR_CUDA;
+      if (launch_stage_fp8(cp, n_seq, slots, updated, ctx->n_sm, stream) != cudaSuccess) return HEATKV_ERR_CUDA;
       ctx->launches += 1;
       ctx->kstats.other += 1;
     }

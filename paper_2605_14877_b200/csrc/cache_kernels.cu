@@ -146,12 +146,12 @@ cudaError_t launch_append_fp8(const CopyParams& p, int n_seq, cudaStream_t strea
 
 // `slots` = the largest number of visible half-tiles any sequence of the call has at (step, layer); `update` = the step's
 // rows (p.k_new, p.v_new) are stored too
-cudaError_t launch_stage_fp8(const CopyParams& p, int n_seq, int slots, bool update, cudaStream_t stream) {
+cudaError_t launch_stage_fp8(const CopyParams& p, int n_seq, int slots, bool update, int n_sm, cudaStream_t stream) {
   const int64_t tiles = update ? (p.t_k + HEATKV_PAGE_TOKENS - 1) / HEATKV_PAGE_TOKENS + 1 : 0;
   const int64_t ctas = (int64_t)slots * n_seq * 2 + tiles * p.H * n_seq;
   if (ctas < 1) return cudaSuccess;
   if (ctas > INT32_MAX) return cudaErrorInvalidValue;
-  if (ctas <= 1480) stage_fp8_kernel<true><<<(unsigned)ctas, CP_THREADS, 0, stream>>>(p, slots, n_seq);
+  if (ctas <= 10 * n_sm) stage_fp8_kernel<true><<<(unsigned)ctas, CP_THREADS, 0, stream>>>(p, slots, n_seq);
   else stage_fp8_kernel<false><<<(unsigned)ctas, CP_THREADS, 0, stream>>>(p, slots, n_seq);
   return cudaGetLastError();
 }
