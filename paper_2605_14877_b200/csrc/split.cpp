@@ -27,7 +27,7 @@ SplitShape split_shape(const std::vector<int>& tiles, const std::vector<int>& ns
 // as many items at once as it has SMs.  The searches look at a thousand launches of hundreds of items on the way of a model's first
 // image, so a candidate's total and longest item come from sums per head, and its items are only listed and simulated (in buffers that
 // the whole search shares) where that bound is below the best so far: both searches for every step and layer of a pair of images at 20x
-// (16 heads, 4 layers) take 0.32 ms where listing every candidate took 1.4, with 32 heads of 64 (2 layers) 0.26 and 1.9.
+// (16 heads, 4 layers) take 0.49 ms where listing every candidate took 1.55, with 32 heads of 64 (2 layers) 0.45 and 2.1.
 constexpr double FIXED = 2.0, PUBLISH = 1.0, MERGE_PER_PIECE = 1.5;
 constexpr size_t SIMULATED_ITEMS = 8192;
 struct ItemRun {
@@ -194,6 +194,9 @@ SplitChoice split_search(const std::vector<int>& tiles, int n_qp, int n_seq, int
 // longer than their estimate by what the last piece's way through memory takes and no other item hides (14 launches of 80 to
 // 288 items: whole heads and lone tiles 1.58 us per unit and 2.3, cuts 3.4 to 5.8 us more): 102 items of 256 queries, 30 of 12 tiles, cut
 // in three 20.6 us, lone 15.9; 32 heads x 1024 queries, 4 of 19 tiles, cut in two 27.4, lone 22.6.
+// Items are simulated in the kernel's own order, head by head: with the odd last tiles of equal heads behind all their pairs the estimate was
+// up to a third too short, and 72 heads x 576 queries over 25 key tiles ran lone in 82.9 us (64-wide 74.7) where cut heads take 72.3 (62.0);
+// now 72.5 (61.4), over 15 tiles 54.0 -> 47.2, 136 heads 89.5 -> 76.5.
 constexpr double TILE_SINGLE = 0.55;        // a key tile of such an item
 constexpr double TILE_PADDED = 0.81;        // of a lone query tile run as the first of a pair
 constexpr double LONE_LAUNCH = 0.8;         // a kernel of its own: its code is fetched anew between launches of the other
@@ -215,14 +218,13 @@ void single_search(const std::vector<int>& tiles, int t_q, int n_seq, int n_sm, 
       as_chosen = as_chosen.items_of(TILE_PADDED * c.full + c.fixed, ns - 1).items_of(TILE_PADDED * c.last + c.fixed, 1);
   }
   const double chosen_t = launch.estimate(as_chosen, HUGE_VAL, [&] {
-    for (int i = 0, m; i < H; i += m) {
+    for (int i = 0; i < H; ++i) {
       const int ns = choice->ns[i];
-      for (m = 1; i + m < H && tiles[i + m] == tiles[i] && choice->ns[i + m] == ns;) ++m;  // heads that are alike
       const Cut c(tiles[i], ns);
       for (int pc = 0; pc < ns; ++pc) {
         const int len = pc + 1 < ns ? c.full : c.last;
-        if (n_qp > odd) launch.add(len + c.fixed, m * (n_qp - odd));
-        if (odd) launch.add(TILE_PADDED * len + c.fixed, m);
+        if (n_qp > odd) launch.add(len + c.fixed, n_qp - odd);
+        if (odd) launch.add(TILE_PADDED * len + c.fixed, 1);
       }
     }
   });
@@ -238,16 +240,13 @@ void single_search(const std::vector<int>& tiles, int t_q, int n_seq, int n_sm, 
     if (first < H - last) sum.longest = std::max(sum.longest, n_qp > odd ? tiles[first] + FIXED : TILE_SINGLE * tiles[first] + FIXED);
     if (last > 0) sum.longest = std::max(sum.longest, TILE_SINGLE * tiles[H - last] + FIXED);
     const double t = launch.estimate(sum, take, [&] {
-      for (int i = 0, m; i < H; i += m) {
-        const bool single = i < first || i >= H - last;
-        const int until = i < first ? first : single ? H : H - last;
-        for (m = 1; i + m < until && tiles[i + m] == tiles[i];) ++m;
-        if (single) {
-          launch.add(TILE_SINGLE * tiles[i] + FIXED, m * n_qt);
+      for (int i = 0; i < H; ++i) {
+        if (i < first || i >= H - last) {
+          launch.add(TILE_SINGLE * tiles[i] + FIXED, n_qt);
           continue;
         }
-        if (n_qp > odd) launch.add(tiles[i] + FIXED, m * (n_qp - odd));
-        if (odd) launch.add(TILE_SINGLE * tiles[i] + FIXED, m);
+        if (n_qp > odd) launch.add(tiles[i] + FIXED, n_qp - odd);
+        if (odd) launch.add(TILE_SINGLE * tiles[i] + FIXED, 1);
       }
     });
     if (t >= take) return;
