@@ -354,11 +354,11 @@ int heatkv_split_plan(const int32_t* tiles /*HOST*/, int n_heads, int n_qp, int 
                       double* makespan_cut);
 
 /* The whole choice of such a launch: the search above, then whether query tiles one by one are quicker (pure host code as well).
- * t_q: the step's queries.  pieces[0..n_heads) as heatkv_split_plan; *lone = 1 when the launch cuts nothing and takes some query tiles
+ * t_q: the step's queries, d: the head dimension (64 or 128).  pieces[0..n_heads) as heatkv_split_plan; *lone = 1 when the launch cuts nothing and takes some query tiles
  * of 128 by themselves, 0 when the cut runs; singles[0..n_heads) = 1 for the heads whose query tiles all go one by one (0 for the
  * others: pairs of query tiles, and an odd last one by itself).  Errors: as heatkv_split_plan. */
-int heatkv_lone_plan(const int32_t* tiles /*HOST*/, int n_heads, int t_q, int n_seq, int n_sm, int per_head, uint64_t max_slots,
-                     uint64_t max_ctrs, int32_t* pieces /*HOST*/, int32_t* singles /*HOST*/, int32_t* lone);
+int heatkv_lone_plan(const int32_t* tiles /*HOST*/, int n_heads, int t_q, int n_seq, int n_sm, int d, int per_head,
+                     uint64_t max_slots, uint64_t max_ctrs, int32_t* pieces /*HOST*/, int32_t* singles /*HOST*/, int32_t* lone);
 
 /* Introspection (host state only unless noted). */
 /* (With the fp8 cache a row counts d + 1 bytes instead of 2 d in both figures.)

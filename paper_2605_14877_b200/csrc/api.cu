@@ -400,7 +400,7 @@ void choose_split(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int step, int 
     if (it == ctx->split_choice.end()) {
       const std::vector<int> t = ordered_tiles(pe, step, layer, own_slots, p->runs);
       SplitChoice made = split_search(t, n_qp, n_seq, ctx->n_sm, one_plan, ctx->split_slots, ctx->split_ctrs);
-      single_search(t, p->t_q, n_seq, ctx->n_sm, one_plan, &made);
+      single_search(t, p->t_q, n_seq, ctx->n_sm, ctx->cfg.d, one_plan, &made);
       it = ctx->split_choice.emplace(key, std::move(made)).first;
     }
     return it->second;

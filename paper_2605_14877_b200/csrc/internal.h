@@ -108,7 +108,7 @@ SplitShape split_shape(const std::vector<int>& tiles, const std::vector<int>& ns
 double split_makespan(const std::vector<int>& tiles, const std::vector<int>& ns, int n_qp, int n_seq, int n_sm);
 SplitChoice split_search(const std::vector<int>& tiles, int n_qp, int n_seq, int n_sm, bool per_head, uint64_t max_slots,
                          uint64_t max_ctrs);
-void single_search(const std::vector<int>& tiles, int t_q, int n_seq, int n_sm, bool per_head, SplitChoice* choice);
+void single_search(const std::vector<int>& tiles, int t_q, int n_seq, int n_sm, int d, bool per_head, SplitChoice* choice);
 
 int build_schedule(const heatkv_config& cfg, const double* scas, const double* cas, int policy,
                    int accounting, double b, const double* fraction, Schedule* out);

@@ -200,8 +200,10 @@ SplitChoice split_search(const std::vector<int>& tiles, int n_qp, int n_seq, int
 constexpr double TILE_SINGLE = 0.55;        // a key tile of such an item
 constexpr double TILE_PADDED = 0.81;        // of a lone query tile run as the first of a pair
 constexpr double LONE_LAUNCH = 0.8;         // a kernel of its own: its code is fetched anew between launches of the other
-constexpr double CUT_LAUNCH = 3.0;
-void single_search(const std::vector<int>& tiles, int t_q, int n_seq, int n_sm, bool per_head, SplitChoice* choice) {
+// Of 64-wide heads cuts are that much longer by 1.7 units, not by 3 (152 launches under 45 units against 130 of whole heads, 1.28 us a unit; lone
+// ones 0.2 shorter than those; 128-wide: 3.3, 1.66 us, 0.4 longer), cold launches the same within 0.5.
+constexpr double CUT_LAUNCH_128 = 3.0, CUT_LAUNCH_64 = 1.7;
+void single_search(const std::vector<int>& tiles, int t_q, int n_seq, int n_sm, int d, bool per_head, SplitChoice* choice) {
   const int H = (int)tiles.size(), n_qp = (t_q + 255) / 256, n_qt = (t_q + 127) / 128, odd = n_qt & 1;
   if (H == 0) return;
   Launch launch{n_seq, n_sm};
@@ -229,7 +231,7 @@ void single_search(const std::vector<int>& tiles, int t_q, int n_seq, int n_sm, 
     }
   });
   const bool is_cut = std::any_of(choice->ns.begin(), choice->ns.end(), [](int n) { return n > 1; });
-  double take = BETTER * (chosen_t + (is_cut ? CUT_LAUNCH : 0.0)) - LONE_LAUNCH;
+  double take = BETTER * (chosen_t + (!is_cut ? 0.0 : d == 64 ? CUT_LAUNCH_64 : CUT_LAUNCH_128)) - LONE_LAUNCH;
   auto attempt = [&](int first, int last) {
     // (a sum of differences: the bound it gives may be an ulp off, the simulation decides)
     Load sum = singles[first];
@@ -290,13 +292,14 @@ extern "C" int heatkv_split_plan(const int32_t* tiles, int n_heads, int n_qp, in
   return HEATKV_OK;
 }
 
-extern "C" int heatkv_lone_plan(const int32_t* tiles, int n_heads, int t_q, int n_seq, int n_sm, int per_head, uint64_t max_slots,
-                                uint64_t max_ctrs, int32_t* pieces, int32_t* singles, int32_t* lone) {
-  if (!pieces || !singles || !lone || !valid(tiles, n_heads, t_q, n_seq, n_sm)) return HEATKV_ERR_INVALID_ARG;
+extern "C" int heatkv_lone_plan(const int32_t* tiles, int n_heads, int t_q, int n_seq, int n_sm, int d, int per_head,
+                                uint64_t max_slots, uint64_t max_ctrs, int32_t* pieces, int32_t* singles, int32_t* lone) {
+  if (!pieces || !singles || !lone || (d != 64 && d != 128) || !valid(tiles, n_heads, t_q, n_seq, n_sm))
+    return HEATKV_ERR_INVALID_ARG;
   try {
     const std::vector<int> t(tiles, tiles + n_heads);
     heatkv::SplitChoice ch = heatkv::split_search(t, (t_q + 255) / 256, n_seq, n_sm, per_head != 0, max_slots, max_ctrs);
-    heatkv::single_search(t, t_q, n_seq, n_sm, per_head != 0, &ch);
+    heatkv::single_search(t, t_q, n_seq, n_sm, d, per_head != 0, &ch);
     *lone = !ch.lone.empty();
     for (int i = 0; i < n_heads; ++i) {
       pieces[i] = ch.ns[i];

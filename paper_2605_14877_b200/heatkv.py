@@ -150,7 +150,7 @@ _lib.heatkv_attention_append.argtypes = [_P, C.POINTER(C.c_int), C.c_int, C.c_in
                                          C.POINTER(Strides), _P, _P, _P]
 _lib.heatkv_split_plan.argtypes = [C.POINTER(C.c_int32), C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_uint64, C.c_uint64,
                                    C.POINTER(C.c_int32), C.POINTER(C.c_double), C.POINTER(C.c_double)]
-_lib.heatkv_lone_plan.argtypes = [C.POINTER(C.c_int32), C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_uint64, C.c_uint64,
+_lib.heatkv_lone_plan.argtypes = [C.POINTER(C.c_int32), C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_uint64, C.c_uint64,
                                   C.POINTER(C.c_int32), C.POINTER(C.c_int32), C.POINTER(C.c_int32)]
 _lib.heatkv_attention_split.argtypes = [_P, C.POINTER(C.c_int), C.c_int, C.c_int, C.c_int, C.POINTER(C.c_int32),
                                         C.POINTER(C.c_int32)]
@@ -361,13 +361,13 @@ def heatkv_split_plan(tiles, n_qp: int, n_seq: int, n_sm: int = 148, per_head: b
     return [int(x) for x in out], a.value, b.value
 
 
-def heatkv_lone_plan(tiles, t_q: int, n_seq: int, n_sm: int = 148, per_head: bool = True,
+def heatkv_lone_plan(tiles, t_q: int, n_seq: int, n_sm: int = 148, d: int = 128, per_head: bool = True,
                      max_slots: int = 1 << 40, max_ctrs: int = 1 << 40):
     """(pieces per head, heads whose query tiles go one by one, does the launch take query tiles by themselves instead of cuts)."""
     n = len(tiles)
     t = (C.c_int32 * n)(*[int(x) for x in tiles])
     pieces, singles, lone = (C.c_int32 * n)(), (C.c_int32 * n)(), C.c_int32()
-    _check(_lib.heatkv_lone_plan(t, n, t_q, n_seq, n_sm, int(per_head), max_slots, max_ctrs, pieces, singles, C.byref(lone)),
+    _check(_lib.heatkv_lone_plan(t, n, t_q, n_seq, n_sm, d, int(per_head), max_slots, max_ctrs, pieces, singles, C.byref(lone)),
            "heatkv_lone_plan")
     return [int(x) for x in pieces], [bool(x) for x in singles], bool(lone.value)
 

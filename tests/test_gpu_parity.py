@@ -492,7 +492,8 @@ def test_mixed_schedules_choose_one_form_in_any_order(hk, d, order):
     pairs whichever comes first."""
     from paper_2605_14877_b200.sweep import Session
     H, t = 24, [512, 1024]
-    assert hk.heatkv_lone_plan([12] * H, t[1], 2, per_head=False)[2] and not hk.heatkv_lone_plan([8] * H, t[1], 2, per_head=False)[2]
+    assert hk.heatkv_lone_plan([12] * H, t[1], 2, d=d, per_head=False)[2]
+    assert not hk.heatkv_lone_plan([8] * H, t[1], 2, d=d, per_head=False)[2]
     gen = torch.Generator(device="cuda").manual_seed(d)
     q, k, v = (torch.randn(2, H, sum(t), d, generator=gen, device="cuda").mul_(f).bfloat16() for f in (1, 1, 0.25))
     out = torch.zeros_like(q)

@@ -396,7 +396,8 @@ def _finish(items, n_sm):
 
 @pytest.mark.parametrize("t_q", [1, 128, 129, 256, 257, 576, 1024, 1600])
 @pytest.mark.parametrize("per_head", [True, False])
-def test_lone_plan_follows_its_estimates(t_q, per_head):
+@pytest.mark.parametrize("d", [128, 64])
+def test_lone_plan_follows_its_estimates(t_q, per_head, d):
     """Pairs of query tiles and lone ones against a simulation of single SMs: a lone launch beats the estimate of the cut by what it has to, and
     where the cut runs, neither all query tiles one by one nor only the odd last ones would have."""
     import paper_2605_14877_b200 as hk
@@ -407,7 +408,7 @@ def test_lone_plan_follows_its_estimates(t_q, per_head):
     for _ in range(25):
         H, n_seq = int(rng.integers(1, 20)), int(rng.integers(1, 5))
         tiles = sorted((int(x) for x in rng.choice([4, 8, 12, 19, 34], size=H)), reverse=True)
-        pieces, singles, lone = hk.heatkv_lone_plan(tiles, t_q, n_seq, per_head=per_head)
+        pieces, singles, lone = hk.heatkv_lone_plan(tiles, t_q, n_seq, d=d, per_head=per_head)
         assert pieces == hk.heatkv_split_plan(tiles, n_qp, n_seq, per_head=per_head)[0]
         _pieces_valid(tiles, pieces)
         assert lone or not any(singles)
@@ -427,7 +428,7 @@ def test_lone_plan_follows_its_estimates(t_q, per_head):
             for pc in range(k):
                 size, fixed = min(n, (pc + 1) * full) - pc * full, 2 + (1 + 1.5 * (k - 1) / k if k > 1 else 0.0)
                 cut += [(size + fixed, (n_qp - odd) * n_seq), (0.81 * size + fixed, odd * n_seq)]
-        bar = 0.98 * (_finish(cut, 148) + 3.0 * (max(pieces) > 1)) - 0.8
+        bar = 0.98 * (_finish(cut, 148) + (3.0 if d == 128 else 1.7) * (max(pieces) > 1)) - 0.8
         if lone:
             taken += 1
             assert lone_estimate(singles) < bar + 1e-9
@@ -439,9 +440,9 @@ def test_lone_plan_follows_its_estimates(t_q, per_head):
 
 def test_lone_plan_rejects_bad_input():
     import paper_2605_14877_b200 as hk
-    for tiles, t_q in (([3, 5], 300), ([4, 0], 300), ([4, 4], 0)):
+    for tiles, t_q, d in (([3, 5], 300, 128), ([4, 0], 300, 128), ([4, 4], 0, 64), ([4, 4], 300, 96)):
         with pytest.raises(hk.HeatKVError):
-            hk.heatkv_lone_plan(tiles, t_q, n_seq=1)
+            hk.heatkv_lone_plan(tiles, t_q, n_seq=1, d=d)
 
 
 def test_choosing_a_launch_form_simulates_few_candidates():
