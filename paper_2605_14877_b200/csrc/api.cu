@@ -846,6 +846,7 @@ static int attention_impl(heatkv_ctx* ctx, const int* seq_ids, int n_seq, int la
     // (fp8 cache: a step that does not ride along goes through heatkv_append_compact below, which takes the
     // sequences' pool rows from the context, not from p)
   }
+  p.carries_update = with_update;
   if (fuse) p.append_tiles = (ctx->cfg.t[step] + HEATKV_PAGE_TOKENS - 1) / HEATKV_PAGE_TOKENS + 1;
   cudaError_t e;
   int32_t longest = 0;

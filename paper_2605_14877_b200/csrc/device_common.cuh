@@ -84,6 +84,7 @@ struct AttnParams {
   int32_t runs;                   // no per-scale bias: the plan's merged attention tables (PlanView)
   int32_t lone;                   // tensor-memory kernel: items may be one query tile (1), without a head table all are (2), and
                                   // nothing is cut (split_tiles: the longest run there would be otherwise)
+  int32_t carries_update;         // a heatkv_attention_append call (the launch before it on the stream is attention, too)
   int32_t full_whole;             // calibration with output: work items before this one hold a pair of query tiles, later ones one
 };
 
