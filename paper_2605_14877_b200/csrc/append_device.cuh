@@ -11,6 +11,8 @@ namespace heatkv {
 
 // What half-tile `j` of a head's update is, from the plan alone: `n` rows (0: the head does not store it), the first of them token
 // `tok0` of the step, to pool rows `row` and up.  `u` = (step * L + layer) * H + head; `base_row` is the sequence's first row.
+// Count and place are fetched together: a load behind the test of the count is one more round trip in the stand-alone updates, which have
+// nothing to hide it behind (14 sequences x 3 heads, fp8, 3 layers x 8 steps: 283.8 against 280.5 us a pass; 4 x 2 heads 288.4 and 284.9).
 struct AppendPlace {
   int n, tok0;
   int64_t row;
@@ -18,8 +20,9 @@ struct AppendPlace {
 __device__ __forceinline__ AppendPlace append_place(const int32_t* plan, int64_t base_row, int u, int j) {
   PlanView pv(plan);
   AppendPlace a = {0, 0, 0};
-  if (j >= pv.app_cnt()[u]) return a;
-  const int2* descs = pv.descs() + pv.app_begin()[u];
+  const int cnt = pv.app_cnt()[u], begin = pv.app_begin()[u];        // both on their way at once
+  if (j >= cnt) return a;
+  const int2* descs = pv.descs() + begin;
   for (int i = 0; i < j; ++i) a.tok0 += descs[i].y & 0xff;
   const int2 dsc = descs[j];
   a.n = dsc.y & 0xff;
