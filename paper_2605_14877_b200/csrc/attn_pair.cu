@@ -32,7 +32,7 @@ using namespace tc;
 
 constexpr int THREADS = 384;
 constexpr int STAGES = 4;               // of K and of V
-// What ptxas assigns under __launch_bounds__(384, 1), for either head size; 44 bytes a thread spilled (11 stores, 32 loads), in all
+// What ptxas assigns under __launch_bounds__(384, 1), for either head size; 44 bytes a thread spilled (11 stores, 36 loads), in all
 // roles together.
 constexpr int REGS_LAUNCH = 168;
 constexpr int REGS_SMALL = 72, REGS_SOFTMAX = 216;

@@ -500,7 +500,7 @@ attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ Map
     // one lane instead of branched around.  Measured: a pair generated at 20x 2.395 -> 2.339 ms of GPU time, the largest
     // model's batch 7.025 -> 6.763 ms, 64-wide heads unchanged (1.66 ms); one thread running the whole role lost 5 %.  The lane is
     // elected anew for every tile and the descriptors are a base and a constant: 65 instructions less per tile, 1024 queries x 296
-    // heads x 24 tiles 369.4 -> 363.5 us (64-wide heads 306.7 -> 302.7).  What matters is that the compiler knows the warp to be
+    // heads x 24 tiles 369.4 -> 363.5 us in a burst (64-wide heads 306.7 -> 302.7), 449.0 -> 446.4 under the power limit.  What matters is that the compiler knows the warp to be
     // converged: where it does not (a `continue` past the __syncwarp at the loop's end, a lane mask that a failed wait may clear) it
     // branches around every product, 33 branches and 350 instructions more per tile, and the kernel is 6 % slower.
     const uint32_t lead = elect_one();
