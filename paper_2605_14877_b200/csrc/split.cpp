@@ -238,9 +238,9 @@ void single_search(const std::vector<int>& tiles, int t_q, int n_seq, int n_sm, 
     const Load &mid0 = pairs[first], &mid1 = pairs[H - last], &end0 = singles[H - last], &end1 = singles[H];
     sum.total += mid1.total - mid0.total + end1.total - end0.total;
     sum.items += mid1.items - mid0.items + end1.items - end0.items;
-    // (heads by descending tiles: the first of each kind is the longest)
-    if (first < H - last) sum.longest = std::max(sum.longest, n_qp > odd ? tiles[first] + FIXED : TILE_SINGLE * tiles[first] + FIXED);
-    if (last > 0) sum.longest = std::max(sum.longest, TILE_SINGLE * tiles[H - last] + FIXED);
+    // (the plan's order is by tokens: among heads of nearly as many a later one may have a tile more)
+    for (int i = first; i < H; ++i)
+      sum.longest = std::max(sum.longest, (i < H - last && n_qp > odd ? 1.0 : TILE_SINGLE) * tiles[i] + FIXED);
     const double t = launch.estimate(sum, take, [&] {
       for (int i = 0; i < H; ++i) {
         if (i < first || i >= H - last) {
